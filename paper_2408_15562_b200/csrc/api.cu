@@ -102,7 +102,7 @@ int fspad_create(const fspad_config *cfg, fspad_ctx **out)
         ok = ok && dev_alloc(&dx, B * FSPAD_MAX_FRONTIER * (size_t)fspad_draft_expand_pieces(cfg->vocab) * FSPAD_MAX_FRONTIER);
         ctx->dx_part = dx;
     }
-    ok = ok && dev_alloc(&ctx->lm_parts, (size_t)128 * fspad_lm_head_tiles(cfg->vocab));
+    ok = ok && dev_alloc(&ctx->lm_parts, (rows < FSPAD_LM_SLAB_ROWS ? rows : (size_t)FSPAD_LM_SLAB_ROWS) * fspad_lm_head_tiles(cfg->vocab));
     ok = ok && cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) == cudaSuccess;

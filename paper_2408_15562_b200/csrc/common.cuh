@@ -14,6 +14,7 @@
 #define FSPAD_MAX_FRONTIER 16      /* frontier nodes per sequence, and top-k per row, of a draft step */
 #define FSPAD_HEAD_DIM 128
 #define FSPAD_STATS_THREADS 256
+#define FSPAD_LM_SLAB_ROWS 1024    /* rows of one launch of the LM-head product (more rows: several launches) */
 
 // Scratch and bookkeeping owned by a context (all device pointers unless noted).
 struct fspad_ctx {
@@ -49,7 +50,7 @@ struct fspad_ctx {
     cudaStream_t side;
     cudaEvent_t ev_fork, ev_join;
 
-    // LM head: per-(row, vocabulary tile) partials of one slab of 128 rows, [128][tiles]
+    // LM head: per-(row, vocabulary tile) partials of one slab of rows, [min(max rows, slab)][tiles]
     struct FspadStatsPart *lm_parts;
     int lm_attr_done;
     int fs_attr_done;         // dynamic shared-memory limit raised for the Feature Sampler's product kernel

@@ -60,6 +60,19 @@ def test_stats_small_shapes_ragged_tiles(rows, H, V):
     assert _stats_case(2, rows, H, V, rps, temps, False) <= 1
 
 
+@pytest.mark.parametrize("rows,H,V", [(32, 72, 257), (33, 64, 128), (129, 128, 1025), (256, 200, 513), (257, 64, 38000),
+                                      (300, 64, 777), (544, 72, 641), (1024, 64, 256), (1057, 64, 300)])
+def test_stats_row_tiles(rows, H, V):
+    """Row counts around the 32-row units, the 256-row tiles (equal and unequal ones) and the 1024-row slab; vocabularies
+    with an odd number of tiles, no multiple of four, and more items than pairs of SMs."""
+    temps = [(1.0, 0.7, 0.0, 1.3)[i % 4] for i in range((rows + 31) // 32)]
+    # close calls: the gap of the two largest of V values from N(0, 9) is about exponential with mean
+    # 3 / sqrt(2 ln V) >= 0.65, so a row's lies below 2 LOGIT_TOL with probability about 0.003 (mean 3.3 at 1057 rows)
+    limit = 4 + rows // 100
+    assert _stats_case(rows, rows, H, V, 32, temps, True) <= limit
+    assert _stats_case(rows + 1, rows, H, V, 32, temps, False) <= limit
+
+
 def test_stats_more_rows_than_one_slab():
     assert _stats_case(3, 300, 128, 2000, 60, [1.0, 0.5, 1.0, 2.0, 1.0], True) <= 2
 
