@@ -102,7 +102,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
     __shared__ unsigned long long s_anc[NW == 1 ? FSPAD_MAX_NODES : 1];
 
     fspad_pdl_wait();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     const bool producer = warp >= 8;         // warp 8 copies, warp 9 drives the tensor cores
     const int row = tid & (BM - 1), grp = (tid >> 7) & 1;
     const int split = blockIdx.x;
@@ -306,9 +306,12 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         }
         if (failed) s_fail = 1;
     } else if (warp == 9) {
-        // ================= tensor-core warp: one thread issues every tcgen05.mma =================
-        if (lane == 0) {
-            const uint32_t elect = 1;             // the whole loop is this one thread's
+        // ================= tensor-core warp: the whole warp runs the loop, one lane issues every tcgen05.mma =================
+        // (one lane's branch kept every operand in ordinary registers: 17.4 against 19.0 us per call at 4 heads per KV head
+        // and 2 K keys, 35.8 against 37.8 at 8 and 8 K, 99.3 against 101.4 on the ragged batch of 16)
+        {
+            const bool issuer = elect_one();
+            const uint32_t elect = 1;             // the instructions stand in the issuer's branch
             // low words of the shared-memory descriptors (start address and leading byte offset);
             // the high word (8-row group stride, version, swizzle mode) is the same for all
             const uint32_t hi = (uint32_t)(make_desc(0, 16) >> 32);
@@ -319,8 +322,8 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             // S(c) = Q K(c)^T into score buffer c & 1 (columns 0..63 of it belong to group 0, 64..127 to
             // group 1); K(c) sits in ring slot kbuf, which the second commit releases
             auto issue_s = [&](int c) {
-                if (!failed && !mbar_wait_thread(kfull(kbuf), kph)) failed = true;
-                if (!failed) {
+                if (!failed && !mbar_wait_warp(kfull(kbuf), kph)) failed = true;
+                if (!failed && issuer) {
                     // no tcgen05 fence here: the K chunk comes through the barrier's own acquire, and the
                     // score buffer's last readers and writers (softmax of chunk c - 2) were ordered before this
                     // thread's instructions by the fence behind its pfull wait of that chunk
@@ -334,6 +337,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                     mma_commit_if(sfull(c & 1), elect);
                     mma_commit_if(kfree(kbuf), elect);
                 }
+                __syncwarp();
                 if (++kbuf == NS) { kbuf = 0; kph ^= 1u; }
             };
             issue_s(0);
@@ -346,9 +350,9 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                 for (int g2 = 0; g2 < 2; ++g2) {
                     // O[g2] += P_g2(c) V(c)[64 g2 .. 64 g2 + 63]: P from the four warps of group g2 (in tensor
                     // memory, over the scores it was computed from) and the V chunk
-                    if (g2 == 0 && !failed && !mbar_wait_thread(pfull(p), ph)) failed = true;
-                    if (g2 == 0 && !failed && !mbar_wait_thread(vfull(vbuf), vph)) failed = true;
-                    if (!failed) {
+                    if (g2 == 0 && !failed && !mbar_wait_warp(pfull(p), ph)) failed = true;
+                    if (g2 == 0 && !failed && !mbar_wait_warp(vfull(vbuf), vph)) failed = true;
+                    if (!failed && issuer) {
                         if (g2 == 0) tc_fence_after();
                         const uint32_t a_t = tmem + (uint32_t)p * 128u + (uint32_t)g2 * 64u;
 #pragma unroll
@@ -360,6 +364,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                         mma_commit_if(odone(g2, p), elect);
                         if (g2 == 1) mma_commit_if(vfree(vbuf), elect);
                     }
+                    __syncwarp();
                 }
                 // tensor-core work completes in issue order, so the scores of chunk c + 2 may replace P(c)
                 if (c + 2 < n_ch) issue_s(c + 2);
