@@ -15,7 +15,8 @@
 // and the CTAs exchanging partial sums through distributed shared memory.
 // Only rows on the realised path are ever read.  The first sweep at a node
 // evaluates exp((x - max)/T) in fp64 once per token and parks the values (and
-// the draft row) in shared memory, so later sweeps at that node are cheap.
+// the draft row) in shared memory, from where each thread takes its share into
+// registers for the sweeps that follow at that node.
 //
 // The residual after k rejections at a node is kept in closed form instead of
 // as a vector: for a token j that has not been rejected,
@@ -31,6 +32,14 @@
 // of exponentials is fp32-accurate and is trusted only when a decision clears
 // a 1e-4 relative margin, otherwise (and before any residual) the exact sum is
 // swept here.
+//
+// What bounds it is latency: a chain of sweeps, exchanges and scalar decisions on
+// 16 SMs, and the fetching of its own instructions, which each launch does anew (at
+// 149 KB of code a third of the warps' active time went into waiting for them; rare
+// paths are therefore single, non-inlined copies, loops are not unrolled unless
+// they are the hot ones).  Measured on a 128256-token row: a rejection after a
+// node's first 5.3 -> 2.0 us (sweep 2.0 -> 0.8, exchange 2.4 -> 0.7, decision 0.9 ->
+// 0.5), the walk of a 60-node sampling step with eight rejections 53 -> 29 us.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -40,16 +49,19 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kMaxCluster = 16;
-constexpr int kWalkThreads = 1024;
+constexpr int kWalkThreads = 512;          // 128 registers each: a thread keeps 16 tokens of the node's rows in them
 constexpr int kWarps = kWalkThreads / 32;
+constexpr int kTile = 16;                  // tokens of a thread's chunk that later residual sweeps take from registers
 constexpr int kSmemBudget = 200 * 1024;   // dynamic shared memory for the per-node cache
-constexpr int kSmemBudgetWide = 188 * 1024;   // the same for the instance with room for 256 nodes (its static part is larger)
+constexpr int kSmemBudgetWide = 176 * 1024;   // the same for the instance with room for 256 nodes (its static part is larger)
 constexpr double kAmbiguous = 1e-4;
 constexpr double kScanRel = 1e-6;          // bound taken for the relative error of the scan's sum of exponentials
 constexpr double kFusedTol = 1e-9;         // relative error the fused first-rejection sweep may leave in the residual mass
+constexpr double k256OverLn2 = 369.3299304675746;   // steps of the exponential's table per unit of its argument
 constexpr float kLog2eF = 1.4426950408889634f;
 constexpr int kPieceSlots = 16;            // pieces of a row whose scan sums are kept for the bonus draw
-enum { REQ_DONE = 0, REQ_EXP = 1, REQ_EXP_Q = 2, REQ_FUSED = 3, REQ_RESID = 4 };
+constexpr int kExpTable = 256;             // entries of the exponential's table
+enum { REQ_DONE = 0, REQ_EXP = 1, REQ_FUSED = 2, REQ_RESID = 3 };
 
 // 2^(i/64), i = 0..63, correctly rounded
 __constant__ double kExp2Tbl[64] = {
@@ -85,276 +97,476 @@ struct WalkArgs {
     int kv_layers, kv_B, kv_H, kv_max_len;
 };
 
-// A set of tree nodes as a bit mask of W 64-bit words (W = 1: trees of up to 64 nodes, the common case;
-// W = 4: up to 256).
-template <int W> struct NodeSet {
-    unsigned long long w[W];
-    __device__ __forceinline__ bool any() const
-    {
-        unsigned long long o = 0ull;
-#pragma unroll
-        for (int i = 0; i < W; ++i) o |= w[i];
-        return o != 0ull;
-    }
-    __device__ __forceinline__ int first() const          // lowest member (the set is not empty)
-    {
-#pragma unroll
-        for (int i = 0; i < W; ++i)
-            if (w[i]) return i * 64 + __ffsll((long long)w[i]) - 1;
-        return -1;
-    }
-    __device__ __forceinline__ void drop_first()
-    {
-#pragma unroll
-        for (int i = 0; i < W; ++i)
-            if (w[i]) { w[i] &= w[i] - 1; return; }
-    }
-    __device__ __forceinline__ bool single() const        // exactly one member
-    {
-        NodeSet t = *this;
-        t.drop_first();
-        return any() && !t.any();
-    }
+// The walk's state at the current node; thread 0's own, in shared memory while the CTA sweeps.  Weights and masses of
+// the target's side are kept times the softmax denominator S.
+struct WalkState {
+    double S, C, U, D, invD, F;     // denominator, coefficient of the draft row, residual mass, draft mass and its
+                                    // inverse, sum of the weights that rejected tokens keep
+    double Cp;                      // coefficient of the rejection under way
+    int cur, nrem, len, ch, ridx;   // ch: child under test (0: none left); ridx: its token's place in the list of rejected ones, or -1
+    int exact, parked;              // S is exact; e and q of the node's rows are parked (first rejection done)
+};
+// What the test of a child needs.
+struct Child {
+    int ch, next, tok, dup;         // next: the sibling after it (0: none)
+    double ex, qx, rq;              // exponential and draft probability of its token, uniform times the latter
 };
 
 // MAXN: capacity in tree nodes of this instance of the kernel (64 or FSPAD_MAX_NODES_WIDE)
-template <int MAXN> struct SharedT {
-    static constexpr int W = MAXN / 64;
-    static constexpr int kPieceRows = (MAXN == 64) ? 64 : 1;   // the per-piece masses are kept only by the 64-node instance
-    double exp_tbl[64];             // 2^(i/64)
+template <int MAXN> struct TreeShared {
     int parent[MAXN];
     int tok[MAXN];
     int path[MAXN];
-    // state of the current node (written by thread 0, read by all after a barrier)
-    double S, invS, c, U, D, m, invT;
-    NodeSet<W> child_mask[MAXN];    // c in child_mask[i] iff parent[c] == i
-    int exact, nrem, decision, xnew, ridx, next, len, cur, have_e, have_q, sel;
-    double cprime, ex, qx;
-    int rem_tok[MAXN];
+    int rowA[MAXN];                 // argmax of every row
+    int next[MAXN];                 // greedy: the child that carries it, MAXN if none
+    int len;
+    int kv_L;                       // prefix length (where the walk compacts the cache)
+};
+template <int MAXN> struct SharedT {
+    TreeShared<MAXN> t;
+    double exp_tbl[kExpTable];      // 2^(i/256)
+    // what thread 0 asks for and about which node (written by thread 0, read by all after a barrier)
+    double S, C;                    // sum of exponentials in use, coefficient of the draft row
+    double S_exact;                 // what the first rejection's sweep found
+    WalkState state;
+    int req, cur, xnew, parked;
+    int nrem, sel;
+    int rem_tok[MAXN];              // tokens rejected at the current node and the weights they keep
     double rem_frozen[MAXN];
+    double node_D[MAXN], node_invD[MAXN];   // draft mass left once node c and its earlier siblings are rejected, its inverse
     // gathered once, in parallel, before the walk: the scan result of every row and, for
-    // every node, its parent's logit and draft probability at the node's token and its uniform
+    // every node, its draft probability in its parent's row and its uniform
     float rowM[MAXN];
     double rowS[MAXN];
-    double rowInvS[MAXN];   // 1 / rowS, so that no division sits on the serial path
-    int rowA[MAXN];
-    float cx[MAXN], cq[MAXN], cu[MAXN];
-    double cex[MAXN];    // exp((logit - row max)/T) of each node's token in its parent's row
+    float cq[MAXN], cu[MAXN];
+    double cex[MAXN];               // exp((logit - row max)/T) of each node's token in its parent's row
+    double later_q[MAXN];           // draft mass of the tokens that only siblings after node c carry
+    int first_child[MAXN], next_sib[MAXN];   // 0: none
+    unsigned char dup[MAXN];        // an earlier sibling carries the same token
     float ubonus;
-    int want_q;
     int bonus_ok;                   // the last residual sweep already holds the bonus draw's per-thread sums
-    // reductions
-    double warp_a[kWarps], warp_b[kWarps], warp_off[kWarps];
-    double slot[2][kMaxCluster][2]; // partial sums received from every CTA of the cluster, by pass parity
-    double tot[2];                  // cluster totals
-    double warp5[kWarps][5], slot5[2][kMaxCluster][5], tot5[5];   // the same exchange for five values
-    int fused_fallback;
-    double cta_total[2][kMaxCluster];  // bonus draw: every CTA's total, received from the peers (by attempt)
-    int verdict[2];                    // bonus draw from one piece of the row: 1 = settled, 2 = the whole row must be swept
-    // serial walk -> sweeps: what thread 0 asks the CTA to do next
-    int req, req_child, req_last;
-    NodeSet<W> rem;                    // children of the current node not tested yet
+    int fail;
+    // reductions: warp totals, totals received from every CTA of the cluster (by exchange parity), their barriers
+    double warp_v[4][kWarps], warp_off[kWarps], warp_total;
+    double slot[2][4][kMaxCluster];
+    unsigned long long bar[2];
+    int verdict;                    // bonus draw from one piece of the row: 1 = settled, 2 = the whole row must be swept
     // approximate mass of every (row, CTA) piece of the vocabulary scan, relative to the row maximum;
     // piece_cnt[row] = 0 when the row has more than kPieceSlots pieces (the draw then sweeps the whole row)
-    double piece_w[kPieceRows][kPieceSlots];
-    int piece_cnt[kPieceRows];
+    float piece_w[MAXN][kPieceSlots];
+    int piece_cnt[MAXN];
 };
 
-// exp(a) for a <= 0 in double precision: a = (64 n + i) ln2/64 + r, |r| <= ln2/128,
-// exp(a) = 2^n * 2^(i/64) * (1 + r + r^2/2 + r^3/6 + r^4/24); relative error below 5e-14
-// (truncation r^5/120 < 4e-14, one-step argument reduction < 3e-14 at the far end of the range).
-// Every operation is an fp64 multiply-add: the rounding to the nearest integer is done by adding
-// and subtracting 1.5 * 2^52 (the integer then sits in the low word of the sum), because the
-// conversions between integers and doubles cost as much as an fp64 operation each.
-__device__ __forceinline__ double exp_neg(double a, const double *tbl)
+// ---- where the scan's partial results of a row are ----
+// first CTA and number of CTAs that share row `row` (rows not cut evenly)
+__device__ __noinline__ int flat_first(const FspadStatsGeom &g, int row, int *cnt)
 {
-    if (!(a > -700.0)) return 0.0;                        // also -inf and NaN
-    const double magic = 6755399441055744.0;              // 1.5 * 2^52
-    const double tm = fma(a, 92.33248261689366, magic);   // a * 64 / ln 2, rounded to an integer
-    const int k = __double2loint(tm);
-    const double kd = tm - magic;
-    const double r = fma(-kd, 0.010830424696249145, a);   // ln2/64
-    double p = fma(r, 1.0 / 24.0, 1.0 / 6.0);
-    p = fma(p, r, 0.5);
-    p = fma(p, r, 1.0);
-    p = fma(p, r, 1.0);
-    const double y = tbl[k & 63] * p;
-    const int n = k >> 6;                                  // floor(k / 64), n in [-1010, 0]
-    return __hiloint2double(__double2hiint(y) + (n << 20), __double2loint(y));
+    const long long r0 = (long long)row * g.upr;
+    if (g.total <= 0xffffffffll) {
+        const unsigned ch = (unsigned)g.chunk, f = (unsigned)r0 / ch;
+        *cnt = (int)(((unsigned)r0 + (unsigned)g.upr - 1u) / ch - f) + 1;
+        return (int)f;
+    }
+    const long long first = r0 / g.chunk, last = (r0 + g.upr - 1) / g.chunk;
+    *cnt = (int)(last - first) + 1;
+    return (int)first;
+}
+__device__ __forceinline__ int row_pieces(const FspadStatsGeom &g, int row)
+{
+    if (g.per_row > 0) return g.per_row;
+    int cnt;
+    flat_first(g, row, &cnt);
+    return cnt;
+}
+// tokens [lo, hi) of piece `pick` of row `row`
+__device__ __noinline__ void piece_bounds(const FspadStatsGeom &g, int row, int pick, int V, int *lo, int *hi)
+{
+    long long u_lo = pick * g.chunk, u_hi = u_lo + g.chunk;
+    if (g.per_row == 0) {
+        int cnt;
+        const long long first = flat_first(g, row, &cnt), row_lo = (long long)row * g.upr;
+        u_lo = max(0ll, (first + pick) * g.chunk - row_lo);
+        u_hi = (first + pick + 1) * g.chunk - row_lo;
+    }
+    *lo = (int)u_lo * g.unit;
+    *hi = (int)min((long long)V, u_hi * g.unit);
 }
 
-__device__ __forceinline__ double warp_sum(double v)
+// The scan's partials of one row, merged by eight lanes (slots lane, lane + 8 at once; any further ones in a loop).
+// The whole warp calls it; `valid` is false for lanes without a row.  piece_w (may be NULL): mass of each piece relative
+// to the row's maximum.
+__device__ __forceinline__ void merge_row(const FspadStatsPart *__restrict__ parts, const FspadStatsGeom &g, int row, bool valid,
+                                          float k, int l8, float &M, double &S, int &A, float *piece_w, int *piece_cnt)
 {
+    const int cnt = valid ? row_pieces(g, row) : 0;
+    const FspadStatsPart *p = parts + (size_t)(valid ? row : 0) * g.slots;
+    float m0 = -INFINITY, s0 = 0.f, m1 = -INFINITY, s1 = 0.f;
+    int a0 = 0x7fffffff, a1 = 0x7fffffff;
+    if (l8 < cnt) {
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(p + l8));
+        m0 = __int_as_float(v.x); s0 = __int_as_float(v.y); a0 = v.z;
+    }
+    if (l8 + 8 < cnt) {
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(p + l8 + 8));
+        m1 = __int_as_float(v.x); s1 = __int_as_float(v.y); a1 = v.z;
+    }
+    float m = m0;
+    int a = a0;
+    if (m1 > m || (m1 == m && a1 < a)) { m = m1; a = a1; }
+#pragma unroll 1
+    for (int sl = l8 + 16; sl < cnt; sl += 8) {
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(p + sl));
+        if (__int_as_float(v.x) > m || (__int_as_float(v.x) == m && v.z < a)) { m = __int_as_float(v.x); a = v.z; }
+    }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
+    for (int off = 4; off > 0; off >>= 1) {
+        const float om = __shfl_xor_sync(0xffffffffu, m, off);
+        const int oa = __shfl_xor_sync(0xffffffffu, a, off);
+        if (om > m || (om == m && oa < a)) { m = om; a = oa; }
+    }
+    const float w0 = (m0 != -INFINITY) ? s0 * exp2f((m0 - m) * k) : 0.f;
+    const float w1 = (m1 != -INFINITY) ? s1 * exp2f((m1 - m) * k) : 0.f;
+    if (piece_w != nullptr && valid) {
+        piece_w[l8] = w0;
+        piece_w[l8 + 8] = w1;
+        if (l8 == 0) *piece_cnt = (cnt <= kPieceSlots) ? cnt : 0;
+    }
+    double s = (double)w0 + (double)w1;
+#pragma unroll 1
+    for (int sl = l8 + 16; sl < cnt; sl += 8) {
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(p + sl));
+        if (__int_as_float(v.x) != -INFINITY) s += (double)(__int_as_float(v.y) * exp2f((__int_as_float(v.x) - m) * k));
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    M = m;
+    S = s;
+    A = (a == 0x7fffffff) ? 0 : a;
 }
 
-__device__ __forceinline__ double weight(double e, double q, double invS, double c)
+// exp((x - m) / T) for x <= m in double precision, by table and polynomial (the scheme of Tang's 1989 paper): with
+// t = (x - m) 256 / (T ln 2) = 256 n + i + f, |f| <= 1/2, the value is 2^n 2^(i/256) exp(f ln2/256).  The exponential
+// of the remainder is a cubic: its Taylor series with the fourth-order term economised into the constant and the
+// square (error below 1.8e-14).  The caller hands over s = 256 / (T ln 2) and off = -m s.  The rounding to the nearest
+// integer is done by adding and subtracting 1.5 * 2^52 (the integer then sits in the low word of the sum): conversions
+// run at a quarter of the fp64 rate (16 against 63 per clock and SM).  Values below e^-700 are taken as zero.
+struct ExpArg {
+    double s, off;
+    float x_min;
+};
+__device__ __forceinline__ ExpArg exp_arg(float m, double invT, float T)
 {
-    const double w = e * invS - c * q;
+    const double s = invT * k256OverLn2;
+    return ExpArg{s, -(double)m * s, m - 700.0f * T};
+}
+__device__ __forceinline__ double exp_neg(float x, const ExpArg &g, const double *tbl)
+{
+    const double magic = 6755399441055744.0;              // 1.5 * 2^52
+    const double t = fma((double)x, g.s, g.off);
+    const double tm = t + magic;
+    const double f = t - (tm - magic);
+    const int k = __double2loint(tm);
+    double p = fma(f, 3.3083026805413713e-09, 3.665566156758904e-06);
+    p = fma(p, f, 0.0027076061740622863);
+    p = fma(p, f, 0.9999999999999825);
+    const double y = tbl[k & (kExpTable - 1)] * p;
+    const double e = __hiloint2double(__double2hiint(y) + ((k >> 8) << 20), __double2loint(y));
+    return x > g.x_min ? e : 0.0;                          // also -inf and NaN
+}
+
+__device__ __forceinline__ double pair_of(float hi, float lo) { return __hiloint2double(__float_as_int(hi), __float_as_int(lo)); }
+
+// All weights are kept times the softmax denominator S: w = max(e - C q, 0) with e = exp((x - m)/T) and C = c S.
+__device__ __forceinline__ double weight(double e, double q, double C)
+{
+    const double w = fma(-C, q, e);
     return w > 0.0 ? w : 0.0;
+}
+
+// ---- how a row is shared out ----
+// Every CTA of the cluster takes a contiguous stretch, every thread of it per_thr positions, a multiple of four.  The
+// boundaries are multiples of 16 bytes from the array's start, whatever V is (both arrays start on one): positions before
+// the row's first token (at most three, of the first thread) and past its last one are empty.
+struct Chunk {
+    int lo, hi;                     // first position (may be -1 .. -3), end of the tokens
+};
+__device__ __forceinline__ Chunk chunk_of(size_t row_start, int V, int per_cta, int per_thr, int rank, int tid)
+{
+    const int ph = (int)(row_start & 3);
+    const int end = (rank + 1) * per_cta;
+    const int u = min(end, rank * per_cta + tid * per_thr);
+    return Chunk{u - ph, min(V, min(end, u + per_thr) - ph)};
+}
+// positions j .. j + 3 where some lie outside the row
+__device__ __noinline__ float4 edge4(const float *__restrict__ x, int j, int hi, float pad)
+{
+    float4 r = make_float4(pad, pad, pad, pad);
+    if (j >= 0 && j < hi) r.x = x[j];
+    if (j + 1 >= 0 && j + 1 < hi) r.y = x[j + 1];
+    if (j + 2 >= 0 && j + 2 < hi) r.z = x[j + 2];
+    if (j + 3 >= 0 && j + 3 < hi) r.w = x[j + 3];
+    return r;
+}
+__device__ __forceinline__ float4 load4(const float *__restrict__ x, int j, int hi, float pad)
+{
+    if (j >= 0 && j + 4 <= hi) return __ldg(reinterpret_cast<const float4 *>(x + j));
+    if (j + 4 <= 0 || j >= hi) return make_float4(pad, pad, pad, pad);
+    return edge4(x, j, hi, pad);
 }
 
 enum { MODE_EXP = 0, MODE_RESID = 1, MODE_CDF = 2 };
 
-struct Sweep {
-    double a, b;
-};
-
-// One sweep of this thread's contiguous chunk [lo, hi) of the vocabulary.
-//   MODE_EXP  : a = sum of e_j = exp((x_j - m)/T); e_j parked in shared memory
-//   MODE_RESID: a = sum of residual weights at coefficient c (tokens already
-//               rejected contribute their frozen value), b = sum of q over
-//               tokens neither rejected before nor equal to xnew
-//   MODE_CDF  : a = sum of the weights the bonus token is drawn from
-//               (nothing rejected at this node: the e_j themselves)
-// With `locate` the running sum starts at run0 and *found receives the first
-// token where base + run exceeds target (else the last positive-weight token).
-template <int MODE, class Shared>
-__device__ Sweep sweep_chunk(const Shared &sh, const float *__restrict__ x, const float *__restrict__ q,
-                             double *__restrict__ se, float *__restrict__ sq, int tid, int nthr, int lo, int hi,
-                             bool vec, bool cache_ok, bool have_e, bool have_q, double c, int xnew,
-                             bool locate, double base, double run0, double target, int *found)
+// The sweeps that are not on the usual path, over this thread's chunk, from the arrays in global memory or, with
+// `parked`, from the e_j and q_j the first rejection's sweep left in shared memory (one copy, not inlined).
+//   MODE_EXP  : sum of e_j
+//   MODE_RESID: sum of the weights at coefficient C over the tokens neither rejected before nor equal to xnew
+//               (rows that do not fit into shared memory)
+//   MODE_CDF  : sum of the weights the bonus token is drawn from (a rejected token's is the one it keeps)
+// With `found` the running sum starts at run and *found receives the first token where it exceeds target (else the
+// last positive-weight token).
+template <class Shared>
+__device__ __noinline__ double sweep_row(int mode, const Shared &sh, const float *__restrict__ x, const float *__restrict__ q,
+                                         const double *__restrict__ se, const float *__restrict__ sq, int stride, Chunk ck,
+                                         bool parked, const ExpArg &arg, double C, int xnew, double run, double target, int *found)
 {
-    const double m = sh.m, invT = sh.invT;
-    const int nrem = sh.nrem;
-    // bonus draw with nothing rejected at this node: the weights are the e_j themselves
-    const double invS = (MODE == MODE_CDF && c == 0.0 && nrem == 0) ? 1.0 : sh.invS;
-    // the exact-sum sweep that precedes a rejection also parks the draft row for the sweeps to come
-    const bool need_q = (MODE == MODE_RESID) || (MODE == MODE_CDF && c != 0.0) || (MODE == MODE_EXP && xnew == -2);
-    bool special = false;
-    if (MODE != MODE_EXP) {
-        for (int r = 0; r < nrem; ++r) special |= (sh.rem_tok[r] >= lo && sh.rem_tok[r] < hi);
-        if (MODE == MODE_RESID) special |= (xnew >= lo && xnew < hi);
-    }
-    double a = 0.0, b = 0.0, run = run0;
+    const int nrem = mode == MODE_EXP ? 0 : sh.nrem;
+    bool special = mode == MODE_RESID && xnew >= ck.lo && xnew < ck.hi;
+#pragma unroll 1
+    for (int r = 0; r < nrem; ++r) special |= (sh.rem_tok[r] >= ck.lo && sh.rem_tok[r] < ck.hi);
+    double a = 0.0;
     int last_pos = -1, hit = -1;
-    for (int j = lo; j < hi; j += 4) {
-        const int n = min(4, hi - j);
-        double ev[4];
-        float qv[4] = {0.f, 0.f, 0.f, 0.f};
-        if (have_e) {
-#pragma unroll
-            for (int t = 0; t < 4; ++t) ev[t] = (t < n) ? se[(j - lo + t) * nthr + tid] : 0.0;
-        } else {
-            float xv[4];
-            if (vec && n == 4) {
-                const float4 t4 = __ldg(reinterpret_cast<const float4 *>(x + j));
-                xv[0] = t4.x; xv[1] = t4.y; xv[2] = t4.z; xv[3] = t4.w;
-            } else {
-#pragma unroll
-                for (int t = 0; t < 4; ++t) xv[t] = (t < n) ? x[j + t] : -INFINITY;
-            }
+#pragma unroll 1
+    for (int j = ck.lo; j < ck.hi; j += 4) {
+        double ev[4], qv[4] = {0.0, 0.0, 0.0, 0.0};
+        if (parked) {
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                ev[t] = exp_neg(((double)xv[t] - m) * invT, sh.exp_tbl);
-                if (cache_ok && t < n) se[(j - lo + t) * nthr + tid] = ev[t];
+                ev[t] = se[(j - ck.lo + t) * stride];
+                qv[t] = (double)sq[(j - ck.lo + t) * stride];
             }
-        }
-        if (need_q) {
-            if (have_q) {
-#pragma unroll
-                for (int t = 0; t < 4; ++t) qv[t] = (t < n) ? sq[(j - lo + t) * nthr + tid] : 0.f;
-            } else {
-                if (vec && n == 4) {
-                    const float4 u4 = __ldg(reinterpret_cast<const float4 *>(q + j));
-                    qv[0] = u4.x; qv[1] = u4.y; qv[2] = u4.z; qv[3] = u4.w;
-                } else {
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) qv[t] = (t < n) ? q[j + t] : 0.f;
-                }
-                if (cache_ok) {
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) if (t < n) sq[(j - lo + t) * nthr + tid] = qv[t];
-                }
+        } else {
+            const float4 xs = load4(x, j, ck.hi, -INFINITY);
+            ev[0] = exp_neg(xs.x, arg, sh.exp_tbl); ev[1] = exp_neg(xs.y, arg, sh.exp_tbl);
+            ev[2] = exp_neg(xs.z, arg, sh.exp_tbl); ev[3] = exp_neg(xs.w, arg, sh.exp_tbl);
+            if (C != 0.0) {
+                const float4 qs = load4(q, j, ck.hi, 0.f);
+                qv[0] = (double)qs.x; qv[1] = (double)qs.y; qv[2] = (double)qs.z; qv[3] = (double)qs.w;
             }
         }
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            if (t >= n) break;
-            if (MODE == MODE_EXP) {
-                a += ev[t];
-                continue;
-            }
-            double w = weight(ev[t], (double)qv[t], invS, c);
-            bool q_counts = true;
+            double w = weight(ev[t], qv[t], C);
             if (special) {
-                const int id = j + t;
+#pragma unroll 1
                 for (int r = 0; r < nrem; ++r)
-                    if (sh.rem_tok[r] == id) { w = sh.rem_frozen[r]; q_counts = false; }
-                if (id == xnew) q_counts = false;
+                    if (sh.rem_tok[r] == j + t) w = mode == MODE_CDF ? sh.rem_frozen[r] : 0.0;
+                if (mode == MODE_RESID && j + t == xnew) w = 0.0;
             }
             a += w;
-            if (MODE == MODE_RESID) {
-                if (q_counts) b += (double)qv[t];
-            } else if (locate) {
-                run += w;
-                if (w > 0.0) last_pos = j + t;
-                if (hit < 0 && base + run > target) hit = j + t;
-            }
+            run += w;
+            if (w > 0.0) last_pos = j + t;
+            if (hit < 0 && w > 0.0 && run > target) hit = j + t;
         }
     }
-    if (locate) *found = (hit >= 0) ? hit : last_pos;
-    return Sweep{a, b};
+    if (found != nullptr) *found = (hit >= 0) ? hit : last_pos;
+    return a;
 }
 
-// The first rejection at a node, in one sweep instead of two.  The exact denominator S is not known
-// yet, but the residual sum_j max(e_j / S - c q_j, 0) is linear in 1 / S over a fixed set of positive
-// terms: with P = { j : e_j / S' - c q_j > 0 } taken at the scan's S' it equals (sum_P e_j) / S -
-// c sum_P q_j for every S that leaves P unchanged.  The sweep returns
-//   v[0] = sum e_j (= S)      v[1] = sum_P e_j      v[2] = sum_P q_j
-//   v[3] = sum of q_j over j != xnew (the next draft mass)
-//   v[4] = sum of e_j / S' over the tokens whose sign a relative error kScanRel of S' could flip;
-// a flipped token changes the result by at most kScanRel times its probability, so kScanRel * v[4]
-// bounds the error and the caller falls back to the two-sweep path when that is not negligible.
-// e_j and q_j are parked in shared memory as in the exact-sum sweep.
-struct Sweep5 {
-    double v[5];
-};
-template <class Shared>
-__device__ Sweep5 fused_reject_sweep(const Shared &sh, const float *__restrict__ x, const float *__restrict__ q,
-                                     double *__restrict__ se, float *__restrict__ sq, int tid, int nthr, int lo, int hi,
-                                     bool vec, bool cache_ok, double inv_s_scan, double c, int xnew)
+// The residual sweep over the values parked in shared memory (rows of more than kTile tokens a thread): sum of
+// max(e_j - C q_j, 0) over this thread's chunk without the tokens rejected so far, whose parked values are zero (as are
+// the empty positions).
+__device__ __noinline__ double parked_sweep(double *__restrict__ se, float *__restrict__ sq, int stride, Chunk ck, int per_thr,
+                                            double C, int xnew)
 {
-    const double m = sh.m, invT = sh.invT;
-    Sweep5 r{{0.0, 0.0, 0.0, 0.0, 0.0}};
-    for (int j = lo; j < hi; j += 4) {
-        const int n = min(4, hi - j);
-        float xv[4], qv[4];
-        if (vec && n == 4) {
-            const float4 t4 = __ldg(reinterpret_cast<const float4 *>(x + j));
-            const float4 u4 = __ldg(reinterpret_cast<const float4 *>(q + j));
-            xv[0] = t4.x; xv[1] = t4.y; xv[2] = t4.z; xv[3] = t4.w;
-            qv[0] = u4.x; qv[1] = u4.y; qv[2] = u4.z; qv[3] = u4.w;
-        } else {
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                xv[t] = (t < n) ? x[j + t] : -INFINITY;
-                qv[t] = (t < n) ? q[j + t] : 0.f;
-            }
-        }
+    if (xnew >= ck.lo && xnew < ck.hi) {
+        se[(xnew - ck.lo) * stride] = 0.0;
+        sq[(xnew - ck.lo) * stride] = 0.f;
+    }
+    double a[2] = {0.0, 0.0};
+#pragma unroll 1
+    for (int k = 0; k < per_thr; k += 4) {
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            if (t >= n) break;
-            const double e = exp_neg(((double)xv[t] - m) * invT, sh.exp_tbl);
-            const double qd = (double)qv[t];
-            if (cache_ok) {
-                se[(j - lo + t) * nthr + tid] = e;
-                sq[(j - lo + t) * nthr + tid] = qv[t];
-            }
-            const double pe = e * inv_s_scan;
-            const double w = pe - c * qd;
-            r.v[0] += e;
-            if (w > 0.0) { r.v[1] += e; r.v[2] += qd; }
-            if (j + t != xnew) r.v[3] += qd;
-            // |w| <= kScanRel * pe needs the binary exponent of w at least 19 below that of pe: an
-            // integer comparison sorts out all but a handful of tokens
-            if ((__double2hiint(w) & 0x7ff00000) <= (__double2hiint(pe) & 0x7ff00000) - (19 << 20))
-                if (pe > 0.0 && fabs(w) <= kScanRel * pe) r.v[4] += pe;
+            const double w = fma(-C, (double)sq[(k + t) * stride], se[(k + t) * stride]);
+            if (__double2hiint(w) >= 0) a[t & 1] += w;
         }
     }
-    return r;
+    return a[0] + a[1];
+}
+
+// A probability in double precision by three integer operations (the conversion instruction runs at 16 per clock and SM).
+// Zero and the denormals come out between 2^-127 and 2^-126: next to the other terms of a sum of at least one, nothing.
+__device__ __forceinline__ double widen(float q)
+{
+    const unsigned u = __float_as_uint(q);
+    return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
+// The same from registers: a multiply-add, a look at the sign in the high word and an addition per token, no
+// shared-memory traffic and no conversion.
+__device__ __forceinline__ double residual_of_tile(const double (&er)[kTile], const float (&qr)[kTile], int per_thr, double C)
+{
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int b = 0; b < kTile; b += 4) {
+        if (b < per_thr) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const double w = fma(-C, widen(qr[b + t]), er[b + t]);
+                if (__double2hiint(w) >= 0) a[t] += w;
+            }
+        }
+    }
+    return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
+// The first rejection at a node, in one sweep.  The exact denominator S is not known yet and the residual is taken at
+// C = S: with P = { j : e_j - S' q_j > 0 } taken at the scan's S',
+//   sum_j max(e_j - S q_j, 0) = sum_P (e_j - S' q_j) - (S - S') sum_P q_j        for every S that leaves P unchanged.
+// The sweep returns (j = xnew, the token being rejected, counts in the first and, parked, is zero from here on)
+//   v[0] = sum e_j (= S)                    v[1] = sum_P (e_j - S' q_j), xnew left out
+//   v[2] = sum of q_j over the tokens that no child of the node carries (the draft mass left by any rejections here is
+//          this plus what the siblings still to be tested carry)
+//   v[3] = two floats: sum_P q_j (it is multiplied by S - S', a millionth of S at most), and the sum of e_j over the
+//          tokens whose sign a relative error kScanRel of S' could flip;
+// a flipped token changes the result by at most kScanRel times its e_j, so kScanRel times that sum bounds the error and the
+// caller sweeps again at the exact S when that is not negligible.
+// e_j and q_j are parked in shared memory, zeros in the empty positions.  The loop is kept short (four tokens, the next
+// four in flight): it runs two or three times per launch, and eight unrolled tokens spent longer on their first pass
+// through the instruction cache (3 us) than on the work.
+template <class Shared>
+__device__ __forceinline__ void fused_reject_sweep(const Shared &sh, const float *__restrict__ x, const float *__restrict__ q,
+                                                   double *__restrict__ se, float *__restrict__ sq, int stride, Chunk ck,
+                                                   int per_thr, bool park, const ExpArg &arg, double S, int xnew, int node,
+                                                   int n_nodes, double (&v)[4])
+{
+    // Which of this thread's first 64 positions hold a child's token: the warp's lanes look at the nodes side by side, and
+    // only for the few tokens that fall into the warp's stretch is the owner told.
+    unsigned long long kids = 0ull;
+    bool far = false;                            // (a position from 64 on: the token is compared with the children one by one)
+    {
+        const int lane = threadIdx.x & 31;
+        const int w_lo = __shfl_sync(0xffffffffu, ck.lo, 0), w_hi = __shfl_sync(0xffffffffu, ck.hi, 31);
+#pragma unroll 1
+        for (int n0 = 0; n0 < n_nodes; n0 += 32) {
+            const int c = n0 + lane;
+            const int t = (c < n_nodes && sh.t.parent[c] == node) ? sh.t.tok[c] : -8;
+#pragma unroll 1
+            for (unsigned m = __ballot_sync(0xffffffffu, t >= w_lo && t < w_hi && t >= 0); m; m &= m - 1) {
+                const int ct = __shfl_sync(0xffffffffu, t, __ffs((int)m) - 1);
+                if (ct >= ck.lo && ct < ck.hi) {
+                    if (ct - ck.lo < 64) kids |= 1ull << (ct - ck.lo);
+                    else far = true;
+                }
+            }
+        }
+    }
+    v[0] = v[1] = v[2] = 0.0;
+    float qp = 0.f, flips = 0.f;
+    float4 x4 = load4(x, ck.lo, ck.hi, -INFINITY), q4 = load4(q, ck.lo, ck.hi, 0.f);
+#pragma unroll 1
+    for (int k = 0; k < per_thr; k += 4) {
+        float4 xn = x4, qn = q4;
+        if (k + 4 < per_thr) {
+            xn = load4(x, ck.lo + k + 4, ck.hi, -INFINITY);
+            qn = load4(q, ck.lo + k + 4, ck.hi, 0.f);
+        }
+        double ev[4] = {exp_neg(x4.x, arg, sh.exp_tbl), exp_neg(x4.y, arg, sh.exp_tbl), exp_neg(x4.z, arg, sh.exp_tbl),
+                        exp_neg(x4.w, arg, sh.exp_tbl)};
+        float qv[4] = {q4.x, q4.y, q4.z, q4.w};
+        v[0] += (ev[0] + ev[1]) + (ev[2] + ev[3]);
+        double qd = ((double)qv[0] + (double)qv[1]) + ((double)qv[2] + (double)qv[3]);   // what counts towards the draft mass
+        if (k < 64 ? ((unsigned)(kids >> k) & 15u) != 0u : far) {
+            qd = 0.0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int id = ck.lo + k + t;
+                bool kid = k < 64 && ((kids >> (k + t)) & 1ull) != 0ull;
+                if (k >= 64)
+#pragma unroll 1
+                    for (int c = 1; c < n_nodes; ++c) kid |= sh.t.parent[c] == node && sh.t.tok[c] == id;
+                if (!kid) qd += (double)qv[t];
+                if (id == xnew) { ev[t] = 0.0; qv[t] = 0.f; }
+            }
+        }
+        v[2] += qd;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const double e = ev[t];
+            if (park) {
+                se[(k + t) * stride] = e;
+                sq[(k + t) * stride] = qv[t];
+            }
+            const double w = fma(-S, (double)qv[t], e);
+            if (__double2hiint(w) >= 0) { v[1] += w; qp += qv[t]; }
+            // |w| <= kScanRel * e needs the binary exponent of w at least 19 below that of e: an
+            // integer comparison sorts out all but a handful of tokens
+            if ((__double2hiint(w) & 0x7ff00000) <= (__double2hiint(e) & 0x7ff00000) - (19 << 20))
+                if (e > 0.0 && fabs(w) <= kScanRel * e) flips += (float)e;
+        }
+        x4 = xn;
+        q4 = qn;
+    }
+    v[3] = pair_of(qp, flips);
+}
+
+// ---- sums over the cluster ----
+// A CTA's totals go to every CTA of the cluster as asynchronous remote stores that count their bytes on the receiver's
+// barrier; only warp 0 waits.  (With remote stores, a cluster-wide barrier of all threads and two more CTA barriers an
+// exchange took 2.4 us.)  The wait is bounded like every other.
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void send_double(uint32_t dst, uint32_t bar, int peer, double v)
+{
+    asm volatile("{\n\t.reg .b32 d, b;\n\tmapa.shared::cluster.u32 d, %0, %2;\n\tmapa.shared::cluster.u32 b, %1, %2;\n\t"
+                 "st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [d], %3, [b];\n\t}\n"
+                 :: "r"(dst), "r"(bar), "r"(peer), "l"(__double_as_longlong(v)) : "memory");
+}
+__device__ __forceinline__ void expect_bytes(uint32_t bar, int bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity)
+{
+#pragma unroll 1
+    for (uint32_t i = 0; i < 2000000; ++i) {         // about 50 ms
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
+// block-wide scan of one value per thread (index order): this thread's exclusive and inclusive prefix and the CTA total
+template <class Shared>
+__device__ __noinline__ double block_scan(Shared &sh, double v, double *excl_out, double *total)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double incl = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const double t2 = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += t2;
+    }
+    const double prev_incl = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane == 31) sh.warp_v[0][wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+        // exclusive scan of the warp totals; the last inclusive value is the CTA total
+        double sc = (lane < kWarps) ? sh.warp_v[0][lane] : 0.0;
+#pragma unroll
+        for (int off = 1; off < kWarps; off <<= 1) {
+            const double t2 = __shfl_up_sync(0xffffffffu, sc, off);
+            if (lane >= off) sc += t2;
+        }
+        const double excl = __shfl_up_sync(0xffffffffu, sc, 1);
+        if (lane < kWarps) sh.warp_off[lane] = (lane == 0) ? 0.0 : excl;
+        if (lane == kWarps - 1) sh.warp_total = sc;
+    }
+    __syncthreads();
+    const double woff = sh.warp_off[wid];
+    *excl_out = (lane == 0) ? woff : woff + prev_incl;
+    *total = sh.warp_total;
+    return woff + incl;
 }
 
 // Compaction of the accepted path by the CTAs that walked it (every CTA of the cluster holds the same path in
@@ -362,13 +574,12 @@ __device__ Sweep5 fused_reject_sweep(const Shared &sh, const float *__restrict__
 // per slice, eight rows in flight, every load of a batch before any of its stores (path[j] >= j and the path
 // is increasing, so moves in index order never overwrite a row that is still to be read).  The same moves as
 // the stand-alone compaction kernel makes; doing them here saves the step one dependent launch.
-template <typename Shared>
-__device__ __forceinline__ void compact_accepted(const WalkArgs &args, const Shared &sh, int b, int rank, int C, int tid, int nthr)
+template <typename Tree>
+__device__ __noinline__ void compact_accepted(const WalkArgs &args, const Tree &sh, int b, int rank, int C, int tid, int nthr)
 {
-    if (args.kv_cache == nullptr) return;
     const int lane = tid & 31, n_warps = nthr >> 5;
     int n = sh.len;
-    const int L = args.kv_prefix[b];
+    const int L = sh.kv_L;
     if (L < 0 || n < 1 || L + sh.path[n - 1] >= args.kv_max_len) {
         if (rank == 0 && tid == 0) fspad_report(args.status, FSPAD_ERR_RANGE);
         n = 0;
@@ -376,9 +587,11 @@ __device__ __forceinline__ void compact_accepted(const WalkArgs &args, const Sha
     if (rank == 0 && tid == 0 && args.kv_new_len) args.kv_new_len[b] = max(L, 0) + n;
     const int per_seq = args.kv_layers * 2 * args.kv_H;
     const int chunk = lane & 15, half = lane >> 4;
-    for (int s = rank * n_warps + (tid >> 5); s < per_seq; s += C * n_warps) {
+#pragma unroll 1
+    for (int s = (tid >> 5) * C + rank; s < per_seq; s += C * n_warps) {
         const int lk = s / args.kv_H, h = s % args.kv_H;
         uint4 *base = args.kv_cache + ((((size_t)lk * args.kv_B + b) * args.kv_H + h) * args.kv_max_len + L) * 16;
+#pragma unroll 1
         for (int j0 = 0; j0 < n; j0 += 8) {
             uint4 v[4];
             int dst[4];
@@ -402,28 +615,97 @@ __device__ __forceinline__ void compact_accepted(const WalkArgs &args, const Sha
     }
 }
 
+// Node c of the tree (its thread's), checked: the parent is a lower node, the token lies in the vocabulary.
+__device__ __forceinline__ void check_node(int c, int V, int &p, int &t, int *status)
+{
+    if (c == 0 ? p != -1 : (p < 0 || p >= c)) {
+        fspad_report(status, FSPAD_ERR_BAD_TREE);
+        p = 0;
+    }
+    if (c == 0) p = -1;
+    if (t < 0 || t >= V) {
+        fspad_report(status, FSPAD_ERR_RANGE);
+        t = 0;
+    }
+}
+
+// Greedy walk of one sequence by one CTA: strict comparison of the draft tokens with the target's argmax.  Every node looks
+// at its parent's argmax side by side; what is left for one thread is to follow the chain of matches.
+template <int MAXN>
+__device__ __forceinline__ void greedy_walk(TreeShared<MAXN> &t, const WalkArgs &args, int b, int N, int tid, int nthr, bool writer)
+{
+    if (tid < MAXN) t.next[tid] = MAXN;
+    __syncthreads();
+    if (tid >= 1 && tid < N && t.tok[tid] == t.rowA[t.parent[tid]]) atomicMin(&t.next[t.parent[tid]], tid);   // lowest node index
+    __syncthreads();
+    if (tid == 0) {                               // every CTA of a cluster: same data, same path
+        int cur = 0, len = 1;
+        t.path[0] = 0;
+#pragma unroll 1
+        for (int nx = t.next[0]; nx < MAXN; nx = t.next[nx]) {
+            t.path[len++] = nx;
+            cur = nx;
+        }
+        t.len = len;
+        if (writer) { args.n_acc[b] = len; args.bonus[b] = t.rowA[cur]; }
+    }
+    __syncthreads();
+    if (writer) {
+        int *out_path = args.path + (size_t)b * args.path_stride;
+#pragma unroll 1
+        for (int i = tid; i < args.path_stride; i += nthr) out_path[i] = (i < t.len) ? t.path[i] : -1;
+    }
+}
+
+// All sequences greedy: one CTA per sequence, nothing of the sampling walk's apparatus.
+template <int MAXN>
+__global__ void __launch_bounds__(kWalkThreads)
+accept_greedy_kernel(const __grid_constant__ WalkArgs args)
+{
+    __shared__ TreeShared<MAXN> t;
+    const int b = blockIdx.x, tid = threadIdx.x, nthr = blockDim.x, N = args.N;
+    fspad_pdl_trigger();
+    // (read before the scan has finished: see the sampling kernel)
+    const float Tf = args.temperature[b];
+    int p = -1, tk = 0;
+    if (tid < N) {
+        p = args.parent[(size_t)b * N + tid];
+        tk = args.tokens[(size_t)b * N + tid];
+        check_node(tid, args.V, p, tk, args.status);
+        t.parent[tid] = p;
+        t.tok[tid] = tk;
+    }
+    if (tid == 0 && !(Tf >= 0.0f)) fspad_report(args.status, FSPAD_ERR_RANGE);
+    if (tid == 0 && Tf > 0.0f) fspad_report(args.status, FSPAD_ERR_NULL);      // a sampling sequence without draft rows
+    fspad_pdl_wait();
+    const int l8 = tid & 7;
+#pragma unroll 1
+    for (int r0 = 0; r0 < N; r0 += nthr >> 3) {      // whole warps iterate together
+        const int row = r0 + (tid >> 3);
+        float M; double S; int A;
+        merge_row(args.parts, args.geom, b * N + row, row < N, 0.f, l8, M, S, A, nullptr, nullptr);
+        if (l8 == 0 && row < N) t.rowA[row] = A;
+    }
+    __syncthreads();
+    greedy_walk(t, args, b, N, tid, nthr, true);
+}
+
 template <int MAXN>
 __global__ void __launch_bounds__(kWalkThreads, 1)
-accept_walk_kernel(const WalkArgs args)
+accept_walk_kernel(const __grid_constant__ WalkArgs args)
 {
     typedef SharedT<MAXN> Shared;
-    constexpr int W = Shared::W;
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
     const int b = blockIdx.x / C;
-    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int N = args.N, V = args.V;
 
     __shared__ Shared sh;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
 
     fspad_pdl_trigger();
-    if (tid < 64) sh.exp_tbl[tid] = kExp2Tbl[tid];
-    if (tid < MAXN) {
-#pragma unroll
-        for (int i = 0; i < W; ++i) sh.child_mask[tid].w[i] = 0ull;
-    }
     // The vocabulary scan that precedes this kernel in the stream lets it start only after the scan's
     // own predecessor has completed, and the scan writes nothing but its partial results.  So the
     // caller's arrays may be read before the scan has finished: the prologue's two round trips of
@@ -436,40 +718,39 @@ accept_walk_kernel(const WalkArgs args)
         p = args.parent[(size_t)b * N + tid];
         t = args.tokens[(size_t)b * N + tid];
     }
-    if (args.uniforms != nullptr && tid <= N)      // thread c: node c's uniform; thread 0: the bonus uniform
-        uval = args.uniforms[(size_t)b * (N + 1) + (tid == 0 ? N : tid)];
+    if (tid <= N) uval = args.uniforms[(size_t)b * (N + 1) + (tid == 0 ? N : tid)];   // thread c: node c's uniform; thread 0: the bonus uniform
+    if (tid == 32 && args.kv_cache != nullptr) sh.t.kv_L = args.kv_prefix[b];
+    // (the loads above are under way)
+    if (tid < kExpTable)
+        sh.exp_tbl[tid] = kExp2Tbl[tid >> 2] * ((tid & 2) ? ((tid & 1) ? 1.0081558981184175 : 1.0054299011128027) : ((tid & 1) ? 1.0027112750502025 : 1.0));
+    if (tid < MAXN) sh.first_child[tid] = MAXN;
+    if (tid == 0) {
+        sh.fail = 0;
+        for (int i = 0; i < 2; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(&sh.bar[i])));
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncthreads();
+    // (the peers' barriers are initialised before anything is sent to them: waited for below)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
     if (!(Tf >= 0.0f)) {
         if (tid == 0 && rank == 0) fspad_report(args.status, FSPAD_ERR_RANGE);
         Tf = 0.0f;
     }
-    const bool sampling = Tf > 0.0f && args.draft != nullptr && args.uniforms != nullptr;
-    if (Tf > 0.0f && !sampling && tid == 0 && rank == 0) fspad_report(args.status, FSPAD_ERR_NULL);
-    __syncthreads();                             // child masks are zeroed
+    const bool sampling = Tf > 0.0f;
+    const size_t row0 = (size_t)b * N;           // the sequence's first row
+    const float *lg = args.logits + row0 * V, *dp = args.draft + row0 * V;
+    const float kT = kLog2eF / (sampling ? Tf : 1.0f);
 
-    const float *lg = args.logits + (size_t)b * N * V;
-    const float *dp = args.draft ? args.draft + (size_t)b * N * V : nullptr;
-    int *out_path = args.path + (size_t)b * args.path_stride;
-    const float kT = kLog2eF / (Tf > 0.0f ? Tf : 1.0f);
-
-    // Round trip 2: thread c owns node c (tree arrays, the child bit of its parent and the scalars
-    // its accept test needs: target logit and draft probability of its token in its parent's row).
+    // Round trip 2: thread c owns node c (tree arrays, and the scalars its accept test needs: target logit and draft
+    // probability of its token in its parent's row).
     float xv = 0.f, qv = 0.f;
     if (tid < N) {
-        if (tid == 0) {
-            if (p != -1) fspad_report(args.status, FSPAD_ERR_BAD_TREE);
-            p = -1;
-        } else if (p < 0 || p >= tid) {
-            fspad_report(args.status, FSPAD_ERR_BAD_TREE);
-            p = 0;
-        }
-        if (t < 0 || t >= V) {
-            fspad_report(args.status, FSPAD_ERR_RANGE);
-            t = 0;
-        }
-        sh.parent[tid] = p;
-        sh.tok[tid] = t;
+        check_node(tid, V, p, t, args.status);
+        sh.t.parent[tid] = p;
+        sh.t.tok[tid] = t;
         if (tid >= 1) {
-            atomicOr(&sh.child_mask[p].w[tid >> 6], 1ull << (tid & 63));
+            atomicMin(&sh.first_child[p], tid);
             if (sampling) {
                 const size_t at = (size_t)p * V + t;
                 xv = lg[at];
@@ -477,449 +758,513 @@ accept_walk_kernel(const WalkArgs args)
             }
         }
     }
-    // The root's draft row is the one most likely to be swept: ask for it now (a hint, no register
-    // is tied up and nothing waits for it).
-    const bool vec = (V % 4 == 0) && ((reinterpret_cast<uintptr_t>(args.logits) & 15) == 0) &&
-                     ((reinterpret_cast<uintptr_t>(args.draft) & 15) == 0);
-    // contiguous slice per CTA, contiguous chunk per thread (multiples of 4 tokens)
-    const int per_cta = (((V + C - 1) / C) + 3) & ~3;
-    const int per_thr = (((per_cta + nthr - 1) / nthr) + 3) & ~3;
-    const int cta_lo = rank * per_cta, cta_hi = min(V, cta_lo + per_cta);
-    const int lo = min(cta_hi, cta_lo + tid * per_thr), hi = min(cta_hi, lo + per_thr);
-    if (sampling && lo < hi)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + lo));
-    if (sampling && tid < N) {
-        if (tid >= 1) { sh.cx[tid] = xv; sh.cq[tid] = qv; sh.cu[tid] = uval; }
-        else sh.ubonus = uval;
+    // how a row is shared out (positions of the row plus up to three in front of it)
+    const int per_cta = (((V + 3 + C - 1) / C) + 3) & ~3;
+    const int per_thr = (((per_cta + kWalkThreads - 1) / kWalkThreads) + 3) & ~3;
+    {
+        // The root's draft row is the one most likely to be swept: ask for it now (a hint, no register
+        // is tied up and nothing waits for it).
+        const Chunk ck = chunk_of(row0 * V, V, per_cta, per_thr, rank, tid);
+        if (sampling && ck.lo >= 0 && ck.lo < ck.hi) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + ck.lo));
+            if (per_thr > 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + min(ck.hi - 1, ck.lo + 8)));
+        }
+    }
+    __syncthreads();
+    const int l8 = tid & 7;
+    if (sampling) {
+        // eight lanes per node: the sibling after it, and whether one before it carries its token
+#pragma unroll 1
+        for (int c0 = 0; c0 < N; c0 += kWalkThreads / 8) {       // whole warps iterate together
+            const int c = c0 + (tid >> 3);
+            int nx = MAXN;
+            unsigned d = 0;
+            if (c >= 1 && c < N) {
+                const int pc = sh.t.parent[c], tc = sh.t.tok[c];
+                for (int o = 1 + l8; o < N; o += 8) {
+                    const bool sib = sh.t.parent[o] == pc;
+                    if (sib && o > c) nx = min(nx, o);
+                    if (sib && o < c && sh.t.tok[o] == tc) d = 1;
+                }
+            }
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) {
+                nx = min(nx, __shfl_xor_sync(0xffffffffu, nx, off));
+                d |= __shfl_xor_sync(0xffffffffu, d, off);
+            }
+            if (l8 == 0 && c < N) { sh.next_sib[c] = nx < MAXN ? nx : 0; sh.dup[c] = (unsigned char)d; }
+        }
     }
 
     fspad_pdl_wait();                            // from here on the scan's partial results may be read
-    {
-        // half-warps merge the scan partials of the rows
-        const int lane16 = tid & 15, n_half = nthr >> 4;
-        for (int r0 = 0; r0 < N; r0 += n_half) {                 // whole warps iterate together
-            const int row = r0 + (tid >> 4);
-            float M; double S; int A;
-            if (MAXN == 64)
-                fspad_stats_merge_half(args.parts, args.geom, b * N + row, row < N, kT, lane16, M, S, A,
-                                       sh.piece_w[row < N ? row : 0], &sh.piece_cnt[row < N ? row : 0]);
-            else
-                fspad_stats_merge_half(args.parts, args.geom, b * N + row, row < N, kT, lane16, M, S, A);
-            if (lane16 == 0 && row < N) { sh.rowM[row] = M; sh.rowS[row] = S; sh.rowInvS[row] = 1.0 / S; sh.rowA[row] = A; }
-        }
+#pragma unroll 1
+    for (int r0 = 0; r0 < N; r0 += kWalkThreads / 8) {           // whole warps iterate together
+        const int row = r0 + (tid >> 3), rs = row < N ? row : 0;
+        float M; double S; int A;
+        merge_row(args.parts, args.geom, b * N + row, row < N, kT, l8, M, S, A, sh.piece_w[rs], &sh.piece_cnt[rs]);
+        if (l8 == 0 && row < N) { sh.rowM[row] = M; sh.rowS[row] = S; sh.t.rowA[row] = A; }
     }
+    const double invT = 1.0 / (double)(sampling ? Tf : 1.0f);
     __syncthreads();
-    if (sampling && tid >= 1 && tid < N)
-        sh.cex[tid] = exp_neg(((double)sh.cx[tid] - (double)sh.rowM[sh.parent[tid]]) * (1.0 / (double)Tf), sh.exp_tbl);
+    if (sampling && tid < N) {
+        if (tid >= 1) {
+            sh.cq[tid] = qv;
+            sh.cu[tid] = uval;
+            sh.cex[tid] = exp_neg(xv, exp_arg(sh.rowM[p], invT, Tf), sh.exp_tbl);
+        } else {
+            sh.ubonus = uval;
+        }
+        if (sh.first_child[tid] == MAXN) sh.first_child[tid] = 0;
+    }
+    // the peers' barriers are initialised (every CTA arrived at the top of the kernel)
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     __syncthreads();
 
     if (!sampling) {
-        // ---- greedy: strict token comparison against the target argmax ----
-        if (tid == 0) {                               // every CTA of the cluster: same data, same path
-            int cur = 0, len = 1;
-            sh.path[0] = 0;
-            for (;;) {
-                const int want = sh.rowA[cur];
-                int next = -1;
-                for (NodeSet<W> rem = sh.child_mask[cur]; rem.any(); rem.drop_first()) {
-                    const int c = rem.first();
-                    if (sh.tok[c] == want) { next = c; break; }
-                }
-                if (next < 0) { if (rank == 0) args.bonus[b] = want; break; }
-                sh.path[len++] = next;
-                cur = next;
-            }
-            if (rank == 0) args.n_acc[b] = len;
-            sh.len = len;
-        }
-        __syncthreads();
-        if (rank == 0)
-            for (int i = tid; i < args.path_stride; i += nthr) out_path[i] = (i < sh.len) ? sh.path[i] : -1;
-        compact_accepted(args, sh, b, rank, C, tid, nthr);
+        greedy_walk(sh.t, args, b, N, tid, kWalkThreads, rank == 0);
+        if (args.kv_cache != nullptr) compact_accepted(args, sh.t, b, rank, C, tid, kWalkThreads);
         return;   // the whole cluster takes this branch together; no peer memory is touched
     }
 
     // ---- sampling ----
-    const bool cache_ok = args.cache_ok != 0;
-    double *se = reinterpret_cast<double *>(dyn_smem);
-    // the cache is laid out [k][thread] (k-th token of each thread's chunk): conflict-free
-    float *sq = reinterpret_cast<float *>(dyn_smem + (size_t)per_thr * nthr * sizeof(double));
-    int parity = 0;
-
-    // cluster-wide reduction of (a, b); result in sh.tot[] (read by thread 0 only).  Every level
-    // is a warp butterfly; the CTAs exchange by remote stores (each writes its pair into every
-    // peer's slot before the barrier), so after the barrier all reads are local, and every CTA
-    // performs the same operations on the same values.
-    auto reduce_exchange = [&](double a, double bb) {
-        const int lane = tid & 31, wid = tid >> 5, nwarps = nthr >> 5;
-        a = warp_sum(a);
-        bb = warp_sum(bb);
-        if (lane == 0) { sh.warp_a[wid] = a; sh.warp_b[wid] = bb; }
+    const bool cache_ok = args.cache_ok != 0, in_regs = cache_ok && per_thr <= kTile;
+    // parked values: [k][thread] (k-th position of each thread's chunk), conflict-free
+    double *se = reinterpret_cast<double *>(dyn_smem) + tid;
+    float *sq = reinterpret_cast<float *>(dyn_smem + (size_t)per_thr * kWalkThreads * sizeof(double)) + tid;
+    int n_exch = 0;                              // exchanges so far
+    // Sums of NV values (one or four) over the cluster, in every lane of warp 0 (the other warps' values are not defined).
+    // Every CTA performs the same operations on the same values.  Four values are summed in groups of eight lanes, one
+    // value to a group, after two steps in which a lane passes on the values of the other groups; the fourth is a pair of
+    // floats in the words of a double.  A slot is written again two exchanges later, by peers that have by then received
+    // this CTA's next totals, which it sends only after it has read the slot.
+    // Warp 0 runs `meanwhile` while the peers' totals are on their way.
+    auto exchange = [&](auto &v, auto meanwhile) {
+        constexpr int NV = sizeof(v) / sizeof(double);
+        constexpr int kGroup = 32 / NV;          // lanes that end up with the same value
+        const int item = lane / kGroup, sub = lane % kGroup;
+        const int par = n_exch & 1;
+        const uint32_t phase = (uint32_t)(n_exch >> 1) & 1u;
+        ++n_exch;
+        auto add = [&](double x2, double y2, bool pair) {
+            if (NV == 4 && pair)
+                return pair_of(__int_as_float(__double2hiint(x2)) + __int_as_float(__double2hiint(y2)),
+                               __int_as_float(__double2loint(x2)) + __int_as_float(__double2loint(y2)));
+            return x2 + y2;
+        };
+        const bool pair = item == 3;
+        double one = v[0];
+        if (NV == 4) {
+            const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
+            const double a0 = (up ? v[2 % NV] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2 % NV], 16);
+            const double a1 = add(up ? v[3 % NV] : v[1 % NV], __shfl_xor_sync(0xffffffffu, up ? v[1 % NV] : v[3 % NV], 16), up);
+            one = add(odd ? a1 : a0, __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8), pair);
+        }
+#pragma unroll
+        for (int off = kGroup / 2; off > 0; off >>= 1) one = add(one, __shfl_xor_sync(0xffffffffu, one, off), pair);
+        if (sub == 0) sh.warp_v[item][wid] = one;
         __syncthreads();
         if (wid == 0) {
-            double sa = (lane < nwarps) ? sh.warp_a[lane] : 0.0;
-            double sb = (lane < nwarps) ? sh.warp_b[lane] : 0.0;
-            sa = warp_sum(sa);
-            sb = warp_sum(sb);
-            if (lane < C) {
-                double *peer = cluster.map_shared_rank(&sh.slot[parity][rank][0], lane);
-                peer[0] = sa;
-                peer[1] = sb;
-            }
+            one = sub < kWarps ? sh.warp_v[item][sub] : 0.0;
+            if (kGroup < kWarps) one = add(one, sh.warp_v[item][(sub + kGroup) % kWarps], pair);
+            static_assert(kGroup >= kWarps / 2, "at most two warp totals per lane");
+#pragma unroll
+            for (int off = (kGroup < kWarps ? kGroup : kWarps) / 2; off > 0; off >>= 1)
+                one = add(one, __shfl_xor_sync(0xffffffffu, one, off), pair);
+            if (NV == 1) one = __shfl_sync(0xffffffffu, one, 0);
+            const uint32_t bar = smem_addr(&sh.bar[par]);
+            if (lane == 0) expect_bytes(bar, C * NV * 8);
+            if (sub < C) send_double(smem_addr(&sh.slot[par][item][rank]), bar, sub, one);
+            if (kGroup < kMaxCluster && sub + kGroup < C) send_double(smem_addr(&sh.slot[par][item][rank]), bar, sub + kGroup, one);
+            meanwhile();
+            if (!wait_cluster(bar, phase)) sh.fail = 1;
+            __syncwarp();
+            one = sub < C ? sh.slot[par][item][sub] : 0.0;
+            if (kGroup < kMaxCluster && sub + kGroup < C) one = add(one, sh.slot[par][item][(sub + kGroup) % kMaxCluster], pair);
+#pragma unroll
+            for (int off = (kGroup < kMaxCluster ? kGroup : kMaxCluster) / 2; off > 0; off >>= 1)
+                one = add(one, __shfl_xor_sync(0xffffffffu, one, off), pair);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) v[k] = __shfl_sync(0xffffffffu, one, k * kGroup);
         }
-        cluster.sync();
-        if (wid == 0) {
-            double ta = (lane < C) ? sh.slot[parity][lane][0] : 0.0;
-            double tb = (lane < C) ? sh.slot[parity][lane][1] : 0.0;
-            ta = warp_sum(ta);
-            tb = warp_sum(tb);
-            if (lane == 0) { sh.tot[0] = ta; sh.tot[1] = tb; }
-        }
-        __syncthreads();
-        parity ^= 1;
     };
 
-    const double invT = 1.0 / (double)Tf;        // every thread: off the serial path of thread 0
-    // the same exchange for the five sums of the fused sweep; result in sh.tot5[]
-    auto reduce_exchange5 = [&](const Sweep5 &in) {
-        const int lane = tid & 31, wid = tid >> 5, nwarps = nthr >> 5;
-        double v[5];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = warp_sum(in.v[k]);
-        if (lane == 0) {
-#pragma unroll
-            for (int k = 0; k < 5; ++k) sh.warp5[wid][k] = v[k];
-        }
-        __syncthreads();
-        if (wid == 0) {
-#pragma unroll
-            for (int k = 0; k < 5; ++k) v[k] = warp_sum((lane < nwarps) ? sh.warp5[lane][k] : 0.0);
-            if (lane < C) {
-                double *peer = cluster.map_shared_rank(&sh.slot5[parity][rank][0], lane);
-#pragma unroll
-                for (int k = 0; k < 5; ++k) peer[k] = v[k];
-            }
-        }
-        cluster.sync();
-        if (wid == 0) {
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                const double t5 = warp_sum((lane < C) ? sh.slot5[parity][lane][k] : 0.0);
-                if (lane == 0) sh.tot5[k] = t5;
-            }
-        }
-        __syncthreads();
-        parity ^= 1;
-    };
+    // draft mass of the tokens that only later siblings of node c carry (read after the first exchange; warp 0 has the
+    // walk to begin)
+    for (int c = tid - 31; wid > 0 && c < N; c += kWalkThreads - 32) {
+        double later = 0.0;
+#pragma unroll 1
+        for (int o = sh.next_sib[c]; o > 0; o = sh.next_sib[o])
+            if (!sh.dup[o]) later += (double)sh.cq[o];
+        sh.later_q[c] = later;
+    }
 
     // Thread 0 of every CTA (all on identical data, so all take identical steps) walks ahead through
     // every decision that needs nothing but scalars, and stops only to ask the CTA for a sweep of the
-    // current node's rows.  enter() makes a node the current one.
-    auto enter = [&](int node) {
-        sh.cur = node;
-        sh.m = (double)sh.rowM[node];
-        sh.S = sh.rowS[node];
-        sh.invS = sh.rowInvS[node];
-        sh.exact = 0; sh.have_e = 0; sh.have_q = 0;
-        sh.c = 0.0; sh.U = 1.0; sh.D = 1.0;
-        sh.nrem = 0;
-        sh.bonus_ok = 0;
-        sh.rem = sh.child_mask[node];
+    // current node's rows.
+    WalkState w;
+    Child nx;                                    // the child to be tested next, fetched ahead
+    double fx = 0.0, next_rhs = 0.0;             // weight of the token being rejected; the next test's right side
+    double next_D = 0.0, next_invD = 0.0;        // draft mass left when the child under test is rejected too
+    auto fetch_child = [&](int c) {
+        nx.ch = c;
+        nx.next = sh.next_sib[c];
+        nx.tok = sh.t.tok[c];
+        nx.dup = sh.dup[c];
+        nx.ex = sh.cex[c];
+        nx.qx = (double)sh.cq[c];
+        nx.rq = (double)sh.cu[c] * nx.qx;
     };
-    if (tid == 0) { sh.len = 1; sh.path[0] = 0; sh.invT = invT; enter(0); }
+    // while a residual's total is on its way: the state, and everything that does not depend on that total
+    auto fetch_ahead = [&]() {
+        w = sh.state;
+        fx = weight(sh.cex[w.ch], (double)sh.cq[w.ch], w.Cp);
+        next_D = sh.node_D[w.ch];
+        next_invD = sh.node_invD[w.ch];
+        fetch_child(sh.next_sib[w.ch]);          // (node 0 where there is none)
+        next_rhs = weight(nx.ex, nx.qx, w.Cp) * (next_D > 0.0 ? next_D : w.D);
+    };
+    enum { GOT_NOTHING, GOT_SUM, GOT_RESIDUAL };
+    int got = GOT_NOTHING;
+    double R = 0.0;                              // warp 0: the sum asked for last
     double last_a = 0.0;                         // this thread's sum of weights in the latest residual sweep
+    double er[kTile];                            // this thread's chunk of the node's rows, after the first rejection there
+    float qr[kTile];
+#pragma unroll
+    for (int i = 0; i < kTile; ++i) { er[i] = 0.0; qr[i] = 0.f; }
 
     for (;;) {
         if (tid == 0) {
+            int go = -1;                                      // node to be entered
+            bool ahead = false;                               // nx and next_rhs hold for the next test
+            if (got == GOT_NOTHING) {
+                go = 0;
+                w.len = 0;
+                w.nrem = 0;
+            } else if (got == GOT_SUM) {
+                w.S = w.U = R;
+                w.exact = 1;
+            } else {
+                // When this was the node's last child, the weights just summed (residual at the new coefficient, the
+                // rejected tokens at the weights they keep) are the ones the bonus token is drawn from, thread by thread
+                // in the same order: the draw reuses the sums (last_a).
+                const double Wt = R + (w.ridx < 0 ? w.F + fx : w.F);
+                double frozen = fx;
+                if (Wt > 0.0) {
+                    w.C = w.Cp;
+                    w.U = Wt;
+                    ahead = true;
+                    sh.bonus_ok = nx.ch > 0 ? 0 : 1;
+                } else {
+                    frozen = weight(sh.cex[w.ch], (double)sh.cq[w.ch], w.C);   // residual vanished: p is kept
+                    if (w.C == 0.0) w.U = w.S;
+                }
+                if (next_D > 0.0) { w.D = next_D; w.invD = next_invD; }
+                if (w.ridx < 0 && w.nrem < MAXN) {
+                    sh.rem_tok[w.nrem] = sh.t.tok[w.ch];
+                    sh.rem_frozen[w.nrem] = frozen;
+                    w.F += frozen;
+                    w.nrem++;
+                }
+                w.ch = nx.ch;
+            }
             int req = REQ_DONE;
-            while (sh.rem.any()) {
-                const int ch = sh.rem.first();
-                const int xt = sh.tok[ch];
-                const double r = (double)sh.cu[ch];
-                const double qx = (double)sh.cq[ch];
-                const double ex = sh.cex[ch];
-                int ridx = -1;
-                for (int k = 0; k < sh.nrem; ++k) if (sh.rem_tok[k] == xt) ridx = k;
+#pragma unroll 1
+            for (;;) {
+                if (go >= 0) {
+                    sh.t.path[w.len++] = go;
+                    w.cur = go;
+                    w.S = w.U = sh.rowS[go];
+                    w.exact = w.parked = 0;
+                    w.C = 0.0; w.D = 1.0; w.invD = 1.0; w.F = 0.0;
+                    w.nrem = 0;
+                    w.ch = sh.first_child[go];
+                    sh.bonus_ok = 0;
+                    go = -1;
+                }
+                if (w.ch == 0 || sh.fail != 0) break;
+                if (!ahead) fetch_child(w.ch);
+                w.ridx = -1;
+                if (w.nrem > 0 && nx.dup)
+#pragma unroll 1
+                    for (int k = 0; k < w.nrem; ++k) if (sh.rem_tok[k] == nx.tok) w.ridx = k;
                 // accept iff r * q_k(x) < p_k(x) with q_k = qx / D and p_k = u / U: compared as
                 // r * qx * U < u * D (both normalisers are positive), so no division is needed
-                const double u = (ridx >= 0) ? sh.rem_frozen[ridx] : weight(ex, qx, sh.invS, sh.c);
-                const double lhs = (ridx >= 0) ? 0.0 : r * qx * sh.U;
-                const double rhs = u * sh.D;
-                const bool acc = lhs < rhs;
-                if (!sh.exact) {
+                double lhs = nx.rq * w.U, rhs = next_rhs;
+                if (!ahead) rhs = weight(nx.ex, nx.qx, w.C) * w.D;
+                if (w.ridx >= 0) {
+                    lhs = 0.0;
+                    rhs = sh.rem_frozen[w.ridx] * w.D;
+                }
+                ahead = false;
+                if (!w.exact) {
                     // the scan's sum of exponentials is trusted only outside a margin around the boundary
                     const double big = fmax(lhs, rhs);
                     if (big > 0.0 && fabs(lhs - rhs) <= kAmbiguous * big) {
-                        req = acc ? REQ_EXP : REQ_EXP_Q;      // exact denominator first (and park the draft row if a rejection is likely)
+                        req = REQ_EXP;                        // exact denominator first
                         break;
                     }
                 }
-                if (acc) {
-                    sh.path[sh.len++] = ch;
-                    enter(ch);
+                if (lhs < rhs) {
+                    go = nx.ch;
                     continue;
                 }
-                // rejected: one sweep gives the new residual mass and the new draft mass
-                sh.ex = ex; sh.qx = qx; sh.ridx = ridx; sh.xnew = xt;
-                sh.cprime = sh.c + sh.U / sh.D;
-                req = sh.exact ? REQ_RESID : REQ_FUSED;       // first rejection at a node: exact denominator and residual in one sweep
+                // rejected: a sweep gives the new residual mass
+                w.Cp = fma(w.U, w.invD, w.C);
+                req = w.parked ? REQ_RESID : REQ_FUSED;
                 break;
             }
             sh.req = req;
-            if (req != REQ_DONE) {
-                sh.req_child = sh.rem.first();
-                sh.req_last = sh.rem.single() ? 1 : 0;
-            }
+            sh.C = req == REQ_DONE ? w.C : w.Cp;
+            sh.xnew = nx.tok;
+            sh.cur = w.cur;
+            sh.S = w.S;
+            sh.nrem = w.nrem;
+            sh.t.len = w.len;
+            sh.parked = w.parked && cache_ok;
+            sh.state = w;
         }
         __syncthreads();
+        w = WalkState{}; nx = Child{}; fx = next_rhs = next_D = next_invD = 0.0;   // (no register is tied up by the state during the sweeps)
         const int req = sh.req;
         if (req == REQ_DONE) break;                           // uniform
-        const int cur = sh.cur;
-        const float *x = lg + (size_t)cur * V;
-        const float *q = dp + (size_t)cur * V;
-        if (req == REQ_EXP || req == REQ_EXP_Q) {
-            // exact softmax denominator of this node (parks e_j in shared memory)
-            const bool with_q = req == REQ_EXP_Q;
-            Sweep sw = sweep_chunk<MODE_EXP>(sh, x, q, se, sq, tid, nthr, lo, hi, vec, cache_ok, false, false, 0.0,
-                                             with_q ? -2 : -1, false, 0, 0, 0, nullptr);
-            reduce_exchange(sw.a, 0.0);
-            if (tid == 0) {
-                sh.S = sh.tot[0]; sh.invS = 1.0 / sh.S; sh.exact = 1; sh.have_e = cache_ok;
-                if (with_q) sh.have_q = cache_ok;
-            }
-            continue;                                         // thread 0 repeats the test with the exact sum
-        }
-        const int xt = sh.xnew;
-        bool fused_done = false;
+        const int cur = sh.cur, xn = sh.xnew;
+        const float *x = lg + (size_t)cur * V, *q = dp + (size_t)cur * V;
+        const Chunk ck = chunk_of((row0 + cur) * V, V, per_cta, per_thr, rank, tid);
+        const ExpArg arg = exp_arg(sh.rowM[cur], invT, Tf);
+        got = GOT_RESIDUAL;
+        bool again = req != REQ_FUSED;
         if (req == REQ_FUSED) {
-            // first rejection at this node, nothing exact yet (c = 0, U = D = 1, nothing removed)
-            const double cp = sh.cprime;
-            const Sweep5 f = fused_reject_sweep(sh, x, q, se, sq, tid, nthr, lo, hi, vec, cache_ok, sh.invS, cp, xt);
-            reduce_exchange5(f);
-            if (tid == 0) {
-                const double S = sh.tot5[0], invS = 1.0 / S;
-                const double W = sh.tot5[1] * invS - cp * sh.tot5[2];
-                sh.S = S; sh.invS = invS; sh.exact = 1; sh.have_e = cache_ok; sh.have_q = cache_ok;
-                sh.fused_fallback = !(W > 0.0 && kScanRel * sh.tot5[4] <= kFusedTol * W);
-                if (!sh.fused_fallback) {
-                    sh.tot[0] = W;
-                    sh.tot[1] = sh.tot5[3];
+            // first rejection at this node, nothing exact yet (nothing removed, C = S)
+            double v[4];
+            const double s_scan = sh.S;
+            fused_reject_sweep(sh, x, q, se, sq, kWalkThreads, ck, per_thr, cache_ok, arg, s_scan, xn, cur, N, v);
+            double tot[4] = {v[0], v[1], v[2], v[3]};
+            exchange(tot, []() {});
+            if (wid == 0) {
+                // what the draft row keeps after each child of the node in turn
+#pragma unroll 1
+                for (int c = lane; c < N; c += 32) {
+                    if (c == 0 || sh.t.parent[c] != cur) continue;
+                    const double d = tot[2] + sh.later_q[c];
+                    sh.node_D[c] = d;
+                    sh.node_invD[c] = 1.0 / d;
+                }
+                const double s_exact = tot[0];
+                const float qp = __int_as_float(__double2hiint(tot[3])), flips = __int_as_float(__double2loint(tot[3]));
+                R = tot[1] - (s_exact - s_scan) * (double)qp;
+                if (R < 0.0) R = 0.0;
+                if (lane == 0) {
+                    sh.state.S = sh.state.Cp = s_exact;
+                    sh.state.exact = sh.state.parked = 1;
+                    const int c = sh.state.ch;
+                    const double Wt = R + weight(sh.cex[c], (double)sh.cq[c], s_exact);
+                    sh.sel = !(Wt > 0.0 && kScanRel * (double)flips <= kFusedTol * Wt);
+                    sh.C = s_exact;                           // the coefficient of the repeated sweep
+                    sh.S_exact = s_exact;
+                }
+                __syncwarp();
+                fetch_ahead();
+            }
+            if (in_regs) {                                    // (each thread its own values: nothing to wait for)
+#pragma unroll
+                for (int i = 0; i < kTile; ++i) {
+                    er[i] = i < per_thr ? se[i * kWalkThreads] : 0.0;
+                    qr[i] = i < per_thr ? sq[i * kWalkThreads] : 0.f;
                 }
             }
             __syncthreads();
-            fused_done = !sh.fused_fallback;
-            // (the exact sum is taken from the exchange's result, which nothing rewrites before the next
-            // exchange; thread 0 may already be changing the walk's state)
-            if (fused_done) last_a = f.v[1] * (1.0 / sh.tot5[0]) - cp * f.v[2];
+            again = sh.sel != 0;
+            // this thread's share of that sum (nothing rewrites S_exact before the next first rejection; thread 0 may
+            // already be changing the rest of the walk's state)
+            if (!again) last_a = v[1] - (sh.S_exact - s_scan) * (double)__int_as_float(__double2hiint(v[3]));
         }
-        if (!fused_done) {
-            Sweep sw = sweep_chunk<MODE_RESID>(sh, x, q, se, sq, tid, nthr, lo, hi, vec, cache_ok, sh.have_e != 0,
-                                               sh.have_q != 0, sh.cprime, xt, false, 0, 0, 0, nullptr);
-            last_a = sw.a;
-            reduce_exchange(sw.a, sw.b);
-        }
-        // When this was the node's last child, the weights just summed (residual at the new
-        // coefficient, the rejected tokens at their frozen values) are the ones the bonus token is
-        // drawn from, thread by thread in the same order: the draw reuses the sums (last_a).
-        if (tid == 0) {
-            const double W = sh.tot[0], Dn = sh.tot[1];
-            double frozen;
-            if (W > 0.0) {
-                frozen = weight(sh.ex, sh.qx, sh.invS, sh.cprime);
-                sh.c = sh.cprime;
-                sh.U = W;
-                sh.bonus_ok = sh.req_last;
+        if (again) {
+            const double Cn = sh.C;
+            if (req == REQ_EXP) {
+                // exact softmax denominator of this node; thread 0 then repeats the test with it
+                last_a = sweep_row(MODE_EXP, sh, x, q, se, sq, kWalkThreads, ck, false, arg, 0.0, -1, 0.0, 0.0, nullptr);
+                got = GOT_SUM;
+            } else if (in_regs) {
+                if (xn >= ck.lo && xn < ck.hi) {
+#pragma unroll
+                    for (int i = 0; i < kTile; ++i) {
+                        er[i] = i == xn - ck.lo ? 0.0 : er[i];
+                        qr[i] = i == xn - ck.lo ? 0.f : qr[i];
+                    }
+                }
+                last_a = residual_of_tile(er, qr, per_thr, Cn);
+            } else if (cache_ok) {
+                last_a = parked_sweep(se, sq, kWalkThreads, ck, per_thr, Cn, xn);
             } else {
-                frozen = weight(sh.ex, sh.qx, sh.invS, sh.c);   // residual vanished: p is kept
+                last_a = sweep_row(MODE_RESID, sh, x, q, se, sq, kWalkThreads, ck, false, arg, Cn, xn, 0.0, 0.0, nullptr);
             }
-            if (sh.ridx < 0 && sh.nrem < MAXN) {
-                sh.rem_tok[sh.nrem] = xt;
-                sh.rem_frozen[sh.nrem] = frozen;
-                sh.nrem++;
-            }
-            if (Dn > 0.0) sh.D = Dn;
-            sh.have_q = cache_ok;
-            sh.rem.drop_first();                                // this child is done
+            double v[1] = {last_a};
+            exchange(v, fetch_ahead);
+            R = v[0];
         }
         // no barrier here: only thread 0 touches the walk's state until the next request is published
     }
+    if (sh.fail != 0) {
+        // a wait ran out: nobody leaves while a peer may still write to its shared memory
+        if (tid == 0) fspad_report(args.status, FSPAD_ERR_TIMEOUT);
+        cluster.sync();
+        return;
+    }
 
     // ---- bonus token: inverse CDF of the current residual at the last node ----
-    {
-        const int cur = sh.cur;
-        const float *x = lg + (size_t)cur * V;
-        const float *q = dp + (size_t)cur * V;
-        const double c = sh.c;
-        const bool have_e = sh.have_e != 0, have_q = sh.have_q != 0;
-        const int lane = tid & 31, wid = tid >> 5;
-
-        // block-wide scan of one value per thread (index order): this thread's exclusive and inclusive
-        // prefix, the CTA total in sh.warp_a[kWarps - 1] ... returned through `total` (valid in every thread)
-        auto block_scan = [&](double v, double &excl_out, double &incl_out, double &total) {
-            double incl = v;
+    const int cur = sh.cur;
+    const float *x = lg + (size_t)cur * V, *q = dp + (size_t)cur * V;
+    const double c = sh.C;
+    // A draw at a node where nothing was rejected (a leaf, typically) is taken from the softmax
+    // of the row itself.  The scan left the mass of every piece of the row, accurate to kScanRel:
+    // enough to name the piece the target falls into and the mass in front of it.  That piece is
+    // then swept with single-precision exponentials - by every CTA on its own, all on the same
+    // data with the same arithmetic, so all reach the same verdict and nothing is exchanged - and
+    // the token is taken when the target clears both ends of its interval by more than the
+    // uncertainty of all the approximations together.  Otherwise, and for every other kind of
+    // draw, the cluster sweeps the whole row exactly.
+    bool settled = false;
+    const int n_piece = sh.piece_cnt[cur];
+    if (!sh.bonus_ok && c == 0.0 && sh.nrem == 0 && n_piece > 0) {
+        // every warp scans the pieces' masses: prefix of the piece the target falls into
+        double cum = lane < n_piece ? (double)sh.piece_w[cur][lane & (kPieceSlots - 1)] : 0.0;
+        const double own = cum;
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const double t2 = __shfl_up_sync(0xffffffffu, incl, off);
-                if (lane >= off) incl += t2;
+        for (int off = 1; off < kPieceSlots; off <<= 1) {
+            const double t2 = __shfl_up_sync(0xffffffffu, cum, off);
+            if (lane >= off) cum += t2;
+        }
+        const double Zs = __shfl_sync(0xffffffffu, cum, n_piece - 1), target = (double)sh.ubonus * Zs;
+        const int pick = __ffs((int)__ballot_sync(0xffffffffu, lane < n_piece && cum > target)) - 1;
+        const double top = __shfl_sync(0xffffffffu, cum, max(pick, 0)), mass = __shfl_sync(0xffffffffu, own, max(pick, 0));
+        const double pre = top - mass;
+        // error budget: the masses in front of the piece and the total (scan, kScanRel each, doubled
+        // for slack) and the single-precision sums inside the piece (argument rounding of the
+        // exponential 1.3e-7 per unit of |log2 e_j|, the approximation itself 2.4e-7, the partial sums)
+        const double tol = 4.0 * kScanRel * Zs + 4e-6 * mass;
+        if (pick >= 0 && target - pre > tol && top - target > tol) {
+            int p_lo, p_hi;
+            piece_bounds(args.geom, b * N + cur, pick, V, &p_lo, &p_hi);
+            const int a_lo = p_lo - (int)(((row0 + cur) * V + p_lo) & 3);       // 16-byte aligned
+            const int pt = ((((p_hi - a_lo) + kWalkThreads - 1) / kWalkThreads) + 3) & ~3;
+            const int t_lo = min(p_hi, a_lo + tid * pt), t_hi = min(p_hi, t_lo + pt);
+            const float Mf = sh.rowM[cur];
+            // weights relative to the row maximum, as the table's: e_j = exp2((x_j - max) * log2(e) / T)
+            auto e32 = [&](float xv2) {
+                float y;
+                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((xv2 - Mf) * kT));
+                return xv2 == -INFINITY ? 0.f : y;
+            };
+            // (tokens of the piece only: what an aligned group of four holds before p_lo is left out)
+            auto in4 = [&](int j) {
+                if (j >= p_lo && j + 4 <= t_hi) return __ldg(reinterpret_cast<const float4 *>(x + j));
+                const int sh_lo = max(p_lo - j, 0);
+                float4 r = edge4(x + j, sh_lo > 0 ? -8 : 0, 0, -INFINITY);
+                if (sh_lo <= 0 && j < t_hi) r.x = x[j];
+                if (sh_lo <= 1 && j + 1 < t_hi) r.y = x[j + 1];
+                if (sh_lo <= 2 && j + 2 < t_hi) r.z = x[j + 2];
+                if (sh_lo <= 3 && j + 3 < t_hi) r.w = x[j + 3];
+                return r;
+            };
+            double mine = 0.0;
+#pragma unroll 1
+            for (int j = t_lo; j < t_hi; j += 4) {
+                const float4 xs = in4(j);
+                mine += (double)((e32(xs.x) + e32(xs.y)) + (e32(xs.z) + e32(xs.w)));
             }
-            const double prev_incl = __shfl_up_sync(0xffffffffu, incl, 1);
-            if (lane == 31) sh.warp_a[wid] = incl;
+            double E, total;
+            const double P = block_scan(sh, mine, &E, &total);
+            const double tgt = target - pre;                  // within the piece
+            if (tid == 0) { sh.sel = 0x7fffffff; sh.verdict = 2; }
             __syncthreads();
-            if (wid == 0) {
-                // exclusive scan of the warp totals; the last inclusive value is the CTA total
-                const int nwarps = nthr >> 5;
-                const double wv = (lane < nwarps) ? sh.warp_a[lane] : 0.0;
-                double sc = wv;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const double t2 = __shfl_up_sync(0xffffffffu, sc, off);
-                    if (lane >= off) sc += t2;
-                }
-                const double excl = __shfl_up_sync(0xffffffffu, sc, 1);
-                if (lane < nwarps) sh.warp_off[lane] = (lane == 0) ? 0.0 : excl;
-                if (lane == nwarps - 1) sh.warp_b[0] = sc;
-            }
+            if (P > tgt) atomicMin(&sh.sel, tid);
             __syncthreads();
-            const double woff = sh.warp_off[wid];
-            incl_out = woff + incl;
-            excl_out = (lane == 0) ? woff : woff + prev_incl;
-            total = sh.warp_b[0];
-        };
-
-        // A draw at a node where nothing was rejected (a leaf, typically) is taken from the softmax
-        // of the row itself.  The scan left the mass of every piece of the row, accurate to kScanRel:
-        // enough to name the piece the target falls into and the mass in front of it.  That piece is
-        // then swept with single-precision exponentials - by every CTA on its own, all on the same
-        // data with the same arithmetic, so all reach the same verdict and nothing is exchanged - and
-        // the token is taken when the target clears both ends of its interval by more than the
-        // uncertainty of all the approximations together.  Otherwise, and for every other kind of
-        // draw, the cluster sweeps the whole row exactly.
-        bool settled = false;
-        const int n_piece = (MAXN == 64) ? sh.piece_cnt[MAXN == 64 ? cur : 0] : 0;
-        if (!sh.bonus_ok && c == 0.0 && sh.nrem == 0 && n_piece > 0) {
-            double Zs = 0.0;
-            for (int i = 0; i < n_piece; ++i) Zs += sh.piece_w[MAXN == 64 ? cur : 0][i];
-            const double target = (double)sh.ubonus * Zs;
-            int pick = -1;
-            double pre = 0.0;
-            for (int i = 0; i < n_piece; ++i) {
-                const double nxt = pre + sh.piece_w[MAXN == 64 ? cur : 0][i];
-                if (nxt > target) { pick = i; break; }
-                pre = nxt;
-            }
-            // error budget: the masses in front of the piece and the total (scan, kScanRel each, doubled
-            // for slack) and the single-precision sums inside the piece (argument rounding of the
-            // exponential 1.3e-7 per unit of |log2 e_j|, the approximation itself 2.4e-7, the partial sums)
-            const double tol = 4.0 * kScanRel * Zs + (pick >= 0 ? 4e-6 * sh.piece_w[MAXN == 64 ? cur : 0][pick] : 0.0);
-            if (pick >= 0 && target - pre > tol && pre + sh.piece_w[MAXN == 64 ? cur : 0][pick] - target > tol) {
-                // token range of that piece: CTA `first + pick` of the scan, clipped to the row
-                const FspadStatsGeom &g = args.geom;
-                const long long row_lo = (long long)(b * N + cur) * g.upr;
-                const long long first = row_lo / g.chunk;
-                const long long u_lo = max(row_lo, (first + pick) * g.chunk), u_hi = min(row_lo + g.upr, (first + pick + 1) * g.chunk);
-                const int p_lo = (int)(u_lo - row_lo) * g.unit, p_hi = (int)(u_hi - row_lo) * g.unit;
-                const int pt = ((((p_hi - p_lo) + nthr - 1) / nthr) + 3) & ~3;
-                const int t_lo = min(p_hi, p_lo + tid * pt), t_hi = min(p_hi, t_lo + pt);
-                const float Mf = sh.rowM[cur];
-                // weights relative to the row maximum, as the table's: e_j = exp2((x_j - max) * log2(e) / T)
-                auto e32 = [&](float xv2) {
-                    float y;
-                    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((xv2 - Mf) * kT));
-                    return xv2 == -INFINITY ? 0.f : y;
-                };
-                double mine = 0.0;
-                for (int j = t_lo; j < t_hi; j += 4) {
-                    float xs[4];
-                    if (vec && j + 4 <= t_hi) {
-                        const float4 t4 = __ldg(reinterpret_cast<const float4 *>(x + j));
-                        xs[0] = t4.x; xs[1] = t4.y; xs[2] = t4.z; xs[3] = t4.w;
-                    } else {
-#pragma unroll
-                        for (int t2 = 0; t2 < 4; ++t2) xs[t2] = (j + t2 < t_hi) ? x[j + t2] : -INFINITY;
-                    }
-                    mine += (double)((e32(xs[0]) + e32(xs[1])) + (e32(xs[2]) + e32(xs[3])));
-                }
-                double E, P, total;
-                block_scan(mine, E, P, total);
-                const double tgt = target - pre;                  // within the piece
-                if (tid == 0) { sh.sel = 0x7fffffff; sh.verdict[0] = 2; }
-                __syncthreads();
-                if (P > tgt) atomicMin(&sh.sel, tid);
-                __syncthreads();
-                if (tid == sh.sel) {
-                    double run = E;
-                    for (int j = t_lo; j < t_hi; ++j) {
-                        const double before = run;
-                        run += (double)e32(x[j]);
-                        if (run > tgt) {
-                            if (tgt - before > tol && run - tgt > tol) {
-                                sh.verdict[0] = 1;
-                                if (rank == 0) args.bonus[b] = j;
-                            }
-                            break;
+            if (tid == sh.sel) {
+                double run = E;
+#pragma unroll 1
+                for (int j = max(t_lo, p_lo); j < t_hi; ++j) {
+                    const double before = run;
+                    run += (double)e32(x[j]);
+                    if (run > tgt) {
+                        if (tgt - before > tol && run - tgt > tol) {
+                            sh.verdict = 1;
+                            if (rank == 0) args.bonus[b] = j;
                         }
+                        break;
                     }
                 }
-                __syncthreads();
-                settled = sh.verdict[0] == 1;
             }
+            __syncthreads();
+            settled = sh.verdict == 1;                        // uniform over the cluster
         }
-        if (rank == 0) {
-            if (tid == 0) args.n_acc[b] = sh.len;
-            for (int i = tid; i < args.path_stride; i += nthr) out_path[i] = (i < sh.len) ? sh.path[i] : -1;
-        }
-        compact_accepted(args, sh, b, rank, C, tid, nthr);   // the path is final; only the bonus token may still be open
-        if (settled) return;                                // uniform over the cluster; no peer memory is touched after the walk's last exchange
-
-        // ---- exact draw over the whole row: every CTA a contiguous slice, every thread a contiguous chunk ----
-        {
-            // with nothing rejected at this node (c == 0) the weights are the e_j themselves and the
-            // denominator cancels, so no separate exact-sum sweep is needed
-            Sweep sw{last_a, 0.0};
-            if (!sh.bonus_ok)
-                sw = sweep_chunk<MODE_CDF>(sh, x, q, se, sq, tid, nthr, lo, hi, vec, cache_ok, have_e, have_q, c, -1, false, 0, 0,
-                                           0, nullptr);
-            double E, P, total;
-            block_scan(sw.a, E, P, total);
-            // the CTA total goes to every CTA of the cluster (remote stores; read locally after the barrier)
-            if (tid < C) *cluster.map_shared_rank(&sh.cta_total[0][rank], tid) = total;
-            cluster.sync();
-            double Z = 0.0, base = 0.0;
-            for (int r = 0; r < C; ++r) {
-                if (r == rank) base = Z;
-                Z = Z + sh.cta_total[0][r];
-            }
-            const double target = (double)sh.ubonus * Z;
-            int owner = -1;
-            {
-                double cum = 0.0;
-                for (int r = 0; r < C; ++r) {
-                    cum = cum + sh.cta_total[0][r];
-                    if (cum > target) { owner = r; break; }
-                }
-            }
-            if (owner == rank) {
-                // the first thread (index order) whose inclusive prefix passes the target owns the draw
-                if (tid == 0) sh.sel = 0x7fffffff;
-                __syncthreads();
-                if (base + P > target) atomicMin(&sh.sel, tid);
-                __syncthreads();
-                // rounding of the two-level prefix can leave no thread above the target although the
-                // CTA total is: the last non-empty chunk then takes the draw
-                if (tid == 0 && sh.sel == 0x7fffffff) sh.sel = max(0, (cta_hi - cta_lo - 1) / per_thr);
-                __syncthreads();
-                if (tid == sh.sel) {
-                    int found = -1;
-                    sweep_chunk<MODE_CDF>(sh, x, q, se, sq, tid, nthr, lo, hi, vec, false, cache_ok, cache_ok && (c != 0.0),
-                                          c, -1, true, base, E, target, &found);
-                    if (found < 0) found = min(lo, V - 1);
-                    args.bonus[b] = found;
-                }
-            }
-            if (owner < 0 && rank == 0 && tid == 0) args.bonus[b] = 0;   // no positive weight anywhere
-        }
-        // no CTA touches a peer's shared memory after the cluster barrier above, so each may leave on its own
     }
+    if (rank == 0) {
+        if (tid == 0) args.n_acc[b] = sh.t.len;
+        int *out_path = args.path + (size_t)b * args.path_stride;
+#pragma unroll 1
+        for (int i = tid; i < args.path_stride; i += kWalkThreads) out_path[i] = (i < sh.t.len) ? sh.t.path[i] : -1;
+    }
+    if (!settled) {
+        // ---- exact draw over the whole row: every CTA a contiguous slice, every thread a contiguous chunk ----
+        const Chunk ck = chunk_of((row0 + cur) * V, V, per_cta, per_thr, rank, tid);
+        const ExpArg arg = exp_arg(sh.rowM[cur], invT, Tf);
+        const bool parked = sh.parked != 0;
+        // with nothing rejected at this node (c == 0) the weights are the e_j themselves and the
+        // denominator cancels, so no separate exact-sum sweep is needed
+        double mine = last_a;
+        if (sh.bonus_ok) {
+#pragma unroll 1
+            for (int k = 0; k < sh.nrem; ++k)
+                if (sh.rem_tok[k] >= ck.lo && sh.rem_tok[k] < ck.hi) mine += sh.rem_frozen[k];
+        } else {
+            mine = sweep_row(MODE_CDF, sh, x, q, se, sq, kWalkThreads, ck, parked, arg, c, -1, 0.0, 0.0, nullptr);
+        }
+        double E, total;
+        const double P = block_scan(sh, mine, &E, &total);
+        // the CTA total goes to every CTA of the cluster, as in exchange(); every warp waits for the peers' itself
+        const int par = n_exch & 1;
+        const uint32_t bar = smem_addr(&sh.bar[par]);
+        if (tid == 0) expect_bytes(bar, C * 8);
+        if (tid < C) send_double(smem_addr(&sh.slot[par][0][rank]), bar, tid, total);
+        if (!wait_cluster(bar, (uint32_t)(n_exch >> 1) & 1u)) {
+            fspad_report(args.status, FSPAD_ERR_TIMEOUT);
+            sh.fail = 1;
+        }
+        __syncwarp();
+        // every warp scans the CTA totals side by side: mass in front of this CTA, whole mass, owner of the target
+        double cum = (lane < C) ? sh.slot[par][0][lane & (kMaxCluster - 1)] : 0.0;
+#pragma unroll
+        for (int off = 1; off < kMaxCluster; off <<= 1) {
+            const double t2 = __shfl_up_sync(0xffffffffu, cum, off);
+            if (lane >= off) cum += t2;
+        }
+        const double Z = __shfl_sync(0xffffffffu, cum, C - 1), target = (double)sh.ubonus * Z;
+        const double before = __shfl_sync(0xffffffffu, cum, rank > 0 ? rank - 1 : 0);
+        const double base = rank > 0 ? before : 0.0;
+        const int owner = __ffs((int)__ballot_sync(0xffffffffu, lane < C && cum > target)) - 1;
+        if (owner == rank) {
+            // the first thread (index order) whose inclusive prefix passes the target owns the draw
+            if (tid == 0) sh.sel = 0x7fffffff;
+            __syncthreads();
+            if (base + P > target) atomicMin(&sh.sel, tid);
+            __syncthreads();
+            // rounding of the two-level prefix can leave no thread above the target although the
+            // CTA total is: the last non-empty chunk then takes the draw
+            const bool tail = sh.sel == 0x7fffffff && ck.lo < ck.hi && (tid == kWalkThreads - 1 || ck.hi == V || ck.hi - ck.lo < per_thr ||
+                                                                       (tid + 1) * per_thr >= per_cta);
+            if (tid == sh.sel || tail) {
+                int found = -1;
+                sweep_row(MODE_CDF, sh, x, q, se, sq, kWalkThreads, ck, parked, arg, c, -1, base + E, target, &found);
+                args.bonus[b] = found < 0 ? min(max(ck.lo, 0), V - 1) : found;
+            }
+        }
+        if (owner < 0 && rank == 0 && tid == 0) args.bonus[b] = 0;   // no positive weight anywhere
+    }
+    if (args.kv_cache != nullptr) compact_accepted(args, sh.t, b, rank, C, tid, kWalkThreads);   // (the CTAs that do not own the draw are at it meanwhile)
+    // every CTA has received every peer's total by now, so each may leave on its own - unless a wait ran out
+    __syncthreads();
+    if (sh.fail != 0) cluster.sync();
 }
 
 }  // namespace
@@ -978,22 +1323,21 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     a.N = N; a.V = V; a.path_stride = ctx->cfg.max_nodes; a.cache_ok = 0;
     a.path = path; a.n_acc = n_acc; a.bonus = bonus; a.status = ctx->d_status;
 
-    const bool sampling = draft != nullptr && uniforms != nullptr;
-    int cluster = 1, threads = 256;
-    size_t smem = 0;
-    if (sampling) {
-        threads = kWalkThreads;
-        cluster = walk_cluster_size(ctx, B, V);
-        const size_t per_cta = (size_t)((((V + cluster - 1) / cluster) + 3) & ~3);
-        const size_t per_thr = ((per_cta + kWalkThreads - 1) / kWalkThreads + 3) & ~(size_t)3;
-        const size_t need = per_thr * kWalkThreads * (sizeof(double) + sizeof(float));
-        if (need <= (size_t)(N <= 64 ? kSmemBudget : kSmemBudgetWide)) { smem = need; a.cache_ok = 1; }
-    }
     ctx->launches++;
-    // trees of up to 64 nodes (one mask word per node, per-piece masses kept for the bonus draw) and up to
-    // FSPAD_MAX_NODES_WIDE nodes are two instances of the kernel
+    if (draft == nullptr || uniforms == nullptr) {               // every sequence greedy
+        if (N <= FSPAD_MAX_NODES)
+            return fspad_launch(accept_greedy_kernel<FSPAD_MAX_NODES>, dim3((unsigned)B), dim3(kWalkThreads), 0, st, 0, a);
+        return fspad_launch(accept_greedy_kernel<FSPAD_MAX_NODES_WIDE>, dim3((unsigned)B), dim3(kWalkThreads), 0, st, 0, a);
+    }
+    const int cluster = walk_cluster_size(ctx, B, V);
+    const size_t per_cta = (size_t)((((V + 3 + cluster - 1) / cluster) + 3) & ~3);       // as the kernel shares a row out
+    const size_t per_thr = ((per_cta + kWalkThreads - 1) / kWalkThreads + 3) & ~(size_t)3;
+    const size_t need = per_thr * kWalkThreads * (sizeof(double) + sizeof(float));
+    size_t smem = 0;
+    if (need <= (size_t)(N <= 64 ? kSmemBudget : kSmemBudgetWide)) { smem = need; a.cache_ok = 1; }
+    // trees of up to 64 nodes and of up to FSPAD_MAX_NODES_WIDE nodes are two instances of the kernel
     if (N <= 64)
-        return fspad_launch(accept_walk_kernel<64>, dim3((unsigned)(B * cluster)), dim3(threads), smem, st, (unsigned)cluster, a);
-    return fspad_launch(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, dim3((unsigned)(B * cluster)), dim3(threads), smem, st,
+        return fspad_launch(accept_walk_kernel<64>, dim3((unsigned)(B * cluster)), dim3(kWalkThreads), smem, st, (unsigned)cluster, a);
+    return fspad_launch(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, dim3((unsigned)(B * cluster)), dim3(kWalkThreads), smem, st,
                         (unsigned)cluster, a);
 }

@@ -80,6 +80,7 @@ struct FspadStatsGeom {
     int slots;         // partial slots per row (capacity)
     long long chunk;   // units per CTA
     long long total;   // rows * upr
+    int per_row;       // > 0: ranges are cut at the rows, this many per row (the last may be shorter); 0: they may cross rows
     int threads;       // threads per CTA of the scan: FSPAD_STATS_THREADS, or half of it for a small array
 };
 
@@ -120,6 +121,7 @@ static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, boo
     const long long min_chunk = (g.upr + (slots - 2) - 1) / (slots - 2);
     if (g.chunk < min_chunk) g.chunk = min_chunk;
     g.n_cta = (int)((g.total + g.chunk - 1) / g.chunk);
+    g.per_row = g.upr % g.chunk == 0 ? (int)(g.upr / g.chunk) : 0;
     return g;
 }
 
@@ -165,61 +167,6 @@ __device__ __forceinline__ void fspad_stats_merge_warp(const FspadStatsPart *__r
     A = (a == 0x7fffffff) ? 0 : a;
 }
 
-// The same merge by a half-warp (16 lanes, up to four slots per lane), so that one warp
-// serves two rows at once.  Both halves of the warp must call it together; `valid` is false
-// for a half that has no row (it only takes part in the shuffles).  With `piece_w` given, the
-// mass of each of the row's pieces relative to the row maximum (what it adds to S) is stored
-// there, slot by slot, when the row has at most 16 pieces; *piece_cnt is the number of pieces,
-// or 0 when there are more than 16.
-__device__ __forceinline__ void fspad_stats_merge_half(const FspadStatsPart *__restrict__ parts,
-                                                       const FspadStatsGeom &g, int row, bool valid, float k,
-                                                       int lane16, float &M, double &S, int &A,
-                                                       double *piece_w = nullptr, int *piece_cnt = nullptr)
-{
-    int cnt = 0;
-    const FspadStatsPart *p = parts;
-    if (valid) {
-        const long long r0 = (long long)row * g.upr;
-        const int first = (int)(r0 / g.chunk), last = (int)((r0 + g.upr - 1) / g.chunk);
-        cnt = last - first + 1;
-        p = parts + (size_t)row * g.slots;
-    }
-    float mi[4], si[4];
-    int ai[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        mi[u] = -INFINITY; si[u] = 0.f; ai[u] = 0x7fffffff;
-        const int sl = lane16 + 16 * u;
-        if (sl < cnt) {
-            const int4 v = __ldcg(reinterpret_cast<const int4 *>(p + sl));
-            mi[u] = __int_as_float(v.x); si[u] = __int_as_float(v.y); ai[u] = v.z;
-        }
-    }
-    float m = mi[0];
-    int a = ai[0];
-#pragma unroll
-    for (int u = 1; u < 4; ++u)
-        if (mi[u] > m || (mi[u] == m && ai[u] < a)) { m = mi[u]; a = ai[u]; }
-#pragma unroll
-    for (int off = 8; off > 0; off >>= 1) {
-        const float om = __shfl_xor_sync(0xffffffffu, m, off, 16);
-        const int oa = __shfl_xor_sync(0xffffffffu, a, off, 16);
-        if (om > m || (om == m && oa < a)) { m = om; a = oa; }
-    }
-    double s = 0.0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const double w = (mi[u] != -INFINITY) ? (double)si[u] * (double)exp2f((mi[u] - m) * k) : 0.0;
-        s += w;
-        if (u == 0 && piece_w != nullptr && valid && lane16 < cnt && cnt <= 16) piece_w[lane16] = w;
-    }
-    if (piece_cnt != nullptr && valid && lane16 == 0) *piece_cnt = (cnt <= 16) ? cnt : 0;
-#pragma unroll
-    for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off, 16);
-    M = m;
-    S = s;
-    A = (a == 0x7fffffff) ? 0 : a;
-}
 #endif
 
 // ---- programmatic dependent launch -----------------------------------------------------

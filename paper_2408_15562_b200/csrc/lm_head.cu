@@ -321,24 +321,22 @@ lm_head_merge_kernel(const FspadStatsPart *__restrict__ tile_parts, int R, int n
                      FspadStatsPart *__restrict__ out_parts, float *__restrict__ row_max, double *__restrict__ row_sum,
                      int *__restrict__ row_arg)
 {
-    fspad_pdl_trigger();
+    // Wait first, then let the successor start: the acceptance walk reads logits in its prologue, and they are complete
+    // only when the product kernel is.
     fspad_pdl_wait();
+    fspad_pdl_trigger();
     const int lane = threadIdx.x & 31;
     const long long wi = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
     const bool as_rows = out_parts == nullptr;
-    const int per_row = as_rows ? 1 : g.slots;
+    const int per_row = as_rows ? 1 : g.per_row;
     if (wi >= (long long)R * per_row) return;
     const int r = (int)(wi / per_row), p = (int)(wi % per_row);     // r: row inside this slab
     const int grow = row0 + r;                                       // row in the caller's numbering
     int t0 = 0, t1 = n_tiles;
     if (!as_rows) {
-        // piece p of the row in the flat geometry: units [max(row_lo, (first+p) chunk), min(row_hi, (first+p+1) chunk))
-        const long long row_lo = (long long)grow * g.upr, row_hi = row_lo + g.upr;
-        const long long first = row_lo / g.chunk;
-        const long long u_lo = max(row_lo, (first + p) * g.chunk), u_hi = min(row_hi, (first + p + 1) * g.chunk);
-        if (u_lo >= u_hi) return;                                    // the row has fewer pieces
-        t0 = (int)((u_lo - row_lo) / tile_units);
-        t1 = (int)((u_hi - row_lo + tile_units - 1) / tile_units);
+        const int tiles = (int)(g.chunk / tile_units);               // pieces are whole tiles, the last may be shorter
+        t0 = p * tiles;
+        t1 = min(n_tiles, t0 + tiles);
     }
     float T = temperature ? temperature[grow / rows_per_seq] : 1.0f;
     if (!(T > 0.0f)) T = 1.0f;
@@ -394,8 +392,8 @@ lm_head_merge_kernel(const FspadStatsPart *__restrict__ tile_parts, int R, int n
 
 int fspad_lm_head_tiles(int V) { return (V + lmh::BN - 1) / lmh::BN; }
 
-// Geometry under which the walk reads the merged partials: pieces of whole tiles, at most 16 per row,
-// when the rows are whole numbers of tiles; one piece per row otherwise.
+// Geometry under which the walk reads the merged partials: pieces of whole tiles, at most 14 per row (the walk keeps the
+// masses of 16), cut at the rows; the last piece of a row may be shorter.
 FspadStatsGeom fspad_lm_head_geom(int rows, int V, bool vec, int slots)
 {
     FspadStatsGeom g;
@@ -404,15 +402,10 @@ FspadStatsGeom fspad_lm_head_geom(int rows, int V, bool vec, int slots)
     g.slots = slots;
     g.total = (long long)rows * g.upr;
     g.threads = FSPAD_STATS_THREADS;            // no scan kernel runs on this geometry; the walk reads the pieces only
-    const int tile_units = lmh::BN / g.unit;
-    if (V % lmh::BN == 0) {
-        const int n_tiles = V / lmh::BN;
-        const int tp = (n_tiles + 13) / 14;               // tiles per piece: a row then spans at most 16 pieces
-        g.chunk = (long long)tp * tile_units;
-    } else {
-        g.chunk = g.upr;
-    }
-    g.n_cta = (int)((g.total + g.chunk - 1) / g.chunk);
+    const int n_tiles = fspad_lm_head_tiles(V), tiles = (n_tiles + 13) / 14;
+    g.chunk = (long long)tiles * (lmh::BN / g.unit);
+    g.per_row = (n_tiles + tiles - 1) / tiles;
+    g.n_cta = rows * g.per_row;
     return g;
 }
 
@@ -460,7 +453,7 @@ cudaError_t fspad_launch_lm_head(fspad_ctx *ctx, const fspad_bf16 *hidden, const
         ctx->launches++;
         const bool as_rows = walk_geom == nullptr;
         FspadStatsGeom g = as_rows ? FspadStatsGeom() : *walk_geom;
-        const long long warps = (long long)rs * (as_rows ? 1 : g.slots);
+        const long long warps = (long long)rs * (as_rows ? 1 : g.per_row);
         e = fspad_launch(lmh::lm_head_merge_kernel, dim3((unsigned)((warps + 3) / 4)), dim3(128), 0, st, 0,
                          (const FspadStatsPart *)ctx->lm_parts, rs, n_tiles, rows_per_seq, temperature, r0, g,
                          as_rows ? 1 : lmh::BN / g.unit, as_rows ? (FspadStatsPart *)nullptr : ctx->st_part, row_max, row_sum,
