@@ -297,23 +297,6 @@ __device__ __forceinline__ Chunk chunk_of(size_t row_start, int V, int per_cta, 
     const int u = min(end, rank * per_cta + tid * per_thr);
     return Chunk{u - ph, min(V, min(end, u + per_thr) - ph)};
 }
-// positions j .. j + 3 where some lie outside the row
-__device__ __noinline__ float4 edge4(const float *__restrict__ x, int j, int hi, float pad)
-{
-    float4 r = make_float4(pad, pad, pad, pad);
-    if (j >= 0 && j < hi) r.x = x[j];
-    if (j + 1 >= 0 && j + 1 < hi) r.y = x[j + 1];
-    if (j + 2 >= 0 && j + 2 < hi) r.z = x[j + 2];
-    if (j + 3 >= 0 && j + 3 < hi) r.w = x[j + 3];
-    return r;
-}
-__device__ __forceinline__ float4 load4(const float *__restrict__ x, int j, int hi, float pad)
-{
-    if (j >= 0 && j + 4 <= hi) return __ldg(reinterpret_cast<const float4 *>(x + j));
-    if (j + 4 <= 0 || j >= hi) return make_float4(pad, pad, pad, pad);
-    return edge4(x, j, hi, pad);
-}
-
 enum { MODE_EXP = 0, MODE_RESID = 1, MODE_CDF = 2 };
 
 // The sweeps that are not on the usual path, over this thread's chunk, from the arrays in global memory or, with
@@ -345,11 +328,11 @@ __device__ __noinline__ double sweep_row(int mode, const Shared &sh, const float
                 qv[t] = (double)sq[(j - ck.lo + t) * stride];
             }
         } else {
-            const float4 xs = load4(x, j, ck.hi, -INFINITY);
+            const float4 xs = fspad_load4(x, j, ck.hi, -INFINITY);
             ev[0] = exp_neg(xs.x, arg, sh.exp_tbl); ev[1] = exp_neg(xs.y, arg, sh.exp_tbl);
             ev[2] = exp_neg(xs.z, arg, sh.exp_tbl); ev[3] = exp_neg(xs.w, arg, sh.exp_tbl);
             if (C != 0.0) {
-                const float4 qs = load4(q, j, ck.hi, 0.f);
+                const float4 qs = fspad_load4(q, j, ck.hi, 0.f);
                 qv[0] = (double)qs.x; qv[1] = (double)qs.y; qv[2] = (double)qs.z; qv[3] = (double)qs.w;
             }
         }
@@ -462,13 +445,13 @@ __device__ __forceinline__ void fused_reject_sweep(const Shared &sh, const float
     }
     v[0] = v[1] = v[2] = 0.0;
     float qp = 0.f, flips = 0.f;
-    float4 x4 = load4(x, ck.lo, ck.hi, -INFINITY), q4 = load4(q, ck.lo, ck.hi, 0.f);
+    float4 x4 = fspad_load4(x, ck.lo, ck.hi, -INFINITY), q4 = fspad_load4(q, ck.lo, ck.hi, 0.f);
 #pragma unroll 1
     for (int k = 0; k < per_thr; k += 4) {
         float4 xn = x4, qn = q4;
         if (k + 4 < per_thr) {
-            xn = load4(x, ck.lo + k + 4, ck.hi, -INFINITY);
-            qn = load4(q, ck.lo + k + 4, ck.hi, 0.f);
+            xn = fspad_load4(x, ck.lo + k + 4, ck.hi, -INFINITY);
+            qn = fspad_load4(q, ck.lo + k + 4, ck.hi, 0.f);
         }
         double ev[4] = {exp_neg(x4.x, arg, sh.exp_tbl), exp_neg(x4.y, arg, sh.exp_tbl), exp_neg(x4.z, arg, sh.exp_tbl),
                         exp_neg(x4.w, arg, sh.exp_tbl)};
@@ -1160,7 +1143,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             auto in4 = [&](int j) {
                 if (j >= p_lo && j + 4 <= t_hi) return __ldg(reinterpret_cast<const float4 *>(x + j));
                 const int sh_lo = max(p_lo - j, 0);
-                float4 r = edge4(x + j, sh_lo > 0 ? -8 : 0, 0, -INFINITY);
+                float4 r = fspad_edge4(x + j, sh_lo > 0 ? -8 : 0, 0, -INFINITY);
                 if (sh_lo <= 0 && j < t_hi) r.x = x[j];
                 if (sh_lo <= 1 && j + 1 < t_hi) r.y = x[j + 1];
                 if (sh_lo <= 2 && j + 2 < t_hi) r.z = x[j + 2];

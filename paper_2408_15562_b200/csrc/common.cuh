@@ -56,6 +56,7 @@ struct fspad_ctx {
     int fs_attr_done;         // dynamic shared-memory limit raised for the Feature Sampler's product kernel
 
     void *dx_part;            // draft step: per-piece top-k lists [max_batch * 16 rows][pieces][16] (value, token)
+    int *dx_done;             // draft step: finished pieces of each sequence [max_batch]; zero between calls
 
     // device staging for the host entry point (h_ready: every buffer below is allocated)
     int h_ready;
@@ -126,6 +127,25 @@ static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, boo
 }
 
 #ifdef __CUDACC__
+// ---- rows read 16 bytes at a time whatever their length ----
+// Positions j .. j + 3 of a row whose valid positions are [0, hi); x + j is 16-byte aligned.  A group that reaches past either
+// end is read element by element (nothing outside the row is touched), with `pad` for the rest.
+static __device__ __noinline__ float4 fspad_edge4(const float *__restrict__ x, int j, int hi, float pad)
+{
+    float4 r = make_float4(pad, pad, pad, pad);
+    if (j >= 0 && j < hi) r.x = x[j];
+    if (j + 1 >= 0 && j + 1 < hi) r.y = x[j + 1];
+    if (j + 2 >= 0 && j + 2 < hi) r.z = x[j + 2];
+    if (j + 3 >= 0 && j + 3 < hi) r.w = x[j + 3];
+    return r;
+}
+__device__ __forceinline__ float4 fspad_load4(const float *__restrict__ x, int j, int hi, float pad)
+{
+    if (j >= 0 && j + 4 <= hi) return __ldg(reinterpret_cast<const float4 *>(x + j));
+    if (j + 4 <= 0 || j >= hi) return make_float4(pad, pad, pad, pad);
+    return fspad_edge4(x, j, hi, pad);
+}
+
 // Merge the per-CTA partials of one row (warp-collective: all 32 lanes call it and all get
 // the result): maximum, its lowest index, and the sum of exponentials rescaled to that
 // maximum (k = log2(e)/T).  Every lane fetches up to two partial slots, so the loads of a

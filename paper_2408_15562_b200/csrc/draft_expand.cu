@@ -2,168 +2,258 @@
 // paragraph: the output of each draft step is truncated to its top-k and every
 // token carries the joint probability of its path).
 //
-// Three small kernels per call:
-//   1. draft_topk_partial_kernel - grid (pieces of 4096 tokens, rows): the top-k of the
-//      piece from one pass: a lower bound of the k-th largest value from the half-warp
-//      maxima, the few tokens that reach it listed in shared memory and ranked by
-//      counting; the one HBM pass over the rows.
-//   2. draft_topk_row_kernel - one CTA per row: the pieces' lists (at most 1024
-//      entries) through the sorting network; the first k become candidates
-//      base + f k + r with the frontier node as parent and the joint
-//      log-probability frontier_logp + value, one single-precision addition.
-//   3. draft_frontier_kernel - one CTA per sequence: the F k new joint values
-//      through the network; the first `width` are the next frontier.
+// One kernel per call, grid (pieces of a row, rows):
+//   1. every CTA streams its piece: the half-warp maxima of the first 4096 tokens give a lower
+//      bound of the piece's k-th largest value, the tokens that reach it are listed in
+//      shared memory, and the list's members are ranked by counting; the one HBM pass over the rows;
+//   2. the CTA that finishes a sequence's last piece (told by a counter per sequence that it then puts back to zero; nobody
+//      waits for anybody) takes one warp to a row and ranks the pieces' lists the same way; the first k
+//      become candidates base + f k + r with the frontier node as parent and the joint
+//      log-probability frontier_logp + value, one single-precision addition;
+//   3. it ranks the F k new joint values; the first `width` are the next frontier.
 // Comparisons and one addition only, so every decision is the oracle's bit for bit.
+//
+// What bounds it: HBM with many rows, otherwise a chain of latencies.  As three kernels (one CTA per 4096 tokens, then a
+// 1024-entry sorting network per row, then one per sequence) a level of ten rows took 15 us at V = 32000 and 40 us with
+// 16 sequences at V = 128256 (82 MB); now 8.5 and 23.  Pieces are as long as one wave of four CTAs per SM allows (a short piece
+// pays the ranking for few tokens), and at most 16 per row, so that the lists merged for a row stay short.
 #include "common.cuh"
-#include "sort_network.cuh"
+#include "sort_key.cuh"
 
 namespace {
 
-constexpr int kThreads = kSortThreads;                 // 256
-constexpr int kPerThread = 16;                         // tokens per thread in the partial kernel
-constexpr int kPiece = kThreads * kPerThread;          // 4096 tokens per CTA
+constexpr int kThreads = 512;                          // one warp for each of a sequence's up to 16 rows
+constexpr int kPerThread = 8;                         // tokens per thread and round
+constexpr int kRound = kThreads * kPerThread;          // 4096 tokens
+constexpr int kKeep = 512;                             // longest list that is ranked by counting
+constexpr int kMaxPieces = 16;
 
-// The top-k of one piece of one row.  The k-th largest of the 16 half-warp maxima is a lower bound of
-// the piece's k-th largest value, because k tokens at least that large exist; every token whose value
-// reaches the bound goes to a shared list (a few dozen entries on ordinary data, the whole piece at
-// worst) as a 64-bit key (order-preserving image of the value, complemented token index: larger key
-// = larger value, or equal value and lower token), and the list's members are ranked by counting.
-// One pass over the data: per token one maximum and one comparison.
-__global__ void __launch_bounds__(kThreads)
-draft_topk_partial_kernel(const float *__restrict__ logprobs, int V, int k, int pieces, uint2 *__restrict__ part)
+struct DraftArgs {
+    const float *logprobs, *frontier_logp;
+    const int *frontier_cand;
+    int V, F, k, width, base, cap, pieces, len;        // len: tokens of a piece (a multiple of kRound / 4)
+    uint2 *part;                                       // [rows][pieces][k] (value, token)
+    int *seq_done;                                     // pieces of a sequence's rows that have finished
+    int *cand_parent, *cand_token;
+    float *cand_logp;
+    int *next_cand;
+    float *next_logp;
+};
+
+struct DraftShared {
+    unsigned long long list[kKeep + kRound];           // keys of the tokens that reach the bound
+    unsigned long long top[FSPAD_MAX_FRONTIER];
+    float hmax[kThreads / 16];
+    float joint[FSPAD_MAX_FRONTIER * FSPAD_MAX_FRONTIER];
+    float bound;
+    int cnt, n, hits, last;
+};
+
+// The list cut to its k largest keys (a list of more than kKeep: ascending or constant values).  The k-th largest key is
+// found bit by bit: 64 counts, whatever the list holds.
+__device__ __noinline__ void cut_list(DraftShared &s, int k, int tid)
 {
-    __shared__ unsigned long long s_list[kPiece];               // tokens whose value reaches the bound
-    __shared__ float s_hmax[kThreads / 16];
-    __shared__ float s_bound;
-    __shared__ int s_cnt;
+    const int n = s.cnt;
+    unsigned long long t = 0ull;
+    for (int bit = 63; bit >= 0; --bit) {
+        const unsigned long long with = t | (1ull << bit);
+        int c = 0;
+        for (int i = tid; i < n; i += kThreads) c += s.list[i] >= with ? 1 : 0;
+        if (tid == 0) s.hits = 0;
+        __syncthreads();
+        if (c) atomicAdd(&s.hits, c);
+        __syncthreads();
+        if (s.hits >= k) t = with;
+        __syncthreads();
+    }
+    if (tid == 0) s.n = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += kThreads)
+        if (s.list[i] >= t) s.top[atomicAdd(&s.n, 1)] = s.list[i];       // keys differ: exactly k of them
+    __syncthreads();
+    if (tid < k) s.list[tid] = s.top[tid];
+    if (tid == 0) { s.cnt = k; s.bound = fspad_key_value(t); }
+    __syncthreads();
+}
+
+// place of key `me` among the n keys of the list
+__device__ __forceinline__ int rank_of(const unsigned long long *list, int n, unsigned long long me)
+{
+    int rank = 0;
+#pragma unroll 4
+    for (int o = 0; o < n; ++o) rank += list[o] > me ? 1 : 0;
+    return rank;
+}
+
+__global__ void __launch_bounds__(kThreads, 4)
+draft_expand_kernel(const DraftArgs a)
+{
+    __shared__ DraftShared s;
     fspad_pdl_trigger();
     fspad_pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31;
-    const int piece = blockIdx.x, row = blockIdx.y;
-    const float *x = logprobs + (size_t)row * V;
-    const int e0 = piece * kPiece;
-    const bool vec = (V % 4 == 0) && ((reinterpret_cast<uintptr_t>(logprobs) & 15) == 0);
-    if (tid == 0) s_cnt = 0;
-    float val[kPerThread];                                       // positions past the row's end hold -inf
-    float bv = -INFINITY;
+    const int piece = blockIdx.x, row = blockIdx.y, V = a.V, k = a.k;
+    const float *x = a.logprobs + (size_t)row * V;
+    // Positions count from the 16-byte boundary at or before the row's first token: loads are aligned whatever V is.
+    const int ph = (int)((reinterpret_cast<uintptr_t>(x) >> 2) & 3);
+    const int lo = piece * a.len - ph, hi = min(V, lo + a.len);      // positions before token 0 and past `hi` are empty
+    const float *__restrict__ xp = x;
+    if (tid == 0) s.cnt = 0;
+    float4 cur[kPerThread / 4], nxt[kPerThread / 4];
+    auto fetch = [&](int e0, float4 (&v)[kPerThread / 4]) {
 #pragma unroll
-    for (int i = 0; i < kPerThread / 4; ++i) {
-        const int e = e0 + 4 * (i * kThreads + tid);
-        if (vec && e + 3 < V) {
-            const float4 t4 = __ldg(reinterpret_cast<const float4 *>(x + e));
-            val[4 * i] = t4.x; val[4 * i + 1] = t4.y; val[4 * i + 2] = t4.z; val[4 * i + 3] = t4.w;
-        } else {
+        for (int i = 0; i < kPerThread / 4; ++i) v[i] = fspad_load4(xp, e0 + 4 * (i * kThreads + tid), hi, -INFINITY);
+    };
+    // the tokens of one round that reach the bound go to the list (where there is room: the count goes on in any case)
+    auto push = [&](int e0) {
+        const float bound = s.bound;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) val[4 * i + c] = (e + c < V) ? x[e + c] : -INFINITY;
+        for (int i = 0; i < kPerThread / 4; ++i) {
+            const int tok = e0 + 4 * (i * kThreads + tid);
+            const float v4[4] = {cur[i].x, cur[i].y, cur[i].z, cur[i].w};
+            if (fmaxf(fmaxf(v4[0], v4[1]), fmaxf(v4[2], v4[3])) >= bound) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (v4[c] >= bound && tok + c >= 0 && tok + c < hi) {
+                        const int at = atomicAdd(&s.cnt, 1);
+                        if (at < kKeep + kRound) s.list[at] = fspad_sort_key(v4[c], (uint32_t)(tok + c));
+                    }
+            }
         }
+    };
+    fetch(lo, cur);
+    {
+        // The k-th largest of the 32 half-warp maxima is a lower bound of the piece's k-th largest value, because k
+        // tokens at least that large exist (a half-warp without any token reports -inf, which can only
+        // lower the bound and so lengthen the list, never lose a token).
+        float bv = -INFINITY;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) bv = fmaxf(bv, val[4 * i + c]);
+        for (int i = 0; i < kPerThread / 4; ++i) bv = fmaxf(fmaxf(bv, fmaxf(cur[i].x, cur[i].y)), fmaxf(cur[i].z, cur[i].w));
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) bv = fmaxf(bv, __shfl_xor_sync(0xffffffffu, bv, off));
+        if ((lane & 15) == 0) s.hmax[tid >> 4] = bv;
+        __syncthreads();
+        if (tid < kThreads / 16) {
+            const float me = s.hmax[tid];
+            int rank = 0;
+#pragma unroll
+            for (int o = 0; o < kThreads / 16; ++o) {
+                const float ot = s.hmax[o];
+                rank += (ot > me || (ot == me && o < tid)) ? 1 : 0;
+            }
+            if (rank == k - 1) s.bound = me;                     // k <= 16: exactly one thread
+        }
+        __syncthreads();
     }
-    // maxima of the 16 half-warps (a half-warp without any token reports -inf, which can only lower
-    // the bound and so lengthen the list, never lose a token)
+    for (int e0 = lo; e0 < hi; e0 += kRound) {
+        if (e0 + kRound < hi) fetch(e0 + kRound, nxt);
+        push(e0);
 #pragma unroll
-    for (int off = 8; off > 0; off >>= 1) bv = fmaxf(bv, __shfl_xor_sync(0xffffffffu, bv, off));
-    if ((lane & 15) == 0) s_hmax[tid >> 4] = bv;
+        for (int i = 0; i < kPerThread / 4; ++i) cur[i] = nxt[i];
+    }
     __syncthreads();
-    if (tid < kThreads / 16) {
-        const float me = s_hmax[tid];
-        int rank = 0;
-#pragma unroll
-        for (int o = 0; o < kThreads / 16; ++o) {
-            const float ot = s_hmax[o];
-            rank += (ot > me || (ot == me && o < tid)) ? 1 : 0;
+    if (s.cnt > kKeep + kRound) {                                // (uniform) ascending or constant values: once more, the list cut between rounds
+        __syncthreads();
+        if (tid == 0) s.cnt = 0;
+        for (int e0 = lo; e0 < hi; e0 += kRound) {
+            fetch(e0, cur);
+            __syncthreads();
+            push(e0);
+            __syncthreads();
+            if (s.cnt > kKeep) cut_list(s, k, tid);
         }
-        if (rank == k - 1) s_bound = me;                         // k <= 16: exactly one thread
+    } else if (s.cnt > kKeep) {
+        cut_list(s, k, tid);
     }
     __syncthreads();
-    const float bound = s_bound;
-#pragma unroll
-    for (int u = 0; u < kPerThread; ++u) {
-        if (val[u] >= bound) {
-            const int tok = e0 + 4 * ((u >> 2) * kThreads + tid) + (u & 3);
-            if (tok < V) s_list[atomicAdd(&s_cnt, 1)] = fspad_sort_key(val[u], (uint32_t)tok);
+    {
+        const int n = s.cnt;
+        uint2 *out = a.part + ((size_t)row * a.pieces + piece) * k;
+        for (int i = tid; i < n; i += kThreads) {
+            const unsigned long long me = s.list[i];
+            const int rank = rank_of(s.list, n, me);
+            if (rank < k) __stcg(out + rank, make_uint2(__float_as_uint(fspad_key_value(me)), fspad_key_index(me)));
         }
+        for (int r = n + tid; r < k; r += kThreads) __stcg(out + r, make_uint2(__float_as_uint(-INFINITY), 0x7fffffffu));   // empty slots
+    }
+    // ---- the last piece of the sequence ----
+    const int b = row / a.F;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        s.last = atomicAdd(a.seq_done + b, 1) == a.F * a.pieces - 1;
+        if (s.last) a.seq_done[b] = 0;
+        __threadfence();
     }
     __syncthreads();
-    const int n = s_cnt;
-    uint2 *out = part + ((size_t)row * pieces + piece) * k;
-    for (int i = tid; i < n; i += kThreads) {
-        const unsigned long long me = s_list[i];
-        int rank = 0;
-        for (int o = 0; o < n; ++o) rank += (s_list[o] > me) ? 1 : 0;
-        if (rank < k) out[rank] = make_uint2(__float_as_uint(fspad_key_value(me)), fspad_key_index(me));
-    }
-    for (int r = n + tid; r < k; r += kThreads) out[r] = make_uint2(__float_as_uint(-INFINITY), 0x7fffffffu);   // empty slots
-}
-
-// one row: partial lists -> top-k -> candidates
-__global__ void __launch_bounds__(kThreads)
-draft_topk_row_kernel(const uint2 *__restrict__ part, const float *__restrict__ frontier_logp,
-                      const int *__restrict__ frontier_cand, int F, int k, int pieces, int base, int cap,
-                      int *__restrict__ cand_parent, int *__restrict__ cand_token, float *__restrict__ cand_logp)
-{
-    __shared__ unsigned long long s_key[kSortEntries];
-    fspad_pdl_trigger();
-    fspad_pdl_wait();
-    const int tid = threadIdx.x, row = blockIdx.x;
-    const int b = row / F, f = row % F;
-    const int n = pieces * k;                                    // <= 1024 (checked on the host)
-    const uint2 *in = part + (size_t)row * n;
-    unsigned long long v[kSortPerThread];
+    if (s.last == 0) return;
+    // the pieces' lists of a row -> candidates, one warp to a row
+    const int n2 = a.pieces * k;                                     // at most 256: eight entries per lane
+    unsigned long long *list = s.list + (tid >> 5) * (kMaxPieces * FSPAD_MAX_FRONTIER);
+    for (int f = tid >> 5; f < a.F; f += kThreads / 32) {
+        const uint2 *in = a.part + (size_t)(b * a.F + f) * n2;
+        const float above = a.frontier_logp[b * a.F + f];
+        const int parent = a.frontier_cand[b * a.F + f];
+        uint2 e[kMaxPieces * FSPAD_MAX_FRONTIER / 32];
 #pragma unroll
-    for (int r = 0; r < kSortPerThread; ++r) {
-        const int i = kSortPerThread * tid + r;
-        unsigned long long key = 0ull;
-        if (i < n) {
-            const uint2 e = in[i];
-            if (e.y != 0x7fffffffu) key = fspad_sort_key(__uint_as_float(e.x), e.y);   // empty slots stay padding
+        for (int u = 0; u < kMaxPieces * FSPAD_MAX_FRONTIER / 32; ++u) {
+            e[u] = make_uint2(0u, 0x7fffffffu);
+            if (lane + 32 * u < n2) e[u] = __ldcg(in + lane + 32 * u);
         }
-        v[r] = key;
-    }
-    fspad_bitonic_sort_desc(v, s_key, tid);
+        // The lists are in descending order: at least k entries are as large as the smallest of the pieces' j-th, j = k / pieces
+        // rounded up.  What is below that needs no ranking.
+        uint2 jth = make_uint2(0u, 0x7fffffffu);
+        if (lane < a.pieces) jth = __ldcg(in + lane * k + (k + a.pieces - 1) / a.pieces - 1);
+        const uint32_t low = jth.y == 0x7fffffffu ? 0u : fspad_orderable(__uint_as_float(jth.x) + 0.0f);
+        const uint32_t bound = __reduce_min_sync(0xffffffffu, lane < a.pieces ? low : 0xffffffffu);
+        int n = 0;
 #pragma unroll
-    for (int r = 0; r < kSortPerThread; ++r) {
-        const int i = kSortPerThread * tid + r;
-        if (i < k && v[r] != 0ull) {
-            const size_t c = (size_t)b * cap + base + f * k + i;
-            cand_parent[c] = frontier_cand[row];
-            cand_token[c] = (int)fspad_key_index(v[r]);
-            cand_logp[c] = __fadd_rn(frontier_logp[row], fspad_key_value(v[r]));   // one fp32 addition
+        for (int u = 0; u < kMaxPieces * FSPAD_MAX_FRONTIER / 32; ++u) {
+            const unsigned long long key = e[u].y == 0x7fffffffu ? 0ull : fspad_sort_key(__uint_as_float(e[u].x), e[u].y);
+            const bool in_list = key != 0ull && (uint32_t)(key >> 32) >= bound;
+            const unsigned m = __ballot_sync(0xffffffffu, in_list);
+            if (in_list) list[n + __popc(m & ((1u << lane) - 1u))] = key;
+            n += __popc(m);
         }
+        __syncwarp();
+        if (lane < k) s.joint[f * k + lane] = -INFINITY;
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) {
+            const unsigned long long me = list[i];
+            const int rank = rank_of(list, n, me);
+            if (rank < k) {
+                const size_t c = (size_t)b * a.cap + a.base + f * k + rank;
+                const float v = __fadd_rn(above, fspad_key_value(me));    // one fp32 addition
+                a.cand_parent[c] = parent;
+                a.cand_token[c] = (int)fspad_key_index(me);
+                a.cand_logp[c] = v;
+                s.joint[f * k + rank] = v;
+            }
+        }
+        __syncwarp();
     }
-}
-
-// one sequence: F k new joint values -> next frontier
-__global__ void __launch_bounds__(kThreads)
-draft_frontier_kernel(const float *__restrict__ cand_logp, int n_new, int width, int base, int cap,
-                      int *__restrict__ next_cand, float *__restrict__ next_logp)
-{
-    __shared__ unsigned long long s_key[kSortEntries];
-    fspad_pdl_trigger();
-    fspad_pdl_wait();
-    const int tid = threadIdx.x, b = blockIdx.x;
-    const float *cl = cand_logp + (size_t)b * cap + base;
-    unsigned long long v[kSortPerThread];
-#pragma unroll
-    for (int r = 0; r < kSortPerThread; ++r) {
-        const int i = kSortPerThread * tid + r;
-        v[r] = (i < n_new) ? fspad_sort_key(cl[i], (uint32_t)i) : 0ull;
+    __syncthreads();
+    // the new joint values -> next frontier
+    const int n_new = a.F * k;                                       // at most 256: one entry per thread
+    unsigned long long me = 0ull;
+    if (tid < n_new) {
+        me = fspad_sort_key(s.joint[tid], (uint32_t)tid);
+        s.list[tid] = me;
     }
-    fspad_bitonic_sort_desc(v, s_key, tid);
-#pragma unroll
-    for (int r = 0; r < kSortPerThread; ++r) {
-        const int i = kSortPerThread * tid + r;
-        if (i < width) {
-            const int c = (int)fspad_key_index(v[r]);
-            next_cand[(size_t)b * width + i] = base + c;
-            next_logp[(size_t)b * width + i] = cl[c];
+    __syncthreads();
+    if (tid < n_new) {
+        const int rank = rank_of(s.list, n_new, me);
+        if (rank < a.width) {
+            a.next_cand[(size_t)b * a.width + rank] = a.base + tid;
+            a.next_logp[(size_t)b * a.width + rank] = s.joint[tid];
         }
     }
 }
 
 }  // namespace
 
-int fspad_draft_expand_pieces(int V) { return (V + kPiece - 1) / kPiece; }
+// pieces of 4096 tokens: the limit on vocabulary times k is stated in them
+int fspad_draft_expand_pieces(int V) { return (V + kRound - 1) / kRound; }
 
 cudaError_t fspad_launch_draft_expand(fspad_ctx *ctx, const float *logprobs, const float *frontier_logp,
                                       const int *frontier_cand, int F, int k, int width, int base, int cap, int B,
@@ -171,15 +261,25 @@ cudaError_t fspad_launch_draft_expand(fspad_ctx *ctx, const float *logprobs, con
                                       float *next_logp, cudaStream_t st)
 {
     if (B == 0) return cudaSuccess;
-    const int V = ctx->cfg.vocab, pieces = fspad_draft_expand_pieces(V), rows = B * F;
-    uint2 *part = reinterpret_cast<uint2 *>(ctx->dx_part);
-    ctx->launches += 3;
-    cudaError_t e = fspad_launch(draft_topk_partial_kernel, dim3(pieces, rows), dim3(kThreads), 0, st, 0, logprobs, V,
-                                 k, pieces, part);
-    if (e != cudaSuccess) return e;
-    e = fspad_launch(draft_topk_row_kernel, dim3(rows), dim3(kThreads), 0, st, 0, (const uint2 *)part, frontier_logp,
-                     frontier_cand, F, k, pieces, base, cap, cand_parent, cand_token, cand_logp);
-    if (e != cudaSuccess) return e;
-    return fspad_launch(draft_frontier_kernel, dim3(B), dim3(kThreads), 0, st, 0, (const float *)cand_logp, F * k,
-                        width, base, cap, next_cand, next_logp);
+    static_assert(kMaxPieces * FSPAD_MAX_FRONTIER <= kThreads && FSPAD_MAX_FRONTIER * FSPAD_MAX_FRONTIER <= kThreads,
+                  "the merged lists have at most one entry per thread");
+    DraftArgs a;
+    a.V = ctx->cfg.vocab;
+    const int rows = B * F;
+    int pieces = (int)((long long)ctx->sm_count * 4 / rows);         // one wave of four CTAs per SM
+    const int most = fspad_draft_expand_pieces(a.V);                 // about a round of 4096 tokens at least (and what `part` is sized for)
+    if (pieces > most) pieces = most;
+    if (pieces > kMaxPieces) pieces = kMaxPieces;
+    if (pieces < 1) pieces = 1;
+    const int quantum = kRound / 4;
+    a.len = (((a.V + 3 + pieces - 1) / pieces) + quantum - 1) / quantum * quantum;    // (up to three empty positions in front)
+    a.pieces = (a.V + 3 + a.len - 1) / a.len;
+    a.logprobs = logprobs; a.frontier_logp = frontier_logp; a.frontier_cand = frontier_cand;
+    a.F = F; a.k = k; a.width = width; a.base = base; a.cap = cap;
+    a.part = reinterpret_cast<uint2 *>(ctx->dx_part);
+    a.seq_done = ctx->dx_done;
+    a.cand_parent = cand_parent; a.cand_token = cand_token; a.cand_logp = cand_logp;
+    a.next_cand = next_cand; a.next_logp = next_logp;
+    ctx->launches++;
+    return fspad_launch(draft_expand_kernel, dim3(a.pieces, rows), dim3(kThreads), 0, st, 0, a);
 }

@@ -95,3 +95,22 @@ def test_host_detected_errors():
         ctx.draft_expand(lp, *args, 17, 4, 0, *arrs)         # top_k beyond 16
     with pytest.raises(binding.FspadError):
         ctx.draft_expand(lp, *args, 2, 5, 0, *arrs)          # width beyond the new candidates
+
+
+@pytest.mark.parametrize("vocab,batch,F,k,width", [(4095, 1, 1, 16, 16), (4096, 1, 16, 16, 40), (4097, 2, 3, 1, 3), (8193, 1, 2, 4, 8),
+                                                   (50257, 16, 10, 10, 10), (128256, 16, 16, 16, 256), (128256, 1, 1, 10, 10)])
+@pytest.mark.parametrize("order", ["random", "ascending", "constant"])
+def test_piece_lengths_and_long_lists(vocab, batch, F, k, width, order):
+    """One to sixteen pieces per row of one or several rounds of 4096 tokens, row starts at every alignment; ascending rows (every
+    token of a later round reaches the first round's bound, so the lists have to be cut) and constant ones (all are ties)."""
+    ctx = binding.Context(8, 2, vocab, 256, max_nodes=64, max_batch=batch)
+    rng = np.random.default_rng(vocab + F)
+    lp = rng.standard_normal((batch, F, vocab), dtype=np.float32)
+    if order == "ascending":
+        lp.sort(-1)
+    elif order == "constant":
+        lp[:] = -2.5
+    flp = rng.standard_normal((batch, F)).astype(np.float32)
+    fc = rng.integers(0, 5, (batch, F)).astype(np.int32)
+    for _ in range(2):                                       # the counters are back at zero after a call
+        _check(ctx, lp, flp, fc, k, width, 7, 7 + F * k)
