@@ -50,6 +50,7 @@ struct Args {
     int table_stride, n_blocks;
     float scale_log2;
     float *part_o, *part_ml;
+    fspad_bf16 *out;                    // one key range per row: the result itself, and no partials (NULL otherwise)
     int *status;
 };
 
@@ -414,12 +415,20 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             return (uint32_t)v;
         };
         const float scale = a.scale_log2;
+        const bool live = mt * BM + (warp & 3) * 32 < M;   // the last row tile may end before this warp's rows
         float m_run = -INFINITY, l_run = 0.f;
 
         for (int c = 0; c < n_ch; ++c) {
             const int ch = c0 + c, p = c & 1;
             const uint32_t tS = tmem + lanes + (uint32_t)p * 128u + (uint32_t)grp * 64u;   // scores, then P
             if (!failed && !mbar_wait(sfull(p), (uint32_t)(c >> 1) & 1u)) failed = true;
+            if (!live) {
+                // (no row of this warp exists: its scores are not looked at, and what its lanes' P holds stays in their
+                // own rows of O, which nobody stores)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(pfull(p));
+                continue;
+            }
             tc_fence_after();
             const bool masked = (ch + 1) * BK > L;   // only chunks that reach past the cached prefix
             // Validity of this group's 64 keys for this row as two 32-bit words: prefix keys are
@@ -521,6 +530,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         const bool any_fail = s_fail != 0;
         if (any_fail && tid == 0) fspad_report(a.status, FSPAD_ERR_TIMEOUT);
         const bool store = row_ok && !any_fail;
+        float *s_inv = reinterpret_cast<float *>(s_ml + 2 * BM);             // (the Q tile, too)
         const float2 ml0 = s_ml[row], ml1 = s_ml[BM + row];
         const float m_all = fmaxf(ml0.x, ml1.x);
         const float m_fin = (m_all == -INFINITY) ? 0.f : m_all;
@@ -543,16 +553,25 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             for (int j = 0; j < 32; j += 4)
                 *reinterpret_cast<float4 *>(ps + q2 * 32 + j) = make_float4(o[j], o[j + 1], o[j + 2], o[j + 3]);
         }
-        if (store && grp == 0) {
+        const float l_all = ml0.y * f0 + ml1.y * f1;
+        if (a.out != nullptr) {
+            if (grp == 0) s_inv[row] = l_all > 0.f ? 1.f / l_all : 0.f;
+        } else if (store && grp == 0) {
             float *ml = a.part_ml + (prow * M + gr) * 2;
             ml[0] = m_all;
-            ml[1] = ml0.y * f0 + ml1.y * f1;
+            ml[1] = l_all;
         }
         asm volatile("bar.sync 1, 256;\n" ::: "memory");   // the eight softmax warps
         if (!any_fail) {
             for (int r = warp; r < BM; r += 8) {
                 const int grr = mt * BM + r;
-                if (grr < M)
+                if (grr < M && a.out != nullptr) {
+                    const float4 o4 = *reinterpret_cast<const float4 *>(stg + r * SROW + lane * 4);
+                    const float inv = s_inv[r];
+                    const int nd = grr / G, hh = grr % G;
+                    *reinterpret_cast<uint2 *>(a.out + (((size_t)b * N + nd) * a.Hq + g * G + hh) * D + lane * 4) =
+                        make_uint2(pack_bf16(o4.x * inv, o4.y * inv), pack_bf16(o4.z * inv, o4.w * inv));
+                } else if (grr < M)
                     *reinterpret_cast<float4 *>(a.part_o + (prow * M + grr) * D + lane * 4) =
                         *reinterpret_cast<const float4 *>(stg + r * SROW + lane * 4);
             }
@@ -673,7 +692,7 @@ static bool make_plane_map(CUtensorMap *map, const fspad_bf16 *plane, size_t row
 cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 *kc,
                                          const fspad_bf16 *vc, const fspad_bf16 *tk, const fspad_bf16 *tv,
                                          const int *parent, const int *prefix_len, int N, int B, int n_splits,
-                                         float scale_log2, cudaStream_t st, FspadPaged paged)
+                                         float scale_log2, fspad_bf16 *out, cudaStream_t st, FspadPaged paged)
 {
     const fspad_config &c = ctx->cfg;
     umma::Args a;
@@ -685,7 +704,7 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     // (every CTA ranks all sequences itself, B loads each for B / 320 of its threads: kept to batches where that is small change)
     a.longest_first = (B > 1 && B <= 128 && (long long)B * c.n_kv_heads * a.mtiles * n_splits > ctx->sm_count) ? 1 : 0;
     a.scale_log2 = scale_log2;
-    a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.status = ctx->d_status;
+    a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.out = n_splits == 1 ? out : nullptr; a.status = ctx->d_status;
     if (!ctx->attn_attr_done) {
         cudaError_t e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              umma::SMEM_BYTES);
