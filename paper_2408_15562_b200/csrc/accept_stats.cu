@@ -75,15 +75,18 @@ template <> struct Unit<1> {
     static __device__ __forceinline__ int first_eq(const T &v, float bm, int j, int a) { return v == bm ? j : a; }
 };
 
-template <int UNIT, int kThreads>
+// SHIFT: rows of a length that is no multiple of 4, one piece of one row per CTA; position j of unit i is 4 i + j - (up to three),
+// aligned loads all the same (read float by float, 520 rows of 50257 took 39 us, now 23)
+template <int UNIT, bool SHIFT, int kThreads>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ temperature,
-                    int rows_per_seq, const FspadStatsGeom g, FspadStatsPart *__restrict__ parts)
+                    int rows_per_seq, int V, const FspadStatsGeom g, FspadStatsPart *__restrict__ parts)
 {
     typedef typename Unit<UNIT>::T U;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const long long lo = (long long)blockIdx.x * g.chunk;
-    const long long hi = min(g.total, lo + g.chunk);
+    const int piece = SHIFT ? (int)blockIdx.x % g.per_row : 0;
+    const long long lo = SHIFT ? ((long long)blockIdx.x / g.per_row) * g.upr + piece * g.chunk : (long long)blockIdx.x * g.chunk;
+    const long long hi = SHIFT ? lo - piece * g.chunk + min((long long)g.upr, (piece + 1) * g.chunk) : min(g.total, lo + g.chunk);
     __shared__ Acc wacc[kThreads / 32];
     __shared__ float s_bmax;
     __shared__ int s_barg;
@@ -101,17 +104,36 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
         const int n = (int)(seg_hi - seg_lo);                 // units in this piece of the row
         const int off = (int)(seg_lo - row_lo);               // position of the piece inside the row
         const U *px = reinterpret_cast<const U *>(logits) + seg_lo;
+        const float *xrow = logits + (size_t)row * V;         // SHIFT: unit i of this piece is xrow[j0 + 4 i ..], empty outside the row
+        const int j0 = SHIFT ? 4 * off - (int)(((size_t)row * V) & 3) : 0;
+        // units [i0, i1) lie inside the row; a first and a last one that do not are thread 0's and thread 32's to begin with
+        const int i0 = SHIFT && j0 < 0 ? 1 : 0, i1 = SHIFT ? min(n, (V - j0) >> 2) : n;
+        auto fetch = [&](int i) -> U {
+            if constexpr (SHIFT) return __ldg(reinterpret_cast<const U *>(xrow + j0) + i);
+            else return __ldg(px + i);
+        };
         float T = temperature ? temperature[row / rows_per_seq] : 1.0f;
         if (!(T > 0.0f)) T = 1.0f;
         const float k = kLog2e / T;
 
         // software pipeline: the next batch of loads is in flight while this one is reduced
         Acc p{-INFINITY, 0.f, 0x7fffffff};
+        int edge = -1;                                        // SHIFT: this thread's unit at an end of the row
+        if constexpr (SHIFT) {
+            if (tid == 0 && i0 > 0) edge = 0;
+            if (tid == 32 && i1 < n) edge = i1;
+            if (edge >= 0) {
+                const U v = fspad_edge4(xrow, j0 + 4 * edge, V, -INFINITY);
+                p.m = Unit<UNIT>::vmax(v);
+                p.s = p.m == -INFINITY ? 0.f : Unit<UNIT>::vsum(v, p.m, k);
+                p.a = -1;
+            }
+        }
         U cur[kDeep], nxt[kDeep];
 #pragma unroll
         for (int u = 0; u < kDeep; ++u) {
             const int i = u * kThreads + tid;
-            cur[u] = (i < n) ? __ldg(px + i) : Unit<UNIT>::pad();
+            cur[u] = (i >= i0 && i < i1) ? fetch(i) : Unit<UNIT>::pad();
         }
         for (int base = 0; base < n; base += kThreads * kDeep) {
             const int nb = base + kThreads * kDeep;
@@ -119,13 +141,13 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
 #pragma unroll
                 for (int u = 0; u < kDeep; ++u) {
                     const int i = nb + u * kThreads + tid;
-                    nxt[u] = (i < n) ? __ldg(px + i) : Unit<UNIT>::pad();
+                    nxt[u] = (i < i1) ? fetch(i) : Unit<UNIT>::pad();
                 }
             }
             float bm = Unit<UNIT>::vmax(cur[0]);
 #pragma unroll
             for (int u = 1; u < kDeep; ++u) bm = fmaxf(bm, Unit<UNIT>::vmax(cur[u]));
-            if (bm > p.m) {
+            if (bm > p.m || (SHIFT && p.a < 0 && bm == p.m)) {        // (an equal value in a batch comes before the row's last unit)
                 // only the batch is remembered; the position inside it is looked up once, at the
                 // end, by the threads that hold the block's maximum
                 p.s = (p.m == -INFINITY) ? 0.f : p.s * ex2((p.m - bm) * k);
@@ -170,19 +192,22 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
         if (my_m == bmax && bmax != -INFINITY) {
             // this thread's batch `my_base` holds the maximum: fetch it again (cache hit) and scan it
             int a = 0x7fffffff;
+            if constexpr (SHIFT)                              // (only a batch with a larger value has displaced it: it may hold the maximum too)
+                if (edge >= 0) a = Unit<UNIT>::first_eq(fspad_edge4(xrow, j0 + 4 * edge, V, -INFINITY), bmax, j0 + 4 * edge, a);
+            int b = 0x7fffffff;
 #pragma unroll
             for (int u = kDeep - 1; u >= 0; --u) {
                 const int i = my_base + u * kThreads + tid;
-                if (i < n) a = Unit<UNIT>::first_eq(__ldg(px + i), bmax, (off + i) * UNIT, a);
+                if (my_base >= 0 && i >= i0 && i < i1) b = Unit<UNIT>::first_eq(fetch(i), bmax, SHIFT ? j0 + 4 * i : (off + i) * UNIT, b);
             }
-            atomicMin(&s_barg, a);
+            atomicMin(&s_barg, min(a, b));
         }
         __syncthreads();
         if (tid == 0) {
-            const int first = (int)(row_lo / g.chunk);
+            const int slot = SHIFT ? piece : (int)(blockIdx.x - (int)(row_lo / g.chunk));
             FspadStatsPart out;
             out.m = wacc[0].m; out.s = wacc[0].s; out.a = s_barg; out.pad = 0;
-            parts[(size_t)row * g.slots + (blockIdx.x - first)] = out;
+            parts[(size_t)row * g.slots + slot] = out;
         }
         __syncthreads();
         seg_lo = seg_hi;
@@ -213,21 +238,20 @@ accept_stats_merge_kernel(const FspadStatsPart *__restrict__ parts, const FspadS
     }
 }
 
-cudaError_t launch_partials(const float *logits, const float *temperature, int rows_per_seq,
+template <int kT>
+cudaError_t launch_partials_t(const float *logits, const float *temperature, int rows_per_seq, int V, const FspadStatsGeom &g,
+                              FspadStatsPart *parts, cudaStream_t st, bool pdl)
+{
+    const dim3 grid(g.n_cta), block(kT);
+    if (g.shift) return fspad_launch_opt(pdl, accept_stats_kernel<4, true, kT>, grid, block, 0, st, 0, logits, temperature, rows_per_seq, V, g, parts);
+    if (g.unit == 4) return fspad_launch_opt(pdl, accept_stats_kernel<4, false, kT>, grid, block, 0, st, 0, logits, temperature, rows_per_seq, V, g, parts);
+    return fspad_launch_opt(pdl, accept_stats_kernel<1, false, kT>, grid, block, 0, st, 0, logits, temperature, rows_per_seq, V, g, parts);
+}
+cudaError_t launch_partials(const float *logits, const float *temperature, int rows_per_seq, int V,
                             const FspadStatsGeom &g, FspadStatsPart *parts, cudaStream_t st, bool pdl = true)
 {
-    if (g.threads == kThreads / 2) {
-        if (g.unit == 4)
-            return fspad_launch_opt(pdl, accept_stats_kernel<4, kThreads / 2>, dim3(g.n_cta), dim3(kThreads / 2), 0, st, 0, logits,
-                                    temperature, rows_per_seq, g, parts);
-        return fspad_launch_opt(pdl, accept_stats_kernel<1, kThreads / 2>, dim3(g.n_cta), dim3(kThreads / 2), 0, st, 0, logits,
-                                temperature, rows_per_seq, g, parts);
-    }
-    if (g.unit == 4)
-        return fspad_launch_opt(pdl, accept_stats_kernel<4, kThreads>, dim3(g.n_cta), dim3(kThreads), 0, st, 0, logits, temperature,
-                            rows_per_seq, g, parts);
-    return fspad_launch_opt(pdl, accept_stats_kernel<1, kThreads>, dim3(g.n_cta), dim3(kThreads), 0, st, 0, logits, temperature,
-                            rows_per_seq, g, parts);
+    return g.threads == kThreads / 2 ? launch_partials_t<kThreads / 2>(logits, temperature, rows_per_seq, V, g, parts, st, pdl)
+                                     : launch_partials_t<kThreads>(logits, temperature, rows_per_seq, V, g, parts, st, pdl);
 }
 
 }  // namespace
@@ -236,11 +260,11 @@ cudaError_t fspad_launch_stats_partials(fspad_ctx *ctx, const float *logits, con
                                         int rows, int rows_per_seq, int V, FspadStatsGeom *geom,
                                         cudaStream_t st, bool pdl, int sms)
 {
-    const bool vec = (V % 4 == 0) && ((reinterpret_cast<uintptr_t>(logits) & 15) == 0);
+    const bool aligned = (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
-    *geom = fspad_stats_geom(sms, rows, V, vec, ctx->stats_slots, true);
+    *geom = fspad_stats_geom(sms, rows, V, aligned, ctx->stats_slots, true);
     ctx->launches++;
-    return launch_partials(logits, temperature, rows_per_seq, *geom, ctx->st_part, st, pdl);
+    return launch_partials(logits, temperature, rows_per_seq, V, *geom, ctx->st_part, st, pdl);
 }
 
 cudaError_t fspad_launch_accept_stats(fspad_ctx *ctx, const float *logits, const float *temperature,
@@ -311,12 +335,12 @@ extern "C" int fspad_accept_stats_noalloc(const float *logits, const float *temp
         nd.scratch.store(scratch, std::memory_order_release);
     }
     cudaStream_t st = fspad_stream(stream);
-    const bool vec = (vocab % 4 == 0) && ((reinterpret_cast<uintptr_t>(logits) & 15) == 0);
-    const FspadStatsGeom g = fspad_stats_geom(nd.sm_count, rows, vocab, vec, kNoAllocSlots);
+    const bool aligned = (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
+    const FspadStatsGeom g = fspad_stats_geom(nd.sm_count, rows, vocab, aligned, kNoAllocSlots);
     FspadStatsPart *parts = reinterpret_cast<FspadStatsPart *>(scratch);
     // every slot the merge reads is rewritten by this call's first kernel, so the contents an
     // earlier call left in the shared array never need clearing
-    if (launch_partials(logits, temperature, rows_per_seq, g, parts, st) != cudaSuccess) return FSPAD_ERR_CUDA;
+    if (launch_partials(logits, temperature, rows_per_seq, vocab, g, parts, st) != cudaSuccess) return FSPAD_ERR_CUDA;
     return fspad_launch(accept_stats_merge_kernel, dim3((rows + 3) / 4), dim3(128), 0, st, 0,
                         (const FspadStatsPart *)parts, g, temperature, rows, rows_per_seq, row_max, row_sum,
                         (int *)row_arg) == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;

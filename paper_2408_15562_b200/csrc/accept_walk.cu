@@ -188,8 +188,9 @@ __device__ __noinline__ void piece_bounds(const FspadStatsGeom &g, int row, int 
         u_lo = max(0ll, (first + pick) * g.chunk - row_lo);
         u_hi = (first + pick + 1) * g.chunk - row_lo;
     }
-    *lo = (int)u_lo * g.unit;
-    *hi = (int)min((long long)V, u_hi * g.unit);
+    const int before = g.shift ? (int)(((size_t)row * V) & 3) : 0;         // positions in front of the row's first token
+    *lo = max(0, (int)u_lo * g.unit - before);
+    *hi = (int)min((long long)V, u_hi * g.unit - before);
 }
 
 // The scan's partials of one row, merged by eight lanes (slots lane, lane + 8 at once; any further ones in a loop).

@@ -76,7 +76,8 @@ struct FspadStatsPart {
 // How the flat [rows x V] logits array is cut into equal per-CTA ranges.
 struct FspadStatsGeom {
     int unit;          // floats per load unit: 4 (128-bit loads) or 1
-    int upr;           // units per row
+    int shift;         // 1: V is no multiple of 4, a row's units count from the 16-byte boundary at or before its first token
+    int upr;           // units per row (with shift: room for up to three positions in front of it)
     int n_cta;         // CTAs in the grid
     int slots;         // partial slots per row (capacity)
     long long chunk;   // units per CTA
@@ -88,11 +89,13 @@ struct FspadStatsGeom {
 // small_ctas: the scan may use CTAs of half the size when the array is small (the pieces, one of which the
 // acceptance walk's bonus draw sweeps, halve with them; on a large array the smaller CTAs cost bandwidth:
 // 5.93 against 6.20 TB/s on 960 rows of 128256)
-static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, bool vec, int slots, bool small_ctas = false)
+// aligned: the array starts on a 16-byte boundary (otherwise it is read float by float)
+static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, bool aligned, int slots, bool small_ctas = false)
 {
     FspadStatsGeom g;
-    g.unit = vec ? 4 : 1;
-    g.upr = V / g.unit;
+    g.unit = aligned ? 4 : 1;
+    g.shift = aligned && V % 4 != 0;
+    g.upr = g.shift ? (V + 6) / 4 : V / g.unit;
     g.slots = slots;
     g.total = (long long)rows * g.upr;
     g.threads = FSPAD_STATS_THREADS;
@@ -102,6 +105,26 @@ static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, boo
     const long long by_size = (g.total + g.threads - 1) / g.threads;   // at least one unit per thread
     if (n > by_size) n = by_size;
     if (n < 1) n = 1;
+    if (g.shift) {
+        // Rows that start anywhere are always cut at the rows: into 16 pieces where every SM gets a CTA that way (see
+        // below), else into what one wave holds; with more rows than CTAs in a wave, into the number of pieces (up to
+        // 8) that leaves the last wave fullest.
+        long long k = n / rows;
+        if (k > 16 && (long long)rows * 16 >= sm_count) k = 16;
+        if (k > slots - 2) k = slots - 2;
+        if (k < 1) {
+            double best = 0.0;
+            for (int t = 1; t <= 8; ++t) {
+                const long long waves = ((long long)rows * t + n - 1) / n;
+                const double full = (double)rows * t / (double)(waves * n);
+                if (full > best + 0.02) { best = full; k = t; }
+            }
+        }
+        g.chunk = (g.upr + k - 1) / k;
+        g.per_row = (int)((g.upr + g.chunk - 1) / g.chunk);
+        g.n_cta = rows * g.per_row;
+        return g;
+    }
     g.chunk = (g.total + n - 1) / n;
     // A CTA whose range crosses a row boundary runs its reduction sequence twice and finishes about a
     // microsecond behind the others.  Where a row divides evenly into a whole number k of pieces such that
@@ -154,9 +177,11 @@ __device__ __forceinline__ void fspad_stats_merge_warp(const FspadStatsPart *__r
                                                        const FspadStatsGeom &g, int row, float k, int lane,
                                                        float &M, double &S, int &A)
 {
-    const long long r0 = (long long)row * g.upr;
-    const int first = (int)(r0 / g.chunk), last = (int)((r0 + g.upr - 1) / g.chunk);
-    const int cnt = last - first + 1;                       // <= g.slots <= 64
+    int cnt = g.per_row;                                    // <= g.slots <= 64
+    if (cnt == 0) {
+        const long long r0 = (long long)row * g.upr;
+        cnt = (int)((r0 + g.upr - 1) / g.chunk) - (int)(r0 / g.chunk) + 1;
+    }
     const FspadStatsPart *p = parts + (size_t)row * g.slots;
     float m0 = -INFINITY, m1 = -INFINITY, s0 = 0.f, s1 = 0.f;
     int a0 = 0x7fffffff, a1 = 0x7fffffff;

@@ -102,7 +102,11 @@ draft_expand_kernel(const DraftArgs a)
     float4 cur[kPerThread / 4], nxt[kPerThread / 4];
     auto fetch = [&](int e0, float4 (&v)[kPerThread / 4]) {
 #pragma unroll
-        for (int i = 0; i < kPerThread / 4; ++i) v[i] = fspad_load4(xp, e0 + 4 * (i * kThreads + tid), hi, -INFINITY);
+        for (int i = 0; i < kPerThread / 4; ++i) {
+            const int j = e0 + 4 * (i * kThreads + tid);             // (groups that reach past an end of the row are looked at apart)
+            v[i] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            if (j >= 0 && j + 4 <= hi) v[i] = __ldg(reinterpret_cast<const float4 *>(xp + j));
+        }
     };
     // the tokens of one round that reach the bound go to the list (where there is room: the count goes on in any case)
     auto push = [&](int e0) {
@@ -111,10 +115,10 @@ draft_expand_kernel(const DraftArgs a)
         for (int i = 0; i < kPerThread / 4; ++i) {
             const int tok = e0 + 4 * (i * kThreads + tid);
             const float v4[4] = {cur[i].x, cur[i].y, cur[i].z, cur[i].w};
-            if (fmaxf(fmaxf(v4[0], v4[1]), fmaxf(v4[2], v4[3])) >= bound) {
+            if (fmaxf(fmaxf(v4[0], v4[1]), fmaxf(v4[2], v4[3])) >= bound && tok >= 0 && tok + 4 <= hi) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (v4[c] >= bound && tok + c >= 0 && tok + c < hi) {
+                    if (v4[c] >= bound) {
                         const int at = atomicAdd(&s.cnt, 1);
                         if (at < kKeep + kRound) s.list[at] = fspad_sort_key(v4[c], (uint32_t)(tok + c));
                     }
@@ -145,6 +149,17 @@ draft_expand_kernel(const DraftArgs a)
         }
         __syncthreads();
     }
+    // the up to three tokens at either end of the row that no aligned group of four covers
+    auto push_ends = [&]() {
+        if (tid >= 6) return;
+        const int tok = tid < 3 ? lo + 1 + tid : hi - 1 - (tid - 3);
+        const bool end = tid < 3 ? lo < 0 && tok >= 0 && tok < min(lo + 4, hi) : tok >= max(lo, 0) && tok >= hi - ((hi - lo) & 3) && (lo >= 0 || tok >= lo + 4);
+        if (end && x[tok] >= s.bound) {
+            const int at = atomicAdd(&s.cnt, 1);
+            if (at < kKeep + kRound) s.list[at] = fspad_sort_key(x[tok], (uint32_t)tok);
+        }
+    };
+    push_ends();
     for (int e0 = lo; e0 < hi; e0 += kRound) {
         if (e0 + kRound < hi) fetch(e0 + kRound, nxt);
         push(e0);
@@ -155,6 +170,8 @@ draft_expand_kernel(const DraftArgs a)
     if (s.cnt > kKeep + kRound) {                                // (uniform) ascending or constant values: once more, the list cut between rounds
         __syncthreads();
         if (tid == 0) s.cnt = 0;
+        __syncthreads();
+        push_ends();
         for (int e0 = lo; e0 < hi; e0 += kRound) {
             fetch(e0, cur);
             __syncthreads();

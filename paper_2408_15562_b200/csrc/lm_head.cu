@@ -398,6 +398,7 @@ FspadStatsGeom fspad_lm_head_geom(int rows, int V, bool vec, int slots)
 {
     FspadStatsGeom g;
     g.unit = vec ? 4 : 1;
+    g.shift = 0;
     g.upr = V / g.unit;
     g.slots = slots;
     g.total = (long long)rows * g.upr;

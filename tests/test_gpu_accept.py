@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import oracle
-from paper_2408_15562_b200 import synth
+from paper_2408_15562_b200 import binding, synth
 from tests import helpers
 
 pytestmark = pytest.mark.gpu
@@ -136,6 +136,25 @@ def test_stats_pass_matches_oracle_rows():
         np.testing.assert_array_equal(a[sl].cpu().numpy(), oa)
         np.testing.assert_allclose(s[sl].cpu().numpy(), os_, rtol=2e-6)
     assert int(a[3]) == min(777, int(np.argmax(inp.target_logits[0, 3])))
+
+
+@pytest.mark.parametrize("rows,vocab", [(1, 5), (3, 33), (7, 4097), (60, 32001), (130, 50257), (700, 2049), (1300, 1003), (64, 50258)])
+def test_stats_rows_of_any_length(rows, vocab):
+    """Vocabularies that are no multiple of four (rows start at every alignment), one piece per row and many, more rows than one
+    wave of CTAs holds; the maximum sits at a random position, at the first and at the last.  Maximum and index exact; the sum is
+    fp32 with ex2.approx: 2e-6 relative."""
+    rng = np.random.default_rng(rows)
+    x = (rng.standard_normal((rows, vocab)) * 3).astype(np.float32)
+    x[::3, 0] = 20.0
+    x[1::3, -1] = 20.0
+    ctx = binding.Context(8, 2, vocab, 512, max_nodes=min(rows, 256), max_batch=(rows + 255) // 256)
+    temp = torch.full(((rows + 9) // 10,), 0.8, device="cuda")
+    m, s, a = ctx.accept_stats(helpers.dev(x), temp, 10)
+    ctx.check()
+    om, os_, oa = oracle.row_stats(x, 0.8)
+    assert np.array_equal(m.cpu().numpy(), om.astype(np.float32))
+    assert np.array_equal(a.cpu().numpy(), oa)
+    np.testing.assert_allclose(s.cpu().numpy(), os_, rtol=2e-6)
 
 
 @pytest.mark.parametrize("name", ["tiny_greedy", "llama3_8b_2k", "vicuna_33b_4k_greedy",
