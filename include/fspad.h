@@ -445,11 +445,14 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
  * One whole verify step from HOST buffers: copies the step's inputs to device
  * staging owned by the context (allocated by the first call, which therefore
  * must not be made inside a stream capture), writes the tree rows into cache
- * rows L_b.. of layer 0, runs fspad_verify_step (attention over layer 0) on
- * `stream`, copies the results back and synchronises the stream.  The KV cache
+ * rows L_b.. of layer 0, does what fspad_verify_step does (attention over layer
+ * 0; it runs while the logits are on their way) on `stream` and the context's
+ * second stream, copies the results back and synchronises the stream.  The KV cache
  * is device-resident state that persists between steps (the caller's device
  * pointer `cache`, layout as in fspad_kv_compact); everything else is host
- * memory (pinned memory makes the copies asynchronous).  Host outputs:
+ * memory (pinned memory makes the copies asynchronous; pinned draft_probs that
+ * start on a 16-byte boundary are not copied at all: the kernel reads the rows
+ * it needs where they are, before the call returns).  Host outputs:
  * attn_out [batch][n_nodes][Hq][d] bf16, accepted_path [batch][max_nodes],
  * n_accepted, bonus_token, new_len [batch].  draft_probs/uniforms may be NULL
  * when every temperature is 0.  Returns the first host- or device-detected error.

@@ -89,6 +89,7 @@ struct WalkArgs {
     const FspadStatsPart *parts;
     FspadStatsGeom geom;
     int N, V, path_stride, cache_ok;
+    int draft_far;                      // the draft rows lie in host memory: not asked for ahead of need
     int *path, *n_acc, *bonus, *status;
     // optional: the cluster that has walked a sequence also moves its accepted K/V rows up (NULL: not asked for)
     uint4 *kv_cache;                    // [layers][2][B][Hkv][max_len][d] bf16 as 16-byte chunks
@@ -749,7 +750,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         // The root's draft row is the one most likely to be swept: ask for it now (a hint, no register
         // is tied up and nothing waits for it).
         const Chunk ck = chunk_of(row0 * V, V, per_cta, per_thr, rank, tid);
-        if (sampling && ck.lo >= 0 && ck.lo < ck.hi) {
+        if (sampling && !args.draft_far && ck.lo >= 0 && ck.lo < ck.hi) {
             asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + ck.lo));
             if (per_thr > 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(dp + min(ck.hi - 1, ck.lo + 8)));
         }
@@ -1295,7 +1296,7 @@ int fspad_walk_ctas(fspad_ctx *ctx, int B, int V) { return B * walk_cluster_size
 cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const float *draft,
                                      const int *tokens, const int *parent, const float *temperature,
                                      const float *uniforms, const FspadStatsGeom &geom, int N, int B, int V,
-                                     int *path, int *n_acc, int *bonus, cudaStream_t st, FspadWalkCompact kv)
+                                     int *path, int *n_acc, int *bonus, cudaStream_t st, FspadWalkCompact kv, bool draft_far)
 {
     if (B == 0) return cudaSuccess;
     WalkArgs a;
@@ -1304,7 +1305,7 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     a.logits = logits; a.draft = draft; a.temperature = temperature; a.uniforms = uniforms;
     a.tokens = tokens; a.parent = parent;
     a.parts = ctx->st_part; a.geom = geom;
-    a.N = N; a.V = V; a.path_stride = ctx->cfg.max_nodes; a.cache_ok = 0;
+    a.N = N; a.V = V; a.path_stride = ctx->cfg.max_nodes; a.cache_ok = 0; a.draft_far = draft_far ? 1 : 0;
     a.path = path; a.n_acc = n_acc; a.bonus = bonus; a.status = ctx->d_status;
 
     ctx->launches++;

@@ -529,6 +529,7 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
         return FSPAD_ERR_NULL;
     if ((draft_probs == nullptr) != (uniforms == nullptr)) return FSPAD_ERR_NULL;
     if (misaligned(cache)) return FSPAD_ERR_ALIGN;
+    if (n_nodes > ctx->cfg.max_len) return FSPAD_ERR_RANGE;
     if (batch == 0) return FSPAD_OK;
     const fspad_config &c = ctx->cfg;
     cudaStream_t st = fspad_stream(stream);
@@ -574,32 +575,57 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     auto d2h = [&](void *dst, const void *src, size_t bytes) {
         ok = ok && cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
     };
-    h2d(ctx->h_q, q, q_bytes);
+    // The walk reads draft rows only where it rejects, and one probability per node: page-locked draft rows are left where they
+    // are and read over the link by the kernel (60 rows of 128256 copied whole took 557 us, as long as the logits).  The
+    // kernel wants them on a 16-byte boundary, and pageable ones have to be copied.
+    const float *draft = nullptr;
+    if (draft_probs) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, draft_probs) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer != nullptr &&
+            !misaligned(at.devicePointer))
+            draft = static_cast<const float *>(at.devicePointer);
+        else
+            (void)cudaGetLastError();
+    }
+    const bool draft_in_place = draft != nullptr;
+    h2d(ctx->h_prefix, prefix_len, B * sizeof(int));
+    h2d(ctx->h_parent, parent, B * N * sizeof(int));
     h2d(ctx->h_tk, tree_k, t_bytes);
     h2d(ctx->h_tv, tree_v, t_bytes);
-    h2d(ctx->h_parent, parent, B * N * sizeof(int));
-    h2d(ctx->h_prefix, prefix_len, B * sizeof(int));
-    h2d(ctx->h_tokens, draft_tokens, B * N * sizeof(int));
-    h2d(ctx->h_temp, temperature, B * sizeof(float));
-    h2d(ctx->h_logits, target_logits, lg_bytes);
-    if (draft_probs) {
-        h2d(ctx->h_draft, draft_probs, lg_bytes);
-        h2d(ctx->h_unif, uniforms, B * (N + 1) * sizeof(float));
-    }
+    h2d(ctx->h_q, q, q_bytes);
     if (!ok) return FSPAD_ERR_CUDA;
-
-    // the tree rows go into cache rows L_b .. of layer 0 (K at [0][0], V at [0][1]); the step then
-    // takes them from there
+    // the tree rows go into cache rows L_b .. of layer 0 (K at [0][0], V at [0][1]); the attention then takes them from there
     if (fspad_launch_tree_scatter(ctx, cache, ctx->h_tk, ctx->h_tv, ctx->h_prefix, n_nodes, batch, st) !=
         cudaSuccess)
         return FSPAD_ERR_CUDA;
-    rc = fspad_verify_step(ctx, cache, 0, ctx->h_q, nullptr, nullptr, ctx->h_parent, ctx->h_prefix, ctx->h_logits,
-                           draft_probs ? ctx->h_draft : nullptr, ctx->h_tokens, ctx->h_temp,
-                           draft_probs ? ctx->h_unif : nullptr, n_nodes, batch, ctx->h_out, ctx->h_path, ctx->h_nacc,
-                           ctx->h_bonus, ctx->h_newlen, stream);
-    if (rc) return rc;
+    // fork: the attention and its result's way back run beside the copy of the logits
+    if (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess)
+        return FSPAD_ERR_CUDA;
+    const size_t plane = (size_t)batch * c.n_kv_heads * (size_t)c.max_len * FSPAD_HEAD_DIM;
+    const bool attn_ok = fspad_launch_tree_attn(ctx, ctx->h_q, cache, cache + plane, nullptr, nullptr, ctx->h_parent, ctx->h_prefix,
+                                                n_nodes, batch, ctx->h_out, ctx->side) == cudaSuccess;
+    h2d(ctx->h_tokens, draft_tokens, B * N * sizeof(int));
+    h2d(ctx->h_temp, temperature, B * sizeof(float));
+    if (draft_probs) h2d(ctx->h_unif, uniforms, B * (N + 1) * sizeof(float));
+    h2d(ctx->h_logits, target_logits, lg_bytes);
+    if (draft_probs && !draft_in_place) {
+        h2d(ctx->h_draft, draft_probs, lg_bytes);
+        draft = ctx->h_draft;
+    }
+    ok = ok && attn_ok &&
+         cudaMemcpyAsync(attn_out, ctx->h_out, q_bytes, cudaMemcpyDeviceToHost, ctx->side) == cudaSuccess;
+    // the join is queued whatever happened in between: the caller's stream ends behind everything
+    const bool joined = cudaEventRecord(ctx->ev_join, ctx->side) == cudaSuccess;
+    FspadStatsGeom geom;
+    ok = ok && fspad_launch_stats_partials(ctx, ctx->h_logits, ctx->h_temp, batch * n_nodes, n_nodes, c.vocab, &geom, st) == cudaSuccess;
+    ok = ok && fspad_launch_accept_walk(ctx, ctx->h_logits, draft, ctx->h_tokens, ctx->h_parent, ctx->h_temp,
+                                        draft_probs ? ctx->h_unif : nullptr, geom, n_nodes, batch, c.vocab, ctx->h_path, ctx->h_nacc,
+                                        ctx->h_bonus, st, FspadWalkCompact(), draft_in_place) == cudaSuccess;
+    // the compaction rewrites cache rows that the attention reads
+    if (!joined || cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess || !ok) return FSPAD_ERR_CUDA;
+    if (fspad_launch_kv_compact(ctx, cache, ctx->h_path, ctx->h_nacc, ctx->h_prefix, batch, ctx->h_newlen, st, false) != cudaSuccess)
+        return FSPAD_ERR_CUDA;
 
-    d2h(attn_out, ctx->h_out, q_bytes);
     // the device path array has max_nodes entries per sequence, and so has the host one
     d2h(accepted_path, ctx->h_path, B * (size_t)c.max_nodes * sizeof(int));
     d2h(n_accepted, ctx->h_nacc, B * sizeof(int));

@@ -280,7 +280,8 @@ struct FspadWalkCompact {
 cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const float *draft,
                                      const int *tokens, const int *parent, const float *temperature,
                                      const float *uniforms, const FspadStatsGeom &geom, int N, int B, int V,
-                                     int *path, int *n_acc, int *bonus, cudaStream_t st, FspadWalkCompact kv = {});
+                                     int *path, int *n_acc, int *bonus, cudaStream_t st, FspadWalkCompact kv = {},
+                                     bool draft_far = false);   // draft_far: the draft rows lie in host memory
 // pdl = false: launched as a plain dependent of what precedes it in the stream (griddepcontrol.wait is
 // then a no-op; the guarantee its successor relies on holds either way)
 cudaError_t fspad_launch_stats_partials(fspad_ctx *ctx, const float *logits, const float *temperature,

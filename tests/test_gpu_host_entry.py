@@ -72,3 +72,30 @@ def test_host_entry_equals_device_calls(mode):
             assert torch.equal(hpath[b, :k], path_d[b, :k].cpu())
             rows = int(hl[b])
             assert torch.equal(cache_h[:, :, b, :, :rows].view(torch.int16), cache_d[:, :, b, :, :rows].view(torch.int16))
+
+
+@pytest.mark.parametrize("vocab,n_nodes", [(3000, 24), (3001, 70)])
+def test_draft_rows_in_place_or_copied(vocab, n_nodes):
+    """Draft rows that the kernel reads where they are (pinned, on a 16-byte boundary) and ones that have to be copied (pinned off the
+    boundary; pageable): the same walk, bit for bit, against the oracle."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=3, prefix=(40, 300), n_nodes=n_nodes, depth=5, branch=6, vocab=vocab,
+                     temperatures=(1.0, 0.0, 0.7))
+    inp = synth.generate(w, 9)
+    B, N = inp.parent.shape
+    ctx = helpers.make_ctx(inp, n_layers=1)
+    r = oracle.tree_accept(inp.target_logits, inp.draft_probs, inp.draft_tokens, inp.parent, inp.temperature, inp.uniforms)
+    pin = lambda a: torch.from_numpy(np.ascontiguousarray(a)).pin_memory()   # noqa: E731
+    flat = torch.from_numpy(np.ascontiguousarray(inp.draft_probs))
+    off = torch.empty(flat.numel() + 4, dtype=torch.float32).pin_memory()[1:1 + flat.numel()].view(flat.shape)
+    off.copy_(flat)
+    for draft in (flat.pin_memory(), off, flat):
+        cache = binding.bf16_tensor(synth.make_cache(inp, 1))
+        out = torch.empty(inp.q.shape, dtype=torch.bfloat16).pin_memory()
+        path = torch.empty((B, N), dtype=torch.int32)
+        n, bonus, new_len = (torch.empty((B,), dtype=torch.int32) for _ in range(3))
+        ctx.verify_step_host(cache, *(binding.bf16_tensor(a, "cpu").pin_memory() for a in (inp.q, inp.tree_k, inp.tree_v)),
+                             pin(inp.parent), pin(inp.prefix_len), pin(inp.target_logits), draft, pin(inp.draft_tokens),
+                             pin(inp.temperature), pin(inp.uniforms), out, path, n, bonus, new_len)
+        assert np.array_equal(path.numpy(), r["accepted_path"])
+        assert np.array_equal(n.numpy(), r["n_accepted"]) and np.array_equal(bonus.numpy(), r["bonus_token"])
+        assert np.array_equal(new_len.numpy(), inp.prefix_len + r["n_accepted"])
