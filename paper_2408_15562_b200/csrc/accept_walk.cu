@@ -660,6 +660,7 @@ accept_greedy_kernel(const __grid_constant__ WalkArgs args)
         t.parent[tid] = p;
         t.tok[tid] = tk;
     }
+    if (tid == 0 && args.kv_cache != nullptr) t.kv_L = args.kv_prefix[b];
     if (tid == 0 && !(Tf >= 0.0f)) fspad_report(args.status, FSPAD_ERR_RANGE);
     if (tid == 0 && Tf > 0.0f) fspad_report(args.status, FSPAD_ERR_NULL);      // a sampling sequence without draft rows
     fspad_pdl_wait();
@@ -673,6 +674,7 @@ accept_greedy_kernel(const __grid_constant__ WalkArgs args)
     }
     __syncthreads();
     greedy_walk(t, args, b, N, tid, nthr, true);
+    if (args.kv_cache != nullptr) compact_accepted(args, t, b, 0, 1, tid, nthr);
 }
 
 template <int MAXN>
