@@ -57,30 +57,17 @@ constexpr int kSmemBudgetWide = 176 * 1024;   // the same for the instance with 
 constexpr double kAmbiguous = 1e-4;
 constexpr double kScanRel = 1e-6;          // bound taken for the relative error of the scan's sum of exponentials
 constexpr double kFusedTol = 1e-9;         // relative error the fused first-rejection sweep may leave in the residual mass
-constexpr double k256OverLn2 = 369.3299304675746;   // steps of the exponential's table per unit of its argument
+constexpr double k16OverLn2 = 23.083120654223414;   // steps of the exponential's table per unit of its argument
 constexpr float kLog2eF = 1.4426950408889634f;
 constexpr int kPieceSlots = 16;            // pieces of a row whose scan sums are kept for the bonus draw
-constexpr int kExpTable = 256;             // entries of the exponential's table
+constexpr int kExpTable = 16;              // entries of the exponential's table: one per pair of shared-memory banks
 enum { REQ_DONE = 0, REQ_EXP = 1, REQ_FUSED = 2, REQ_RESID = 3 };
 
-// 2^(i/64), i = 0..63, correctly rounded
-__constant__ double kExp2Tbl[64] = {
-    1.0, 1.0108892860517005, 1.0218971486541166, 1.0330248790212284,
-    1.0442737824274138, 1.0556451783605572, 1.0671404006768237, 1.0787607977571199,
-    1.0905077326652577, 1.102382583307841, 1.1143867425958924, 1.1265216186082418,
-    1.1387886347566916, 1.1511892299529827, 1.1637248587775775, 1.1763969916502812,
-    1.189207115002721, 1.202156731452703, 1.215247359980469, 1.22848053610687,
-    1.241857812073484, 1.255380757024691, 1.2690509571917332, 1.2828700160787783,
-    1.2968395546510096, 1.3109612115247644, 1.3252366431597413, 1.339667524053303,
-    1.3542555469368927, 1.3690024229745905, 1.383909881963832, 1.3989796725383112,
-    1.4142135623730951, 1.42961333839197, 1.4451808069770467, 1.460917794180647,
-    1.4768261459394993, 1.4929077282912648, 1.5091644275934228, 1.5255981507445384,
-    1.5422108254079407, 1.559004400237837, 1.5759808451078865, 1.593142151342267,
-    1.6104903319492543, 1.6280274218573478, 1.645755478153965, 1.6636765803267364,
-    1.681792830507429, 1.7001063537185235, 1.718619298122478, 1.7373338352737062,
-    1.7562521603732995, 1.7753764925265212, 1.7947090750031072, 1.8142521755003989,
-    1.8340080864093424, 1.8539791250833855, 1.8741676341103, 1.8945759815869656,
-    1.9152065613971474, 1.9360617934922943, 1.9571441241754002, 1.978456026387951,
+// 2^(i/16), i = 0..15, correctly rounded
+__constant__ double kExp2Tbl[16] = {
+    1.0, 1.0442737824274138, 1.0905077326652577, 1.1387886347566916, 1.189207115002721, 1.241857812073484,
+    1.2968395546510096, 1.3542555469368927, 1.4142135623730951, 1.4768261459394993, 1.5422108254079407,
+    1.6104903319492543, 1.681792830507429, 1.7562521603732995, 1.8340080864093424, 1.9152065613971474,
 };
 
 struct WalkArgs {
@@ -104,6 +91,7 @@ struct WalkState {
     double S, C, U, D, invD, F;     // denominator, coefficient of the draft row, residual mass, draft mass and its
                                     // inverse, sum of the weights that rejected tokens keep
     double Cp;                      // coefficient of the rejection under way
+    double base;                    // draft mass of the tokens that no child carries (after the first rejection)
     int cur, nrem, len, ch, ridx;   // ch: child under test (0: none left); ridx: its token's place in the list of rejected ones, or -1
     int exact, parked;              // S is exact; e and q of the node's rows are parked (first rejection done)
 };
@@ -125,7 +113,7 @@ template <int MAXN> struct TreeShared {
 };
 template <int MAXN> struct SharedT {
     TreeShared<MAXN> t;
-    double exp_tbl[kExpTable];      // 2^(i/256)
+    alignas(128) double exp_tbl[kExpTable];      // 2^(i/16)
     // what thread 0 asks for and about which node (written by thread 0, read by all after a barrier)
     double S, C;                    // sum of exponentials in use, coefficient of the draft row
     double S_exact;                 // what the first rejection's sweep found
@@ -134,14 +122,13 @@ template <int MAXN> struct SharedT {
     int nrem, sel;
     int rem_tok[MAXN];              // tokens rejected at the current node and the weights they keep
     double rem_frozen[MAXN];
-    double node_D[MAXN], node_invD[MAXN];   // draft mass left once node c and its earlier siblings are rejected, its inverse
     // gathered once, in parallel, before the walk: the scan result of every row and, for
     // every node, its draft probability in its parent's row and its uniform
     float rowM[MAXN];
     double rowS[MAXN];
     float cq[MAXN], cu[MAXN];
     double cex[MAXN];               // exp((logit - row max)/T) of each node's token in its parent's row
-    double later_q[MAXN];           // draft mass of the tokens that only siblings after node c carry
+    double later_q[MAXN];           // draft mass of the tokens that only siblings after node c carry (children of nodes with a rejection)
     int first_child[MAXN], next_sib[MAXN];   // 0: none
     unsigned char dup[MAXN];        // an earlier sibling carries the same token
     float ubonus;
@@ -247,18 +234,19 @@ __device__ __forceinline__ void merge_row(const FspadStatsPart *__restrict__ par
 }
 
 // exp((x - m) / T) for x <= m in double precision, by table and polynomial (the scheme of Tang's 1989 paper): with
-// t = (x - m) 256 / (T ln 2) = 256 n + i + f, |f| <= 1/2, the value is 2^n 2^(i/256) exp(f ln2/256).  The exponential
-// of the remainder is a cubic: its Taylor series with the fourth-order term economised into the constant and the
-// square (error below 1.8e-14).  The caller hands over s = 256 / (T ln 2) and off = -m s.  The rounding to the nearest
-// integer is done by adding and subtracting 1.5 * 2^52 (the integer then sits in the low word of the sum): conversions
-// run at a quarter of the fp64 rate (16 against 63 per clock and SM).  Values below e^-700 are taken as zero.
+// t = (x - m) 16 / (T ln 2) = 16 n + i + f, |f| <= 1/2, the value is 2^n 2^(i/16) exp(f ln2/16).  The exponential
+// of the remainder is its Taylor series to the fifth order with the sixth economised into the lower ones (error below
+// 5e-15).  Sixteen entries lie in sixteen pairs of banks, so that a warp's look-ups never collide (with 256 entries and a
+// cubic each cost six shared-memory cycles).  The caller hands over s = 16 / (T ln 2) and off = -m s.  The rounding to
+// the nearest integer is done by adding and subtracting 1.5 * 2^52 (the integer then sits in the low word of the sum):
+// conversions run at a quarter of the fp64 rate (16 against 63 per clock and SM).  Values below e^-700 are taken as zero.
 struct ExpArg {
     double s, off;
     float x_min;
 };
 __device__ __forceinline__ ExpArg exp_arg(float m, double invT, float T)
 {
-    const double s = invT * k256OverLn2;
+    const double s = invT * k16OverLn2;
     return ExpArg{s, -(double)m * s, m - 700.0f * T};
 }
 __device__ __forceinline__ double exp_neg(float x, const ExpArg &g, const double *tbl)
@@ -268,12 +256,21 @@ __device__ __forceinline__ double exp_neg(float x, const ExpArg &g, const double
     const double tm = t + magic;
     const double f = t - (tm - magic);
     const int k = __double2loint(tm);
-    double p = fma(f, 3.3083026805413713e-09, 3.665566156758904e-06);
-    p = fma(p, f, 0.0027076061740622863);
-    p = fma(p, f, 0.9999999999999825);
+    double p = fma(f, 1.2715871950558131e-09, 1.4676444618653448e-07);
+    p = fma(p, f, 1.3550807779497457e-05);
+    p = fma(p, f, 0.0009383847924862099);
+    p = fma(p, f, 0.04332169878499658);
+    p = fma(p, f, 1.0000000000000044);
     const double y = tbl[k & (kExpTable - 1)] * p;
-    const double e = __hiloint2double(__double2hiint(y) + ((k >> 8) << 20), __double2loint(y));
+    const double e = __hiloint2double(__double2hiint(y) + ((k >> 4) << 20), __double2loint(y));
     return x > g.x_min ? e : 0.0;                          // also -inf and NaN
+}
+
+// w where it is not negative, else zero, without a branch (tokens of a warp are of both kinds)
+__device__ __forceinline__ double positive(double w)
+{
+    const int keep = ~(__double2hiint(w) >> 31);
+    return __hiloint2double(__double2hiint(w) & keep, __double2loint(w) & keep);
 }
 
 __device__ __forceinline__ double pair_of(float hi, float lo) { return __hiloint2double(__float_as_int(hi), __float_as_int(lo)); }
@@ -372,8 +369,7 @@ __device__ __noinline__ double parked_sweep(double *__restrict__ se, float *__re
     for (int k = 0; k < per_thr; k += 4) {
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            const double w = fma(-C, (double)sq[(k + t) * stride], se[(k + t) * stride]);
-            if (__double2hiint(w) >= 0) a[t & 1] += w;
+            a[t & 1] += positive(fma(-C, (double)sq[(k + t) * stride], se[(k + t) * stride]));
         }
     }
     return a[0] + a[1];
@@ -396,8 +392,7 @@ __device__ __forceinline__ double residual_of_tile(const double (&er)[kTile], co
         if (b < per_thr) {
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                const double w = fma(-C, widen(qr[b + t]), er[b + t]);
-                if (__double2hiint(w) >= 0) a[t] += w;
+                a[t] += positive(fma(-C, widen(qr[b + t]), er[b + t]));
             }
         }
     }
@@ -482,7 +477,8 @@ __device__ __forceinline__ void fused_reject_sweep(const Shared &sh, const float
                 sq[(k + t) * stride] = qv[t];
             }
             const double w = fma(-S, (double)qv[t], e);
-            if (__double2hiint(w) >= 0) { v[1] += w; qp += qv[t]; }
+            v[1] += positive(w);
+            qp += __double2hiint(w) >= 0 ? qv[t] : 0.f;
             // |w| <= kScanRel * e needs the binary exponent of w at least 19 below that of e: an
             // integer comparison sorts out all but a handful of tokens
             if ((__double2hiint(w) & 0x7ff00000) <= (__double2hiint(e) & 0x7ff00000) - (19 << 20))
@@ -708,8 +704,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     if (tid <= N) uval = args.uniforms[(size_t)b * (N + 1) + (tid == 0 ? N : tid)];   // thread c: node c's uniform; thread 0: the bonus uniform
     if (tid == 32 && args.kv_cache != nullptr) sh.t.kv_L = args.kv_prefix[b];
     // (the loads above are under way)
-    if (tid < kExpTable)
-        sh.exp_tbl[tid] = kExp2Tbl[tid >> 2] * ((tid & 2) ? ((tid & 1) ? 1.0081558981184175 : 1.0054299011128027) : ((tid & 1) ? 1.0027112750502025 : 1.0));
+    if (tid < kExpTable) sh.exp_tbl[tid] = kExp2Tbl[tid];
     if (tid < MAXN) sh.first_child[tid] = MAXN;
     if (tid == 0) {
         sh.fail = 0;
@@ -876,16 +871,6 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         }
     };
 
-    // draft mass of the tokens that only later siblings of node c carry (read after the first exchange; warp 0 has the
-    // walk to begin)
-    for (int c = tid - 31; wid > 0 && c < N; c += kWalkThreads - 32) {
-        double later = 0.0;
-#pragma unroll 1
-        for (int o = sh.next_sib[c]; o > 0; o = sh.next_sib[o])
-            if (!sh.dup[o]) later += (double)sh.cq[o];
-        sh.later_q[c] = later;
-    }
-
     // Thread 0 of every CTA (all on identical data, so all take identical steps) walks ahead through
     // every decision that needs nothing but scalars, and stops only to ask the CTA for a sweep of the
     // current node's rows.
@@ -906,8 +891,8 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     auto fetch_ahead = [&]() {
         w = sh.state;
         fx = weight(sh.cex[w.ch], (double)sh.cq[w.ch], w.Cp);
-        next_D = sh.node_D[w.ch];
-        next_invD = sh.node_invD[w.ch];
+        next_D = w.base + sh.later_q[w.ch];
+        next_invD = 1.0 / next_D;
         fetch_child(sh.next_sib[w.ch]);          // (node 0 where there is none)
         next_rhs = weight(nx.ex, nx.qx, w.Cp) * (next_D > 0.0 ? next_D : w.D);
     };
@@ -1027,22 +1012,25 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             const double s_scan = sh.S;
             fused_reject_sweep(sh, x, q, se, sq, kWalkThreads, ck, per_thr, cache_ok, arg, s_scan, xn, cur, N, v);
             double tot[4] = {v[0], v[1], v[2], v[3]};
-            exchange(tot, []() {});
-            if (wid == 0) {
-                // what the draft row keeps after each child of the node in turn
-#pragma unroll 1
-                for (int c = lane; c < N; c += 32) {
-                    if (c == 0 || sh.t.parent[c] != cur) continue;
-                    const double d = tot[2] + sh.later_q[c];
-                    sh.node_D[c] = d;
-                    sh.node_invD[c] = 1.0 / d;
+            auto load_tile = [&]() {                          // (each thread its own values: nothing to wait for)
+                if (in_regs) {
+#pragma unroll
+                    for (int i = 0; i < kTile; ++i) {
+                        er[i] = i < per_thr ? se[i * kWalkThreads] : 0.0;
+                        qr[i] = i < per_thr ? sq[i * kWalkThreads] : 0.f;
+                    }
                 }
+            };
+            exchange(tot, load_tile);
+            if (wid > 0) load_tile();
+            if (wid == 0) {
                 const double s_exact = tot[0];
                 const float qp = __int_as_float(__double2hiint(tot[3])), flips = __int_as_float(__double2loint(tot[3]));
                 R = tot[1] - (s_exact - s_scan) * (double)qp;
                 if (R < 0.0) R = 0.0;
                 if (lane == 0) {
                     sh.state.S = sh.state.Cp = s_exact;
+                    sh.state.base = tot[2];
                     sh.state.exact = sh.state.parked = 1;
                     const int c = sh.state.ch;
                     const double Wt = R + weight(sh.cex[c], (double)sh.cq[c], s_exact);
@@ -1050,17 +1038,20 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
                     sh.C = s_exact;                           // the coefficient of the repeated sweep
                     sh.S_exact = s_exact;
                 }
-                __syncwarp();
-                fetch_ahead();
-            }
-            if (in_regs) {                                    // (each thread its own values: nothing to wait for)
-#pragma unroll
-                for (int i = 0; i < kTile; ++i) {
-                    er[i] = i < per_thr ? se[i * kWalkThreads] : 0.0;
-                    qr[i] = i < per_thr ? sq[i * kWalkThreads] : 0.f;
+            } else {
+                // while warp 0 waits for the peers: for each child of the node, the draft mass of the tokens that only
+                // siblings after it carry
+                for (int c = tid - 31; c < N; c += kWalkThreads - 32) {
+                    if (sh.t.parent[c] != cur) continue;
+                    double later = 0.0;
+#pragma unroll 1
+                    for (int o = sh.next_sib[c]; o > 0; o = sh.next_sib[o])
+                        if (!sh.dup[o]) later += (double)sh.cq[o];
+                    sh.later_q[c] = later;
                 }
             }
             __syncthreads();
+            if (wid == 0) fetch_ahead();
             again = sh.sel != 0;
             // this thread's share of that sum (nothing rewrites S_exact before the next first rejection; thread 0 may
             // already be changing the rest of the walk's state)
