@@ -424,8 +424,7 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
     // the free SMs.  Otherwise the scan goes first on all SMs and the attention is forked behind it, sized
     // to leave the walk's SMs alone, so that the walk (the longer chain) and the attention run side by side.
     const int sms = ctx->sm_count;
-    const int G = c.n_q_heads / c.n_kv_heads;
-    const long long attn_ctas = (long long)batch * c.n_kv_heads * ((n_nodes * G + 127) / 128) *
+    const long long attn_ctas = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch) *
                                 fspad_attn_umma_splits(ctx, n_nodes, batch);
     const bool may_sample = draft_probs != nullptr;
     const bool scan_first = may_sample && sms - attn_ctas < sms / 4;
@@ -469,7 +468,7 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
         // its SM taken waits for a scan CTA's whole life.
         int scan_sms = 0;
         if (may_sample || both_sms > 0) {
-            const long long attn_now = (long long)batch * c.n_kv_heads * ((n_nodes * G + 127) / 128) *
+            const long long attn_now = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch, both_sms) *
                                        fspad_attn_umma_splits(ctx, n_nodes, batch, both_sms);
             scan_sms = sms - (int)(attn_now < sms ? attn_now : sms);
             if (scan_sms < sms / 8) scan_sms = sms / 8;

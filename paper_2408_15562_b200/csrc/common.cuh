@@ -32,6 +32,7 @@ struct fspad_ctx {
     // TMA descriptors of the K and V cache planes last seen (re-encoded when they change)
     alignas(64) unsigned char attn_tmap_k[128];
     alignas(64) unsigned char attn_tmap_v[128];
+    alignas(64) unsigned char attn_tmap_k_half[128];
     const void *attn_tmap_kptr, *attn_tmap_vptr;
     size_t attn_tmap_rows;
     int attn_tmap_ok;
@@ -316,6 +317,8 @@ cudaError_t fspad_launch_tree_scatter(fspad_ctx *ctx, fspad_bf16 *cache, const f
                                       const fspad_bf16 *tv, const int *prefix_len, int N, int B,
                                       cudaStream_t st);
 int fspad_attn_umma_splits(const fspad_ctx *ctx, int N, int B, int sms = 0);
+bool fspad_attn_pairs(const fspad_ctx *ctx, int N, int B, int sms = 0);      // row tiles go in pairs of CTAs
+int fspad_attn_mtiles(const fspad_ctx *ctx, int N, int B, int sms = 0);     // row tiles (CTAs) per kv head and key range
 int fspad_lm_head_tiles(int V);
 size_t fspad_feature_sampler_scratch_floats(int rows, int H, int I);
 cudaError_t fspad_launch_feature_sampler(fspad_ctx *ctx, const fspad_bf16 *f, const fspad_bf16 *e, const fspad_bf16 *wup,
@@ -331,7 +334,7 @@ int fspad_walk_ctas(fspad_ctx *ctx, int B, int V);   // CTAs of the sampling wal
 cudaError_t fspad_launch_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t st);
 cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 *kc,
                                          const fspad_bf16 *vc, const fspad_bf16 *tk, const fspad_bf16 *tv,
-                                         const int *parent, const int *prefix_len, int N, int B, int n_splits,
+                                         const int *parent, const int *prefix_len, int N, int B, int sms, int n_splits,
                                          float scale_log2, fspad_bf16 *out, cudaStream_t st, FspadPaged paged);
 cudaError_t fspad_launch_kv_append(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *tree_kv, const int *path,
                                    const int *n_acc, const int *prefix_len, int N, int B, int *new_len, cudaStream_t st);

@@ -111,7 +111,7 @@ cudaError_t fspad_launch_tree_attn(fspad_ctx *ctx, const fspad_bf16 *q, const fs
     a.mtiles = (a.M + 127) / 128;
     a.scale_log2 = ctx->scale * kLog2e;
     a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.out = out; a.status = ctx->d_status;
-    cudaError_t e = fspad_launch_attn_umma_split(ctx, q, kc, vc, tk, tv, parent, prefix_len, N, B, a.n_splits,
+    cudaError_t e = fspad_launch_attn_umma_split(ctx, q, kc, vc, tk, tv, parent, prefix_len, N, B, sms, a.n_splits,
                                                  a.scale_log2, out, st, paged);
     // One key range per row (a batch that fills the SMs): the attention kernel has written the result, nothing to merge
     // (the merge pass took 14.6 us on 16 sequences of 60 nodes and 32 heads).

@@ -34,8 +34,9 @@ constexpr int BK = 128;                // keys per chunk
 constexpr int NT = 320;                // threads per CTA: two per query row + a copy warp + a tensor-core warp
 constexpr int HALF = 128 * 128;        // bytes of one [128 rows][64 bf16] half tile
 constexpr int TILE = 2 * HALF;         // bytes of one [128][128] bf16 tile
-constexpr int NS = 3;                  // K / V chunks in flight per CTA
-constexpr int SMEM_BYTES = (1 + 2 * NS) * TILE + 1024;   // Q, K[NS], V[NS] + alignment slack
+// K / V chunks in flight: a lone CTA holds whole ones, a pair's CTA half of each
+__host__ __device__ constexpr int ring_slots(bool pair) { return pair ? 5 : 3; }
+constexpr int smem_bytes(bool pair) { return TILE + 2 * ring_slots(pair) * (pair ? HALF : TILE) + 1024; }   // Q, K ring, V ring + alignment slack
 constexpr uint32_t TMEM_COLS = 512;    // S/P of group 0, of group 1: columns 0..255; O of group 0, of group 1: 256..511
 constexpr int kMaxBlocksPerCta = 128;  // paged cache: chunks (= blocks) one CTA may be given
 constexpr float kLazyLog2 = 8.f;        // a row's reference maximum may lag its true maximum by this much (log2)
@@ -86,13 +87,23 @@ __device__ __forceinline__ uint32_t tile_off(int r, int c)
 // A new phase of a barrier can only begin after every side that waits on it has seen the previous
 // one (a parity wait must never fall two phases behind).
 // Tensor-core order: S(0) S(1) | PV_0(0) PV_1(0) S(2) | PV_0(1) PV_1(1) S(3) | ...
+// PAIR: two CTAs of a cluster (two SMs) take two neighbouring row tiles of the same keys as one 256-row tile
+// (cta_group::2): each keeps its own rows' Q, scores, P and O, and holds keys 64 r .. 64 r + 63 of every K chunk and
+// columns 64 r .. 64 r + 63 of every V chunk (r: its rank), which the tensor cores of both read.  Rank 0's thread issues
+// for both; K / V and P barriers that it waits on are its own (rank 1 arrives remotely), the others exist in both CTAs.
+// What a lone CTA's loop is short of is shared-memory bandwidth: 96 KB read and 64 KB filled per chunk, 1280 of its 2050
+// cycles; in a pair 80 and 32 KB.
 // NW: 64-bit words of a node's ancestor mask.  NW = 1 (trees of up to 64 nodes): the masks are built once per
 // CTA in shared memory.  NW = 4 (up to 256 nodes): there is no shared memory left for them, so every softmax
 // thread follows its own node's parent chain in global memory (a few cached loads) and keeps the mask in registers.
-template <int NW>
+template <int NW, bool PAIR>
 __global__ void __launch_bounds__(NT, 1)
 tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV)
 {
+    constexpr int NS = ring_slots(PAIR);                     // ring slots
+    constexpr int SLOT = PAIR ? HALF : TILE;                 // bytes of this CTA's share of a K or V chunk
+    constexpr int KROWS = PAIR ? BK / 2 : BK;                // keys of its share of a K chunk
+    constexpr int KSUB = KROWS * 128;                        // bytes of one 64-column half of that share
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long s_bar[4 * NS + 13];
     __shared__ uint32_t s_tmem;
@@ -106,8 +117,9 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
     const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     const bool producer = warp >= 8;         // warp 8 copies, warp 9 drives the tensor cores
     const int row = tid & (BM - 1), grp = (tid >> 7) & 1;
-    const int split = blockIdx.x;
-    const int g = blockIdx.y / a.mtiles, mt = blockIdx.y % a.mtiles;
+    const int split = PAIR ? blockIdx.y : blockIdx.x, tile_g = PAIR ? blockIdx.x : blockIdx.y;
+    const int g = tile_g / a.mtiles, mt = tile_g % a.mtiles;
+    const int rank = PAIR ? mt & 1 : 0;           // a.mtiles is even then, so a pair has one kv head
     int b = blockIdx.z;
     if (a.longest_first) {
         // CTAs are dispatched in index order as SMs come free, so with more CTAs than SMs the sequences
@@ -151,7 +163,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
 
     // 1024-byte aligned tiles: Q | K[NS] | V[NS]
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t sQ = base, sK = base + TILE, sV = base + (1 + NS) * TILE;
+    const uint32_t sQ = base, sK = base + TILE, sV = base + TILE + NS * SLOT;
     const uint32_t bar0 = smem_u32(&s_bar[0]);
     auto kfull = [&](int buf) { return bar0 + 8u * (uint32_t)buf; };
     auto vfull = [&](int buf) { return bar0 + 8u * (uint32_t)(NS + buf); };
@@ -163,13 +175,22 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
     const uint32_t drain = bar0 + 8u * (uint32_t)(4 * NS + 12);   // used only when a wait has run out
     const bool tma_ok = a.use_tma != 0;
     // The thread that issues the first TMA copies also initialises the barriers, so those copies
-    // leave as soon as the prefix length is known, ahead of the CTA's first barrier.
+    // leave as soon as the prefix length is known, ahead of the CTA's first barrier (a pair's: as soon as both CTAs'
+    // barriers are initialised).
     if (tid == 256) {
 #pragma unroll
-        for (int i = 0; i < 4 * NS + 13; ++i) mbar_init(bar0 + 8u * i, (i >= 4 * NS + 4 && i < 4 * NS + 6) ? 8 : 1);
+        for (int i = 0; i < 4 * NS + 13; ++i)
+            mbar_init(bar0 + 8u * i, (i >= 4 * NS + 4 && i < 4 * NS + 6) ? (PAIR ? 16 : 8) : (PAIR && i < 2 * NS) ? 2 : 1);
         s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    if (PAIR) {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    }
+    // arrivals on the barriers of the side that issues
+    auto arrive0 = [&](uint32_t bar) { if (PAIR) mbar_arrive_rank0(bar); else mbar_arrive(bar); };
+    auto arrive_p = [&](uint32_t bar) { if (PAIR && rank != 0) mbar_arrive_rank0_light(bar); else mbar_arrive(bar); };
 
     const bool paged = a.block_table != nullptr;
     if (paged) {
@@ -200,29 +221,55 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
     // with 16-byte asynchronous copies by the threads t0, t0 + nt, ... that the caller names (the
     // whole CTA in the prologue, the producer warp alone inside the loop).
     auto gather = [&](int ch, int buf, bool is_v, int t0, int nt) {
-        const uint32_t dst = (is_v ? sV : sK) + buf * TILE;
+        const uint32_t dst = (is_v ? sV : sK) + buf * SLOT;
         const fspad_bf16 *cb = is_v ? a.vc : a.kc, *tb = is_v ? tvb : tkb;
-        for (int i = t0; i < BK * 16; i += nt) {
-            const int r = i >> 4, c = i & 15;
-            const int key = ch * BK + r;
+        for (int i = t0; i < SLOT / 16; i += nt) {
+            // row r of the share and 16-byte chunk c of the whole row (a pair's K share: half the keys; its V share: half the columns)
+            const int r = PAIR && is_v ? i >> 3 : i >> 4, cl = PAIR && is_v ? i & 7 : i & 15;
+            const int c = PAIR && is_v ? cl + 8 * rank : cl;
+            const int key = ch * BK + r + (PAIR && !is_v ? KROWS * rank : 0);
             const bool ok = key < Ltot;
             const fspad_bf16 *src = cb;
             // prefix rows, and tree rows that live in the cache, come from the planes; explicit tree rows from their array
             if (ok) src = (key < L || tb == nullptr) ? cb + phys_row(key) * D + c * 8 : tb + (size_t)(key - L) * D + c * 8;
-            cp_async16(dst + tile_off(r, c), src, ok);
+            const uint32_t off = PAIR ? (uint32_t)((cl >> 3) * KSUB + r * 128 + (((cl & 7) ^ (r & 7)) << 4)) : tile_off(r, c);
+            cp_async16(dst + off, src, ok);
         }
     };
     auto tma_fill = [&](int ch, int buf, bool is_v) {       // one lane
-        const uint32_t dst = (is_v ? sV : sK) + buf * TILE;
+        const uint32_t dst = (is_v ? sV : sK) + buf * SLOT;
         const uint32_t bar = is_v ? vfull(buf) : kfull(buf);
         const CUtensorMap *map = is_v ? &tmV : &tmK;
-        mbar_expect_tx(bar, TILE);
         const int y = (int)phys_row(ch * BK);
-        tma_load_2d(dst, map, 0, y, bar);
-        tma_load_2d(dst + HALF, map, 64, y, bar);
+        if constexpr (PAIR) {
+            mbar_expect_tx_rank0(bar, SLOT);
+            if (is_v) {
+                tma_load_2d_pair(dst, map, 64 * rank, y, bar);                    // 128 keys x 64 columns
+            } else {
+                tma_load_2d_pair(dst, map, 0, y + KROWS * rank, bar);             // 64 keys x 64 columns, twice
+                tma_load_2d_pair(dst + KSUB, map, 64, y + KROWS * rank, bar);
+            }
+        } else {
+            mbar_expect_tx(bar, TILE);
+            tma_load_2d(dst, map, 0, y, bar);
+            tma_load_2d(dst + HALF, map, 64, y, bar);
+        }
     };
 
-    // ---- prologue: the first NS chunks and Q go out first, the rest hides under their latency ----
+    // ---- prologue: Q and the first NS chunks go out first, the rest hides under their latency (Q ahead of the chunks: behind
+    // the ring's fill on every SM it arrives when that has, 6 us later on a long context) ----
+    for (int i = tid; i < BM * 16; i += NT) {
+        const int r = i >> 4, c = i & 15;
+        const int grr = mt * BM + r;
+        const bool ok = grr < M;
+        const int nd = ok ? grr / G : 0, hh = ok ? grr % G : 0;
+        const fspad_bf16 *src = a.q + (((size_t)b * N + nd) * a.Hq + g * G + hh) * D + c * 8;
+        cp_async16(sQ + tile_off(r, c), src, ok);
+    }
+    if (PAIR) {
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");     // both CTAs' barriers are initialised
+    }
 #pragma unroll
     for (int u = 0; u < NS; ++u) {
         if (u >= n_ch) break;
@@ -233,22 +280,20 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             gather(c0 + u, u, true, tid, NT);
         }
     }
-    for (int i = tid; i < BM * 16; i += NT) {
-        const int r = i >> 4, c = i & 15;
-        const int grr = mt * BM + r;
-        const bool ok = grr < M;
-        const int nd = ok ? grr / G : 0, hh = ok ? grr % G : 0;
-        const fspad_bf16 *src = a.q + (((size_t)b * N + nd) * a.Hq + g * G + hh) * D + c * 8;
-        cp_async16(sQ + tile_off(r, c), src, ok);
-    }
     cp_async_commit();
     if (NW == 1 && tid < N) s_par[tid] = a.parent[(size_t)b * N + tid];
     __syncthreads();                              // barriers initialised, parents staged
     if (warp == 9) {
         __syncwarp();
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
-                     :: "r"(smem_u32(&s_tmem)), "r"(TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n"
+                         :: "r"(smem_u32(&s_tmem)), "r"(TMEM_COLS) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
+                         :: "r"(smem_u32(&s_tmem)), "r"(TMEM_COLS) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+        }
     } else if (NW == 1 && tid < N) {
         // tree -> ancestor-or-self masks (parents were staged in shared memory above)
         unsigned long long mask = 0ull;
@@ -268,9 +313,11 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_sync_all();                 // both CTAs have their Q and their tensor memory
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t idesc_s = make_idesc(false, 128), idesc_o = make_idesc(true, 128);
+    const uint32_t idesc_s = PAIR ? make_idesc_m256(128) : make_idesc(false, 128);
+    const uint32_t idesc_o = PAIR ? make_idesc_m256(128) | (1u << 16) : make_idesc(true, 128);      // B (= V) MN-major
     const uint32_t tO = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256u + (uint32_t)grp * 128u;   // this group's O row
     bool failed = false;
     int filled_k = min(n_ch, NS), filled_v = filled_k;   // copy warp: chunks whose K (V) fill has been started
@@ -280,7 +327,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         // chunks gathered by the whole CTA in the prologue are announced here
         if (lane == 0) {
             for (int u = 0; u < NS && u < n_ch; ++u)
-                if (!is_tma(c0 + u)) { mbar_arrive(kfull(u)); mbar_arrive(vfull(u)); }
+                if (!is_tma(c0 + u)) { arrive0(kfull(u)); arrive0(vfull(u)); }
         }
         auto fill = [&](int ch, int buf, bool is_v) {
             if (is_tma(ch)) {
@@ -291,7 +338,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                 cp_async_wait<0>();
                 fence_async_smem();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(is_v ? vfull(buf) : kfull(buf));
+                if (lane == 0) arrive0(is_v ? vfull(buf) : kfull(buf));
             }
             __syncwarp();
         };
@@ -310,9 +357,10 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         // ================= tensor-core warp: the whole warp runs the loop, one lane issues every tcgen05.mma =================
         // (one lane's branch kept every operand in ordinary registers: 17.4 against 19.0 us per call at 4 heads per KV head
         // and 2 K keys, 35.8 against 37.8 at 8 and 8 K, 99.3 against 101.4 on the ragged batch of 16)
-        {
+        if (rank == 0) {
             const bool issuer = elect_one();
             const uint32_t elect = 1;             // the instructions stand in the issuer's branch
+            auto commit = [&](uint32_t bar) { if (PAIR) mma_commit_pair(bar); else mma_commit_if(bar, elect); };
             // low words of the shared-memory descriptors (start address and leading byte offset);
             // the high word (8-row group stride, version, swizzle mode) is the same for all
             const uint32_t hi = (uint32_t)(make_desc(0, 16) >> 32);
@@ -328,15 +376,16 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                     // no tcgen05 fence here: the K chunk comes through the barrier's own acquire, and the
                     // score buffer's last readers and writers (softmax of chunk c - 2) were ordered before this
                     // thread's instructions by the fence behind its pfull wait of that chunk
-                    const uint32_t kb = k_lo + (uint32_t)kbuf * (TILE >> 4);
+                    const uint32_t kb = k_lo + (uint32_t)kbuf * (SLOT >> 4);
                     const uint32_t d = tmem + (uint32_t)(c & 1) * 128u;
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) { // K = 16 per instruction over d = 128
-                        const uint32_t koff = ((ks >> 2) * HALF + (ks & 3) * 32) >> 4;
-                        mma_f16_lo(d, q_lo + koff, hi, kb + koff, hi, idesc_s, ks > 0, elect);
+                        const uint32_t qoff = ((ks >> 2) * HALF + (ks & 3) * 32) >> 4, koff = ((ks >> 2) * KSUB + (ks & 3) * 32) >> 4;
+                        if constexpr (PAIR) mma_f16_pair(d, q_lo + qoff, kb + koff, hi, idesc_s, ks > 0);
+                        else mma_f16_lo(d, q_lo + qoff, hi, kb + koff, hi, idesc_s, ks > 0, elect);
                     }
-                    mma_commit_if(sfull(c & 1), elect);
-                    mma_commit_if(kfree(kbuf), elect);
+                    commit(sfull(c & 1));
+                    commit(kfree(kbuf));
                 }
                 __syncwarp();
                 if (++kbuf == NS) { kbuf = 0; kph ^= 1u; }
@@ -346,7 +395,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             for (int c = 0; c < n_ch; ++c) {
                 const int p = c & 1;
                 const uint32_t ph = (uint32_t)(c >> 1) & 1u;
-                const uint32_t vb = v_lo + (uint32_t)vbuf * (TILE >> 4);
+                const uint32_t vb = v_lo + (uint32_t)vbuf * (SLOT >> 4);
 #pragma unroll
                 for (int g2 = 0; g2 < 2; ++g2) {
                     // O[g2] += P_g2(c) V(c)[64 g2 .. 64 g2 + 63]: P from the four warps of group g2 (in tensor
@@ -359,11 +408,14 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) { // K = 16 keys per instruction = 8 columns of packed bf16 pairs
                             // V as an MN-major operand: d is contiguous, the two 64-wide halves are HALF bytes apart
-                            mma_f16_ts(tmem + 256u + (uint32_t)g2 * 128u, a_t + (uint32_t)ks * 8u,
-                                       vb + (uint32_t)((g2 * 64 + ks * 16) * 128 >> 4), hi, idesc_o, (c > 0) || (ks > 0), elect);
+                            // (a pair's CTA holds one of those halves)
+                            const uint32_t od = tmem + 256u + (uint32_t)g2 * 128u, at = a_t + (uint32_t)ks * 8u;
+                            const uint32_t vk = vb + (uint32_t)((g2 * 64 + ks * 16) * 128 >> 4);
+                            if constexpr (PAIR) mma_f16_ts_pair(od, at, vk, hi, idesc_o, (c > 0) || (ks > 0));
+                            else mma_f16_ts(od, at, vk, hi, idesc_o, (c > 0) || (ks > 0), elect);
                         }
-                        mma_commit_if(odone(g2, p), elect);
-                        if (g2 == 1) mma_commit_if(vfree(vbuf), elect);
+                        commit(odone(g2, p));
+                        if (g2 == 1) commit(vfree(vbuf));
                     }
                     __syncwarp();
                 }
@@ -426,7 +478,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                 // (no row of this warp exists: its scores are not looked at, and what its lanes' P holds stays in their
                 // own rows of O, which nobody stores)
                 __syncwarp();
-                if (lane == 0) mbar_arrive(pfull(p));
+                if (lane == 0) arrive_p(pfull(p));
                 continue;
             }
             tc_fence_after();
@@ -488,27 +540,37 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                 }
             }
             // ---- P = exp2(s * scale - m) as bf16 pairs, written over the group's score columns (every score
-            // is in registers by now); the row sum as four independent chains ----
-            float rs4[4] = {0.f, 0.f, 0.f, 0.f};
+            // is in registers by now); the row sum as four pairs of chains; multiply-adds and sums two to an instruction
+            // (33.6 against 34.1 us on 52 heads and 4 K keys, 75.9 against 77.2 on the ragged batch; taking the exponentials
+            // against the old reference while the maximum is being found cost registers: 2 us more on every shape) ----
+            float rs;
+            {
+                const uint64_t scale2 = f32x2(scale, scale), neg = f32x2(-m_safe, -m_safe);
+                uint64_t acc[4];
 #pragma unroll
-            for (int blk = 0; blk < 2; ++blk) {
-                uint32_t w[16];
+                for (int blk = 0; blk < 2; ++blk) {
+                    uint32_t w[16];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const float p0 = ex2f(fmaf(v[blk * 32 + 2 * e], scale, -m_safe));
-                    const float p1 = ex2f(fmaf(v[blk * 32 + 2 * e + 1], scale, -m_safe));
-                    rs4[e & 3] += p0 + p1;
-                    w[e] = pack_bf16(p0, p1);
+                    for (int e = 0; e < 16; ++e) {
+                        float x0, x1;
+                        f32x2_split(f32x2_fma(f32x2(v[blk * 32 + 2 * e], v[blk * 32 + 2 * e + 1]), scale2, neg), x0, x1);
+                        const float p0 = ex2f(x0), p1 = ex2f(x1);
+                        const uint64_t pp = f32x2(p0, p1);
+                        acc[e & 3] = blk == 0 && e < 4 ? pp : f32x2_add(acc[e & 3], pp);
+                        w[e] = pack_bf16(p0, p1);
+                    }
+                    tmem_st16(tS + (uint32_t)blk * 16u, w);
                 }
-                tmem_st16(tS + (uint32_t)blk * 16u, w);
+                float lo, hi;
+                f32x2_split(f32x2_add(f32x2_add(acc[0], acc[1]), f32x2_add(acc[2], acc[3])), lo, hi);
+                rs = lo + hi;
             }
-            const float rs = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
             l_run = l_run * alpha + rs;
             m_run = m_new;
             asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(pfull(p));
+            if (lane == 0) arrive_p(pfull(p));
         }
         // ---- each group waits for its own last product (tensor-core work completes in order, so the
         // one before it is complete too); the CTA-wide barrier below then orders both accumulators
@@ -579,6 +641,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         fspad_pdl_trigger();                      // partial written: the merge kernel may start launching
         tc_fence_before();
         __syncthreads();
+        if (PAIR) cluster_sync_all();             // neither CTA leaves while the other may still reach it
         return;
     }
     // copy and tensor-core warps: meet the softmax warps at their two CTA-wide barriers; the warp
@@ -591,21 +654,24 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         // waits for the last fill it started in every ring slot, the tensor-core warp for everything
         // its thread has issued (one more commit on a barrier of its own).
         if (warp == 8) {
-            for (int sl = 0; sl < NS; ++sl) {
+            for (int sl = 0; sl < NS && rank == 0; ++sl) {    // (a pair's fills are all counted by rank 0's barriers)
                 const int nk = (filled_k - sl + NS - 1) / NS, nv = (filled_v - sl + NS - 1) / NS;   // fills of slot sl
                 if (nk > 0) (void)mbar_wait(kfull(sl), (uint32_t)(nk - 1) & 1u);
                 if (nv > 0) (void)mbar_wait(vfull(sl), (uint32_t)(nv - 1) & 1u);
             }
-        } else {
-            mma_commit_if(drain, lane == 0);
+        } else if (rank == 0) {
+            if constexpr (PAIR) { if (lane == 0) mma_commit_pair(drain); }
+            else mma_commit_if(drain, lane == 0);
             (void)mbar_wait(drain, 0u);
         }
     }
     __syncthreads();
+    if (PAIR) cluster_sync_all();
     if (warp != 9) return;
     tc_fence_after();
     __syncwarp();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(TMEM_COLS) : "memory");
+    if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(TMEM_COLS) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
 // Self-test of the bounded wait: one warp waits, with a small cap, on a barrier that nothing ever
@@ -632,18 +698,38 @@ cudaError_t fspad_launch_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t s
                             (uint32_t)polls);
 }
 
-int fspad_attn_umma_splits(const fspad_ctx *ctx, int N, int B, int sms)
+// Key ranges per row: one CTA per SM, never a partial second wave.
+static int ranges_per_row(const fspad_ctx *ctx, int B, int mtiles, int sms)
 {
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
-    const int G = ctx->cfg.n_q_heads / ctx->cfg.n_kv_heads;
-    const int mtiles = (N * G + umma::BM - 1) / umma::BM;
     const long long base = (long long)B * ctx->cfg.n_kv_heads * mtiles;
-    long long s = sms / base;                     // one CTA per SM, never a partial second wave
+    long long s = sms / base;
     const int max_chunks = (ctx->cfg.max_len + umma::BK - 1) / umma::BK;
     if (s > max_chunks) s = max_chunks;
     if (s > 64) s = 64;
     if (s < 1) s = 1;
     return (int)s;
+}
+
+// Row tiles of a kv head.  Where they alone fill the SMs (a batch: one key range per row, long loops) two or more go in pairs,
+// the last pair possibly with an empty half: 86 -> 77 us on 16 sequences of 240 rows a head, 93 -> 74 us on 4 of 520
+// (five tiles, six in pairs).  Where the keys are split as well, the loops are short and the pair's hand-shakes cost more than
+// it saves: 23.6 against 19.5 us with two chunks a CTA, 40 against 38 us with 17.
+bool fspad_attn_pairs(const fspad_ctx *ctx, int N, int B, int sms)
+{
+    if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
+    const int mtiles = (N * (ctx->cfg.n_q_heads / ctx->cfg.n_kv_heads) + umma::BM - 1) / umma::BM;
+    return mtiles > 1 && 2ll * B * ctx->cfg.n_kv_heads * mtiles > sms;          // (no room for two ranges)
+}
+int fspad_attn_mtiles(const fspad_ctx *ctx, int N, int B, int sms)
+{
+    const int mtiles = (N * (ctx->cfg.n_q_heads / ctx->cfg.n_kv_heads) + umma::BM - 1) / umma::BM;
+    return fspad_attn_pairs(ctx, N, B, sms) ? (mtiles + 1) & ~1 : mtiles;
+}
+
+int fspad_attn_umma_splits(const fspad_ctx *ctx, int N, int B, int sms)
+{
+    return ranges_per_row(ctx, B, fspad_attn_mtiles(ctx, N, B, sms), sms);
 }
 
 // ---- TMA descriptors of the K and V cache planes ----------------------------------------
@@ -691,7 +777,7 @@ static bool make_plane_map(CUtensorMap *map, const fspad_bf16 *plane, size_t row
 
 cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 *kc,
                                          const fspad_bf16 *vc, const fspad_bf16 *tk, const fspad_bf16 *tv,
-                                         const int *parent, const int *prefix_len, int N, int B, int n_splits,
+                                         const int *parent, const int *prefix_len, int N, int B, int sms, int n_splits,
                                          float scale_log2, fspad_bf16 *out, cudaStream_t st, FspadPaged paged)
 {
     const fspad_config &c = ctx->cfg;
@@ -700,16 +786,18 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     a.N = N; a.Hq = c.n_q_heads; a.Hkv = c.n_kv_heads; a.G = c.n_q_heads / c.n_kv_heads;
     a.M = N * a.G; a.max_len = paged.table ? paged.stride * umma::BK : c.max_len; a.n_splits = n_splits;
     a.block_table = paged.table; a.table_stride = paged.stride; a.n_blocks = paged.n_blocks;
-    a.mtiles = (a.M + umma::BM - 1) / umma::BM;
+    a.mtiles = fspad_attn_mtiles(ctx, N, B, sms);
+    const bool pair = fspad_attn_pairs(ctx, N, B, sms);
     // (every CTA ranks all sequences itself, B loads each for B / 320 of its threads: kept to batches where that is small change)
     a.longest_first = (B > 1 && B <= 128 && (long long)B * c.n_kv_heads * a.mtiles * n_splits > ctx->sm_count) ? 1 : 0;
     a.scale_log2 = scale_log2;
     a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.out = n_splits == 1 ? out : nullptr; a.status = ctx->d_status;
     if (!ctx->attn_attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             umma::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, umma::SMEM_BYTES);
+        const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<1, false>, at, umma::smem_bytes(false));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<4, false>, at, umma::smem_bytes(false));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<1, true>, at, umma::smem_bytes(true));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<4, true>, at, umma::smem_bytes(true));
         if (e != cudaSuccess) return e;
         ctx->attn_attr_done = 1;
     }
@@ -717,16 +805,18 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     static_assert(sizeof(CUtensorMap) <= sizeof(ctx->attn_tmap_k), "tensor map storage");
     CUtensorMap *mk = reinterpret_cast<CUtensorMap *>(ctx->attn_tmap_k);
     CUtensorMap *mv = reinterpret_cast<CUtensorMap *>(ctx->attn_tmap_v);
+    CUtensorMap *mk_half = reinterpret_cast<CUtensorMap *>(ctx->attn_tmap_k_half);     // boxes of 64 keys: a pair's CTA loads half a K chunk
     // rows of the plane matrix: every sequence's cache, or the whole pool of blocks
     const size_t rows = paged.table ? (size_t)paged.n_blocks * c.n_kv_heads * umma::BK : (size_t)B * c.n_kv_heads * c.max_len;
     if (ctx->attn_tmap_kptr != kc || ctx->attn_tmap_vptr != vc || ctx->attn_tmap_rows != rows) {
-        ctx->attn_tmap_ok = make_plane_map(mk, kc, rows) && make_plane_map(mv, vc, rows);
+        ctx->attn_tmap_ok = make_plane_map(mk, kc, rows) && make_plane_map(mv, vc, rows) &&
+                            fspad_make_tmap_bf16_2d(mk_half, kc, (size_t)umma::D, rows, (unsigned)umma::BK / 2);
         ctx->attn_tmap_kptr = kc; ctx->attn_tmap_vptr = vc; ctx->attn_tmap_rows = rows;
     }
     a.use_tma = ctx->attn_tmap_ok ? 1 : 0;
-    dim3 grid(n_splits, c.n_kv_heads * a.mtiles, B);
+    const dim3 grid = pair ? dim3(c.n_kv_heads * a.mtiles, n_splits, B) : dim3(n_splits, c.n_kv_heads * a.mtiles, B);
     ctx->launches++;
-    if (N <= FSPAD_MAX_NODES)
-        return fspad_launch_opt(false, umma::tree_attn_umma_kernel<1>, grid, dim3(umma::NT), umma::SMEM_BYTES, st, 0, a, *mk, *mv);
-    return fspad_launch_opt(false, umma::tree_attn_umma_kernel<4>, grid, dim3(umma::NT), umma::SMEM_BYTES, st, 0, a, *mk, *mv);
+    auto kernel = N <= FSPAD_MAX_NODES ? (pair ? umma::tree_attn_umma_kernel<1, true> : umma::tree_attn_umma_kernel<1, false>)
+                                       : (pair ? umma::tree_attn_umma_kernel<4, true> : umma::tree_attn_umma_kernel<4, false>);
+    return fspad_launch_opt(false, kernel, grid, dim3(umma::NT), umma::smem_bytes(pair), st, pair ? 2u : 0u, a, pair ? *mk_half : *mk, *mv);
 }

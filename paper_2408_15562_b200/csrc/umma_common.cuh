@@ -164,6 +164,18 @@ __device__ __forceinline__ void mbar_arrive_rank0(uint32_t bar)
     asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\t"
                  "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n\t}\n" ::"r"(bar) : "memory");
 }
+// The same for an arrival that only orders tensor memory (the tcgen05 fences do that): no release of the cluster's memory,
+// which costs a warp hundreds of cycles.
+__device__ __forceinline__ void mbar_arrive_rank0_light(uint32_t bar)
+{
+    asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\t"
+                 "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_rank0(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\t"
+                 "mbarrier.arrive.expect_tx.shared::cluster.b64 _, [ra], %1;\n\t}\n" ::"r"(bar), "r"(bytes) : "memory");
+}
 // one box into this CTA's shared memory, its bytes counted by the barrier at `bar`'s offset in rank 0's
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
 {
@@ -184,6 +196,14 @@ __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint32_t a_lo, uin
                  "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
                  "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}\n"
                  :: "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+// the pair's product with A from each CTA's own tensor memory
+__device__ __forceinline__ void mma_f16_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                                uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 db, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], db, %4, p;\n\t}\n"
+                 :: "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
 // what has been issued so far arrives, when complete, on the barrier at this offset in both CTAs
 __device__ __forceinline__ void mma_commit_pair(uint32_t bar)
@@ -236,6 +256,30 @@ __device__ __forceinline__ float ex2f(float x)
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// two single-precision operations in one instruction
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void f32x2_split(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)

@@ -109,6 +109,28 @@ def test_more_ctas_than_sms_sequences_taken_longest_first(lengths):
     _check(inp)
 
 
+@pytest.mark.parametrize("n_nodes,group", [(33, 4), (64, 4), (60, 5), (60, 8), (130, 3), (200, 2)])
+@pytest.mark.parametrize("alias", [False, True])
+def test_row_tiles_in_pairs(n_nodes, group, alias):
+    """Calls whose row tiles alone fill the SMs run on pairs of CTAs: 2 to 4 row tiles of a kv head (an empty half of the last pair
+    with 3), the boundary between the tiles inside a node's heads, 1 .. 12 chunks a sequence (every wrap state of the pair's
+    five-deep ring), the gathered boundary chunks first, in the middle and last; tree rows apart and in the cache."""
+    B = 12
+    L = np.array([0, 100, 128, 129, 383, 500, 640, 700, 900, 1151, 1280, 1400], np.int32)
+    w = synth.scaled(W["batch16_ragged"], batch=B, n_q_heads=8 * group, n_kv_heads=8, n_nodes=n_nodes, depth=6, branch=12,
+                     prefix=(int(L.max()), int(L.max())), temperatures=(0.0,) * B, vocab=16, n_layers=1)
+    inp = synth.generate(w, n_nodes, with_accept=False)
+    if inp.parent.shape[1] != n_nodes:
+        pytest.skip("the expansion gave fewer nodes")
+    inp.prefix_len[:] = L
+    _shrink_values(inp)                         # (the first sequences have few keys)
+    if alias:
+        for b in range(B):
+            inp.k_cache[b, :, L[b]:L[b] + n_nodes] = inp.tree_k[b]
+            inp.v_cache[b, :, L[b]:L[b] + n_nodes] = inp.tree_v[b]
+    _check(inp, alias_cache=alias)
+
+
 def test_equal_value_rows_reproduce_exactly():
     """All V rows equal to one bf16 row: the softmax weights sum to 1, so the output is that row."""
     w = synth.scaled(W["llama3_8b_2k"], prefix=(300, 300), vocab=16)
