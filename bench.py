@@ -526,9 +526,9 @@ def main():
                                   "note": "one level of the draft phase (three kernels); not part of value"},
             "lm_head_call": None if lm is None else dict(lm, **{
                 "rows": B * N, "hidden": lm_H, "vocab": w.vocab, "weight_bytes": 2.0 * lm_H * w.vocab,
-                "slabs_of_128_rows": (B * N + 127) // 128,
-                "stats_gbs": 2.0 * lm_H * w.vocab * ((B * N + 127) // 128) / (lm["stats_us"] * 1e-6) / 1e9,
-                "stats_frac_of_hbm_peak": 2.0 * lm_H * w.vocab * ((B * N + 127) // 128) / (lm["stats_us"] * 1e-6) / 1e9 / peak,
+                "slabs_of_1024_rows": (B * N + 1023) // 1024,
+                "stats_gbs": 2.0 * lm_H * w.vocab * ((B * N + 1023) // 1024) / (lm["stats_us"] * 1e-6) / 1e9,
+                "stats_frac_of_hbm_peak": 2.0 * lm_H * w.vocab * ((B * N + 1023) // 1024) / (lm["stats_us"] * 1e-6) / 1e9 / peak,
                 "note": "LM head with the scan as its epilogue (stats) and with the walk behind it (accept); weights are "
                         "streamed once per slab; not part of value"}),
             "feature_sampler_call": None if fs is None else dict(fs, **{
