@@ -77,6 +77,7 @@ struct WalkArgs {
     FspadStatsGeom geom;
     int N, V, path_stride, cache_ok;
     int draft_far;                      // the draft rows lie in host memory: not asked for ahead of need
+    int B, sampled_first;               // sequences; clusters take the sampling ones first
     int *path, *n_acc, *bonus, *status;
     // optional: the cluster that has walked a sequence also moves its accepted K/V rows up (NULL: not asked for)
     uint4 *kv_cache;                    // [layers][2][B][Hkv][max_len][d] bf16 as 16-byte chunks
@@ -681,7 +682,6 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
-    const int b = blockIdx.x / C;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int N = args.N, V = args.V;
 
@@ -689,12 +689,32 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     extern __shared__ __align__(16) unsigned char dyn_smem[];
 
     fspad_pdl_trigger();
+    int b = blockIdx.x / C;
+    if (args.sampled_first) {
+        // More clusters than the SMs hold at once: they are dispatched in index order, so the long walks should come first.
+        // Every CTA takes the sequence whose place in that order (sampling ones, then greedy ones, by index) is its own.
+        const bool samples = tid < args.B && args.temperature[tid] > 0.0f;
+        const unsigned m = __ballot_sync(0xffffffffu, samples);
+        if (lane == 0) sh.warp_off[wid] = (double)__popc(m);
+        __syncthreads();
+        int before = __popc(m & ((1u << lane) - 1u)), total = 0;
+#pragma unroll 1
+        for (int w = 0; w < kWarps; ++w) {
+            const int n = (int)sh.warp_off[w];
+            if (w < wid) before += n;
+            total += n;
+        }
+        if (tid < args.B && (samples ? before : total + tid - before) == b) sh.cur = tid;
+        __syncthreads();
+        b = sh.cur;
+    }
     // The vocabulary scan that precedes this kernel in the stream lets it start only after the scan's
     // own predecessor has completed, and the scan writes nothing but its partial results.  So the
     // caller's arrays may be read before the scan has finished: the prologue's two round trips of
     // dependent loads run under the scan's tail.
     // Round trip 1: everything that depends on nothing - temperature, tree arrays, uniforms.
     float Tf = args.temperature[b];
+    if (!(Tf > 0.0f) && rank > 0) return;        // a greedy sequence is one CTA's work: the others make room for the next cluster
     int p = -1, t = 0;
     float uval = 0.f;
     if (tid < N) {
@@ -804,9 +824,9 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     __syncthreads();
 
     if (!sampling) {
-        greedy_walk(sh.t, args, b, N, tid, kWalkThreads, rank == 0);
-        if (args.kv_cache != nullptr) compact_accepted(args, sh.t, b, rank, C, tid, kWalkThreads);
-        return;   // the whole cluster takes this branch together; no peer memory is touched
+        greedy_walk(sh.t, args, b, N, tid, kWalkThreads, true);
+        if (args.kv_cache != nullptr) compact_accepted(args, sh.t, b, 0, 1, tid, kWalkThreads);
+        return;   // (rank 0 of the cluster; no peer memory is touched)
     }
 
     // ---- sampling ----
@@ -1298,7 +1318,7 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     a.logits = logits; a.draft = draft; a.temperature = temperature; a.uniforms = uniforms;
     a.tokens = tokens; a.parent = parent;
     a.parts = ctx->st_part; a.geom = geom;
-    a.N = N; a.V = V; a.path_stride = ctx->cfg.max_nodes; a.cache_ok = 0; a.draft_far = draft_far ? 1 : 0;
+    a.N = N; a.V = V; a.path_stride = ctx->cfg.max_nodes; a.cache_ok = 0; a.draft_far = draft_far ? 1 : 0; a.B = B; a.sampled_first = 0;
     a.path = path; a.n_acc = n_acc; a.bonus = bonus; a.status = ctx->d_status;
 
     ctx->launches++;
@@ -1308,6 +1328,9 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
         return fspad_launch(accept_greedy_kernel<FSPAD_MAX_NODES_WIDE>, dim3((unsigned)B), dim3(kWalkThreads), 0, st, 0, a);
     }
     const int cluster = walk_cluster_size(ctx, B, V);
+    // (16 sequences, half of them sampling: the walk 75 -> 68 us beside the attention, the step 202 -> 199; with one wave of clusters
+    // the order does not matter and the look at the temperatures is saved)
+    a.sampled_first = B > 1 && B <= kWalkThreads && B * cluster > ctx->sm_count;     // (one thread looks at each sequence)
     const size_t per_cta = (size_t)((((V + 3 + cluster - 1) / cluster) + 3) & ~3);       // as the kernel shares a row out
     const size_t per_thr = ((per_cta + kWalkThreads - 1) / kWalkThreads + 3) & ~(size_t)3;
     const size_t need = per_thr * kWalkThreads * (sizeof(double) + sizeof(float));

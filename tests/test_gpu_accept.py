@@ -170,6 +170,17 @@ def test_full_size_batch16_mixed():
     _assert_parity(inp, allow_near=1)
 
 
+@pytest.mark.parametrize("pattern", ["alternating", "greedy_last", "one_sampling", "all_sampling"])
+def test_more_clusters_than_the_sms_hold(pattern):
+    """20 sequences of 16 CTAs each: the sampling ones are taken first, wherever they stand in the batch, and a greedy one is one
+    CTA's work; every sequence gets its own result."""
+    B = 20
+    temps = {"alternating": (0.0, 1.0) * 10, "greedy_last": (0.8,) * 13 + (0.0,) * 7, "one_sampling": (0.0,) * 11 + (1.0,) + (0.0,) * 8,
+             "all_sampling": (1.0, 0.7, 1.3, 0.9) * 5}[pattern]
+    w = synth.scaled(W["llama3_8b_2k"], batch=B, vocab=33000, n_nodes=12, depth=4, branch=4, temperatures=temps, prefix=(8, 8))
+    _assert_parity(synth.generate(w, 1, with_attention=False), allow_near=1)
+
+
 def test_device_detected_errors_are_reported_not_fatal():
     w = synth.scaled(W["tiny_greedy"], vocab=1000, n_nodes=8, prefix=(8, 8))
     inp = synth.generate(w, 0, with_attention=False)
