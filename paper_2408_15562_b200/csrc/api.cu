@@ -28,6 +28,39 @@ int check_common(const fspad_ctx *ctx, int n_nodes, int batch)
     return FSPAD_OK;
 }
 
+// How a step's attention shares the SMs with its acceptance.  Both entry points take it from here: the number of key ranges
+// follows from attn_sms, and with it which reference a probability is rounded against, so that they give the same bits.
+struct StepPlan {
+    bool scan_first;            // the scan goes first on all SMs, the attention behind it beside the walk
+    int attn_sms;               // SMs the attention may fill (0: all)
+};
+StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample)
+{
+    // Which of the two goes first.  The acceptance is a streaming scan over every SM followed by a walk
+    // that one cluster per sampling sequence carries out; the attention is one CTA per SM.  When the
+    // attention's CTAs leave a good part of the SMs free, both start at once and the acceptance lives on
+    // the free SMs.  Otherwise the scan goes first on all SMs and the attention is forked behind it, sized
+    // to leave the walk's SMs alone, so that the walk (the longer chain) and the attention run side by side.
+    const fspad_config &c = ctx->cfg;
+    const int sms = ctx->sm_count;
+    const long long attn_ctas = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch) *
+                                fspad_attn_umma_splits(ctx, n_nodes, batch);
+    StepPlan p = {may_sample && sms - attn_ctas < sms / 4, 0};
+    if (p.scan_first) {
+        const int walk = fspad_walk_ctas(ctx, batch, c.vocab);
+        p.attn_sms = sms - (walk < sms / 2 ? walk : sms / 2);
+    } else if (!may_sample && attn_ctas > sms / 2) {
+        // An all-greedy acceptance is a scan and a one-CTA walk: beside an attention that holds most SMs the
+        // scan's CTAs only get going when the attention's leave.  Where the context is short enough for the
+        // attention to stay short on half the SMs (at most 8 chunks per CTA by the context's max_len), it
+        // gets half and the two really run side by side (17.2 against 20.5 us on the 26-node greedy workload).
+        const int s_half = fspad_attn_umma_splits(ctx, n_nodes, batch, sms / 2);
+        const int max_chunks = (c.max_len + 127) / 128;
+        if ((max_chunks + s_half - 1) / s_half <= 8) p.attn_sms = sms / 2;
+    }
+    return p;
+}
+
 }  // namespace
 
 extern "C" {
@@ -418,21 +451,11 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
     const size_t plane = (size_t)batch * c.n_kv_heads * (size_t)c.max_len * FSPAD_HEAD_DIM;
     const fspad_bf16 *kc = cache + (size_t)attn_layer * 2 * plane, *vc = kc + plane;
 
-    // Which of the two goes first.  The acceptance is a streaming scan over every SM followed by a walk
-    // that one cluster per sampling sequence carries out; the attention is one CTA per SM.  When the
-    // attention's CTAs leave a good part of the SMs free, both start at once and the acceptance lives on
-    // the free SMs.  Otherwise the scan goes first on all SMs and the attention is forked behind it, sized
-    // to leave the walk's SMs alone, so that the walk (the longer chain) and the attention run side by side.
     const int sms = ctx->sm_count;
-    const long long attn_ctas = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch) *
-                                fspad_attn_umma_splits(ctx, n_nodes, batch);
     const bool may_sample = draft_probs != nullptr;
-    const bool scan_first = may_sample && sms - attn_ctas < sms / 4;
-    int attn_sms = 0;
-    if (scan_first) {
-        const int walk = fspad_walk_ctas(ctx, batch, c.vocab);
-        attn_sms = sms - (walk < sms / 2 ? walk : sms / 2);
-    }
+    const StepPlan plan = step_plan(ctx, n_nodes, batch, may_sample);
+    const bool scan_first = plan.scan_first;
+    const int attn_sms = plan.attn_sms;
     cudaError_t ce = cudaSuccess;
     FspadStatsGeom geom;
     const int rows = batch * n_nodes;
@@ -444,18 +467,8 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
         return FSPAD_ERR_CUDA;
     int rc_attn = FSPAD_OK;
     if (!scan_first) {
-        // An all-greedy acceptance is a scan and a one-CTA walk: beside an attention that holds most SMs the
-        // scan's CTAs only get going when the attention's leave.  Where the context is short enough for the
-        // attention to stay short on half the SMs (at most 8 chunks per CTA by the context's max_len), it
-        // gets half and the two really run side by side (17.2 against 20.5 us on the 26-node greedy workload).
-        int both_sms = 0;
-        if (!may_sample && attn_ctas > sms / 2) {
-            const int s_half = fspad_attn_umma_splits(ctx, n_nodes, batch, sms / 2);
-            const int max_chunks = (c.max_len + 127) / 128;
-            if ((max_chunks + s_half - 1) / s_half <= 8) both_sms = sms / 2;
-        }
         rc_attn = fspad_launch_tree_attn(ctx, q, kc, vc, tree_k, tree_v, parent, prefix_len, n_nodes, batch, attn_out,
-                                         ctx->side, both_sms) == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;
+                                         ctx->side, attn_sms) == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;
         // Here the scan is launched as a plain dependent: as a programmatic dependent of the previous
         // step's last kernel it was seen to hold the forked attention back behind the whole acceptance
         // (steps replayed from one CUDA graph: 72.5 us per step against 48.8 on the 52-head shape).
@@ -467,9 +480,9 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
         // full-size scan are the better neighbours (37.6 against 39.0 us): an attention CTA that finds
         // its SM taken waits for a scan CTA's whole life.
         int scan_sms = 0;
-        if (may_sample || both_sms > 0) {
-            const long long attn_now = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch, both_sms) *
-                                       fspad_attn_umma_splits(ctx, n_nodes, batch, both_sms);
+        if (may_sample || attn_sms > 0) {
+            const long long attn_now = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch, attn_sms) *
+                                       fspad_attn_umma_splits(ctx, n_nodes, batch, attn_sms);
             scan_sms = sms - (int)(attn_now < sms ? attn_now : sms);
             if (scan_sms < sms / 8) scan_sms = sms / 8;
         }
@@ -601,8 +614,9 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     if (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess)
         return FSPAD_ERR_CUDA;
     const size_t plane = (size_t)batch * c.n_kv_heads * (size_t)c.max_len * FSPAD_HEAD_DIM;
+    const StepPlan plan = step_plan(ctx, n_nodes, batch, draft_probs != nullptr);
     const bool attn_ok = fspad_launch_tree_attn(ctx, ctx->h_q, cache, cache + plane, nullptr, nullptr, ctx->h_parent, ctx->h_prefix,
-                                                n_nodes, batch, ctx->h_out, ctx->side) == cudaSuccess;
+                                                n_nodes, batch, ctx->h_out, ctx->side, plan.attn_sms) == cudaSuccess;
     h2d(ctx->h_tokens, draft_tokens, B * N * sizeof(int));
     h2d(ctx->h_temp, temperature, B * sizeof(float));
     if (draft_probs) h2d(ctx->h_unif, uniforms, B * (N + 1) * sizeof(float));

@@ -99,3 +99,34 @@ def test_draft_rows_in_place_or_copied(vocab, n_nodes):
         assert np.array_equal(path.numpy(), r["accepted_path"])
         assert np.array_equal(n.numpy(), r["n_accepted"]) and np.array_equal(bonus.numpy(), r["bonus_token"])
         assert np.array_equal(new_len.numpy(), inp.prefix_len + r["n_accepted"])
+
+
+@pytest.mark.parametrize("temps,prefix,nodes,hq,hkv", [((1.0,), 2048, 60, 32, 8), ((0.0,), 2048, 60, 32, 8), ((0.0,), 256, 26, 32, 32)])
+def test_host_entry_gives_the_bits_of_the_device_entry(temps, prefix, nodes, hq, hkv):
+    """Sizes at which the step leaves SMs to the acceptance, so that its attention has fewer key ranges than one alone would have:
+    both entry points take the same ranges, and every output is the same bit for bit."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=1, prefix=(prefix, prefix), n_q_heads=hq, n_kv_heads=hkv, n_nodes=nodes, depth=6,
+                     branch=10, vocab=32000, temperatures=temps, n_layers=1)
+    inp = synth.generate(w, 2)
+    B, N = inp.parent.shape
+    ctx = helpers.make_ctx(inp, n_layers=1)
+    cache_host = synth.make_cache(inp, 1)
+    L = inp.prefix_len
+    cache_host[0, 0, 0, :, L[0]:L[0] + N] = inp.tree_k[0]
+    cache_host[0, 1, 0, :, L[0]:L[0] + N] = inp.tree_v[0]
+    d, cache_d = helpers.upload_accept(inp), binding.bf16_tensor(cache_host)
+    q = binding.bf16_tensor(inp.q)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    want = [torch.empty_like(q), torch.empty((B, N), **i32)] + [torch.empty((B,), **i32) for _ in range(3)]
+    ctx.verify_step(cache_d, q, None, None, d["parent"], helpers.dev(L), d["target_logits"], d["draft_probs"], d["draft_tokens"],
+                    d["temperature"], d["uniforms"], *want)
+    ctx.check()
+    pin = lambda a: None if a is None else torch.from_numpy(np.ascontiguousarray(a)).pin_memory()   # noqa: E731
+    got = [torch.empty(t.shape, dtype=t.dtype).pin_memory() for t in want]
+    cache_h = binding.bf16_tensor(synth.make_cache(inp, 1))
+    ctx.verify_step_host(cache_h, *(binding.bf16_tensor(a, "cpu").pin_memory() for a in (inp.q, inp.tree_k, inp.tree_v)), pin(inp.parent),
+                         pin(L), pin(inp.target_logits), pin(inp.draft_probs), pin(inp.draft_tokens), pin(inp.temperature),
+                         pin(inp.uniforms) if inp.draft_probs is not None else None, *got)
+    torch.cuda.synchronize()
+    for g, t in zip(got, want):
+        assert torch.equal(g.view(torch.int16), t.cpu().view(torch.int16))

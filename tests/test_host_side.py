@@ -1,0 +1,89 @@
+"""The host side of the step's two entry points without a device: api.cu compiled for the CPU against stand-ins for the CUDA
+runtime and the launchers (`host_fake.cpp`) that log every call and can fail on demand."""
+import ctypes
+import os
+import re
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2408_15562_b200 import binding
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CSRC = os.path.join(ROOT, "paper_2408_15562_b200", "csrc")
+STREAM = 0x77
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("host_side") / "libhostside.so")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic",
+                           "-DatomicCAS(p,a,b)=((void)(p),(void)(a),(void)(b))",
+                           "-I" + os.path.join(ROOT, "include"), "-I" + CSRC, "-I/usr/local/cuda/include",
+                           "-x", "c++", os.path.join(CSRC, "api.cu"), os.path.join(HERE, "host_fake.cpp"), "-o", out])
+    lib = ctypes.CDLL(out)
+    vp, ci = ctypes.c_void_p, ctypes.c_int
+    lib.fspad_create.argtypes = [ctypes.POINTER(binding.FspadConfig), ctypes.POINTER(vp)]
+    lib.fspad_destroy.argtypes = [vp]
+    lib.fspad_destroy.restype = None
+    lib.fspad_verify_step.argtypes = [vp, vp, ci] + [vp] * 10 + [ci, ci] + [vp] * 6
+    lib.fspad_verify_step_host.argtypes = [vp] * 12 + [ci, ci] + [vp] * 6
+    lib.fake_log.restype = ctypes.c_char_p
+    lib.fake_fail.argtypes = [ctypes.c_char_p, ci]
+    lib.fake_pin.argtypes = [vp, ctypes.c_size_t]
+    return lib
+
+
+class Step:
+    """One context and one set of (never read) buffers for both entry points."""
+
+    def __init__(self, lib, hq=32, hkv=8, nodes=60, batch=1, vocab=4096, max_len=2176, sampling=True):
+        self.lib, self.n, self.batch, self.vocab, self.sampling = lib, nodes, batch, vocab, sampling
+        cfg = binding.FspadConfig(hq, hkv, 128, nodes, vocab, 1, max_len, batch, 0.0)
+        self.ctx = ctypes.c_void_p()
+        assert lib.fspad_create(ctypes.byref(cfg), ctypes.byref(self.ctx)) == 0
+        raw = np.zeros(batch * nodes * vocab + 8, np.float32)
+        skip = (-raw.ctypes.data // 4) % 4
+        self.draft = raw[skip:skip + batch * nodes * vocab]              # 16-byte aligned
+        self.small = np.zeros(batch * (max(nodes, 64) + 1) + 8, np.int32)
+        lib.fake_reset()
+
+    def __del__(self):
+        self.lib.fspad_destroy(self.ctx)
+
+    def host(self):
+        big = 0x1000                                     # never dereferenced by the stand-ins
+        p = self.small.ctypes.data
+        draft, unif = (self.draft.ctypes.data, p) if self.sampling else (None, None)
+        rc = self.lib.fspad_verify_step_host(self.ctx, big, big, big, big, big, big, big, draft, big, big, unif, self.n, self.batch,
+                                             big, p, p, p, p, STREAM)
+        return rc, self.lib.fake_log().decode().splitlines()
+
+    def device(self):
+        big = 0x1000
+        draft, unif = (big, big) if self.sampling else (None, None)
+        rc = self.lib.fspad_verify_step(self.ctx, big, 0, big, None, None, big, big, big, draft, big, big, unif, self.n, self.batch, big,
+                                        big, big, big, big, STREAM)
+        return rc, self.lib.fake_log().decode().splitlines()
+
+
+def _field(log, name, key):
+    line = next(x for x in log if x.startswith(name + " "))
+    return re.search(key + r"=(\S+)", line).group(1)
+
+
+@pytest.mark.parametrize("sampling", [True, False])
+@pytest.mark.parametrize("hq,hkv,nodes,batch,max_len", [(32, 8, 60, 1, 2176), (52, 52, 60, 1, 4224), (64, 8, 60, 1, 8320),
+                                                        (32, 32, 26, 1, 320), (32, 8, 24, 3, 384), (28, 4, 8, 2, 512)])
+def test_host_entry_cuts_the_attention_as_the_device_entry_does(lib, hq, hkv, nodes, batch, max_len, sampling):
+    """The number of key ranges decides which probabilities are rounded against which reference: the two entry points give the
+    same bits only if they let the attention fill the same number of SMs."""
+    step = Step(lib, hq, hkv, nodes, batch, max_len=max_len, sampling=sampling)
+    rc, log = step.device()
+    want = _field(log, "attention", "sms")
+    lib.fake_reset()
+    rc_h, log_h = step.host()
+    assert rc == 0 and rc_h == 0
+    assert _field(log_h, "attention", "sms") == want
