@@ -98,8 +98,9 @@ long long fspad_launch_count(const fspad_ctx *ctx);
  * library; no passage of the paper).  Every wait of a kernel on a barrier has
  * a poll limit; when it runs out the kernel records FSPAD_ERR_TIMEOUT in the
  * status word and returns.  This call queues one warp that waits, with a limit
- * of `polls` polls (1 .. 4096), on a barrier nothing ever arrives on: after it
- * fspad_status() returns FSPAD_ERR_TIMEOUT, and the context stays usable.
+ * of `polls` polls (1 .. 4096), on a barrier nothing ever arrives on, and then a
+ * pair of CTAs of which one waits in the same way for the other's message: after
+ * it fspad_status() returns FSPAD_ERR_TIMEOUT, and the context stays usable.
  */
 int fspad_selftest_wait_timeout(fspad_ctx *ctx, int polls, void *stream);
 

@@ -506,16 +506,28 @@ __device__ __forceinline__ void expect_bytes(uint32_t bar, int bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity)
+constexpr uint32_t kPolls = 2000000;                 // about 50 ms
+__device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, uint32_t polls = kPolls)
 {
 #pragma unroll 1
-    for (uint32_t i = 0; i < 2000000; ++i) {         // about 50 ms
+    for (uint32_t i = 0; i < polls; ++i) {
         uint32_t ok;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
         if (ok) return true;
     }
     return false;
+}
+
+// The same wait by every thread of the CTA.  What a thread has seen is its own: one may give up just before the last bytes
+// land and the next may not, and barriers of the CTA in what follows would then be reached by some only.  So nobody goes on
+// before all have waited, and all go on (true) or none does.
+template <class Shared>
+__device__ __forceinline__ bool wait_cluster_all(Shared &sh, uint32_t bar, uint32_t parity, uint32_t polls = kPolls)
+{
+    if (!wait_cluster(bar, parity, polls)) sh.fail = 1;
+    __syncthreads();
+    return sh.fail == 0;
 }
 
 // block-wide scan of one value per thread (index order): this thread's exclusive and inclusive prefix and the CTA total
@@ -1220,16 +1232,16 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         }
         double E, total;
         const double P = block_scan(sh, mine, &E, &total);
-        // the CTA total goes to every CTA of the cluster, as in exchange(); every warp waits for the peers' itself
+        // the CTA total goes to every CTA of the cluster, as in exchange(); every thread waits for the peers' itself
         const int par = n_exch & 1;
         const uint32_t bar = smem_addr(&sh.bar[par]);
         if (tid == 0) expect_bytes(bar, C * 8);
         if (tid < C) send_double(smem_addr(&sh.slot[par][0][rank]), bar, tid, total);
-        if (!wait_cluster(bar, (uint32_t)(n_exch >> 1) & 1u)) {
-            fspad_report(args.status, FSPAD_ERR_TIMEOUT);
-            sh.fail = 1;
+        if (!wait_cluster_all(sh, bar, (uint32_t)(n_exch >> 1) & 1u)) {
+            if (tid == 0) fspad_report(args.status, FSPAD_ERR_TIMEOUT);
+            cluster.sync();                                   // nobody leaves while a peer may still write to its shared memory
+            return;
         }
-        __syncwarp();
         // every warp scans the CTA totals side by side: mass in front of this CTA, whole mass, owner of the target
         double cum = (lane < C) ? sh.slot[par][0][lane & (kMaxCluster - 1)] : 0.0;
 #pragma unroll
@@ -1260,12 +1272,41 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         if (owner < 0 && rank == 0 && tid == 0) args.bonus[b] = 0;   // no positive weight anywhere
     }
     if (args.kv_cache != nullptr) compact_accepted(args, sh.t, b, rank, C, tid, kWalkThreads);   // (the CTAs that do not own the draw are at it meanwhile)
-    // every CTA has received every peer's total by now, so each may leave on its own - unless a wait ran out
-    __syncthreads();
-    if (sh.fail != 0) cluster.sync();
+    // every CTA has received every peer's total by now, so each may leave on its own
+}
+
+// Self-test of the last wait: a pair of CTAs, of which the second sends nothing.  The first one's wait runs out after `polls`
+// polls, all its threads leave the same way, and the kernel ends normally.
+struct WaitTestShared {
+    double slot;
+    unsigned long long bar;
+    int fail;
+};
+__global__ void __launch_bounds__(64) walk_wait_selftest_kernel(int *status, uint32_t polls)
+{
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ WaitTestShared sh;
+    const int rank = (int)cluster.block_rank();
+    const uint32_t bar = smem_addr(&sh.bar);
+    if (threadIdx.x == 0) {
+        sh.fail = 0;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar));
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    cluster.sync();
+    if (threadIdx.x == 0) expect_bytes(bar, 8);
+    if (rank == 0 && threadIdx.x == 0) send_double(smem_addr(&sh.slot), bar, 1, 1.0);
+    if (!wait_cluster_all(sh, bar, 0u, rank == 0 ? polls : kPolls) && threadIdx.x == 0) fspad_report(status, FSPAD_ERR_TIMEOUT);
+    cluster.sync();
 }
 
 }  // namespace
+
+cudaError_t fspad_launch_walk_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t st)
+{
+    ctx->launches++;
+    return fspad_launch_opt(false, walk_wait_selftest_kernel, dim3(2), dim3(64), 0, st, 2u, ctx->d_status, (uint32_t)polls);
+}
 
 // Cluster size of the sampling walk.  Once per context: raise the dynamic shared-memory limit and find
 // the largest cluster the device can co-schedule for this kernel: 16 (opt-in), else 8.  Small

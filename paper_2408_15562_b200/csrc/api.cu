@@ -190,7 +190,9 @@ int fspad_selftest_wait_timeout(fspad_ctx *ctx, int polls, void *stream)
 {
     if (!ctx) return FSPAD_ERR_NULL;
     if (polls < 1 || polls > 4096) return FSPAD_ERR_RANGE;
-    return fspad_launch_wait_selftest(ctx, polls, fspad_stream(stream)) == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;
+    return fspad_launch_wait_selftest(ctx, polls, fspad_stream(stream)) == cudaSuccess &&
+                   fspad_launch_walk_wait_selftest(ctx, polls, fspad_stream(stream)) == cudaSuccess
+               ? FSPAD_OK : FSPAD_ERR_CUDA;
 }
 
 int fspad_tree_attn(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 *k_cache,

@@ -332,6 +332,7 @@ cudaError_t fspad_launch_lm_head(fspad_ctx *ctx, const fspad_bf16 *hidden, const
                                  float *row_max, double *row_sum, int *row_arg, cudaStream_t st);
 int fspad_walk_ctas(fspad_ctx *ctx, int B, int V);   // CTAs of the sampling walk for B sequences
 cudaError_t fspad_launch_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t st);
+cudaError_t fspad_launch_walk_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t st);
 cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 *kc,
                                          const fspad_bf16 *vc, const fspad_bf16 *tk, const fspad_bf16 *tv,
                                          const int *parent, const int *prefix_len, int N, int B, int sms, int n_splits,

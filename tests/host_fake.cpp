@@ -139,3 +139,4 @@ cudaError_t fspad_launch_tree_build(fspad_ctx *, const int *, const int *, const
                                     unsigned long long *, int *, cudaStream_t)
 { return cudaErrorUnknown; }
 cudaError_t fspad_launch_wait_selftest(fspad_ctx *, int, cudaStream_t) { return cudaErrorUnknown; }
+cudaError_t fspad_launch_walk_wait_selftest(fspad_ctx *, int, cudaStream_t) { return cudaErrorUnknown; }

@@ -29,3 +29,22 @@ def test_wait_runs_out_and_is_reported_once():
     mx, mean = helpers.attn_errors(out, ref)
     assert mx <= 1e-2 and mean <= 1e-3
     torch.cuda.synchronize()
+
+
+def test_a_cta_whose_peer_is_silent_leaves_as_a_whole():
+    """The walk's last exchange: the wait for a peer that never sends runs out, all threads of the CTA take the same way out, and the
+    next call on the context, a sampling walk, is correct."""
+    w = synth.scaled(synth.WORKLOADS["llama3_8b_2k"], batch=2, prefix=(8, 8), n_nodes=12, depth=3, branch=3, vocab=5000,
+                     temperatures=(1.0, 0.7))
+    inp = synth.generate(w, 0, with_attention=False)
+    ctx = helpers.make_ctx(inp)
+    for polls in (1, 100, 4096):
+        before = ctx.launch_count()
+        assert ctx.selftest_wait_timeout(polls) == 0
+        assert ctx.launch_count() == before + 2       # the lone warp and the pair of CTAs
+        assert ctx.status() == -7 and ctx.status() == 0
+    d = helpers.upload_accept(inp)
+    got = ctx.tree_accept(d["target_logits"], d["draft_probs"], d["draft_tokens"], d["parent"], d["temperature"], d["uniforms"])
+    ctx.check()
+    hard, near, msgs = helpers.compare_accept(inp, *(t.cpu().numpy() for t in got))
+    assert hard == 0, msgs
