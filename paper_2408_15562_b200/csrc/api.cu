@@ -6,6 +6,8 @@
 #include <cstring>
 #include <new>
 
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace {
@@ -26,6 +28,34 @@ int check_common(const fspad_ctx *ctx, int n_nodes, int batch)
     if (n_nodes > FSPAD_MAX_NODES_WIDE || n_nodes > ctx->cfg.max_nodes) return FSPAD_ERR_TREE_TOO_LARGE;
     if (n_nodes < 1 || batch < 0 || batch > ctx->cfg.max_batch) return FSPAD_ERR_SHAPE;
     return FSPAD_OK;
+}
+
+// Device address of host memory [p, p + bytes) if all of it is page-locked and mapped in one piece, else NULL.  The first
+// byte alone says nothing about the rest: of a buffer whose front part only is registered a kernel would read past the mapping.
+const void *mapped_whole(const void *p, size_t bytes)
+{
+    typedef CUresult (*AttrFn)(void *, CUpointer_attribute, CUdeviceptr);
+    static const AttrFn attr = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPoint("cuPointerGetAttribute", &fn, cudaEnableDefault, &q) == cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        (void)cudaGetLastError();
+        return ok ? reinterpret_cast<AttrFn>(fn) : nullptr;
+    }();
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    if (at.type != cudaMemoryTypeHost || at.devicePointer == nullptr || attr == nullptr) return nullptr;
+    CUdeviceptr lo = 0;
+    size_t size = 0;
+    const CUdeviceptr first = reinterpret_cast<CUdeviceptr>(at.devicePointer);
+    if (attr(&lo, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, first) != CUDA_SUCCESS ||
+        attr(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, first) != CUDA_SUCCESS)
+        return nullptr;
+    return first >= lo && first - lo <= size && size - (first - lo) >= bytes ? at.devicePointer : nullptr;
 }
 
 // How a step's attention shares the SMs with its acceptance.  Both entry points take it from here: the number of key ranges
@@ -592,15 +622,8 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     // The walk reads draft rows only where it rejects, and one probability per node: page-locked draft rows are left where they
     // are and read over the link by the kernel (60 rows of 128256 copied whole took 557 us, as long as the logits).  The
     // kernel wants them on a 16-byte boundary, and pageable ones have to be copied.
-    const float *draft = nullptr;
-    if (draft_probs) {
-        cudaPointerAttributes at;
-        if (cudaPointerGetAttributes(&at, draft_probs) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer != nullptr &&
-            !misaligned(at.devicePointer))
-            draft = static_cast<const float *>(at.devicePointer);
-        else
-            (void)cudaGetLastError();
-    }
+    const float *draft = draft_probs ? static_cast<const float *>(mapped_whole(draft_probs, lg_bytes)) : nullptr;
+    if (misaligned(draft)) draft = nullptr;
     const bool draft_in_place = draft != nullptr;
     h2d(ctx->h_prefix, prefix_len, B * sizeof(int));
     h2d(ctx->h_parent, parent, B * N * sizeof(int));

@@ -8,6 +8,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace {
@@ -74,6 +76,22 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p)
     a->type = in ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
     a->devicePointer = in ? const_cast<void *>(p) : nullptr;
     a->hostPointer = const_cast<void *>(p);
+    return cudaSuccess;
+}
+
+CUresult fake_pointer_attribute(void *data, CUpointer_attribute what, CUdeviceptr p)
+{
+    const Range *r = pinned((const void *)p);
+    if (!r) return CUDA_ERROR_INVALID_VALUE;
+    if (what == CU_POINTER_ATTRIBUTE_RANGE_START_ADDR) *(CUdeviceptr *)data = (CUdeviceptr)r->lo;
+    else if (what == CU_POINTER_ATTRIBUTE_RANGE_SIZE) *(size_t *)data = r->bytes;
+    else return CUDA_ERROR_INVALID_VALUE;
+    return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPoint(const char *, void **fn, unsigned long long, cudaDriverEntryPointQueryResult *q)
+{
+    *fn = (void *)fake_pointer_attribute;
+    if (q) *q = cudaDriverEntryPointSuccess;
     return cudaSuccess;
 }
 

@@ -87,3 +87,19 @@ def test_host_entry_cuts_the_attention_as_the_device_entry_does(lib, hq, hkv, no
     rc_h, log_h = step.host()
     assert rc == 0 and rc_h == 0
     assert _field(log_h, "attention", "sms") == want
+
+
+@pytest.mark.parametrize("pins,in_place", [(((0, 1.0),), True), ((), False), (((0, 0.5),), False), (((0, 0.999),), False),
+                                           (((0.5, 0.5),), False), (((0, 0.25), (0.75, 0.25)), False), (((0, 0.5), (0.5, 0.5)), False)])
+def test_draft_rows_are_read_in_place_only_where_all_of_them_are_pinned(lib, pins, in_place):
+    """(first byte, length) of the registered parts, as shares of the draft rows."""
+    step = Step(lib)
+    n = step.draft.nbytes
+    for at, share in pins:
+        lib.fake_pin(step.draft.ctypes.data + int(at * n), int(share * n))
+    rc, log = step.host()
+    assert rc == 0
+    copied = any(x.startswith("h2d host=%x " % step.draft.ctypes.data) for x in log)
+    assert copied != in_place and _field(log, "walk", "far") == str(int(in_place))
+    if in_place:
+        assert int(_field(log, "walk", "draft"), 16) == step.draft.ctypes.data
