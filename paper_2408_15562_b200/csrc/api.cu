@@ -619,6 +619,13 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     auto d2h = [&](void *dst, const void *src, size_t bytes) {
         ok = ok && cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
     };
+    // The caller's memory is read and written by what is queued, the draft rows by the walk itself: an error, too, is returned only
+    // when nothing of it is still under way.
+    auto give_up = [&](int err) {
+        (void)cudaStreamSynchronize(ctx->side);
+        (void)cudaStreamSynchronize(st);
+        return err;
+    };
     // The walk reads draft rows only where it rejects, and one probability per node: page-locked draft rows are left where they
     // are and read over the link by the kernel (60 rows of 128256 copied whole took 557 us, as long as the logits).  The
     // kernel wants them on a 16-byte boundary, and pageable ones have to be copied.
@@ -630,14 +637,14 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     h2d(ctx->h_tk, tree_k, t_bytes);
     h2d(ctx->h_tv, tree_v, t_bytes);
     h2d(ctx->h_q, q, q_bytes);
-    if (!ok) return FSPAD_ERR_CUDA;
+    if (!ok) return give_up(FSPAD_ERR_CUDA);
     // the tree rows go into cache rows L_b .. of layer 0 (K at [0][0], V at [0][1]); the attention then takes them from there
     if (fspad_launch_tree_scatter(ctx, cache, ctx->h_tk, ctx->h_tv, ctx->h_prefix, n_nodes, batch, st) !=
         cudaSuccess)
-        return FSPAD_ERR_CUDA;
+        return give_up(FSPAD_ERR_CUDA);
     // fork: the attention and its result's way back run beside the copy of the logits
     if (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess)
-        return FSPAD_ERR_CUDA;
+        return give_up(FSPAD_ERR_CUDA);
     const size_t plane = (size_t)batch * c.n_kv_heads * (size_t)c.max_len * FSPAD_HEAD_DIM;
     const StepPlan plan = step_plan(ctx, n_nodes, batch, draft_probs != nullptr);
     const bool attn_ok = fspad_launch_tree_attn(ctx, ctx->h_q, cache, cache + plane, nullptr, nullptr, ctx->h_parent, ctx->h_prefix,
@@ -652,7 +659,6 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     }
     ok = ok && attn_ok &&
          cudaMemcpyAsync(attn_out, ctx->h_out, q_bytes, cudaMemcpyDeviceToHost, ctx->side) == cudaSuccess;
-    // the join is queued whatever happened in between: the caller's stream ends behind everything
     const bool joined = cudaEventRecord(ctx->ev_join, ctx->side) == cudaSuccess;
     FspadStatsGeom geom;
     ok = ok && fspad_launch_stats_partials(ctx, ctx->h_logits, ctx->h_temp, batch * n_nodes, n_nodes, c.vocab, &geom, st) == cudaSuccess;
@@ -660,17 +666,18 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
                                         draft_probs ? ctx->h_unif : nullptr, geom, n_nodes, batch, c.vocab, ctx->h_path, ctx->h_nacc,
                                         ctx->h_bonus, st, FspadWalkCompact(), draft_in_place) == cudaSuccess;
     // the compaction rewrites cache rows that the attention reads
-    if (!joined || cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess || !ok) return FSPAD_ERR_CUDA;
+    if (!joined || cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess || !ok) return give_up(FSPAD_ERR_CUDA);
     if (fspad_launch_kv_compact(ctx, cache, ctx->h_path, ctx->h_nacc, ctx->h_prefix, batch, ctx->h_newlen, st, false) != cudaSuccess)
-        return FSPAD_ERR_CUDA;
+        return give_up(FSPAD_ERR_CUDA);
 
     // the device path array has max_nodes entries per sequence, and so has the host one
     d2h(accepted_path, ctx->h_path, B * (size_t)c.max_nodes * sizeof(int));
     d2h(n_accepted, ctx->h_nacc, B * sizeof(int));
     d2h(bonus_token, ctx->h_bonus, B * sizeof(int));
     d2h(new_len, ctx->h_newlen, B * sizeof(int));
-    if (!ok) return FSPAD_ERR_CUDA;
-    return fspad_status(ctx, stream);
+    if (!ok) return give_up(FSPAD_ERR_CUDA);
+    rc = fspad_status(ctx, stream);                // (waits for the stream)
+    return rc == FSPAD_ERR_CUDA ? give_up(rc) : rc;
 }
 
 }  // extern "C"

@@ -103,3 +103,22 @@ def test_draft_rows_are_read_in_place_only_where_all_of_them_are_pinned(lib, pin
     assert copied != in_place and _field(log, "walk", "far") == str(int(in_place))
     if in_place:
         assert int(_field(log, "walk", "draft"), 16) == step.draft.ctypes.data
+
+
+FAILING = [("h2d", k) for k in range(1, 10)] + [("d2h", k) for k in range(1, 7)] + \
+    [(name, 1) for name in ("scatter", "attention", "scan", "walk", "compact", "sync")] + \
+    [("event_record", k) for k in (1, 2)] + [("stream_wait", k) for k in (1, 2)]
+
+
+@pytest.mark.parametrize("name,nth", FAILING)
+def test_host_entry_returns_an_error_only_when_nothing_is_under_way(lib, name, nth):
+    """Copies and the walk use the caller's memory: whatever call fails, both streams have been waited for after the last thing queued."""
+    step = Step(lib)
+    lib.fake_fail(name.encode(), nth)
+    rc, log = step.host()
+    assert rc == -6                                                  # FSPAD_ERR_CUDA
+    side = next((re.search(r"stream=(\S+)", x).group(1) for x in log if x.startswith("attention ")), None)
+    for stream in {"%x" % STREAM, side} - {None}:
+        mine = [k for k, x in enumerate(log) if x.endswith("stream=" + stream) and not x.startswith("sync ")]
+        waits = [k for k, x in enumerate(log) if x == "sync stream=" + stream]
+        assert not mine or (waits and max(waits) > max(mine)), (stream, log)
