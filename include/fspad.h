@@ -301,7 +301,8 @@ int fspad_feature_sampler(fspad_ctx *ctx, const fspad_bf16 *f, const fspad_bf16 
  * cand_logp = frontier_logp[f] + value (one single-precision addition).  The
  * `width` new candidates with the largest joint value (equal values: the lower
  * candidate index first) are returned, in that order, as next_cand / next_logp
- * [batch][width]: the frontier of the next level.  cand_* are [batch][n_cand_cap],
+ * [batch][width]: the frontier of the next level.  next_* may be the buffers of
+ * frontier_* or overlap them in any way.  cand_* are [batch][n_cand_cap],
  * device, owned by the caller; only the new entries are written.  Per-piece
  * lists live in the context's scratch (allocated by fspad_create): one call per
  * context at a time.  Asynchronous on `stream`.  Errors: FSPAD_ERR_SHAPE for

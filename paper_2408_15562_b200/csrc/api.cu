@@ -166,6 +166,7 @@ int fspad_create(const fspad_config *cfg, fspad_ctx **out)
         ctx->dx_part = dx;
     }
     ok = ok && dev_alloc(&ctx->dx_done, B);
+    ok = ok && dev_alloc(&ctx->dx_front, 2 * B * FSPAD_MAX_FRONTIER);
     ok = ok && dev_alloc(&ctx->lm_parts, (rows < FSPAD_LM_SLAB_ROWS ? rows : (size_t)FSPAD_LM_SLAB_ROWS) * fspad_lm_head_tiles(cfg->vocab));
     ok = ok && cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) == cudaSuccess;
@@ -186,7 +187,7 @@ void fspad_destroy(fspad_ctx *ctx)
 {
     if (!ctx) return;
     cudaDeviceSynchronize();
-    void *ptrs[] = {ctx->lm_parts, ctx->dx_part, ctx->dx_done, ctx->d_status, ctx->part_o, ctx->part_ml, ctx->st_part, ctx->row_max, ctx->row_sum, ctx->row_arg, ctx->h_q, ctx->h_tk,
+    void *ptrs[] = {ctx->lm_parts, ctx->dx_part, ctx->dx_done, ctx->dx_front, ctx->d_status, ctx->part_o, ctx->part_ml, ctx->st_part, ctx->row_max, ctx->row_sum, ctx->row_arg, ctx->h_q, ctx->h_tk,
                     ctx->h_tv, ctx->h_out, ctx->h_parent, ctx->h_prefix, ctx->h_tokens, ctx->h_path,
                     ctx->h_nacc, ctx->h_bonus, ctx->h_newlen, ctx->h_logits, ctx->h_draft, ctx->h_temp,
                     ctx->h_unif};

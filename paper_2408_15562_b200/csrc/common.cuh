@@ -58,6 +58,7 @@ struct fspad_ctx {
 
     void *dx_part;            // draft step: per-piece top-k lists [max_batch * 16 rows][pieces][16] (value, token)
     int *dx_done;             // draft step: finished pieces of each sequence [max_batch]; zero between calls
+    float *dx_front;          // draft step: a frontier put aside, values and candidates [2][max_batch][16]
 
     // device staging for the host entry point (h_ready: every buffer below is allocated)
     int h_ready;

@@ -278,6 +278,25 @@ cudaError_t fspad_launch_draft_expand(fspad_ctx *ctx, const float *logprobs, con
                                       float *next_logp, cudaStream_t st)
 {
     if (B == 0) return cudaSuccess;
+    // A sequence's next frontier is written while other sequences may not have read theirs yet.  Where the caller's next_* lie over
+    // frontier_* in any other way than list over list of the same length, the current ones are first put aside.
+    const size_t in_bytes = (size_t)B * F * sizeof(float), out_bytes = (size_t)B * width * sizeof(float);
+    auto overlap = [&](const void *in, const void *out) {
+        const uintptr_t i = reinterpret_cast<uintptr_t>(in), o = reinterpret_cast<uintptr_t>(out);
+        return i < o + out_bytes && o < i + in_bytes;
+    };
+    const bool same_place = F == width && frontier_cand == next_cand && frontier_logp == next_logp;
+    const bool aside = !same_place && (overlap(frontier_cand, next_cand) || overlap(frontier_cand, next_logp) ||
+                                       overlap(frontier_logp, next_cand) || overlap(frontier_logp, next_logp));
+    if (aside) {
+        float *keep_logp = ctx->dx_front;
+        int *keep_cand = reinterpret_cast<int *>(ctx->dx_front + (size_t)ctx->cfg.max_batch * FSPAD_MAX_FRONTIER);
+        cudaError_t e = cudaMemcpyAsync(keep_logp, frontier_logp, in_bytes, cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(keep_cand, frontier_cand, in_bytes, cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return e;
+        frontier_logp = keep_logp;
+        frontier_cand = keep_cand;
+    }
     static_assert(kMaxPieces * FSPAD_MAX_FRONTIER <= kThreads && FSPAD_MAX_FRONTIER * FSPAD_MAX_FRONTIER <= kThreads,
                   "the merged lists have at most one entry per thread");
     DraftArgs a;
@@ -298,5 +317,5 @@ cudaError_t fspad_launch_draft_expand(fspad_ctx *ctx, const float *logprobs, con
     a.cand_parent = cand_parent; a.cand_token = cand_token; a.cand_logp = cand_logp;
     a.next_cand = next_cand; a.next_logp = next_logp;
     ctx->launches++;
-    return fspad_launch(draft_expand_kernel, dim3(a.pieces, rows), dim3(kThreads), 0, st, 0, a);
+    return fspad_launch_opt(!aside, draft_expand_kernel, dim3(a.pieces, rows), dim3(kThreads), 0, st, 0, a);
 }

@@ -114,3 +114,33 @@ def test_piece_lengths_and_long_lists(vocab, batch, F, k, width, order):
     fc = rng.integers(0, 5, (batch, F)).astype(np.int32)
     for _ in range(2):                                       # the counters are back at zero after a call
         _check(ctx, lp, flp, fc, k, width, 7, 7 + F * k)
+
+
+@pytest.mark.parametrize("batch,F,k,width", [(1, 1, 10, 10), (16, 1, 10, 10), (16, 10, 10, 4), (16, 4, 8, 9), (16, 10, 10, 10), (7, 16, 16, 16)])
+@pytest.mark.parametrize("shift", [0, 4])
+def test_next_frontier_over_the_current_one(batch, F, k, width, shift):
+    """The frontier's buffers used for the next one as well, in place or a few entries further: every sequence still starts from its own
+    current frontier, whichever sequence finishes first."""
+    vocab = 20000
+    ctx = binding.Context(8, 2, vocab, 256, max_nodes=64, max_batch=batch)
+    rng = np.random.default_rng(F * 31 + width)
+    lp = rng.standard_normal((batch, F, vocab), dtype=np.float32)
+    flp = rng.standard_normal((batch, F)).astype(np.float32)
+    fc = rng.integers(0, 50, (batch, F)).astype(np.int32)
+    cap = 60 + F * k
+    ref = [np.full((batch, cap), -7, np.int32), np.full((batch, cap), -7, np.int32), np.full((batch, cap), -3.5, np.float32)]
+    nc_ref, nl_ref = oracle.draft_expand(lp, flp, fc, k, width, 60, *ref)
+    dlp, room = _dev(lp), batch * max(F, width) + shift
+    for _ in range(3):
+        bufs = torch.zeros(room, dtype=torch.int32, device="cuda"), torch.zeros(room, dtype=torch.float32, device="cuda")
+        cand, logp = (t[:batch * F].view(batch, F) for t in bufs)
+        nxt = tuple(t[shift:shift + batch * width].view(batch, width) for t in bufs)
+        cand.copy_(_dev(fc))
+        logp.copy_(_dev(flp))
+        got = [_dev(np.full((batch, cap), -7, np.int32)), _dev(np.full((batch, cap), -7, np.int32)),
+               _dev(np.full((batch, cap), -3.5, np.float32))]
+        ctx.draft_expand(dlp, logp, cand, k, width, 60, *got, *nxt)
+        ctx.check()
+        for g, r in zip(got, ref):
+            assert np.array_equal(g.cpu().numpy(), r)
+        assert np.array_equal(nxt[0].cpu().numpy(), nc_ref) and np.array_equal(nxt[1].cpu().numpy(), nl_ref)
