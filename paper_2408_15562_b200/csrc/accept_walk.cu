@@ -376,12 +376,18 @@ __device__ __noinline__ double parked_sweep(double *__restrict__ se, float *__re
     return a[0] + a[1];
 }
 
-// A probability in double precision by three integer operations (the conversion instruction runs at 16 per clock and SM).
-// Zero and the denormals come out between 2^-127 and 2^-126: next to the other terms of a sum of at least one, nothing.
+// A probability in double precision without the conversion instruction (16 per clock and SM): exact for zero and for every
+// positive normal number, which is what a `plain` tile holds.  The coefficient it is multiplied by has no bound (a rejection
+// adds U / D, and D, the draft mass left, may be a denormal itself), so nothing but the exact value will do.
+__device__ __forceinline__ bool widens(float q)
+{
+    const unsigned u = __float_as_uint(q);
+    return u == 0u || u - 0x00800000u < 0x7f000000u;
+}
 __device__ __forceinline__ double widen(float q)
 {
     const unsigned u = __float_as_uint(q);
-    return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+    return __hiloint2double(u == 0u ? 0 : (int)((u >> 3) + 0x38000000u), (int)(u << 29));
 }
 // The same from registers: a multiply-add, a look at the sign in the high word and an addition per token, no
 // shared-memory traffic and no conversion.
@@ -934,6 +940,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     double last_a = 0.0;                         // this thread's sum of weights in the latest residual sweep
     double er[kTile];                            // this thread's chunk of the node's rows, after the first rejection there
     float qr[kTile];
+    bool plain = true;                           // every q of the tile is zero or a positive normal number
 #pragma unroll
     for (int i = 0; i < kTile; ++i) { er[i] = 0.0; qr[i] = 0.f; }
 
@@ -1046,10 +1053,12 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             double tot[4] = {v[0], v[1], v[2], v[3]};
             auto load_tile = [&]() {                          // (each thread its own values: nothing to wait for)
                 if (in_regs) {
+                    plain = true;
 #pragma unroll
                     for (int i = 0; i < kTile; ++i) {
                         er[i] = i < per_thr ? se[i * kWalkThreads] : 0.0;
                         qr[i] = i < per_thr ? sq[i * kWalkThreads] : 0.f;
+                        plain &= widens(qr[i]);
                     }
                 }
             };
@@ -1095,7 +1104,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
                 // exact softmax denominator of this node; thread 0 then repeats the test with it
                 last_a = sweep_row(MODE_EXP, sh, x, q, se, sq, kWalkThreads, ck, false, arg, 0.0, -1, 0.0, 0.0, nullptr);
                 got = GOT_SUM;
-            } else if (in_regs) {
+            } else if (in_regs && plain) {
                 if (xn >= ck.lo && xn < ck.hi) {
 #pragma unroll
                     for (int i = 0; i < kTile; ++i) {
@@ -1104,7 +1113,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
                     }
                 }
                 last_a = residual_of_tile(er, qr, per_thr, Cn);
-            } else if (cache_ok) {
+            } else if (cache_ok) {                            // (also threads whose tile holds a denormal or a negative zero)
                 last_a = parked_sweep(se, sq, kWalkThreads, ck, per_thr, Cn, xn);
             } else {
                 last_a = sweep_row(MODE_RESID, sh, x, q, se, sq, kWalkThreads, ck, false, arg, Cn, xn, 0.0, 0.0, nullptr);

@@ -198,3 +198,49 @@ def test_device_detected_errors_are_reported_not_fatal():
     # the context still works
     path, n_acc, bonus = _run(inp, ctx)
     assert helpers.compare_accept(inp, path, n_acc, bonus)[0] == 0
+
+
+@pytest.mark.parametrize("vocab", [4096, 128256, 151936])
+@pytest.mark.parametrize("rest", ["zero", "denormal", "minus_zero"])
+@pytest.mark.parametrize("temp", [1.0, 0.1])
+def test_draft_rows_with_tiny_children(vocab, rest, temp):
+    """A peaked draft row whose children run from 1 down to the smallest denormal, the other tokens exactly zero, negative zero or
+    denormal: once the large ones are rejected the draft mass left is tiny and the coefficient of the draft row huge, so that even a
+    draft probability of 1e-39 decides weights.  Rows that fit into a thread's registers (4096, 128256) and that do not (151936)."""
+    B, N = 8, 9
+    rng = np.random.default_rng(vocab)
+    w = synth.scaled(W["llama3_8b_2k"], batch=B, vocab=vocab, n_nodes=N, tree="star", temperatures=(temp,) * B, prefix=(8, 8))
+    inp = synth.generate(w, 0, with_attention=False)
+    assert inp.parent.shape == (B, N)
+    sizes = np.array([1.0, 1e-9, 3e-20, 1e-30, 2e-38, 9e-39, 5e-42, 1.5e-45], np.float32)
+    for b in range(B):
+        tok = rng.permutation(vocab)
+        inp.target_logits[b] = -60.0 * temp
+        heavy = tok[N:N + 40]
+        inp.target_logits[b][:, heavy] = (rng.standard_normal(heavy.size) * temp).astype(np.float32)
+        inp.draft_probs[b] = np.float32(-0.0) if rest == "minus_zero" else np.float32(0.0)
+        if rest == "denormal":
+            inp.draft_probs[b][:, heavy[::2]] = (rng.random(heavy[::2].size) * 1e-39).astype(np.float32)
+        kids = tok[:N - 1]
+        keep = N - 1 - b % 4                                     # how many of the tiny ones are listed; the rest repeat the first
+        kids[keep:] = kids[0]
+        inp.draft_probs[b][:, kids[:keep]] = sizes[:keep]
+        inp.draft_tokens[b, 1:] = kids
+        inp.uniforms[b] = rng.random(N + 1)
+    _assert_parity(inp)
+    r = oracle.tree_accept(inp.target_logits, inp.draft_probs, inp.draft_tokens, inp.parent, inp.temperature, inp.uniforms)
+    assert int((r["n_accepted"] == 1).sum()) >= B - 2               # the children are rejected, the bonus token is drawn from what is left
+
+
+def test_zero_draft_probabilities_keep_their_weight():
+    """Two rejected children of 1 and 2e-38 leave two tokens of weight 1 and 0.497 that the draft gives nothing: neither loses any."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=1, vocab=4096, n_nodes=3, tree="star", temperatures=(1.0,), prefix=(8, 8))
+    inp = synth.generate(w, 0, with_attention=False)
+    inp.target_logits[...] = -60.0
+    inp.target_logits[:, :, 100], inp.target_logits[:, :, 3000] = 0.0, -0.7
+    inp.draft_probs[...] = 0.0
+    inp.draft_probs[:, :, 200], inp.draft_probs[:, :, 300] = 1.0, 2e-38
+    inp.draft_tokens[0] = [0, 200, 300]
+    inp.uniforms[...] = [0.5, 0.5, 0.5, 0.8]
+    path, n_acc, bonus = _run(inp)
+    assert int(n_acc[0]) == 1 and int(bonus[0]) == 3000
