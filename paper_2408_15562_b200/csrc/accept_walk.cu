@@ -58,6 +58,7 @@ constexpr double kAmbiguous = 1e-4;
 constexpr double kScanRel = 1e-6;          // bound taken for the relative error of the scan's sum of exponentials
 constexpr double kFusedTol = 1e-9;         // relative error the fused first-rejection sweep may leave in the residual mass
 constexpr double k16OverLn2 = 23.083120654223414;   // steps of the exponential's table per unit of its argument
+constexpr int kExpRange = 0x40cf8f17;      // high word of 700 * 16 / ln 2
 constexpr float kLog2eF = 1.4426950408889634f;
 constexpr int kPieceSlots = 16;            // pieces of a row whose scan sums are kept for the bonus draw
 constexpr int kExpTable = 16;              // entries of the exponential's table: one per pair of shared-memory banks
@@ -238,22 +239,19 @@ __device__ __forceinline__ void merge_row(const FspadStatsPart *__restrict__ par
 // t = (x - m) 16 / (T ln 2) = 16 n + i + f, |f| <= 1/2, the value is 2^n 2^(i/16) exp(f ln2/16).  The exponential
 // of the remainder is its Taylor series to the fifth order with the sixth economised into the lower ones (error below
 // 5e-15).  Sixteen entries lie in sixteen pairs of banks, so that a warp's look-ups never collide (with 256 entries and a
-// cubic each cost six shared-memory cycles).  The caller hands over s = 16 / (T ln 2) and off = -m s.  The rounding to
+// cubic each cost six shared-memory cycles).  The caller hands over s = 16 / (T ln 2) and m; the difference x - m is taken
+// first (of two floats it is exact or nearly so), because the rounding of a product m s has no bound at low temperatures:
+// at T = 1e-12 and m = 20 it is 2 % of a step, at 1e-16 hundreds of steps.  The rounding to
 // the nearest integer is done by adding and subtracting 1.5 * 2^52 (the integer then sits in the low word of the sum):
 // conversions run at a quarter of the fp64 rate (16 against 63 per clock and SM).  Values below e^-700 are taken as zero.
 struct ExpArg {
-    double s, off;
-    float x_min;
+    double s, m;
 };
-__device__ __forceinline__ ExpArg exp_arg(float m, double invT, float T)
-{
-    const double s = invT * k16OverLn2;
-    return ExpArg{s, -(double)m * s, m - 700.0f * T};
-}
+__device__ __forceinline__ ExpArg exp_arg(float m, double invT) { return ExpArg{invT * k16OverLn2, (double)m}; }
 __device__ __forceinline__ double exp_neg(float x, const ExpArg &g, const double *tbl)
 {
     const double magic = 6755399441055744.0;              // 1.5 * 2^52
-    const double t = fma((double)x, g.s, g.off);
+    const double t = ((double)x - g.m) * g.s;
     const double tm = t + magic;
     const double f = t - (tm - magic);
     const int k = __double2loint(tm);
@@ -264,7 +262,8 @@ __device__ __forceinline__ double exp_neg(float x, const ExpArg &g, const double
     p = fma(p, f, 1.0000000000000044);
     const double y = tbl[k & (kExpTable - 1)] * p;
     const double e = __hiloint2double(__double2hiint(y) + ((k >> 4) << 20), __double2loint(y));
-    return x > g.x_min ? e : 0.0;                          // also -inf and NaN
+    // |t| < 16158.2 = 700 * 16 / ln 2, told by the high word alone (to one part in a million): false for -inf and NaN, too
+    return (__double2hiint(t) & 0x7fffffff) < kExpRange ? e : 0.0;
 }
 
 // w where it is not negative, else zero, without a branch (tokens of a warp are of both kinds)
@@ -830,7 +829,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         if (tid >= 1) {
             sh.cq[tid] = qv;
             sh.cu[tid] = uval;
-            sh.cex[tid] = exp_neg(xv, exp_arg(sh.rowM[p], invT, Tf), sh.exp_tbl);
+            sh.cex[tid] = exp_neg(xv, exp_arg(sh.rowM[p], invT), sh.exp_tbl);
         } else {
             sh.ubonus = uval;
         }
@@ -1042,7 +1041,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         const int cur = sh.cur, xn = sh.xnew;
         const float *x = lg + (size_t)cur * V, *q = dp + (size_t)cur * V;
         const Chunk ck = chunk_of((row0 + cur) * V, V, per_cta, per_thr, rank, tid);
-        const ExpArg arg = exp_arg(sh.rowM[cur], invT, Tf);
+        const ExpArg arg = exp_arg(sh.rowM[cur], invT);
         got = GOT_RESIDUAL;
         bool again = req != REQ_FUSED;
         if (req == REQ_FUSED) {
@@ -1227,7 +1226,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     if (!settled) {
         // ---- exact draw over the whole row: every CTA a contiguous slice, every thread a contiguous chunk ----
         const Chunk ck = chunk_of((row0 + cur) * V, V, per_cta, per_thr, rank, tid);
-        const ExpArg arg = exp_arg(sh.rowM[cur], invT, Tf);
+        const ExpArg arg = exp_arg(sh.rowM[cur], invT);
         const bool parked = sh.parked != 0;
         // with nothing rejected at this node (c == 0) the weights are the e_j themselves and the
         // denominator cancels, so no separate exact-sum sweep is needed

@@ -244,3 +244,25 @@ def test_zero_draft_probabilities_keep_their_weight():
     inp.uniforms[...] = [0.5, 0.5, 0.5, 0.8]
     path, n_acc, bonus = _run(inp)
     assert int(n_acc[0]) == 1 and int(bonus[0]) == 3000
+
+
+@pytest.mark.parametrize("temp", [1e-3, 1e-8, 1e-10, 1e-12, 1e-14, 1e-16, 1e-20, 1e-30])
+def test_temperatures_close_to_zero(temp):
+    """Three tokens share the maximum, so p = 1/3 each however low the temperature; every first child is tested at r q = p (1 +- 3e-4),
+    outside the margin inside which the scan's sum is replaced by an exact one."""
+    B, N, V = 8, 7, 3000
+    rng = np.random.default_rng(3)
+    w = synth.scaled(W["llama3_8b_2k"], batch=B, vocab=V, n_nodes=N, tree="star", temperatures=(temp,) * B, prefix=(8, 8))
+    inp = synth.generate(w, 0, with_attention=False)
+    for b in range(B):
+        top = np.float32(20.3 if b % 2 else 7.77)
+        inp.target_logits[b] = top - np.float32(1.0) - rng.random((N, V)).astype(np.float32)
+        tok = rng.permutation(V)[:N]
+        inp.target_logits[b][:, tok[:3]] = top
+        inp.draft_probs[b] = np.float32(0.1 / V)
+        inp.draft_probs[b][:, tok[:N - 1]] = np.array([0.4, 0.5, 0.45, 0.02, 0.02, 0.01], np.float32)
+        inp.draft_tokens[b, 1:] = tok[:N - 1]
+        side = 3e-4 if b % 4 < 2 else -3e-4
+        inp.uniforms[b] = rng.random(N + 1)
+        inp.uniforms[b, 1] = (1.0 / 3.0) * (1.0 + side) / 0.4
+    _assert_parity(inp)
