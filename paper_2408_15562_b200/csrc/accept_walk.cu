@@ -53,7 +53,7 @@ constexpr int kWalkThreads = 512;          // 128 registers each: a thread keeps
 constexpr int kWarps = kWalkThreads / 32;
 constexpr int kTile = 16;                  // tokens of a thread's chunk that later residual sweeps take from registers
 constexpr int kSmemBudget = 200 * 1024;   // dynamic shared memory for the per-node cache
-constexpr int kSmemBudgetWide = 176 * 1024;   // the same for the instance with room for 256 nodes (its static part is larger)
+constexpr int kSmemBudgetWide = 168 * 1024;   // the same for the instance with room for 256 nodes (its other parts are larger)
 constexpr double kAmbiguous = 1e-4;
 constexpr double kScanRel = 1e-6;          // bound taken for the relative error of the scan's sum of exponentials
 constexpr double kFusedTol = 1e-9;         // relative error the fused first-rejection sweep may leave in the residual mass
@@ -61,6 +61,7 @@ constexpr double k16OverLn2 = 23.083120654223414;   // steps of the exponential'
 constexpr int kExpRange = 0x40cf8f17;      // high word of 700 * 16 / ln 2
 constexpr float kLog2eF = 1.4426950408889634f;
 constexpr int kPieceSlots = 16;            // pieces of a row whose scan sums are kept for the bonus draw
+constexpr int kPieceBytes = kPieceSlots * sizeof(double);      // of one row; ahead of the per-node cache in dynamic shared memory
 constexpr int kExpTable = 16;              // entries of the exponential's table: one per pair of shared-memory banks
 enum { REQ_DONE = 0, REQ_EXP = 1, REQ_FUSED = 2, REQ_RESID = 3 };
 
@@ -141,9 +142,8 @@ template <int MAXN> struct SharedT {
     double slot[2][4][kMaxCluster];
     unsigned long long bar[2];
     int verdict;                    // bonus draw from one piece of the row: 1 = settled, 2 = the whole row must be swept
-    // approximate mass of every (row, CTA) piece of the vocabulary scan, relative to the row maximum;
-    // piece_cnt[row] = 0 when the row has more than kPieceSlots pieces (the draw then sweeps the whole row)
-    float piece_w[MAXN][kPieceSlots];
+    // piece_cnt[row]: pieces of the row whose masses are kept (in dynamic shared memory); 0 when it has more than kPieceSlots
+    // (the draw then sweeps the whole row)
     int piece_cnt[MAXN];
 };
 
@@ -187,7 +187,7 @@ __device__ __noinline__ void piece_bounds(const FspadStatsGeom &g, int row, int 
 // The whole warp calls it; `valid` is false for lanes without a row.  piece_w (may be NULL): mass of each piece relative
 // to the row's maximum.
 __device__ __forceinline__ void merge_row(const FspadStatsPart *__restrict__ parts, const FspadStatsGeom &g, int row, bool valid,
-                                          float k, int l8, float &M, double &S, int &A, float *piece_w, int *piece_cnt)
+                                          float k, int l8, float &M, double &S, int &A, double *piece_w, int *piece_cnt)
 {
     const int cnt = valid ? row_pieces(g, row) : 0;
     const FspadStatsPart *p = parts + (size_t)(valid ? row : 0) * g.slots;
@@ -215,18 +215,18 @@ __device__ __forceinline__ void merge_row(const FspadStatsPart *__restrict__ par
         const int oa = __shfl_xor_sync(0xffffffffu, a, off);
         if (om > m || (om == m && oa < a)) { m = om; a = oa; }
     }
-    const float w0 = (m0 != -INFINITY) ? s0 * exp2f((m0 - m) * k) : 0.f;
-    const float w1 = (m1 != -INFINITY) ? s1 * exp2f((m1 - m) * k) : 0.f;
+    const double w0 = (m0 != -INFINITY) ? (double)s0 * (double)exp2f((m0 - m) * k) : 0.0;
+    const double w1 = (m1 != -INFINITY) ? (double)s1 * (double)exp2f((m1 - m) * k) : 0.0;
     if (piece_w != nullptr && valid) {
         piece_w[l8] = w0;
         piece_w[l8 + 8] = w1;
         if (l8 == 0) *piece_cnt = (cnt <= kPieceSlots) ? cnt : 0;
     }
-    double s = (double)w0 + (double)w1;
+    double s = w0 + w1;
 #pragma unroll 1
     for (int sl = l8 + 16; sl < cnt; sl += 8) {
         const int4 v = __ldcg(reinterpret_cast<const int4 *>(p + sl));
-        if (__int_as_float(v.x) != -INFINITY) s += (double)(__int_as_float(v.y) * exp2f((__int_as_float(v.x) - m) * k));
+        if (__int_as_float(v.x) != -INFINITY) s += (double)__int_as_float(v.y) * (double)exp2f((__int_as_float(v.x) - m) * k);
     }
 #pragma unroll
     for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
@@ -704,6 +704,8 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
 
     __shared__ Shared sh;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
+    // mass of every (row, CTA) piece of the vocabulary scan, relative to the row maximum
+    double (*piece_w)[kPieceSlots] = reinterpret_cast<double (*)[kPieceSlots]>(dyn_smem);
 
     fspad_pdl_trigger();
     int b = blockIdx.x / C;
@@ -820,7 +822,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     for (int r0 = 0; r0 < N; r0 += kWalkThreads / 8) {           // whole warps iterate together
         const int row = r0 + (tid >> 3), rs = row < N ? row : 0;
         float M; double S; int A;
-        merge_row(args.parts, args.geom, b * N + row, row < N, kT, l8, M, S, A, sh.piece_w[rs], &sh.piece_cnt[rs]);
+        merge_row(args.parts, args.geom, b * N + row, row < N, kT, l8, M, S, A, piece_w[rs], &sh.piece_cnt[rs]);
         if (l8 == 0 && row < N) { sh.rowM[row] = M; sh.rowS[row] = S; sh.t.rowA[row] = A; }
     }
     const double invT = 1.0 / (double)(sampling ? Tf : 1.0f);
@@ -849,8 +851,9 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     // ---- sampling ----
     const bool cache_ok = args.cache_ok != 0, in_regs = cache_ok && per_thr <= kTile;
     // parked values: [k][thread] (k-th position of each thread's chunk), conflict-free
-    double *se = reinterpret_cast<double *>(dyn_smem) + tid;
-    float *sq = reinterpret_cast<float *>(dyn_smem + (size_t)per_thr * kWalkThreads * sizeof(double)) + tid;
+    unsigned char *node_cache = dyn_smem + N * kPieceBytes;
+    double *se = reinterpret_cast<double *>(node_cache) + tid;
+    float *sq = reinterpret_cast<float *>(node_cache + (size_t)per_thr * kWalkThreads * sizeof(double)) + tid;
     int n_exch = 0;                              // exchanges so far
     // Sums of NV values (one or four) over the cluster, in every lane of warp 0 (the other warps' values are not defined).
     // Every CTA performs the same operations on the same values.  Four values are summed in groups of eight lanes, one
@@ -1146,7 +1149,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     const int n_piece = sh.piece_cnt[cur];
     if (!sh.bonus_ok && c == 0.0 && sh.nrem == 0 && n_piece > 0) {
         // every warp scans the pieces' masses: prefix of the piece the target falls into
-        double cum = lane < n_piece ? (double)sh.piece_w[cur][lane & (kPieceSlots - 1)] : 0.0;
+        double cum = lane < n_piece ? piece_w[cur][lane & (kPieceSlots - 1)] : 0.0;
         const double own = cum;
 #pragma unroll
         for (int off = 1; off < kPieceSlots; off <<= 1) {
@@ -1325,15 +1328,18 @@ static int walk_cluster_size(fspad_ctx *ctx, int B, int V)
 {
     if (ctx->walk_cluster == 0) {
         ctx->walk_cluster = 8;
-        cudaFuncSetAttribute(accept_walk_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-        cudaFuncSetAttribute(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudgetWide);
+        constexpr int most = kSmemBudget + 64 * kPieceBytes, most_wide = kSmemBudgetWide + FSPAD_MAX_NODES_WIDE * kPieceBytes;
+        static_assert(most + sizeof(SharedT<64>) <= 227 * 1024 && most_wide + sizeof(SharedT<FSPAD_MAX_NODES_WIDE>) <= 227 * 1024,
+                      "shared memory of a CTA");
+        cudaFuncSetAttribute(accept_walk_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        cudaFuncSetAttribute(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most_wide);
         if (cudaFuncSetAttribute(accept_walk_kernel<64>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaFuncSetAttribute(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
                 cudaSuccess) {
             cudaLaunchConfig_t probe = {};
             probe.gridDim = dim3(kMaxCluster);
             probe.blockDim = dim3(kWalkThreads);
-            probe.dynamicSmemBytes = kSmemBudget;
+            probe.dynamicSmemBytes = most;
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
             at[0].val.clusterDim.x = kMaxCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -1341,7 +1347,7 @@ static int walk_cluster_size(fspad_ctx *ctx, int B, int V)
             int n = 0;
             int n2 = 0;
             cudaLaunchConfig_t probe2 = probe;
-            probe2.dynamicSmemBytes = kSmemBudgetWide;
+            probe2.dynamicSmemBytes = most_wide;
             if (cudaOccupancyMaxActiveClusters(&n, accept_walk_kernel<64>, &probe) == cudaSuccess && n >= 1 &&
                 cudaOccupancyMaxActiveClusters(&n2, accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, &probe2) == cudaSuccess && n2 >= 1)
                 ctx->walk_cluster = kMaxCluster;
@@ -1383,8 +1389,8 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     const size_t per_cta = (size_t)((((V + 3 + cluster - 1) / cluster) + 3) & ~3);       // as the kernel shares a row out
     const size_t per_thr = ((per_cta + kWalkThreads - 1) / kWalkThreads + 3) & ~(size_t)3;
     const size_t need = per_thr * kWalkThreads * (sizeof(double) + sizeof(float));
-    size_t smem = 0;
-    if (need <= (size_t)(N <= 64 ? kSmemBudget : kSmemBudgetWide)) { smem = need; a.cache_ok = 1; }
+    size_t smem = (size_t)N * kPieceBytes;
+    if (need <= (size_t)(N <= 64 ? kSmemBudget : kSmemBudgetWide)) { smem += need; a.cache_ok = 1; }
     // trees of up to 64 nodes and of up to FSPAD_MAX_NODES_WIDE nodes are two instances of the kernel
     if (N <= 64)
         return fspad_launch(accept_walk_kernel<64>, dim3((unsigned)(B * cluster)), dim3(kWalkThreads), smem, st, (unsigned)cluster, a);
