@@ -138,8 +138,8 @@ template <int MAXN> struct SharedT {
     int bonus_ok;                   // the last residual sweep already holds the bonus draw's per-thread sums
     int fail;
     // reductions: warp totals, totals received from every CTA of the cluster (by exchange parity), their barriers
-    double warp_v[4][kWarps], warp_off[kWarps], warp_total;
-    double slot[2][4][kMaxCluster];
+    double warp_v[5][kWarps], warp_off[kWarps], warp_total;
+    double slot[2][5][kMaxCluster];
     unsigned long long bar[2];
     int verdict;                    // bonus draw from one piece of the row: 1 = settled, 2 = the whole row must be swept
     // piece_cnt[row]: pieces of the row whose masses are kept (in dynamic shared memory); 0 when it has more than kPieceSlots
@@ -272,8 +272,6 @@ __device__ __forceinline__ double positive(double w)
     const int keep = ~(__double2hiint(w) >> 31);
     return __hiloint2double(__double2hiint(w) & keep, __double2loint(w) & keep);
 }
-
-__device__ __forceinline__ double pair_of(float hi, float lo) { return __hiloint2double(__float_as_int(hi), __float_as_int(lo)); }
 
 // All weights are kept times the softmax denominator S: w = max(e - C q, 0) with e = exp((x - m)/T) and C = c S.
 __device__ __forceinline__ double weight(double e, double q, double C)
@@ -412,8 +410,8 @@ __device__ __forceinline__ double residual_of_tile(const double (&er)[kTile], co
 //   v[0] = sum e_j (= S)                    v[1] = sum_P (e_j - S' q_j), xnew left out
 //   v[2] = sum of q_j over the tokens that no child of the node carries (the draft mass left by any rejections here is
 //          this plus what the siblings still to be tested carry)
-//   v[3] = two floats: sum_P q_j (it is multiplied by S - S', a millionth of S at most), and the sum of e_j over the
-//          tokens whose sign a relative error kScanRel of S' could flip;
+//   v[3] = sum_P q_j                        v[4] = sum of e_j over the tokens whose sign a relative error kScanRel of S'
+//                                                  could flip;
 // a flipped token changes the result by at most kScanRel times its e_j, so kScanRel times that sum bounds the error and the
 // caller sweeps again at the exact S when that is not negligible.
 // e_j and q_j are parked in shared memory, zeros in the empty positions.  The loop is kept short (four tokens, the next
@@ -423,7 +421,7 @@ template <class Shared>
 __device__ __forceinline__ void fused_reject_sweep(const Shared &sh, const float *__restrict__ x, const float *__restrict__ q,
                                                    double *__restrict__ se, float *__restrict__ sq, int stride, Chunk ck,
                                                    int per_thr, bool park, const ExpArg &arg, double S, int xnew, int node,
-                                                   int n_nodes, double (&v)[4])
+                                                   int n_nodes, double (&v)[5])
 {
     // Which of this thread's first 64 positions hold a child's token: the warp's lanes look at the nodes side by side, and
     // only for the few tokens that fall into the warp's stretch is the owner told.
@@ -446,8 +444,7 @@ __device__ __forceinline__ void fused_reject_sweep(const Shared &sh, const float
             }
         }
     }
-    v[0] = v[1] = v[2] = 0.0;
-    float qp = 0.f, flips = 0.f;
+    v[0] = v[1] = v[2] = v[3] = v[4] = 0.0;
     float4 x4 = fspad_load4(x, ck.lo, ck.hi, -INFINITY), q4 = fspad_load4(q, ck.lo, ck.hi, 0.f);
 #pragma unroll 1
     for (int k = 0; k < per_thr; k += 4) {
@@ -482,18 +479,17 @@ __device__ __forceinline__ void fused_reject_sweep(const Shared &sh, const float
                 se[(k + t) * stride] = e;
                 sq[(k + t) * stride] = qv[t];
             }
-            const double w = fma(-S, (double)qv[t], e);
+            const double q64 = (double)qv[t], w = fma(-S, q64, e);
             v[1] += positive(w);
-            qp += __double2hiint(w) >= 0 ? qv[t] : 0.f;
+            v[3] += __double2hiint(w) >= 0 ? q64 : 0.0;
             // |w| <= kScanRel * e needs the binary exponent of w at least 19 below that of e: an
             // integer comparison sorts out all but a handful of tokens
             if ((__double2hiint(w) & 0x7ff00000) <= (__double2hiint(e) & 0x7ff00000) - (19 << 20))
-                if (e > 0.0 && fabs(w) <= kScanRel * e) flips += (float)e;
+                if (e > 0.0 && fabs(w) <= kScanRel * e) v[4] += e;
         }
         x4 = xn;
         q4 = qn;
     }
-    v[3] = pair_of(qp, flips);
 }
 
 // ---- sums over the cluster ----
@@ -855,59 +851,72 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     double *se = reinterpret_cast<double *>(node_cache) + tid;
     float *sq = reinterpret_cast<float *>(node_cache + (size_t)per_thr * kWalkThreads * sizeof(double)) + tid;
     int n_exch = 0;                              // exchanges so far
-    // Sums of NV values (one or four) over the cluster, in every lane of warp 0 (the other warps' values are not defined).
-    // Every CTA performs the same operations on the same values.  Four values are summed in groups of eight lanes, one
-    // value to a group, after two steps in which a lane passes on the values of the other groups; the fourth is a pair of
-    // floats in the words of a double.  A slot is written again two exchanges later, by peers that have by then received
+    // Sums of NV values (one or five) over the cluster, in every lane of warp 0 (the other warps' values are not defined).
+    // Every CTA performs the same operations on the same values.  The first four of five are summed in groups of eight lanes,
+    // one value to a group, after two steps in which a lane passes on the values of the other groups; the fifth by all lanes
+    // beside them.  A slot is written again two exchanges later, by peers that have by then received
     // this CTA's next totals, which it sends only after it has read the slot.
     // Warp 0 runs `meanwhile` while the peers' totals are on their way.
     auto exchange = [&](auto &v, auto meanwhile) {
         constexpr int NV = sizeof(v) / sizeof(double);
-        constexpr int kGroup = 32 / NV;          // lanes that end up with the same value
+        constexpr bool kFive = NV == 5;
+        static_assert(NV == 1 || kFive, "one value or five");
+        constexpr int kGroup = kFive ? 8 : 32;   // lanes that end up with the same value
         const int item = lane / kGroup, sub = lane % kGroup;
         const int par = n_exch & 1;
         const uint32_t phase = (uint32_t)(n_exch >> 1) & 1u;
         ++n_exch;
-        auto add = [&](double x2, double y2, bool pair) {
-            if (NV == 4 && pair)
-                return pair_of(__int_as_float(__double2hiint(x2)) + __int_as_float(__double2hiint(y2)),
-                               __int_as_float(__double2loint(x2)) + __int_as_float(__double2loint(y2)));
-            return x2 + y2;
-        };
-        const bool pair = item == 3;
-        double one = v[0];
-        if (NV == 4) {
+        double one = v[0], fifth = v[NV - 1];
+        if (kFive) {
             const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
             const double a0 = (up ? v[2 % NV] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2 % NV], 16);
-            const double a1 = add(up ? v[3 % NV] : v[1 % NV], __shfl_xor_sync(0xffffffffu, up ? v[1 % NV] : v[3 % NV], 16), up);
-            one = add(odd ? a1 : a0, __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8), pair);
+            const double a1 = (up ? v[3 % NV] : v[1 % NV]) + __shfl_xor_sync(0xffffffffu, up ? v[1 % NV] : v[3 % NV], 16);
+            one = (odd ? a1 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) fifth += __shfl_xor_sync(0xffffffffu, fifth, off);
+            if (lane == 0) sh.warp_v[4][wid] = fifth;
         }
 #pragma unroll
-        for (int off = kGroup / 2; off > 0; off >>= 1) one = add(one, __shfl_xor_sync(0xffffffffu, one, off), pair);
+        for (int off = kGroup / 2; off > 0; off >>= 1) one += __shfl_xor_sync(0xffffffffu, one, off);
         if (sub == 0) sh.warp_v[item][wid] = one;
         __syncthreads();
         if (wid == 0) {
             one = sub < kWarps ? sh.warp_v[item][sub] : 0.0;
-            if (kGroup < kWarps) one = add(one, sh.warp_v[item][(sub + kGroup) % kWarps], pair);
-            static_assert(kGroup >= kWarps / 2, "at most two warp totals per lane");
+            if (kGroup < kWarps) one += sh.warp_v[item][(sub + kGroup) % kWarps];
+            static_assert(kGroup >= kWarps / 2 && kWarps == kMaxCluster, "at most two warp or CTA totals per lane");
 #pragma unroll
-            for (int off = (kGroup < kWarps ? kGroup : kWarps) / 2; off > 0; off >>= 1)
-                one = add(one, __shfl_xor_sync(0xffffffffu, one, off), pair);
-            if (NV == 1) one = __shfl_sync(0xffffffffu, one, 0);
+            for (int off = (kGroup < kWarps ? kGroup : kWarps) / 2; off > 0; off >>= 1) one += __shfl_xor_sync(0xffffffffu, one, off);
+            if (!kFive) one = __shfl_sync(0xffffffffu, one, 0);
             const uint32_t bar = smem_addr(&sh.bar[par]);
             if (lane == 0) expect_bytes(bar, C * NV * 8);
             if (sub < C) send_double(smem_addr(&sh.slot[par][item][rank]), bar, sub, one);
             if (kGroup < kMaxCluster && sub + kGroup < C) send_double(smem_addr(&sh.slot[par][item][rank]), bar, sub + kGroup, one);
+            if (kFive) {
+                fifth = lane < kWarps ? sh.warp_v[4][lane % kWarps] : 0.0;
+#pragma unroll
+                for (int off = kWarps / 2; off > 0; off >>= 1) fifth += __shfl_xor_sync(0xffffffffu, fifth, off);
+                if (lane < C) send_double(smem_addr(&sh.slot[par][4][rank]), bar, lane, fifth);
+            }
             meanwhile();
             if (!wait_cluster(bar, phase)) sh.fail = 1;
             __syncwarp();
             one = sub < C ? sh.slot[par][item][sub] : 0.0;
-            if (kGroup < kMaxCluster && sub + kGroup < C) one = add(one, sh.slot[par][item][(sub + kGroup) % kMaxCluster], pair);
+            if (kGroup < kMaxCluster && sub + kGroup < C) one += sh.slot[par][item][(sub + kGroup) % kMaxCluster];
+            if (kFive) {
+                fifth = lane < C ? sh.slot[par][4][lane % kMaxCluster] : 0.0;
+#pragma unroll
+                for (int off = kMaxCluster / 2; off > 0; off >>= 1) fifth += __shfl_xor_sync(0xffffffffu, fifth, off);
+            }
 #pragma unroll
             for (int off = (kGroup < kMaxCluster ? kGroup : kMaxCluster) / 2; off > 0; off >>= 1)
-                one = add(one, __shfl_xor_sync(0xffffffffu, one, off), pair);
+                one += __shfl_xor_sync(0xffffffffu, one, off);
+            if (kFive) {
 #pragma unroll
-            for (int k = 0; k < NV; ++k) v[k] = __shfl_sync(0xffffffffu, one, k * kGroup);
+                for (int k = 0; k < 4; ++k) v[k % NV] = __shfl_sync(0xffffffffu, one, k * 8);
+                v[NV - 1] = __shfl_sync(0xffffffffu, fifth, 0);
+            } else {
+                v[0] = __shfl_sync(0xffffffffu, one, 0);
+            }
         }
     };
 
@@ -1049,10 +1058,10 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         bool again = req != REQ_FUSED;
         if (req == REQ_FUSED) {
             // first rejection at this node, nothing exact yet (nothing removed, C = S)
-            double v[4];
+            double v[5];
             const double s_scan = sh.S;
             fused_reject_sweep(sh, x, q, se, sq, kWalkThreads, ck, per_thr, cache_ok, arg, s_scan, xn, cur, N, v);
-            double tot[4] = {v[0], v[1], v[2], v[3]};
+            double tot[5] = {v[0], v[1], v[2], v[3], v[4]};
             auto load_tile = [&]() {                          // (each thread its own values: nothing to wait for)
                 if (in_regs) {
                     plain = true;
@@ -1068,8 +1077,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             if (wid > 0) load_tile();
             if (wid == 0) {
                 const double s_exact = tot[0];
-                const float qp = __int_as_float(__double2hiint(tot[3])), flips = __int_as_float(__double2loint(tot[3]));
-                R = tot[1] - (s_exact - s_scan) * (double)qp;
+                R = tot[1] - (s_exact - s_scan) * tot[3];
                 if (R < 0.0) R = 0.0;
                 if (lane == 0) {
                     sh.state.S = sh.state.Cp = s_exact;
@@ -1077,7 +1085,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
                     sh.state.exact = sh.state.parked = 1;
                     const int c = sh.state.ch;
                     const double Wt = R + weight(sh.cex[c], (double)sh.cq[c], s_exact);
-                    sh.sel = !(Wt > 0.0 && kScanRel * (double)flips <= kFusedTol * Wt);
+                    sh.sel = !(Wt > 0.0 && kScanRel * tot[4] <= kFusedTol * Wt);
                     sh.C = s_exact;                           // the coefficient of the repeated sweep
                     sh.S_exact = s_exact;
                 }
@@ -1098,7 +1106,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             again = sh.sel != 0;
             // this thread's share of that sum (nothing rewrites S_exact before the next first rejection; thread 0 may
             // already be changing the rest of the walk's state)
-            if (!again) last_a = v[1] - (sh.S_exact - s_scan) * (double)__int_as_float(__double2hiint(v[3]));
+            if (!again) last_a = v[1] - (sh.S_exact - s_scan) * v[3];
         }
         if (again) {
             const double Cn = sh.C;
