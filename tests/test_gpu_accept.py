@@ -266,3 +266,36 @@ def test_temperatures_close_to_zero(temp):
         inp.uniforms[b] = rng.random(N + 1)
         inp.uniforms[b, 1] = (1.0 / 3.0) * (1.0 + side) / 0.4
     _assert_parity(inp)
+
+
+def _check_stats(rows, vocab, noalloc):
+    """Maximum and index exact, sum 2e-6 relative (fp32 with ex2.approx), every row start alignment among the rows."""
+    x = (np.random.default_rng(vocab).standard_normal((rows, vocab)) * 3).astype(np.float32)
+    temp = torch.full(((rows + 9) // 10,), 0.8, device="cuda")
+    if noalloc:
+        got = (torch.empty(rows, device="cuda"), torch.empty(rows, dtype=torch.float64, device="cuda"),
+               torch.empty(rows, dtype=torch.int32, device="cuda"))
+        assert binding.accept_stats_noalloc(helpers.dev(x), temp, 10, got) == 0
+        torch.cuda.synchronize()
+    else:
+        ctx = binding.Context(8, 2, vocab, 512, max_nodes=min(rows, 256), max_batch=(rows + 255) // 256)
+        got = ctx.accept_stats(helpers.dev(x), temp, 10)
+        ctx.check()
+    om, os_, oa = oracle.row_stats(x, 0.8)
+    assert np.array_equal(got[0].cpu().numpy(), om.astype(np.float32))
+    assert np.array_equal(got[2].cpu().numpy(), oa)
+    np.testing.assert_allclose(got[1].cpu().numpy(), os_, rtol=2e-6)
+
+
+@pytest.mark.parametrize("noalloc", [False, True])
+@pytest.mark.parametrize("rows,vocab", [(64, 46), (64, 47), (60, 166), (26, 79), (120, 22), (1000, 30), (512, 6), (300, 101), (60, 167)])
+def test_stats_pieces_that_begin_past_the_end_of_a_row(rows, vocab, noalloc):
+    """Sizes at which a row's last piece is one unit that only a row starting off a 16-byte boundary reaches into."""
+    _check_stats(rows, vocab, noalloc)
+
+
+@pytest.mark.parametrize("vocab", [22, 46, 47])
+def test_sampling_walk_on_rows_of_many_short_pieces(vocab):
+    for variant in range(4):
+        w = synth.scaled(W["llama3_8b_2k"], batch=8, vocab=vocab, n_nodes=15, depth=4, branch=3, temperatures=(1.0, 0.7) * 4, prefix=(8, 8))
+        _assert_parity(synth.generate(w, variant, with_attention=False), allow_near=1)
