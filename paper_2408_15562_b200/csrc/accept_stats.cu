@@ -122,7 +122,7 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
         int edge = -1;                                        // SHIFT: this thread's unit at an end of the row
         if constexpr (SHIFT) {
             if (tid == 0 && i0 > 0) edge = 0;
-            if (tid == 32 && i1 < n && j0 + 4 * i1 < V) edge = i1;
+            if (tid == 32 && i1 >= i0 && i1 < n && j0 + 4 * i1 < V) edge = i1;   // (i1 < i0: the row is one unit, thread 0's)
             if (edge >= 0) {
                 const U v = fspad_edge4(xrow, j0 + 4 * edge, V, -INFINITY);
                 p.m = Unit<UNIT>::vmax(v);

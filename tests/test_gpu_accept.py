@@ -299,3 +299,10 @@ def test_sampling_walk_on_rows_of_many_short_pieces(vocab):
     for variant in range(4):
         w = synth.scaled(W["llama3_8b_2k"], batch=8, vocab=vocab, n_nodes=15, depth=4, branch=3, temperatures=(1.0, 0.7) * 4, prefix=(8, 8))
         _assert_parity(synth.generate(w, variant, with_attention=False), allow_near=1)
+
+
+@pytest.mark.parametrize("noalloc", [False, True])
+@pytest.mark.parametrize("rows,vocab", [(8, 1), (9, 1), (64, 1), (8, 2), (33, 2), (8, 3), (50, 3), (1000, 1), (1024, 3)])
+def test_stats_rows_shorter_than_one_load(rows, vocab, noalloc):
+    """A row's first and last unit may be the same one: its tokens count once."""
+    _check_stats(rows, vocab, noalloc)
