@@ -69,6 +69,28 @@ def test_attention_headline_and_ragged_batch():
     _check_attn(inp, 4, True, seqs=[0, int(np.argmin(inp.prefix_len)), int(np.argmax(inp.prefix_len))])
 
 
+@pytest.mark.parametrize("aliased", [False, True])
+@pytest.mark.parametrize("n_nodes,group", [(130, 4), (200, 2), (70, 4)])
+def test_attention_wide_trees_in_pairs_of_row_tiles(n_nodes, group, aliased):
+    """Blocks, more than 64 nodes and pairs of CTAs at once: 520, 400 and 280 rows a kv head (5, 4 and 3 row tiles, an empty half with
+    the odd ones), enough of them to fill the SMs; prefixes at the edges of blocks and between."""
+    B = 6
+    L = np.array([0, 127, 128, 640, 700, 1151], np.int32)
+    w = synth.scaled(W["llama3_8b_2k"], batch=B, n_q_heads=8 * group, n_kv_heads=8, n_nodes=n_nodes, depth=8, branch=12,
+                     prefix=(int(L.max()), int(L.max())), temperatures=(0.0,) * B, vocab=16, n_layers=1)
+    inp = synth.generate(w, n_nodes, with_accept=False)
+    assert inp.parent.shape[1] == n_nodes
+    inp.prefix_len[:] = L
+    for arr in (inp.v_cache, inp.tree_v):          # few keys in the first sequence: keep the outputs of order one
+        nz = arr & 0x7FFF != 0
+        arr[nz] -= np.uint16(2 << 7)
+    if aliased:
+        for b in range(B):
+            inp.k_cache[b, :, L[b]:L[b] + n_nodes] = inp.tree_k[b]
+            inp.v_cache[b, :, L[b]:L[b] + n_nodes] = inp.tree_v[b]
+    _check_attn(inp, n_nodes, aliased)
+
+
 def test_compaction_paged():
     rng = np.random.default_rng(9)
     B, N, Hkv, nl, nb = 4, 60, 3, 3, 5
