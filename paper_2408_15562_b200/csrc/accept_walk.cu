@@ -1189,7 +1189,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             auto in4 = [&](int j) {
                 if (j >= p_lo && j + 4 <= t_hi) return __ldg(reinterpret_cast<const float4 *>(x + j));
                 const int sh_lo = max(p_lo - j, 0);
-                float4 r = fspad_edge4(x + j, sh_lo > 0 ? -8 : 0, 0, -INFINITY);
+                float4 r = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
                 if (sh_lo <= 0 && j < t_hi) r.x = x[j];
                 if (sh_lo <= 1 && j + 1 < t_hi) r.y = x[j + 1];
                 if (sh_lo <= 2 && j + 2 < t_hi) r.z = x[j + 2];
