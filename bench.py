@@ -523,7 +523,7 @@ def main():
                                   "gbs": dlp_host.nbytes / (draft_expand_us * 1e-6) / 1e9,
                                   "frac_of_hbm_peak": dlp_host.nbytes / (draft_expand_us * 1e-6) / 1e9 / peak,
                                   "bit_exact_vs_oracle": draft_expand_ok, "oracle_us_one_thread": draft_expand_cpu_us,
-                                  "note": "one level of the draft phase (three kernels); not part of value"},
+                                  "note": "one level of the draft phase (one kernel); not part of value"},
             "lm_head_call": None if lm is None else dict(lm, **{
                 "rows": B * N, "hidden": lm_H, "vocab": w.vocab, "weight_bytes": 2.0 * lm_H * w.vocab,
                 "slabs_of_1024_rows": (B * N + 1023) // 1024,

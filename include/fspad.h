@@ -225,8 +225,8 @@ int fspad_accept_stats_noalloc(const float *logits, const float *temperature, in
  *   hidden_dim a multiple of 8;  rows <= max_batch * max_nodes of the context
  *   temperature [rows / rows_per_seq] fp32 or NULL (0 -> 1), as in fspad_accept_stats
  *   logits_out [rows][vocab] fp32 or NULL;  row_max fp32, row_sum fp64, row_arg int32: [rows]
- * All pointers are device pointers, 16-byte aligned.  Rows are processed in slabs of 128; every slab
- * streams the vocabulary matrix once.  Accuracy: the products are exact, the fp32 accumulation over
+ * All pointers are device pointers, 16-byte aligned.  Rows are processed in slabs of 1024 (one launch each); every slab
+ * streams the vocabulary matrix from HBM once.  Accuracy: the products are exact, the fp32 accumulation over
  * hidden_dim terms leaves an absolute error of about 1e-5 (bounded by hidden_dim / 16 roundings of the
  * running sum) in every logit, so row_arg is the exact argmax wherever the maximum leads the runner-up
  * by more than that.
@@ -307,7 +307,7 @@ int fspad_feature_sampler(fspad_ctx *ctx, const fspad_bf16 *f, const fspad_bf16 
  * lists live in the context's scratch (allocated by fspad_create): one call per
  * context at a time.  Asynchronous on `stream`.  Errors: FSPAD_ERR_SHAPE for
  * sizes outside the ranges above, FSPAD_ERR_TOO_LARGE when ceil(vocab / 4096) *
- * top_k exceeds 1024.
+ * top_k exceeds 1024 (a limit of the call; the kernel itself needs none).
  */
 int fspad_draft_expand(fspad_ctx *ctx, const float *logprobs, const float *frontier_logp,
                        const int32_t *frontier_cand, int n_frontier, int top_k, int width, int base, int n_cand_cap,
@@ -424,10 +424,10 @@ int fspad_kv_compact_paged(fspad_ctx *ctx, fspad_bf16 *pool, const int32_t *bloc
  * acceptance directly when tree_k / tree_v are given (attention then never
  * reads the cache rows compaction rewrites); when they are NULL (tree rows
  * taken from cache rows L_b ..) compaction waits for the attention as well.
- * In the first case, when draft_probs is given and a sequence has at most 64
- * (layer, K/V, kv head) slices, the kernel that walks the tree makes the
- * compaction's moves itself (same result; an invalid prefix length is then
- * reported by that kernel).
+ * In the first case, when a sequence has at most 64 (layer, K/V, kv head)
+ * slices, the kernel that walks the tree makes the compaction's moves itself,
+ * greedy or sampling (same result; an invalid prefix length is then reported by
+ * that kernel).
  * Work queued on `stream` after the call sees every output.  The call only
  * enqueues work and records / waits on events, so it may be captured into a
  * CUDA graph.  One call per context at a time.
@@ -449,12 +449,15 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
  * must not be made inside a stream capture), writes the tree rows into cache
  * rows L_b.. of layer 0, does what fspad_verify_step does (attention over layer
  * 0; it runs while the logits are on their way) on `stream` and the context's
- * second stream, copies the results back and synchronises the stream.  The KV cache
+ * second stream, copies the results back and synchronises the stream.  The outputs
+ * are those of fspad_verify_step on the same inputs, bit for bit.  The KV cache
  * is device-resident state that persists between steps (the caller's device
  * pointer `cache`, layout as in fspad_kv_compact); everything else is host
- * memory (pinned memory makes the copies asynchronous; pinned draft_probs that
- * start on a 16-byte boundary are not copied at all: the kernel reads the rows
- * it needs where they are, before the call returns).  Host outputs:
+ * memory (pinned memory makes the copies asynchronous; draft_probs that lie in
+ * one pinned allocation or registration as a whole and start on a 16-byte
+ * boundary are not copied at all: the kernel reads the rows it needs where they
+ * are, before the call returns).  An error, too, is returned only when nothing
+ * queued by the call uses host memory any more.  Host outputs:
  * attn_out [batch][n_nodes][Hq][d] bf16, accepted_path [batch][max_nodes],
  * n_accepted, bonus_token, new_len [batch].  draft_probs/uniforms may be NULL
  * when every temperature is 0.  Returns the first host- or device-detected error.

@@ -217,12 +217,17 @@ __device__ __forceinline__ void fspad_stats_merge_warp(const FspadStatsPart *__r
 #endif
 
 // ---- programmatic dependent launch -----------------------------------------------------
-// Every kernel of the library is launched with the programmatic-serialization attribute and
-// follows one rule: it lets its successor start launching at once (fspad_pdl_trigger) and it
+// Most kernels of the library are launched with the programmatic-serialization attribute and
+// follow one rule: a kernel lets its successor start launching at once (fspad_pdl_trigger) and
 // touches global memory only after the whole preceding kernel of the stream has completed and
 // flushed (fspad_pdl_wait).  Launch latency and the memory-free part of a prologue (barrier
 // set-up, tensor-memory allocation, table fills) then overlap the tail of the previous kernel,
 // while results stay exactly those of plain stream order.
+// The acceptance walk is the exception: it reads the caller's arrays (trees, logits, draft rows) before its wait.  It may,
+// because the two kernels that can precede it, the vocabulary scan and the LM head's merge, let it start only after their own
+// wait, when everything queued before them is complete, and themselves write nothing but scan partials, which the walk reads
+// after its wait.  Kernels whose predecessor is not one kernel of the same stream (behind a fork, a join or a copy) may be
+// launched without the attribute.
 #ifdef __CUDACC__
 __device__ __forceinline__ void fspad_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void fspad_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

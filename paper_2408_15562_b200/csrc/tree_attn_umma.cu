@@ -3,20 +3,23 @@
 // the attention mask built from the tree).
 //
 // Split-KV flash-decode with tcgen05: all query rows that share a kv head (tree
-// node x GQA group member) form the M = 128 operand of one CTA; keys are
-// consumed in chunks of 128.  Per chunk: S = Q K^T is one chain of eight
-// tcgen05.mma (128 x 128 x 16, bf16 -> fp32) into tensor memory; a softmax
-// thread per query row reads its scores back with tcgen05.ld, applies the
-// ancestor mask (only on chunks that reach past the cached prefix) and the
-// softmax in registers, and writes P as packed bf16 pairs back into tensor
-// memory, over the scores; O += P V is a second chain of eight tcgen05.mma whose
-// A operand is read from tensor memory and whose B operand is V in its
-// [key][d] layout (MN-major).  O stays in tensor memory across chunks.  The
-// work is split over three kinds of warps that meet only on mbarriers (see the
-// kernel's comment); K/V chunks go through a three-deep ring of 128-byte-swizzled
-// tiles, filled by TMA for chunks inside the cached prefix and by 16-byte
-// asynchronous copies for Q and the one chunk that mixes prefix, tree rows and
-// zero padding.  Per-split partials are merged by the combine kernel.
+// node x GQA group member) are cut into row tiles of 128, one CTA each; where the
+// row tiles alone fill the SMs, two neighbouring ones go to a pair of CTAs as one
+// tile of 256 rows (cta_group::2).  Keys are consumed in chunks of 128.  Per chunk:
+// S = Q K^T is one chain of eight tcgen05.mma (128 or 256 x 128 x 16, bf16 -> fp32)
+// into tensor memory; two softmax threads per query row, 64 keys each, read its
+// scores back with tcgen05.ld, apply the ancestor mask (only on chunks that reach
+// past the cached prefix) and the softmax in registers, and write P as packed bf16
+// pairs back into tensor memory, over the scores; O += P V is a second chain of
+// eight tcgen05.mma whose A operand is read from tensor memory and whose B operand
+// is V in its [key][d] layout (MN-major).  O stays in tensor memory across chunks.
+// The work is split over three kinds of warps that meet only on mbarriers (see the
+// kernel's comment); K/V chunks go through a ring of 128-byte-swizzled tiles (three
+// whole chunks in a lone CTA, half of each of five in a pair's), filled by TMA for
+// chunks inside the cached prefix and by 16-byte asynchronous copies for Q and the
+// one chunk that mixes prefix, tree rows and zero padding.  Where a row's keys are
+// split over several CTAs the partials are merged by the combine kernel; with one
+// range per row the kernel writes the result itself.
 //
 // Every wait on an mbarrier is bounded; on expiry the CTA records
 // FSPAD_ERR_TIMEOUT, skips the remaining tensor-core work, frees its tensor
@@ -68,8 +71,8 @@ __device__ __forceinline__ uint32_t tile_off(int r, int c)
 // owns keys 64 g .. 64 g + 63 of every chunk: its half of each score buffer, its own running
 // reference maximum, sum and O accumulator, merged with the other group's by log-sum-exp when the
 // loop ends.  Warp 8 is the copy warp: it issues every TMA copy of the loop and gathers
-// the one chunk TMA cannot describe.  Warp 9 is the tensor-core warp: one of its threads issues
-// every tcgen05.mma; the warp owns the tensor memory.
+// the one chunk TMA cannot describe.  Warp 9 is the tensor-core warp: all its lanes run the issue loop and
+// one elected lane issues every tcgen05.mma (in a pair, rank 0's for both); the warp owns the tensor memory.
 // Tensor memory: columns [128 p, 128 p + 128) hold the fp32 scores S of the chunks of parity p, the
 // 64 columns at 128 p + 64 g being group g's, and then, written over the first 32 of those, P_g as
 // packed bf16 pairs, which the second product reads directly as its A operand; columns

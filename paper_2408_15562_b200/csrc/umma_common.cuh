@@ -76,8 +76,8 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, ui
 
 // Warp number as a value the compiler knows to be the same in every lane.  A loop that issues tensor-core instructions
 // is run by a whole warp under this number, with the instructions themselves predicated on elect_one(): descriptors
-// and addresses then live in uniform registers, which is where the instructions take them from.  In a branch of one lane
-// each operand is moved there first (60 against 20 cycles an instruction, 140 against 100 a commit).
+// and addresses are then warp-uniform values.  In a branch of one lane they are not, and an instruction took 60 cycles
+// against 20, a commit 140 against 100.
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 __device__ __forceinline__ bool elect_one()
 {

@@ -71,7 +71,7 @@ def test_tree_rows_taken_from_cache_when_no_tree_arrays():
 @pytest.mark.parametrize("prefix", [0, 100, 128, 200, 256, 300, 511, 640, 1000])
 def test_every_chunk_count_per_cta(prefix):
     """80 kv heads fill the GPU with one key range per head, so a CTA walks all of the sequence's
-    1 .. 9 chunks itself: every wrap state of the three-deep K/V ring and of the parity-doubled
+    1 .. 9 chunks itself: every wrap state of a lone CTA's three-deep K/V ring and of the parity-doubled
     score barriers, with the gathered boundary chunk first, in the middle of the ring, or last."""
     w = synth.scaled(W["llama3_8b_2k"], n_q_heads=80, n_kv_heads=80, prefix=(prefix, prefix), n_nodes=9,
                      depth=3, branch=3, vocab=16)

@@ -45,7 +45,7 @@ def test_paper_sized_candidate_lists(step, n_nodes):
 
 @pytest.mark.parametrize("levels,width,branch", [(1, 1, 1), (2, 1, 3), (3, 3, 5), (6, 12, 14), (9, 14, 9)])
 def test_sizes_across_sorting_network_widths(levels, width, branch):
-    """Candidate counts 1, 6, 35, 854, 972: sorting networks of 2, 8, 64 and 1024 entries, ragged."""
+    """Candidate counts 1, 6, 35, 854, 972: one warp with idle lanes to a full CTA, ragged."""
     ctx = _ctx()
     cp, ct, lp, rt = synth.tree_candidates(7, 3, levels=levels, width=width, branch=branch, vocab=128256, step=0.25)
     assert cp.shape[1] <= 1024
