@@ -108,7 +108,7 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
         const int j0 = SHIFT ? 4 * off - (int)(((size_t)row * V) & 3) : 0;
         // units [i0, i1) lie inside the row; a first and a last one that do not are thread 0's and thread 32's to begin with.
         // (A row has room for one unit more than its tokens may fill, so a piece can begin past the row's end: it is empty.)
-        const int i0 = SHIFT && j0 < 0 ? 1 : 0, i1 = SHIFT ? min(n, max(0, V - j0) >> 2) : n;
+        const int i0 = SHIFT && j0 < 0 ? 1 : 0, i1 = SHIFT ? min(n, (V - j0) >> 2) : n;
         auto fetch = [&](int i) -> U {
             if constexpr (SHIFT) return __ldg(reinterpret_cast<const U *>(xrow + j0) + i);
             else return __ldg(px + i);
@@ -122,7 +122,7 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
         int edge = -1;                                        // SHIFT: this thread's unit at an end of the row
         if constexpr (SHIFT) {
             if (tid == 0 && i0 > 0) edge = 0;
-            if (tid == 32 && i1 >= i0 && i1 < n && j0 + 4 * i1 < V) edge = i1;   // (i1 < i0: the row is one unit, thread 0's)
+            if (tid == 32 && i1 >= i0 && i1 < n) edge = i1;   // (i1 < i0: the row is one unit, thread 0's, or the piece is empty)
             if (edge >= 0) {
                 const U v = fspad_edge4(xrow, j0 + 4 * edge, V, -INFINITY);
                 p.m = Unit<UNIT>::vmax(v);
