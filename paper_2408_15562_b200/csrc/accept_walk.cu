@@ -373,21 +373,13 @@ __device__ __noinline__ double parked_sweep(double *__restrict__ se, float *__re
     return a[0] + a[1];
 }
 
-// A probability in double precision without the conversion instruction (16 per clock and SM): exact for zero and for every
-// positive normal number, which is what a `plain` tile holds.  The coefficient it is multiplied by has no bound (a rejection
-// adds U / D, and D, the draft mass left, may be a denormal itself), so nothing but the exact value will do.
-__device__ __forceinline__ bool widens(float q)
-{
-    const unsigned u = __float_as_uint(q);
-    return u == 0u || u - 0x00800000u < 0x7f000000u;
-}
-__device__ __forceinline__ double widen(float q)
-{
-    const unsigned u = __float_as_uint(q);
-    return __hiloint2double(u == 0u ? 0 : (int)((u >> 3) + 0x38000000u), (int)(u << 29));
-}
-// The same from registers: a multiply-add, a look at the sign in the high word and an addition per token, no
-// shared-memory traffic and no conversion.
+// The same from registers: a conversion, a multiply-add, a look at the sign in the high word and an addition per token, no
+// shared-memory traffic.  q is converted by the instruction, which is exact for zeros, denormals and a negative zero alike: the
+// coefficient it is multiplied by has no bound (a rejection adds U / D, and D, the draft mass left, may be a denormal itself),
+// so no draft probability is too small to matter.  At 16 per clock and SM the conversions take 512 cycles of a sweep of 16
+// tokens a thread, most of them beside the sums; widening zeros and normal numbers by integer operations, with another way
+// for threads that hold anything else, took longer (60-node step at 2 K keys: 42.2 against 40.2 us with many rejections,
+// 34.7 against 34.3 with few; 39.9 and 33.6 with integer operations that are exact for normal numbers only).
 __device__ __forceinline__ double residual_of_tile(const double (&er)[kTile], const float (&qr)[kTile], int per_thr, double C)
 {
     double a[4] = {0.0, 0.0, 0.0, 0.0};
@@ -396,7 +388,7 @@ __device__ __forceinline__ double residual_of_tile(const double (&er)[kTile], co
         if (b < per_thr) {
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                a[t] += positive(fma(-C, widen(qr[b + t]), er[b + t]));
+                a[t] += positive(fma(-C, (double)qr[b + t], er[b + t]));
             }
         }
     }
@@ -951,7 +943,6 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     double last_a = 0.0;                         // this thread's sum of weights in the latest residual sweep
     double er[kTile];                            // this thread's chunk of the node's rows, after the first rejection there
     float qr[kTile];
-    bool plain = true;                           // every q of the tile is zero or a positive normal number
 #pragma unroll
     for (int i = 0; i < kTile; ++i) { er[i] = 0.0; qr[i] = 0.f; }
 
@@ -1064,12 +1055,10 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             double tot[5] = {v[0], v[1], v[2], v[3], v[4]};
             auto load_tile = [&]() {                          // (each thread its own values: nothing to wait for)
                 if (in_regs) {
-                    plain = true;
 #pragma unroll
                     for (int i = 0; i < kTile; ++i) {
                         er[i] = i < per_thr ? se[i * kWalkThreads] : 0.0;
                         qr[i] = i < per_thr ? sq[i * kWalkThreads] : 0.f;
-                        plain &= widens(qr[i]);
                     }
                 }
             };
@@ -1114,7 +1103,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
                 // exact softmax denominator of this node; thread 0 then repeats the test with it
                 last_a = sweep_row(MODE_EXP, sh, x, q, se, sq, kWalkThreads, ck, false, arg, 0.0, -1, 0.0, 0.0, nullptr);
                 got = GOT_SUM;
-            } else if (in_regs && plain) {
+            } else if (in_regs) {
                 if (xn >= ck.lo && xn < ck.hi) {
 #pragma unroll
                     for (int i = 0; i < kTile; ++i) {
@@ -1123,7 +1112,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
                     }
                 }
                 last_a = residual_of_tile(er, qr, per_thr, Cn);
-            } else if (cache_ok) {                            // (also threads whose tile holds a denormal or a negative zero)
+            } else if (cache_ok) {
                 last_a = parked_sweep(se, sq, kWalkThreads, ck, per_thr, Cn, xn);
             } else {
                 last_a = sweep_row(MODE_RESID, sh, x, q, se, sq, kWalkThreads, ck, false, arg, Cn, xn, 0.0, 0.0, nullptr);
