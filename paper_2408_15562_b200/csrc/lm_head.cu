@@ -188,10 +188,10 @@ lm_head_stats_kernel(const Args a, const __grid_constant__ CUtensorMap tmW, cons
                 const uint32_t idesc = make_idesc_m256((uint32_t)units * 32u);
                 const int buf = j & 1;
                 // the accumulator is free once both CTAs' epilogues have read the item that used it two items ago
-                if (j >= 2 && !failed && !mbar_wait_warp(acce(buf), (uint32_t)((j - 2) >> 1) & 1u)) failed = true;
+                if (j >= 2 && !failed && !mbar_wait(acce(buf), (uint32_t)((j - 2) >> 1) & 1u)) failed = true;
                 tc_fence_after();
                 for (int k = 0; k < n_k; ++k) {
-                    if (!failed && !mbar_wait_warp(full(s), ph)) failed = true;
+                    if (!failed && !mbar_wait(full(s), ph)) failed = true;
                     if (!failed) {
                         tc_fence_after();
                         const uint32_t so = w_lo + (((uint32_t)s * stage) >> 4);

@@ -15,11 +15,20 @@
 // is V in its [key][d] layout (MN-major).  O stays in tensor memory across chunks.
 // The work is split over three kinds of warps that meet only on mbarriers (see the
 // kernel's comment); K/V chunks go through a ring of 128-byte-swizzled tiles (three
-// whole chunks in a lone CTA, half of each of five in a pair's), filled by TMA for
-// chunks inside the cached prefix and by 16-byte asynchronous copies for Q and the
-// one chunk that mixes prefix, tree rows and zero padding.  Where a row's keys are
+// whole chunks in a lone CTA, half of each of five in a pair's) from the last chunk
+// down, filled by TMA, as Q is; only the chunks with rows of an explicit tree array or
+// zero padding, which come first, are gathered with 16-byte asynchronous copies, and
+// Q where a group of query heads does not divide the tile.  Where a row's keys are
 // split over several CTAs the partials are merged by the combine kernel; with one
 // range per row the kernel writes the result itself.
+//
+// What bounds it.  A chunk takes a CTA 2000 cycles: the softmax threads' own chain (wait,
+// scores from tensor memory, maximum, 64 exponentials, P back, arrival: 1500 to 1600 busy, of which
+// 1024 are the special-function units' when both groups are at it), beside 1050 of the tensor cores.  Around the
+// loop stand, in cycles, 5000 to the first scores and 5000 from the last product to the end (9600 and
+// 10000 before the tail's gather, the wide prologue's barriers and the row-by-row stores went).  One B200, us a call:
+// 52 heads and 4 K keys 34.8 -> 29.5, 8 heads of 8 and 8 K 33.3 -> 28.4, 16 ragged sequences 84.8 -> 66.6, four paged
+// sequences of 130 nodes 56.9 -> 40.2.
 //
 // Every wait on an mbarrier is bounded; on expiry the CTA records
 // FSPAD_ERR_TIMEOUT, skips the remaining tensor-core work, frees its tensor
@@ -41,12 +50,12 @@ constexpr int TILE = 2 * HALF;         // bytes of one [128][128] bf16 tile
 __host__ __device__ constexpr int ring_slots(bool pair) { return pair ? 5 : 3; }
 constexpr int smem_bytes(bool pair) { return TILE + 2 * ring_slots(pair) * (pair ? HALF : TILE) + 1024; }   // Q, K ring, V ring + alignment slack
 constexpr uint32_t TMEM_COLS = 512;    // S/P of group 0, of group 1: columns 0..255; O of group 0, of group 1: 256..511
-constexpr int kMaxBlocksPerCta = 128;  // paged cache: chunks (= blocks) one CTA may be given
 constexpr float kLazyLog2 = 8.f;        // a row's reference maximum may lag its true maximum by this much (log2)
 struct Args {
     const fspad_bf16 *q, *kc, *vc, *tk, *tv;
     const int *parent, *prefix_len;
-    int N, Hq, Hkv, G, M, max_len, n_splits, mtiles, use_tma;
+    int N, Hq, Hkv, G, M, max_len, n_splits, mtiles, use_tma, q_tma;
+    int early;                          // launched beside its predecessors in the stream: they have read everything this kernel needs to be complete
     int longest_first;                  // the launch needs several waves of CTAs: blockIdx.z counts the sequences from the longest down
     // paged cache: the planes are pools of 128-row blocks [n_blocks][Hkv][128][d] and block_table[b][i] names
     // the block that holds rows 128 i .. 128 i + 127 of sequence b (NULL: contiguous planes)
@@ -70,8 +79,7 @@ __device__ __forceinline__ uint32_t tile_off(int r, int c)
 // thread, a warp reaching the tensor-memory lane quarter given by its index modulo 4).  Group g
 // owns keys 64 g .. 64 g + 63 of every chunk: its half of each score buffer, its own running
 // reference maximum, sum and O accumulator, merged with the other group's by log-sum-exp when the
-// loop ends.  Warp 8 is the copy warp: it issues every TMA copy of the loop and gathers
-// the one chunk TMA cannot describe.  Warp 9 is the tensor-core warp: all its lanes run the issue loop and
+// loop ends; ahead of the loop they gather what TMA cannot describe.  Warp 8 is the copy warp: it issues every TMA copy.  Warp 9 is the tensor-core warp: all its lanes run the issue loop and
 // one elected lane issues every tcgen05.mma (in a pair, rank 0's for both); the warp owns the tensor memory.
 // Tensor memory: columns [128 p, 128 p + 128) hold the fp32 scores S of the chunks of parity p, the
 // 64 columns at 128 p + 64 g being group g's, and then, written over the first 32 of those, P_g as
@@ -84,8 +92,7 @@ __device__ __forceinline__ uint32_t tile_off(int r, int c)
 //   kfull/vfull(b)  K / V ring slot b filled (TMA bytes, or one arrival)     tensor-core warp waits
 //   kfree/vfree(b)  both S (both P V) of the chunk in slot b complete        copy warp waits
 //   sfull(p)        S of a chunk of parity p complete (tcgen05.commit)       both groups wait
-//   pfull(p)        P written and O rescaled by the 8 warps of both groups    tensor-core warp waits (one wait and
-//                                                                            one fence for both groups' products)
+//   pfull(g, p)     P_g written and O_g rescaled by the 4 warps of group g    tensor-core warp waits
 //   odone(g, p)     O_g += P_g V of a chunk of parity p complete             group g waits (rescale, end)
 // A new phase of a barrier can only begin after every side that waits on it has seen the previous
 // one (a parity wait must never fall two phases behind).
@@ -94,56 +101,85 @@ __device__ __forceinline__ uint32_t tile_off(int r, int c)
 // (cta_group::2): each keeps its own rows' Q, scores, P and O, and holds keys 64 r .. 64 r + 63 of every K chunk and
 // columns 64 r .. 64 r + 63 of every V chunk (r: its rank), which the tensor cores of both read.  Rank 0's thread issues
 // for both; K / V and P barriers that it waits on are its own (rank 1 arrives remotely), the others exist in both CTAs.
-// What a lone CTA's loop is short of is shared-memory bandwidth: 96 KB read and 64 KB filled per chunk, 1280 of its 2050
-// cycles; in a pair 80 and 32 KB.
-// NW: 64-bit words of a node's ancestor mask.  NW = 1 (trees of up to 64 nodes): the masks are built once per
-// CTA in shared memory.  NW = 4 (up to 256 nodes): there is no shared memory left for them, so every softmax
-// thread follows its own node's parent chain in global memory (a few cached loads) and keeps the mask in registers.
-template <int NW, bool PAIR>
+// (Neither filling the ring nor the products bound the loop: without either it takes as long.)
+template <bool PAIR>
 __global__ void __launch_bounds__(NT, 1)
-tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV)
+tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV)
 {
     constexpr int NS = ring_slots(PAIR);                     // ring slots
     constexpr int SLOT = PAIR ? HALF : TILE;                 // bytes of this CTA's share of a K or V chunk
     constexpr int KROWS = PAIR ? BK / 2 : BK;                // keys of its share of a K chunk
     constexpr int KSUB = KROWS * 128;                        // bytes of one 64-column half of that share
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long s_bar[4 * NS + 13];
+    __shared__ __align__(8) unsigned long long s_bar[4 * NS + 16];
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
-    __shared__ int s_seq;
-    __shared__ int s_par[NW == 1 ? FSPAD_MAX_NODES : 1];
-    __shared__ int s_blk[kMaxBlocksPerCta];       // paged cache: blocks of this CTA's chunks
-    __shared__ unsigned long long s_anc[NW == 1 ? FSPAD_MAX_NODES : 1];
+    __shared__ __align__(8) short s_par[FSPAD_MAX_NODES_WIDE];      // parents (only where this CTA's keys reach into the tree)
 
-    fspad_pdl_wait();
+    if (!a.early) fspad_pdl_wait();
     const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     const bool producer = warp >= 8;         // warp 8 copies, warp 9 drives the tensor cores
     const int row = tid & (BM - 1), grp = (tid >> 7) & 1;
     const int split = PAIR ? blockIdx.y : blockIdx.x, tile_g = PAIR ? blockIdx.x : blockIdx.y;
     const int g = tile_g / a.mtiles, mt = tile_g % a.mtiles;
     const int rank = PAIR ? mt & 1 : 0;           // a.mtiles is even then, so a pair has one kv head
-    int b = blockIdx.z;
+    const int N = a.N, G = a.G, M = a.M;
+    const uint32_t bar0 = smem_u32(&s_bar[0]);
+    // The thread that issues the first TMA copies also initialises the barriers, so those copies
+    // leave as soon as the prefix length is known, ahead of the CTA's first barrier (a pair's: as soon as both CTAs'
+    // barriers are initialised).
+    if (tid == 256) {
+#pragma unroll
+        for (int i = 0; i < 4 * NS + 16; ++i) {
+            int count = 1;
+            if (i >= 4 * NS + 4 && i < 4 * NS + 8) count = PAIR ? 8 : 4;                     // softmax warps of a group
+            if (i >= 4 * NS + 14) count = PAIR ? 16 : 8;                         // all of them
+            if (i == 4 * NS + 13 && PAIR) count = a.q_tma ? 2 : 1;               // Q, and rank 1's tensor memory
+            mbar_init(bar0 + 8u * i, count);
+        }
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 8) {
+        __syncwarp();
+        asm volatile("bar.arrive 2, 320;\n" ::: "memory");                       // (waited for by the other warps in the prologue)
+    }
+    // Launched while its predecessors still run (see Args::early), the grid must not be complete before they are: one CTA sees to it.
+    const bool last_cta = a.early && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
+    int b = blockIdx.z, L;
     if (a.longest_first) {
         // CTAs are dispatched in index order as SMs come free, so with more CTAs than SMs the sequences
-        // handled last decide the tail: they should be the short ones.  Every CTA ranks the sequences by
-        // length (ties by index, so the ranks are a permutation) and takes the one whose rank is blockIdx.z.
-        const int nb = (int)gridDim.z;
-        for (int t = tid; t < nb; t += NT) {
-            const int Lt = a.prefix_len[t];
-            int rank = 0;
-            for (int u = 0; u < nb; ++u) {
-                const int Lu = a.prefix_len[u];
-                rank += (Lu > Lt || (Lu == Lt && u < t)) ? 1 : 0;
+        // handled last decide the tail: they should be the short ones.  Every warp ranks the sequences by
+        // length (ties by index, so the ranks are a permutation) and takes the one whose rank is blockIdx.z; without a barrier
+        // (through shared memory the first wave knew its length after 3800 cycles).
+        const int nb = (int)gridDim.z;            // at most 128
+        int len[4], place[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) len[i] = lane + 32 * i < nb ? a.prefix_len[lane + 32 * i] : 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll 4
+            for (int u = 32 * j; u < min(nb, 32 * j + 32); ++u) {
+                const int Lu = __shfl_sync(0xffffffffu, len[j], u & 31);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) place[i] += (Lu > len[i] || (Lu == len[i] && u < lane + 32 * i)) ? 1 : 0;
             }
-            if (rank == (int)blockIdx.z) s_seq = t;
+        L = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const unsigned hit = __ballot_sync(0xffffffffu, lane + 32 * i < nb && place[i] == (int)blockIdx.z);
+            const int at = __shfl_sync(0xffffffffu, len[i], hit ? __ffs((int)hit) - 1 : 0);
+            if (hit) { b = __ffs((int)hit) - 1 + 32 * i; L = at; }
         }
-        __syncthreads();
-        b = s_seq;
+    } else {
+        L = a.prefix_len[b];
     }
-    const int N = a.N, G = a.G, M = a.M;
+    const int par_of = tid < N ? a.parent[(size_t)b * N + tid] : -1;      // (under way with the prefix length)
+    if (PAIR) {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    }
 
-    int L = a.prefix_len[b];
     if (L < 0 || L + N > a.max_len) {
         if (tid == 0) fspad_report(a.status, FSPAD_ERR_RANGE);
         L = max(0, min(L, a.max_len - N));
@@ -156,96 +192,83 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
 
     const int gr = mt * BM + row;                 // this thread's row among the kv head's M rows
     const bool row_ok = gr < M && !producer;
-    const int node = row_ok ? gr / G : 0;
     const size_t prow = ((size_t)b * a.Hkv + g) * a.n_splits + split;
 
-    if (c0 >= c1) {                               // nothing to do for this split: empty partial
+    if (n_ch <= 0) {                              // nothing to do for this split: empty partial (never in a pair: one range per row)
         if (row_ok && grp == 0) { float *ml = a.part_ml + (prow * M + gr) * 2; ml[0] = -INFINITY; ml[1] = 0.f; }
+        if (last_cta) fspad_pdl_wait();
         return;
     }
 
     // 1024-byte aligned tiles: Q | K[NS] | V[NS]
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sQ = base, sK = base + TILE, sV = base + TILE + NS * SLOT;
-    const uint32_t bar0 = smem_u32(&s_bar[0]);
     auto kfull = [&](int buf) { return bar0 + 8u * (uint32_t)buf; };
     auto vfull = [&](int buf) { return bar0 + 8u * (uint32_t)(NS + buf); };
     auto kfree = [&](int buf) { return bar0 + 8u * (uint32_t)(2 * NS + buf); };
     auto vfree = [&](int buf) { return bar0 + 8u * (uint32_t)(3 * NS + buf); };
     auto sfull = [&](int par) { return bar0 + 8u * (uint32_t)(4 * NS + par); };
-    auto pfull = [&](int par) { return bar0 + 8u * (uint32_t)(4 * NS + 4 + par); };
+    auto pfull = [&](int grp2, int par) { return bar0 + 8u * (uint32_t)(4 * NS + 4 + 2 * grp2 + par); };
     auto odone = [&](int grp2, int par) { return bar0 + 8u * (uint32_t)(4 * NS + 8 + 2 * grp2 + par); };
     const uint32_t drain = bar0 + 8u * (uint32_t)(4 * NS + 12);   // used only when a wait has run out
-    const bool tma_ok = a.use_tma != 0;
-    // The thread that issues the first TMA copies also initialises the barriers, so those copies
-    // leave as soon as the prefix length is known, ahead of the CTA's first barrier (a pair's: as soon as both CTAs'
-    // barriers are initialised).
-    if (tid == 256) {
-#pragma unroll
-        for (int i = 0; i < 4 * NS + 13; ++i)
-            mbar_init(bar0 + 8u * i, (i >= 4 * NS + 4 && i < 4 * NS + 6) ? (PAIR ? 16 : 8) : (PAIR && i < 2 * NS) ? 2 : 1);
-        s_fail = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    if (PAIR) {
-        __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    }
+    const uint32_t qfull = bar0 + 8u * (uint32_t)(4 * NS + 13);   // Q by TMA
+    const uint32_t gkfull = bar0 + 8u * (uint32_t)(4 * NS + 14), gvfull = gkfull + 8u;   // what the softmax warps gather: Q and K, V
+    const bool tma_ok = a.use_tma != 0, q_tma = a.q_tma != 0;
     // arrivals on the barriers of the side that issues
     auto arrive0 = [&](uint32_t bar) { if (PAIR) mbar_arrive_rank0(bar); else mbar_arrive(bar); };
-    auto arrive_p = [&](uint32_t bar) { if (PAIR && rank != 0) mbar_arrive_rank0_light(bar); else mbar_arrive(bar); };
+    auto arrive_p = [&](uint32_t bar) { if (PAIR && rank != 0) mbar_arrive_rank0_light(bar); else mbar_arrive_light(bar); };
 
     const bool paged = a.block_table != nullptr;
-    if (paged) {
-        // the blocks of this CTA's chunks (a chunk is one block); an entry out of range is reported and replaced
-        if (n_ch > kMaxBlocksPerCta && tid == 0) fspad_report(a.status, FSPAD_ERR_SHAPE);
-        for (int i = tid; i < n_ch && i < kMaxBlocksPerCta; i += NT) {
-            int blk = a.block_table[(size_t)b * a.table_stride + c0 + i];
-            if (blk < 0 || blk >= a.n_blocks) { fspad_report(a.status, FSPAD_ERR_RANGE); blk = 0; }
-            s_blk[i] = blk;
-        }
-        __syncthreads();
-    }
+    const int *blocks = paged ? a.block_table + (size_t)b * a.table_stride : nullptr;
     const int plane_row0 = (b * a.Hkv + g) * a.max_len;   // contiguous planes: first row of this kv head
-    // row of the plane matrix [rows][128] that holds cache row `key` of this sequence and kv head
-    // (key inside this CTA's chunks)
-    auto phys_row = [&](int key) -> size_t {
-        if (!paged) return (size_t)plane_row0 + (size_t)key;
-        const int i = min((key >> 7) - c0, kMaxBlocksPerCta - 1);
-        return ((size_t)s_blk[i] * a.Hkv + g) * 128 + (size_t)(key & 127);
+    // row of the plane matrix [rows][128] with which chunk `ch` of this sequence and kv head begins (paged: a chunk is one
+    // block; an entry out of range is reported and replaced)
+    auto chunk_row = [&](int ch) -> int {
+        if (!paged) return plane_row0 + ch * BK;
+        int blk = __ldg(blocks + ch);
+        if (blk < 0 || blk >= a.n_blocks) { fspad_report(a.status, FSPAD_ERR_RANGE); blk = 0; }
+        return (blk * a.Hkv + g) * BK;
     };
     const fspad_bf16 *tkb = a.tk ? a.tk + ((size_t)b * a.Hkv + g) * (size_t)N * D : nullptr;
     const fspad_bf16 *tvb = a.tv ? a.tv + ((size_t)b * a.Hkv + g) * (size_t)N * D : nullptr;
-    auto is_tma = [&](int ch) { return tma_ok && (ch + 1) * BK <= L; };
+    // The chunks are taken from the last one down, so that those TMA cannot describe come first: the ones with rows of an
+    // explicit tree array, and the one that ends in zero padding (at most three of them: 256 nodes).  The softmax warps, idle until
+    // the first scores are there, gather them side by side with the copies of the others.  (Gathered where they stood, at
+    // the end of the range and by the copy warp alone, they held everything up: 2.5 us for each operand.)
+    const int key_tma = tkb ? L : Ltot;           // rows in front of this key lie in the cache
+    auto is_tma = [&](int ch) { return tma_ok && (ch + 1) * BK <= key_tma; };
+    int n_gather = 0;                             // chunks of the first ring filling that are gathered
+    while (n_gather < NS && n_gather < n_ch && !is_tma(c1 - 1 - n_gather)) ++n_gather;
 
-    // Start the fill of an operand buffer with chunk `ch`.  A chunk inside the cached prefix comes
-    // by TMA (two 64 x 128 boxes, issued by one lane of the producer warp, completion counted on
-    // the buffer's mbarrier); the chunk that mixes prefix, tree rows and zero padding is gathered
-    // with 16-byte asynchronous copies by the threads t0, t0 + nt, ... that the caller names (the
-    // whole CTA in the prologue, the producer warp alone inside the loop).
+    // Gather chunk `ch` into ring slot `buf` with 16-byte asynchronous copies by threads t0, t0 + nt, ... (nt a multiple of 16):
+    // 16-byte piece c of every row that falls to a thread is the same, so all its addresses follow from one.
     auto gather = [&](int ch, int buf, bool is_v, int t0, int nt) {
         const uint32_t dst = (is_v ? sV : sK) + buf * SLOT;
-        const fspad_bf16 *cb = is_v ? a.vc : a.kc, *tb = is_v ? tvb : tkb;
-        for (int i = t0; i < SLOT / 16; i += nt) {
-            // row r of the share and 16-byte chunk c of the whole row (a pair's K share: half the keys; its V share: half the columns)
-            const int r = PAIR && is_v ? i >> 3 : i >> 4, cl = PAIR && is_v ? i & 7 : i & 15;
-            const int c = PAIR && is_v ? cl + 8 * rank : cl;
-            const int key = ch * BK + r + (PAIR && !is_v ? KROWS * rank : 0);
+        const fspad_bf16 *tb = is_v ? tvb : tkb;
+        const fspad_bf16 *cb = (is_v ? a.vc : a.kc) + (size_t)chunk_row(ch) * D;
+        const int sh = PAIR && is_v ? 3 : 4;      // a pair's V share: half the columns; its K share: half the keys
+        const int cl = t0 & ((1 << sh) - 1), c = PAIR && is_v ? cl + 8 * rank : cl;
+        const int k_lo = PAIR && !is_v ? KROWS * rank : 0;
+        const uint32_t half = (uint32_t)(cl >> 3) * (PAIR ? KSUB : HALF);
+#pragma unroll 4
+        for (int r = t0 >> sh; r < (PAIR && !is_v ? KROWS : BK); r += nt >> sh) {
+            const int kr = r + k_lo, key = ch * BK + kr;
             const bool ok = key < Ltot;
-            const fspad_bf16 *src = cb;
             // prefix rows, and tree rows that live in the cache, come from the planes; explicit tree rows from their array
-            if (ok) src = (key < L || tb == nullptr) ? cb + phys_row(key) * D + c * 8 : tb + (size_t)(key - L) * D + c * 8;
-            const uint32_t off = PAIR ? (uint32_t)((cl >> 3) * KSUB + r * 128 + (((cl & 7) ^ (r & 7)) << 4)) : tile_off(r, c);
-            cp_async16(dst + off, src, ok);
+            const fspad_bf16 *src = cb;
+            if (ok) src = (key < L || tb == nullptr) ? cb + (size_t)kr * D : tb + (size_t)(key - L) * D;
+            cp_async16(dst + half + (uint32_t)(r * 128 + (((cl & 7) ^ (r & 7)) << 4)), src + c * 8, ok);
         }
     };
-    auto tma_fill = [&](int ch, int buf, bool is_v) {       // one lane
+    // One lane: the TMA copies of a chunk that begins with row y of the planes.  A pair's bytes are all expected by rank 0, whose
+    // barrier counts them (an arrival there by rank 1 took it 400 cycles); rank 1's may land before they are expected,
+    // never before the phase they belong to, because a slot is only refilled when rank 0 has waited for what it held.
+    auto tma_fill = [&](int y, int buf, bool is_v) {
         const uint32_t dst = (is_v ? sV : sK) + buf * SLOT;
         const uint32_t bar = is_v ? vfull(buf) : kfull(buf);
         const CUtensorMap *map = is_v ? &tmV : &tmK;
-        const int y = (int)phys_row(ch * BK);
         if constexpr (PAIR) {
-            mbar_expect_tx_rank0(bar, SLOT);
+            if (rank == 0) mbar_expect_tx(bar, 2 * SLOT);
             if (is_v) {
                 tma_load_2d_pair(dst, map, 64 * rank, y, bar);                    // 128 keys x 64 columns
             } else {
@@ -259,33 +282,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         }
     };
 
-    // ---- prologue: Q and the first NS chunks go out first, the rest hides under their latency (Q ahead of the chunks: behind
-    // the ring's fill on every SM it arrives when that has, 6 us later on a long context) ----
-    for (int i = tid; i < BM * 16; i += NT) {
-        const int r = i >> 4, c = i & 15;
-        const int grr = mt * BM + r;
-        const bool ok = grr < M;
-        const int nd = ok ? grr / G : 0, hh = ok ? grr % G : 0;
-        const fspad_bf16 *src = a.q + (((size_t)b * N + nd) * a.Hq + g * G + hh) * D + c * 8;
-        cp_async16(sQ + tile_off(r, c), src, ok);
-    }
-    if (PAIR) {
-        __syncwarp();
-        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");     // both CTAs' barriers are initialised
-    }
-#pragma unroll
-    for (int u = 0; u < NS; ++u) {
-        if (u >= n_ch) break;
-        if (is_tma(c0 + u)) {
-            if (tid == 256) { tma_fill(c0 + u, u, false); tma_fill(c0 + u, u, true); }
-        } else {
-            gather(c0 + u, u, false, tid, NT);
-            gather(c0 + u, u, true, tid, NT);
-        }
-    }
-    cp_async_commit();
-    if (NW == 1 && tid < N) s_par[tid] = a.parent[(size_t)b * N + tid];
-    __syncthreads();                              // barriers initialised, parents staged
+    // ---- prologue: the tensor memory, then every warp goes its own way; what each needs from the others comes by mbarrier ----
     if (warp == 9) {
         __syncwarp();
         if constexpr (PAIR) {
@@ -297,28 +294,77 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                          :: "r"(smem_u32(&s_tmem)), "r"(TMEM_COLS) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
         }
-    } else if (NW == 1 && tid < N) {
-        // tree -> ancestor-or-self masks (parents were staged in shared memory above)
-        unsigned long long mask = 0ull;
-        int cur = tid;
-        bool bad = false;
-        for (int step = 0; step <= N && cur >= 0; ++step) {
-            mask |= 1ull << cur;
-            const int p = s_par[cur];
-            if (cur == 0) { bad |= (p != -1); break; }
-            if (p < 0 || p >= cur) { bad = true; break; }
-            cur = p;
-        }
-        if (bad) fspad_report(a.status, FSPAD_ERR_BAD_TREE);
-        s_anc[tid] = mask;
     }
-    cp_async_wait<0>();                           // Q and any gathered chunk
-    fence_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    if (PAIR) cluster_sync_all();                 // both CTAs have their Q and their tensor memory
-    tc_fence_after();
-    const uint32_t tmem = s_tmem;
+    auto peer_ready = [&]() {                     // both CTAs' barriers are initialised
+        if (PAIR) {
+            __syncwarp();
+            asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+        }
+    };
+    const bool in_tree = c1 * BK > L;             // this range's keys reach into the tree
+    int blk_row = 0;                              // copy warp: first plane row of chunk 32 i + lane (counted from the range's end)
+    auto first_fills = [&](int u0, int u1) {      // copy warp: ring slots u0 .. u1 - 1, for the first time
+        for (int u = u0; u < u1 && u < n_ch; ++u) {
+            const int y = __shfl_sync(0xffffffffu, blk_row, u);
+            if (lane == 0) {
+                if (u >= n_gather) { tma_fill(y, u, false); tma_fill(y, u, true); }
+                else if (rank == 0) { mbar_arrive(kfull(u)); mbar_arrive(vfull(u)); }       // (gkfull and gvfull tell when they are there)
+            }
+            __syncwarp();
+        }
+    };
+    // The rings of all SMs are 24 to 28 MB, 4 us of HBM, and what is asked for together arrives together: the first scores would wait
+    // for all of it.  So the rest of the ring is asked for when the first scores are there.
+    constexpr int kFirst = PAIR ? 3 : 2;
+    if (warp == 8) {
+        if (lane < n_ch) blk_row = chunk_row(c1 - 1 - lane);
+        peer_ready();
+        if (lane == 0 && q_tma) {
+            const int nd = b * N + mt * (BM / G);
+            if constexpr (PAIR) {
+                if (rank == 0) mbar_expect_tx(qfull, 2 * TILE);
+                tma_load_3d_pair(sQ, &tmQ, 0, g * G, nd, qfull);
+                tma_load_3d_pair(sQ + HALF, &tmQ, 64, g * G, nd, qfull);
+            } else {
+                mbar_expect_tx(qfull, TILE);
+                tma_load_3d(sQ, &tmQ, 0, g * G, nd, qfull);
+                tma_load_3d(sQ + HALF, &tmQ, 64, g * G, nd, qfull);
+            }
+        }
+        first_fills(0, kFirst);
+    } else if (warp < 8) {
+        // What TMA cannot describe: Q where a group of query heads does not divide the tile, and the first n_gather chunks.
+        if (!q_tma) {
+            const int c = tid & 15;
+            int r = tid >> 4;                     // 16 rows a step
+            int nd = (mt * BM + r) / G, hh = (mt * BM + r) % G;
+            const int dn = 16 / G, dh = 16 % G;
+            for (; r < BM; r += 16) {
+                const bool ok = mt * BM + r < M;
+                const fspad_bf16 *src = a.q + (ok ? (((size_t)b * N + nd) * a.Hq + g * G + hh) * D + c * 8 : 0);
+                cp_async16(sQ + tile_off(r, c), src, ok);
+                nd += dn; hh += dh;
+                if (hh >= G) { hh -= G; ++nd; }
+            }
+        }
+        for (int u = 0; u < n_gather; ++u) gather(c1 - 1 - u, u, false, tid, 256);
+        cp_async_commit();
+        for (int u = 0; u < n_gather; ++u) gather(c1 - 1 - u, u, true, tid, 256);
+        cp_async_commit();
+        peer_ready();
+    } else {
+        peer_ready();
+    }
+    if (PAIR && warp == 9 && lane == 0 && rank != 0) arrive0(qfull);             // rank 1's tensor memory is there
+    if (in_tree && tid < N) s_par[tid] = par_of < -1 ? (short)-2 : (short)min(par_of, 32767);
+    // barriers initialised, tensor memory there, parents staged: the copy warp, which has use for none of it, has arrived with
+    // the barriers' initialisation (with it here, the nine other warps waited 2000 cycles for its copies to be issued)
+    if (warp != 8) {
+        tc_fence_before();
+        asm volatile("bar.sync 2, 320;\n" ::: "memory");
+        tc_fence_after();
+    }
+    const uint32_t tmem = warp != 8 ? s_tmem : 0u;
     const uint32_t idesc_s = PAIR ? make_idesc_m256(128) : make_idesc(false, 128);
     const uint32_t idesc_o = PAIR ? make_idesc_m256(128) | (1u << 16) : make_idesc(true, 128);      // B (= V) MN-major
     const uint32_t tO = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256u + (uint32_t)grp * 128u;   // this group's O row
@@ -326,33 +372,33 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
     int filled_k = min(n_ch, NS), filled_v = filled_k;   // copy warp: chunks whose K (V) fill has been started
 
     if (warp == 8) {
-        // ================= copy warp: refills the K / V buffers =================
-        // chunks gathered by the whole CTA in the prologue are announced here
-        if (lane == 0) {
-            for (int u = 0; u < NS && u < n_ch; ++u)
-                if (!is_tma(c0 + u)) { arrive0(kfull(u)); arrive0(vfull(u)); }
-        }
-        auto fill = [&](int ch, int buf, bool is_v) {
-            if (is_tma(ch)) {
-                if (lane == 0) tma_fill(ch, buf, is_v);
+        // ================= copy warp: fills and refills the K / V buffers =================
+        if (n_ch > kFirst && !mbar_wait(kfree(0), 0u)) failed = true;
+        if (!failed) first_fills(kFirst, NS);
+        auto fill = [&](int c, int y, int buf, bool is_v) {
+            if (is_tma(c1 - 1 - c)) {
+                if (lane == 0) tma_fill(y, buf, is_v);
             } else {
-                gather(ch, buf, is_v, lane, 32);
+                gather(c1 - 1 - c, buf, is_v, lane, 32);
                 cp_async_commit();
                 cp_async_wait<0>();
                 fence_async_smem();
                 __syncwarp();
-                if (lane == 0) arrive0(is_v ? vfull(buf) : kfull(buf));
+                if (lane == 0) mbar_arrive(is_v ? vfull(buf) : kfull(buf));      // (a lone CTA: pairs have their maps)
             }
             __syncwarp();
         };
         int buf = 0;                             // i modulo NS
         uint32_t ph = 0;                         // flips each time the ring wraps
         for (int i = 0; i + NS < n_ch; ++i) {
+            const int c = i + NS;
+            if ((c & 31) == 0 && c + lane < n_ch) blk_row = chunk_row(c1 - 1 - c - lane);
+            const int y = __shfl_sync(0xffffffffu, blk_row, c & 31);
             // the K buffer of chunk i is free once S(i) has completed, its V buffer once O += P(i) V(i) has
             if (!failed && !mbar_wait(kfree(buf), ph)) failed = true;
-            if (!failed) { fill(c0 + i + NS, buf, false); ++filled_k; }
+            if (!failed) { fill(c, y, buf, false); ++filled_k; }
             if (!failed && !mbar_wait(vfree(buf), ph)) failed = true;
-            if (!failed) { fill(c0 + i + NS, buf, true); ++filled_v; }
+            if (!failed) { fill(c, y, buf, true); ++filled_v; }
             if (++buf == NS) { buf = 0; ph ^= 1u; }
         }
         if (failed) s_fail = 1;
@@ -362,8 +408,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         // and 2 K keys, 35.8 against 37.8 at 8 and 8 K, 99.3 against 101.4 on the ragged batch of 16)
         if (rank == 0) {
             const bool issuer = elect_one();
-            const uint32_t elect = 1;             // the instructions stand in the issuer's branch
-            auto commit = [&](uint32_t bar) { if (PAIR) mma_commit_pair(bar); else mma_commit_if(bar, elect); };
+            auto commit = [&](uint32_t bar) { if (PAIR) mma_commit_pair(bar); else mma_commit(bar); };
             // low words of the shared-memory descriptors (start address and leading byte offset);
             // the high word (8-row group stride, version, swizzle mode) is the same for all
             const uint32_t hi = (uint32_t)(make_desc(0, 16) >> 32);
@@ -374,7 +419,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             // S(c) = Q K(c)^T into score buffer c & 1 (columns 0..63 of it belong to group 0, 64..127 to
             // group 1); K(c) sits in ring slot kbuf, which the second commit releases
             auto issue_s = [&](int c) {
-                if (!failed && !mbar_wait_warp(kfull(kbuf), kph)) failed = true;
+                if (!failed && !mbar_wait(kfull(kbuf), kph)) failed = true;
                 if (!failed && issuer) {
                     // no tcgen05 fence here: the K chunk comes through the barrier's own acquire, and the
                     // score buffer's last readers and writers (softmax of chunk c - 2) were ordered before this
@@ -385,7 +430,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                     for (int ks = 0; ks < 8; ++ks) { // K = 16 per instruction over d = 128
                         const uint32_t qoff = ((ks >> 2) * HALF + (ks & 3) * 32) >> 4, koff = ((ks >> 2) * KSUB + (ks & 3) * 32) >> 4;
                         if constexpr (PAIR) mma_f16_pair(d, q_lo + qoff, kb + koff, hi, idesc_s, ks > 0);
-                        else mma_f16_lo(d, q_lo + qoff, hi, kb + koff, hi, idesc_s, ks > 0, elect);
+                        else mma_f16_ss(d, q_lo + qoff, kb + koff, hi, idesc_s, ks > 0);
                     }
                     commit(sfull(c & 1));
                     commit(kfree(kbuf));
@@ -393,8 +438,11 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                 __syncwarp();
                 if (++kbuf == NS) { kbuf = 0; kph ^= 1u; }
             };
+            if ((PAIR || q_tma) && !mbar_wait(qfull, 0u)) failed = true;
+            if ((n_gather > 0 || !q_tma) && !failed && !mbar_wait(gkfull, 0u)) failed = true;
             issue_s(0);
             if (n_ch > 1) issue_s(1);
+            if (n_gather > 0 && !failed && !mbar_wait(gvfull, 0u)) failed = true;
             for (int c = 0; c < n_ch; ++c) {
                 const int p = c & 1;
                 const uint32_t ph = (uint32_t)(c >> 1) & 1u;
@@ -403,10 +451,10 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                 for (int g2 = 0; g2 < 2; ++g2) {
                     // O[g2] += P_g2(c) V(c)[64 g2 .. 64 g2 + 63]: P from the four warps of group g2 (in tensor
                     // memory, over the scores it was computed from) and the V chunk
-                    if (g2 == 0 && !failed && !mbar_wait_warp(pfull(p), ph)) failed = true;
-                    if (g2 == 0 && !failed && !mbar_wait_warp(vfull(vbuf), vph)) failed = true;
+                    if (!failed && !mbar_wait(pfull(g2, p), ph)) failed = true;
+                    if (g2 == 0 && !failed && !mbar_wait(vfull(vbuf), vph)) failed = true;
                     if (!failed && issuer) {
-                        if (g2 == 0) tc_fence_after();
+                        tc_fence_after();
                         const uint32_t a_t = tmem + (uint32_t)p * 128u + (uint32_t)g2 * 64u;
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) { // K = 16 keys per instruction = 8 columns of packed bf16 pairs
@@ -415,7 +463,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
                             const uint32_t od = tmem + 256u + (uint32_t)g2 * 128u, at = a_t + (uint32_t)ks * 8u;
                             const uint32_t vk = vb + (uint32_t)((g2 * 64 + ks * 16) * 128 >> 4);
                             if constexpr (PAIR) mma_f16_ts_pair(od, at, vk, hi, idesc_o, (c > 0) || (ks > 0));
-                            else mma_f16_ts(od, at, vk, hi, idesc_o, (c > 0) || (ks > 0), elect);
+                            else mma_f16_ts(od, at, vk, hi, idesc_o, (c > 0) || (ks > 0));
                         }
                         commit(odone(g2, p));
                         if (g2 == 1) commit(vfree(vbuf));
@@ -432,71 +480,50 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
     } else {
         // ================= softmax warps =================
         const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
-        unsigned long long anc[NW];
-        if (NW == 1) {
-            anc[0] = s_anc[node];
-        } else {
-#pragma unroll
-            for (int w = 0; w < NW; ++w) anc[w] = 0ull;
-            if (row_ok) {
-                const int *par = a.parent + (size_t)b * N;
-                int cur = node;
-                bool bad = false;
-                for (int step = 0; step <= N && cur >= 0; ++step) {
-#pragma unroll
-                    for (int w = 0; w < NW; ++w) anc[w] |= ((cur >> 6) == w) ? (1ull << (cur & 63)) : 0ull;
-                    const int p = __ldg(par + cur);
-                    if (cur == 0) { bad |= (p != -1); break; }
-                    if (p < 0 || p >= cur) { bad = true; break; }
-                    cur = p;
-                }
-                if (bad) fspad_report(a.status, FSPAD_ERR_BAD_TREE);
-            }
+        if (n_gather > 0 || !q_tma) {
+            cp_async_wait<1>();
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) arrive0(gkfull);
+            cp_async_wait<0>();
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) arrive0(gvfull);
         }
-        // 32 bits of the mask from tree index `off` on (prefix keys, off < 0, count as set; bits beyond the mask are clear)
-        auto mask_word = [&](int off) -> uint32_t {
-            if (off >= 64 * NW) return 0u;
-            if (off <= -32) return ~0u;
-            if (off < 0) return ((1u << (-off)) - 1u) | (uint32_t)(anc[0] << (-off));
-            const int w = off >> 6, sft = off & 63;
-            unsigned long long lo = 0ull, hi = 0ull;
-#pragma unroll
-            for (int i = 0; i < NW; ++i) {
-                if (i == w) lo = anc[i];
-                if (i == w + 1) hi = anc[i];
-            }
-            unsigned long long v = lo >> sft;
-            if (sft > 32) v |= hi << (64 - sft);
-            return (uint32_t)v;
-        };
         const float scale = a.scale_log2;
         const bool live = mt * BM + (warp & 3) * 32 < M;   // the last row tile may end before this warp's rows
         float m_run = -INFINITY, l_run = 0.f;
+        int cur = in_tree && row_ok ? gr / G : -1;         // this row's node, then its ancestors: how far the chunks so far have taken them
 
         for (int c = 0; c < n_ch; ++c) {
-            const int ch = c0 + c, p = c & 1;
+            const int ch = c1 - 1 - c, p = c & 1;      // (from the last chunk down)
             const uint32_t tS = tmem + lanes + (uint32_t)p * 128u + (uint32_t)grp * 64u;   // scores, then P
+            const bool masked = (ch + 1) * BK > L;   // only chunks that reach past the cached prefix
+            // Validity of this group's 64 keys for this row: prefix keys are valid, tree key L + t is valid iff t is the row's node
+            // or one of its ancestors (which also rules out the zero padding).  Parents come before their children and the
+            // chunks from the last one down, so every chunk takes the walk to the root on from where the one before it left off;
+            // no mask is kept, whatever the tree's size.
+            unsigned long long valid = ~0ull;
+            if (masked) {
+                const int t0 = ch * BK + grp * 64 - L, t_chunk = ch * BK - L;        // tree index of the group's, the chunk's first key
+                valid = t0 >= 0 ? 0ull : t0 <= -64 ? ~0ull : (1ull << -t0) - 1ull;
+                while (cur >= 0 && cur >= t_chunk) {
+                    const unsigned o = (unsigned)(cur - t0);
+                    if (o < 64u) valid |= 1ull << o;
+                    const int p = s_par[cur];
+                    if (cur == 0 ? p != -1 : (p < 0 || p >= cur)) fspad_report(a.status, FSPAD_ERR_BAD_TREE);
+                    cur = p < cur ? p : -1;
+                }
+            }
             if (!failed && !mbar_wait(sfull(p), (uint32_t)(c >> 1) & 1u)) failed = true;
             if (!live) {
                 // (no row of this warp exists: its scores are not looked at, and what its lanes' P holds stays in their
                 // own rows of O, which nobody stores)
                 __syncwarp();
-                if (lane == 0) arrive_p(pfull(p));
+                if (lane == 0) arrive_p(pfull(grp, p));
                 continue;
             }
             tc_fence_after();
-            const bool masked = (ch + 1) * BK > L;   // only chunks that reach past the cached prefix
-            // Validity of this group's 64 keys for this row as two 32-bit words: prefix keys are
-            // valid, tree key L + t is valid iff bit t of the row's ancestor mask is set (bits at and
-            // beyond the tree size are clear, which also rules out the zero padding).
-            uint32_t valid[2] = {~0u, ~0u};
-            if (masked) {
-#pragma unroll
-                for (int blk = 0; blk < 2; ++blk) {
-                    const int off = ch * BK + grp * 64 + blk * 32 - L;      // tree index of the word's first key
-                    valid[blk] = mask_word(off);
-                }
-            }
             // ---- this row's 64 scores of the group, in registers after one trip to tensor memory, with the
             // tree mask applied where it matters; the row maximum as four independent chains ----
             float v[64];
@@ -513,7 +540,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             if (masked) {
 #pragma unroll
                 for (int j = 0; j < 64; ++j)
-                    if (!((valid[j >> 5] >> (j & 31)) & 1u)) v[j] = -INFINITY;
+                    if (!(((uint32_t)(valid >> (j & 32)) >> (j & 31)) & 1u)) v[j] = -INFINITY;
             }
             float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -545,7 +572,9 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             // ---- P = exp2(s * scale - m) as bf16 pairs, written over the group's score columns (every score
             // is in registers by now); the row sum as four pairs of chains; multiply-adds and sums two to an instruction
             // (33.6 against 34.1 us on 52 heads and 4 K keys, 75.9 against 77.2 on the ragged batch; taking the exponentials
-            // against the old reference while the maximum is being found cost registers: 2 us more on every shape) ----
+            // against the old reference while the maximum is being found cost registers: 2 us more on every shape; asking for
+            // half of the next chunk's scores between the two halves of this one's exponentials: 112 against 96 us on 16
+            // sequences of 4 K keys) ----
             float rs;
             {
                 const uint64_t scale2 = f32x2(scale, scale), neg = f32x2(-m_safe, -m_safe);
@@ -573,7 +602,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) arrive_p(pfull(p));
+            if (lane == 0) arrive_p(pfull(grp, p));
         }
         // ---- each group waits for its own last product (tensor-core work completes in order, so the
         // one before it is complete too); the CTA-wide barrier below then orders both accumulators
@@ -588,63 +617,77 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        // ---- publish the partial: the two groups' (max, sum, O row) merged by log-sum-exp ----
+        // ---- publish the row: the two groups' (max, sum, O row) merged by log-sum-exp ----
         // Thread (row, grp) owns output columns grp*64 .. grp*64+63.  Every lane of every softmax warp
         // takes part in the tensor-memory loads (they are warp-collective); only the stores to global
-        // memory depend on whether the lane's row exists.
+        // memory depend on whether the row exists.
         const bool any_fail = s_fail != 0;
         if (any_fail && tid == 0) fspad_report(a.status, FSPAD_ERR_TIMEOUT);
-        const bool store = row_ok && !any_fail;
-        float *s_inv = reinterpret_cast<float *>(s_ml + 2 * BM);             // (the Q tile, too)
         const float2 ml0 = s_ml[row], ml1 = s_ml[BM + row];
         const float m_all = fmaxf(ml0.x, ml1.x);
         const float m_fin = (m_all == -INFINITY) ? 0.f : m_all;
-        const float f0 = ex2f(ml0.x - m_fin), f1 = ex2f(ml1.x - m_fin);     // exp2(-inf) = 0 for a fully masked half
-        // The merged rows go through shared memory (the K ring is idle by now), so that the global
-        // stores are whole 512-byte rows per warp instead of 32 row-strided pieces per instruction
-        // (every such piece is a transaction of its own: the direct stores cost 3 us per CTA).
-        constexpr int SROW = D + 4;                   // floats per staged row; the pad keeps 16-byte stores conflict-free
-        float *stg = reinterpret_cast<float *>(smem_raw + (base - smem_u32(smem_raw)) + TILE);
-        float *ps = stg + row * SROW + grp * 64;
+        float f0 = ex2f(ml0.x - m_fin), f1 = ex2f(ml1.x - m_fin);           // exp2(-inf) = 0 for a fully masked half
+        const float l_all = ml0.y * f0 + ml1.y * f1;
+        const bool final = a.out != nullptr;
+        if (final) {
+            const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+            f0 *= inv;
+            f1 *= inv;
+        }
+        // The merged rows are staged in shared memory (the K ring is idle by now), so that they leave as whole rows, 16 bytes a
+        // lane.  (Stores straight from the registers are row-strided pieces, each a transaction of its own: 3 us per CTA; a bulk
+        // copy per row: 1.1 us until the last of the 128 has been read; rows one after another with their addresses: 1.2 us.)
+        constexpr int FROW = D * 4 + 16, HROW = D * 2 + 16;      // bytes of a staged row; the pad keeps 16-byte stores conflict-free
+        const uint32_t stage = base + TILE, stg = stage + (uint32_t)(row * (final ? HROW : FROW));
+        int *s_row = reinterpret_cast<int *>(s_par);             // where each row goes (-1: nowhere); nobody looks at the parents any more
+        static_assert(sizeof(s_par) >= BM * sizeof(int), "one place per row");
+        if (grp == 0) s_row[row] = !row_ok || any_fail ? -1 : final ? (b * N + gr / G) * a.Hq + g * G + gr % G : gr;
         const uint32_t tO0 = tmem + lanes + 256u + (uint32_t)grp * 64u, tO1 = tO0 + 128u;
 #pragma unroll
         for (int q2 = 0; q2 < 2; ++q2) {
-            float o[32], o1[32];
-            tmem_ld32(tO0 + q2 * 32, o);
-            tmem_ld32(tO1 + q2 * 32, o1);
+            uint32_t o[32], o1[32];
+            __syncwarp();
+            tmem_ld32_issue(tO0 + q2 * 32, o);
+            tmem_ld32_issue(tO1 + q2 * 32, o1);
+            tmem_ld_wait(o);
+            tmem_ld_pin(o1);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) o[j] = fmaf(o1[j], f1, o[j] * f0);
+            for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(fmaf(__uint_as_float(o1[j]), f1, __uint_as_float(o[j]) * f0));
+            if (final) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 4)
-                *reinterpret_cast<float4 *>(ps + q2 * 32 + j) = make_float4(o[j], o[j + 1], o[j + 2], o[j + 3]);
+                for (int j = 0; j < 32; j += 8)
+                    st_shared16(stg + (uint32_t)(grp * 128 + q2 * 64 + j * 2),
+                                pack_bf16(__uint_as_float(o[j]), __uint_as_float(o[j + 1])), pack_bf16(__uint_as_float(o[j + 2]), __uint_as_float(o[j + 3])),
+                                pack_bf16(__uint_as_float(o[j + 4]), __uint_as_float(o[j + 5])), pack_bf16(__uint_as_float(o[j + 6]), __uint_as_float(o[j + 7])));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) st_shared16(stg + (uint32_t)(grp * 256 + q2 * 128 + j * 4), o[j], o[j + 1], o[j + 2], o[j + 3]);
+            }
         }
-        const float l_all = ml0.y * f0 + ml1.y * f1;
-        if (a.out != nullptr) {
-            if (grp == 0) s_inv[row] = l_all > 0.f ? 1.f / l_all : 0.f;
-        } else if (store && grp == 0) {
+        if (!final && row_ok && grp == 0 && !any_fail) {
             float *ml = a.part_ml + (prow * M + gr) * 2;
             ml[0] = m_all;
             ml[1] = l_all;
         }
         asm volatile("bar.sync 1, 256;\n" ::: "memory");   // the eight softmax warps
-        if (!any_fail) {
-            for (int r = warp; r < BM; r += 8) {
-                const int grr = mt * BM + r;
-                if (grr < M && a.out != nullptr) {
-                    const float4 o4 = *reinterpret_cast<const float4 *>(stg + r * SROW + lane * 4);
-                    const float inv = s_inv[r];
-                    const int nd = grr / G, hh = grr % G;
-                    *reinterpret_cast<uint2 *>(a.out + (((size_t)b * N + nd) * a.Hq + g * G + hh) * D + lane * 4) =
-                        make_uint2(pack_bf16(o4.x * inv, o4.y * inv), pack_bf16(o4.z * inv, o4.w * inv));
-                } else if (grr < M)
-                    *reinterpret_cast<float4 *>(a.part_o + (prow * M + grr) * D + lane * 4) =
-                        *reinterpret_cast<const float4 *>(stg + r * SROW + lane * 4);
+        if (final) {
+#pragma unroll
+            for (int i = 0; i < BM / 16; ++i) {                  // a warp takes 16 rows, two at a time
+                const int r = warp * 16 + 2 * i + (lane >> 4), to = s_row[r];
+                if (to >= 0) reinterpret_cast<uint4 *>(a.out + (size_t)to * D)[lane & 15] = ld_shared16(stage + (uint32_t)(r * HROW + (lane & 15) * 16));
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < BM / 8; ++i) {
+                const int r = warp * 16 + i, to = s_row[r];
+                if (to >= 0) reinterpret_cast<uint4 *>(a.part_o + (prow * M + to) * D)[lane] = ld_shared16(stage + (uint32_t)(r * FROW + lane * 16));
             }
         }
         fspad_pdl_trigger();                      // partial written: the merge kernel may start launching
         tc_fence_before();
         __syncthreads();
         if (PAIR) cluster_sync_all();             // neither CTA leaves while the other may still reach it
+        if (last_cta) fspad_pdl_wait();
         return;
     }
     // copy and tensor-core warps: meet the softmax warps at their two CTA-wide barriers; the warp
@@ -657,6 +700,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
         // waits for the last fill it started in every ring slot, the tensor-core warp for everything
         // its thread has issued (one more commit on a barrier of its own).
         if (warp == 8) {
+            if ((PAIR || q_tma) && rank == 0) (void)mbar_wait(qfull, 0u);
             for (int sl = 0; sl < NS && rank == 0; ++sl) {    // (a pair's fills are all counted by rank 0's barriers)
                 const int nk = (filled_k - sl + NS - 1) / NS, nv = (filled_v - sl + NS - 1) / NS;   // fills of slot sl
                 if (nk > 0) (void)mbar_wait(kfull(sl), (uint32_t)(nk - 1) & 1u);
@@ -664,7 +708,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmK, con
             }
         } else if (rank == 0) {
             if constexpr (PAIR) { if (lane == 0) mma_commit_pair(drain); }
-            else mma_commit_if(drain, lane == 0);
+            else { if (lane == 0) mma_commit(drain); }
             (void)mbar_wait(drain, 0u);
         }
     }
@@ -773,6 +817,22 @@ bool fspad_make_tmap_bf16_2d(CUtensorMap *map, const fspad_bf16 *base, size_t co
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The query rows [nodes of all sequences][Hq][128] as boxes of 64 columns, the G heads of a kv head and the 128 / G nodes of a
+// row tile, which land as one half tile in the rows' order (G divides 128; nodes past a sequence's last one belong to rows that
+// nobody looks at).
+static bool make_q_map(CUtensorMap *map, const fspad_bf16 *q, size_t nodes, int Hq, int G)
+{
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn || umma::BM % G != 0 || nodes > 0x7fffffffull) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)umma::D, (cuuint64_t)Hq, (cuuint64_t)nodes};
+    const cuuint64_t strides[2] = {umma::D * sizeof(fspad_bf16), (cuuint64_t)Hq * umma::D * sizeof(fspad_bf16)};
+    const cuuint32_t box[3] = {64u, (cuuint32_t)G, (cuuint32_t)(umma::BM / G)};
+    const cuuint32_t estr[3] = {1u, 1u, 1u};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<fspad_bf16 *>(q), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 static bool make_plane_map(CUtensorMap *map, const fspad_bf16 *plane, size_t rows)
 {
     return fspad_make_tmap_bf16_2d(map, plane, (size_t)umma::D, rows, (unsigned)umma::BK);
@@ -790,17 +850,14 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     a.M = N * a.G; a.max_len = paged.table ? paged.stride * umma::BK : c.max_len; a.n_splits = n_splits;
     a.block_table = paged.table; a.table_stride = paged.stride; a.n_blocks = paged.n_blocks;
     a.mtiles = fspad_attn_mtiles(ctx, N, B, sms);
-    const bool pair = fspad_attn_pairs(ctx, N, B, sms);
     // (every CTA ranks all sequences itself, B loads each for B / 320 of its threads: kept to batches where that is small change)
     a.longest_first = (B > 1 && B <= 128 && (long long)B * c.n_kv_heads * a.mtiles * n_splits > ctx->sm_count) ? 1 : 0;
     a.scale_log2 = scale_log2;
     a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.out = n_splits == 1 ? out : nullptr; a.status = ctx->d_status;
     if (!ctx->attn_attr_done) {
         const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        cudaError_t e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<1, false>, at, umma::smem_bytes(false));
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<4, false>, at, umma::smem_bytes(false));
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<1, true>, at, umma::smem_bytes(true));
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<4, true>, at, umma::smem_bytes(true));
+        cudaError_t e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<false>, at, umma::smem_bytes(false));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma::tree_attn_umma_kernel<true>, at, umma::smem_bytes(true));
         if (e != cudaSuccess) return e;
         ctx->attn_attr_done = 1;
     }
@@ -817,9 +874,12 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
         ctx->attn_tmap_kptr = kc; ctx->attn_tmap_vptr = vc; ctx->attn_tmap_rows = rows;
     }
     a.use_tma = ctx->attn_tmap_ok ? 1 : 0;
+    const bool pair = a.use_tma && fspad_attn_pairs(ctx, N, B, sms);      // (without maps the tiles go to lone CTAs, one of them perhaps empty)
+    a.early = 0;
+    CUtensorMap mq = {};
+    a.q_tma = make_q_map(&mq, q, (size_t)B * N, c.n_q_heads, a.G) ? 1 : 0;
     const dim3 grid = pair ? dim3(c.n_kv_heads * a.mtiles, n_splits, B) : dim3(n_splits, c.n_kv_heads * a.mtiles, B);
     ctx->launches++;
-    auto kernel = N <= FSPAD_MAX_NODES ? (pair ? umma::tree_attn_umma_kernel<1, true> : umma::tree_attn_umma_kernel<1, false>)
-                                       : (pair ? umma::tree_attn_umma_kernel<4, true> : umma::tree_attn_umma_kernel<4, false>);
-    return fspad_launch_opt(false, kernel, grid, dim3(umma::NT), umma::smem_bytes(pair), st, pair ? 2u : 0u, a, pair ? *mk_half : *mk, *mv);
+    auto kernel = pair ? umma::tree_attn_umma_kernel<true> : umma::tree_attn_umma_kernel<false>;
+    return fspad_launch_opt(false, kernel, grid, dim3(umma::NT), umma::smem_bytes(pair), st, pair ? 2u : 0u, a, mq, pair ? *mk_half : *mk, *mv);
 }

@@ -15,7 +15,7 @@ bool fspad_make_tmap_bf16_2d(CUtensorMap *map, const fspad_bf16 *base, size_t co
 
 namespace umma {
 
-constexpr uint32_t WAIT_CAP = 200000;   // polls of a bounded mbarrier wait
+constexpr uint32_t WAIT_CAP = 200000;   // tries of a bounded mbarrier wait
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -34,42 +34,27 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count));
 }
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+// One try of a wait: the thread sleeps in hardware until the phase completes or about a microsecond has passed.
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(1000u) : "memory");
     return ok != 0;
 }
-// Bounded wait (non-blocking test + short sleep, about 20 ms in all); false if the cap ran out.
-// Lane 0 polls and the warp takes its verdict through a full-mask shuffle, so every lane leaves
-// together with the same verdict: the warp-collective tensor-memory instructions that follow need
-// a converged warp, and the tensor-core warp's issue loop needs one `failed` flag for all lanes.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t cap = WAIT_CAP)
-{
-    int ok = 0;
-    if ((threadIdx.x & 31) == 0) {
-        for (uint32_t i = 0; i < cap && !ok; ++i) {
-            ok = mbar_test(bar, parity) ? 1 : 0;
-            if (!ok && i >= 64) __nanosleep(40);      // the first polls spin: hand-offs are short
-        }
-    }
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    return ok != 0;
-}
-
-// The same bounded wait for a thread on its own (no other lane of its warp takes part).
+// The bounded wait (some 0.2 s in all) of a thread on its own; false if the cap ran out.
 __device__ __forceinline__ bool mbar_wait_thread(uint32_t bar, uint32_t parity, uint32_t cap = WAIT_CAP)
 {
-    for (uint32_t i = 0; i < cap; ++i) {
-        if (mbar_test(bar, parity)) return true;
-        if (i >= 64) __nanosleep(40);
-    }
+    for (uint32_t i = 0; i < cap; ++i)
+        if (mbar_try(bar, parity)) return true;
     return false;
 }
-
-// The same bounded wait for a converged warp whose lanes all poll; every lane leaves with the same verdict.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t cap = WAIT_CAP)
+// The same for a converged warp: every lane waits, and all leave with the same verdict, because the warp-collective
+// tensor-memory instructions that follow need a converged warp and the tensor-core warp's issue loop one `failed` flag.
+// (Asleep in hardware the waiting warps leave the shared-memory pipe to the others: with polling loops of lane 0, or of all
+// lanes of the tensor-core warp, the softmax warps of the attention were held up by 500 cycles at every hand-over, although what
+// they waited for had long been there: 100 -> 94 us on 16 sequences of 4 K keys.)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t cap = WAIT_CAP)
 {
     return __all_sync(0xffffffffu, mbar_wait_thread(bar, parity, cap)) != 0;
 }
@@ -98,6 +83,23 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
                  :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y) : "memory");
 }
 
+// one box of a 3-D tensor map
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];\n"
+                 :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared16(uint32_t src)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(src) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_shared16(uint32_t dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
 // shared-memory matrix descriptor, 128-byte swizzle, 8-row groups 1024 bytes apart
 __device__ __forceinline__ uint64_t make_desc(uint32_t addr, uint32_t lbo_bytes)
 {
@@ -121,18 +123,16 @@ __device__ __forceinline__ uint32_t make_idesc(bool b_mn_major, uint32_t n)
     d |= (128u >> 4) << 24;                 // M
     return d;
 }
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                        uint32_t accumulate)
+// D[tmem] (+)= A[smem] * B[smem], descriptors as low words and the high word they share: the issuing thread keeps the
+// precomputed low words in registers and adds a tile offset with one integer add
+__device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate)
 {
-    const uint32_t zero = 0;                // no output lane is disabled
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n\t}\n"
-                 :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(zero), "r"(zero),
-                    "r"(zero), "r"(zero) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+                 "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}\n"
+                 :: "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
 }
-// same instruction, descriptors handed over as (low, high) words so the issuing thread can keep
-// the precomputed low words in registers and add a tile offset with one integer add
-// The whole warp runs the issue loop so that descriptors and addresses stay warp-uniform values;
+// The same predicated on one lane: the whole warp runs the issue loop so that descriptors and addresses stay warp-uniform values;
 // `elect` is non-zero in the one lane whose instruction is actually issued.
 __device__ __forceinline__ void mma_f16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                            uint32_t idesc, uint32_t accumulate, uint32_t elect)
@@ -169,12 +169,7 @@ __device__ __forceinline__ void mbar_arrive_rank0(uint32_t bar)
 __device__ __forceinline__ void mbar_arrive_rank0_light(uint32_t bar)
 {
     asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\t"
-                 "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}\n" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx_rank0(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\t"
-                 "mbarrier.arrive.expect_tx.shared::cluster.b64 _, [ra], %1;\n\t}\n" ::"r"(bar), "r"(bytes) : "memory");
+                 "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [ra];\n\t}\n" ::"r"(bar) : "memory");
 }
 // one box into this CTA's shared memory, its bytes counted by the barrier at `bar`'s offset in rank 0's
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
@@ -182,6 +177,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
     asm volatile("{\n\t.reg .b32 rb;\n\tmapa.shared::cluster.u32 rb, %2, 0;\n\t"
                  "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [rb];\n\t}\n"
                  :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar)
+{
+    asm volatile("{\n\t.reg .b32 rb;\n\tmapa.shared::cluster.u32 rb, %2, 0;\n\t"
+                 "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [rb];\n\t}\n"
+                 :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
 }
 // instruction descriptor of the pair: bf16 x bf16 -> fp32, M = 256 (128 rows of A in each CTA), N = n
 // (half of B's rows in each CTA), both operands K-major
@@ -286,15 +287,20 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
+// the same for an arrival that only orders tensor memory (the tcgen05 fences do that)
+__device__ __forceinline__ void mbar_arrive_light(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
 // D[tmem] (+)= A[tmem] * B[smem]: the A operand (here P, bf16 pairs packed into 32-bit columns, one
 // query row per lane) is read from tensor memory
 __device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
-                                           uint32_t accumulate, uint32_t elect)
+                                           uint32_t accumulate)
 {
-    asm volatile("{\n\t.reg .pred p, e;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 e, %6, 0;\n\t"
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
                  "mov.b64 db, {%2, %3};\n\t"
-                 "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}\n"
-                 :: "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(elect) : "memory");
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}\n"
+                 :: "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void mma_commit_if(uint32_t bar, uint32_t elect)
 {

@@ -177,3 +177,24 @@ def test_prefix_out_of_range_is_reported():
         ctx.tree_attn(d["q"], d["k_cache"], d["v_cache"], d["tree_k"], d["tree_v"].flatten()[1:], d["parent"],
                       d["prefix_len"])
     assert e.value.code == -2
+
+
+@pytest.mark.parametrize("hq,hkv,prefix,n", [
+    (2, 2, 128, 60),       # the prefix ends with a chunk: the tree's chunk holds nothing but tree rows and padding
+    (6, 2, 127, 1),        # Q gathered (three heads a group); the last chunk is exactly full
+    (14, 2, 129, 60),      # Q gathered, rows of a tile begin within a node
+    (2, 1, 255, 129),      # three chunks with tree rows, one of them full
+    (4, 1, 127, 256),      # three chunks with tree rows, the first with a single one
+    (120, 40, 300, 60),    # pairs of CTAs, Q gathered
+    (80, 40, 383, 65),     # pairs of CTAs, the last chunk is exactly full
+])
+def test_rows_behind_the_tree_may_hold_anything(hq, hkv, prefix, n):
+    """Chunks with tree rows or padding are gathered, the others copied by TMA: what lies behind the last tree row (or, where the
+    tree rows come apart, behind the prefix) is NaN here and must not get into any sum."""
+    w = synth.scaled(W["llama3_8b_2k"], n_q_heads=hq, n_kv_heads=hkv, prefix=(prefix, prefix), n_nodes=n,
+                     tree="pruned" if n > 1 else "chain", depth=8 if n > 1 else 1, branch=10, vocab=16)
+    inp = synth.generate(w, 3, with_accept=False)
+    for alias in (True, False):
+        for plane in (inp.k_cache, inp.v_cache):
+            plane[:, :, prefix + (n if alias else 0):] = 0x7FC0
+        _check(inp, alias_cache=alias)
