@@ -418,14 +418,15 @@ int fspad_kv_compact_paged(fspad_ctx *ctx, fspad_bf16 *pool, const int32_t *bloc
  * loop).  Equivalent to fspad_tree_attn (over the K and V planes of layer
  * `attn_layer` of `cache`), fspad_tree_accept and fspad_kv_compact queued one
  * after the other on `stream`, with the same arguments, outputs and errors, but
- * the attention runs on a second stream owned by the context, forked from and
- * joined back into `stream` with events: attention and acceptance share no
- * data, so their kernels overlap on the device.  Compaction follows the
+ * the attention runs beside the acceptance (they share no data): as a
+ * programmatic dependent in `stream` where it is the longer of the two, else on a
+ * second stream owned by the context, forked from and joined back into `stream`
+ * with events.  Compaction follows the
  * acceptance directly when tree_k / tree_v are given (attention then never
  * reads the cache rows compaction rewrites); when they are NULL (tree rows
  * taken from cache rows L_b ..) compaction waits for the attention as well.
  * In the first case, when a sequence has at most 64 (layer, K/V, kv head)
- * slices, the kernel that walks the tree makes the compaction's moves itself,
+ * slices (256 where a sampling step stays in one stream), the kernel that walks the tree makes the compaction's moves itself,
  * greedy or sampling (same result; an invalid prefix length is then reported by
  * that kernel).
  * Work queued on `stream` after the call sees every output.  The call only

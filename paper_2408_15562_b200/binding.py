@@ -337,7 +337,7 @@ class Context:
     def verify_step(self, cache, q, tree_k, tree_v, parent, prefix_len, target_logits, draft_probs, draft_tokens,
                     temperature, uniforms, attn_out, accepted_path, n_accepted, bonus_token, new_len, attn_layer=0,
                     stream=None):
-        """The whole verify step on device tensors: attention (second stream of the context) beside
+        """The whole verify step on device tensors: attention beside
         acceptance, then compaction; outputs are written in place."""
         B, N = q.shape[0], q.shape[1]
         bf, f32, i32 = torch.bfloat16, torch.float32, torch.int32

@@ -61,32 +61,46 @@ const void *mapped_whole(const void *p, size_t bytes)
 // How a step's attention shares the SMs with its acceptance.  Both entry points take it from here: the number of key ranges
 // follows from attn_sms, and with it which reference a probability is rounded against, so that they give the same bits.
 struct StepPlan {
-    bool scan_first;            // the scan goes first on all SMs, the attention behind it beside the walk
+    bool chain;                 // one stream: scan, walk, and the attention launched beside the walk
+    bool scan_first;            // two streams: the scan goes first on all SMs, the attention behind it beside the walk
     int attn_sms;               // SMs the attention may fill (0: all)
 };
 StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample)
 {
     // Which of the two goes first.  The acceptance is a streaming scan over every SM followed by a walk
-    // that one cluster per sampling sequence carries out; the attention is one CTA per SM.  When the
-    // attention's CTAs leave a good part of the SMs free, both start at once and the acceptance lives on
-    // the free SMs.  Otherwise the scan goes first on all SMs and the attention is forked behind it, sized
-    // to leave the walk's SMs alone, so that the walk (the longer chain) and the attention run side by side.
+    // that one cluster per sampling sequence carries out; the attention is one CTA per SM.  Where the walk's clusters
+    // leave half of the SMs free and the attention is long, the scan goes first on all SMs and the walk and the attention, sized
+    // for the SMs the walk leaves, follow it in the same stream as programmatic dependents: the attention's CTAs come when every
+    // CTA of the walk has its SM.  (On a second stream behind an event the attention was there 3 to 5 us later, or now and then
+    // ahead of a cluster, which then had no 16 SMs side by side before the attention had left: 80 us in place of 38 on 52 heads.
+    // One B200, us a step, two streams against one: 50.7 and 38.1 on 52 heads and 4 K keys, 44.2 and 42.4 on 8 x 8 and 8 K,
+    // both 17 chunks a CTA.)  The merge of the key ranges then comes when the walk is complete, too, which costs its 2.5 us
+    // where the attention would have been through before: 36.5 against 38.9 on 2 chunks a CTA.  An attention of 12 chunks (19 us)
+    // is as long as the shorter walks; with one range there is no merge.
+    // Otherwise, and with more clusters, the attention is forked behind the scan onto the second stream.
     const fspad_config &c = ctx->cfg;
     const int sms = ctx->sm_count;
     const long long attn_ctas = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch) *
                                 fspad_attn_umma_splits(ctx, n_nodes, batch);
-    StepPlan p = {may_sample && sms - attn_ctas < sms / 4, 0};
-    if (p.scan_first) {
+    StepPlan p = {false, false, 0};
+    if (may_sample) {
         const int walk = fspad_walk_ctas(ctx, batch, c.vocab);
-        p.attn_sms = sms - (walk < sms / 2 ? walk : sms / 2);
-    } else if (!may_sample && attn_ctas > sms / 2) {
+        const int beside = sms - (walk < sms / 2 ? walk : sms / 2), ranges = fspad_attn_umma_splits(ctx, n_nodes, batch, beside);
+        p.chain = walk <= sms / 2 && (ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges);
+        p.scan_first = !p.chain && sms - attn_ctas < sms / 4;
+        if (p.chain || p.scan_first) p.attn_sms = beside;
+    } else if (attn_ctas > sms / 2) {
         // An all-greedy acceptance is a scan and a one-CTA walk: beside an attention that holds most SMs the
         // scan's CTAs only get going when the attention's leave.  Where the context is short enough for the
         // attention to stay short on half the SMs (at most 8 chunks per CTA by the context's max_len), it
-        // gets half and the two really run side by side (17.2 against 20.5 us on the 26-node greedy workload).
+        // gets half and the two really run side by side (17.2 against 20.5 us on the 26-node greedy workload); and where the scan
+        // is short, too (8 MB: 1.3 us of HBM, 3.6 us in all), it goes first on all SMs and the attention follows in the same
+        // stream: four launches without an event between them, 17.2 -> 15.0 us on that workload.
         const int s_half = fspad_attn_umma_splits(ctx, n_nodes, batch, sms / 2);
         const int max_chunks = (c.max_len + 127) / 128;
-        if ((max_chunks + s_half - 1) / s_half <= 8) p.attn_sms = sms / 2;
+        const bool short_attn = (max_chunks + s_half - 1) / s_half <= 8;
+        p.chain = short_attn && (long long)batch * n_nodes * c.vocab <= 2 << 20;
+        if (short_attn && !p.chain) p.attn_sms = sms / 2;
     }
     return p;
 }
@@ -492,6 +506,27 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
     cudaError_t ce = cudaSuccess;
     FspadStatsGeom geom;
     const int rows = batch * n_nodes;
+    // With the tree rows given apart from the cache the compaction depends on the walk alone, and when the
+    // sequence's slices are few (one warp each among the 16 x 16 warps of a sampling walk's cluster, four each for the 16
+    // warps of a greedy one) the walk makes the moves itself at its end: one dependent launch less on the step's
+    // longest chain (all-greedy step of 26 nodes and 64 slices: 29.3 -> 23.7 us called one by one, 13.1 against 13.3 from a graph).
+    const bool aliased = tree_k == nullptr;      // attention reads the cache rows that compaction rewrites
+    const bool walk_compacts = !aliased && c.n_layers * 2 * c.n_kv_heads <= (plan.chain && may_sample ? 256 : 64);
+    FspadWalkCompact kv;
+    if (walk_compacts) { kv.cache = cache; kv.prefix_len = prefix_len; kv.new_len = new_len; }
+    if (plan.chain) {
+        // Every kernel's end waits for its predecessor's: what follows this call finds all of it complete.
+        ce = fspad_launch_stats_partials(ctx, target_logits, temperature, rows, n_nodes, c.vocab, &geom, st);
+        if (ce == cudaSuccess)
+            ce = fspad_launch_accept_walk(ctx, target_logits, draft_probs, draft_tokens, parent, temperature, uniforms, geom,
+                                          n_nodes, batch, c.vocab, accepted_path, n_accepted, bonus_token, st, kv);
+        if (ce == cudaSuccess)
+            ce = fspad_launch_tree_attn(ctx, q, kc, vc, tree_k, tree_v, parent, prefix_len, n_nodes, batch, attn_out, st, attn_sms,
+                                        FspadPaged{nullptr, 0, 0, true});
+        if (ce == cudaSuccess && !walk_compacts)
+            ce = fspad_launch_kv_compact(ctx, cache, accepted_path, n_accepted, prefix_len, batch, new_len, st);
+        return ce == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;
+    }
     if (scan_first)
         ce = fspad_launch_stats_partials(ctx, target_logits, temperature, rows, n_nodes, c.vocab, &geom, st);
     // fork: the attention of this step on the context's second stream
@@ -521,14 +556,6 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
         }
         ce = fspad_launch_stats_partials(ctx, target_logits, temperature, rows, n_nodes, c.vocab, &geom, st, false, scan_sms);
     }
-    // With the tree rows given apart from the cache the compaction depends on the walk alone, and when the
-    // sequence's slices are few (one warp each among the 16 x 16 warps of a sampling walk's cluster, four each for the 16
-    // warps of a greedy one) the walk makes the moves itself at its end: one dependent launch less on the step's
-    // longest chain (all-greedy step of 26 nodes and 64 slices: 29.3 -> 23.7 us called one by one, 13.1 against 13.3 from a graph).
-    const bool aliased = tree_k == nullptr;      // attention reads the cache rows that compaction rewrites
-    const bool walk_compacts = !aliased && c.n_layers * 2 * c.n_kv_heads <= 64;
-    FspadWalkCompact kv;
-    if (walk_compacts) { kv.cache = cache; kv.prefix_len = prefix_len; kv.new_len = new_len; }
     if (ce == cudaSuccess)
         ce = fspad_launch_accept_walk(ctx, target_logits, draft_probs, draft_tokens, parent, temperature, uniforms, geom,
                                       n_nodes, batch, c.vocab, accepted_path, n_accepted, bonus_token, st, kv);

@@ -226,7 +226,8 @@ __device__ __forceinline__ void fspad_stats_merge_warp(const FspadStatsPart *__r
 // The acceptance walk is the exception: it reads the caller's arrays (trees, logits, draft rows) before its wait.  It may,
 // because the two kernels that can precede it, the vocabulary scan and the LM head's merge, let it start only after their own
 // wait, when everything queued before them is complete, and themselves write nothing but scan partials, which the walk reads
-// after its wait.  Kernels whose predecessor is not one kernel of the same stream (behind a fork, a join or a copy) may be
+// after its wait.  The attention of a step called as one is the other: launched behind the walk, it starts when every CTA of the
+// walk has, reads what was complete before the scan started, and waits for the walk at its end.  Kernels whose predecessor is not one kernel of the same stream (behind a fork, a join or a copy) may be
 // launched without the attribute.
 #ifdef __CUDACC__
 __device__ __forceinline__ void fspad_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -308,9 +309,12 @@ cudaError_t fspad_launch_kv_compact(fspad_ctx *ctx, fspad_bf16 *cache, const int
                                     cudaStream_t st, bool pdl = true);
 // A cache kept as a pool of 128-row blocks: table[b * stride + i] is the block with rows 128 i .. 128 i + 127
 // of sequence b (table == NULL: contiguous cache).
+// early: the attention is launched beside the kernel before it in the stream, which has only been started when all that
+// precedes the two of them, and so every input of the attention, is complete; the attention's end waits for that kernel's.
 struct FspadPaged {
     const int *table;
     int stride, n_blocks;
+    bool early = false;
 };
 // sms: how many SMs the call may fill with CTAs (0 = all of them).  merge_pdl: the merge kernel is a programmatic
 // dependent of the attention kernel (its CTAs become resident, waiting, as the attention's last CTAs finish).

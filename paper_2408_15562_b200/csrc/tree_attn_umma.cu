@@ -875,11 +875,11 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     }
     a.use_tma = ctx->attn_tmap_ok ? 1 : 0;
     const bool pair = a.use_tma && fspad_attn_pairs(ctx, N, B, sms);      // (without maps the tiles go to lone CTAs, one of them perhaps empty)
-    a.early = 0;
+    a.early = paged.early ? 1 : 0;
     CUtensorMap mq = {};
     a.q_tma = make_q_map(&mq, q, (size_t)B * N, c.n_q_heads, a.G) ? 1 : 0;
     const dim3 grid = pair ? dim3(c.n_kv_heads * a.mtiles, n_splits, B) : dim3(n_splits, c.n_kv_heads * a.mtiles, B);
     ctx->launches++;
     auto kernel = pair ? umma::tree_attn_umma_kernel<true> : umma::tree_attn_umma_kernel<false>;
-    return fspad_launch_opt(false, kernel, grid, dim3(umma::NT), umma::smem_bytes(pair), st, pair ? 2u : 0u, a, mq, pair ? *mk_half : *mk, *mv);
+    return fspad_launch_opt(paged.early, kernel, grid, dim3(umma::NT), umma::smem_bytes(pair), st, pair ? 2u : 0u, a, mq, pair ? *mk_half : *mk, *mv);
 }

@@ -102,6 +102,41 @@ def test_whole_step_headline_shape_in_a_graph():
     _check(inp, outs, cache, ref_o, r, want, want_len)
 
 
+@pytest.mark.parametrize("mode,heads,prefix,n_layers,aliased", [
+    ("sample", 80, 300, 1, False),      # one key range a row; the walk's CTAs compact 160 slices
+    ("sample", 80, 300, 2, False),      # 320 slices: the compaction kernel, behind the attention
+    ("sample", 80, 300, 1, True),       # the compaction rewrites rows that the attention reads
+    ("sample", 70, 3000, 1, False),     # two ranges of 12 chunks: the merge kernel follows
+    ("greedy", 80, 300, 1, False),      # short scan, one-CTA walk
+])
+def test_step_in_one_stream(mode, heads, prefix, n_layers, aliased):
+    """The attention launched beside the walk in the caller's stream: eager, and replayed twice back to back from a graph."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=1, n_q_heads=heads, n_kv_heads=heads, prefix=(prefix, prefix), n_nodes=24,
+                     depth=4, branch=4, vocab=3000, temperatures=(1.0 if mode == "sample" else 0.0,))
+    inp = synth.generate(w, 12)
+    N, L = inp.parent.shape[1], int(inp.prefix_len[0])
+    cache_host = synth.make_cache(inp, n_layers)
+    cache_host[0, 0, 0], cache_host[0, 1, 0] = inp.k_cache[0], inp.v_cache[0]
+    cache_host[0, 0, 0, :, L:L + N], cache_host[0, 1, 0, :, L:L + N] = inp.tree_k[0], inp.tree_v[0]
+    ref = _oracle_step(inp, cache_host, 0)
+    ctx = helpers.make_ctx(inp, n_layers=n_layers)
+    d, a, outs, cache = _device_inputs(inp, cache_host)
+    _call(ctx, cache, a, d, outs, aliased, 0)
+    ctx.check()
+    _check(inp, outs, cache, *ref)
+    again = binding.bf16_tensor(cache_host)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(2):
+            cache.copy_(again)
+            _call(ctx, cache, a, d, outs, aliased, 0)
+    outs["attn_out"].zero_()
+    outs["path"].fill_(-7)
+    g.replay()
+    ctx.check()
+    _check(inp, outs, cache, *ref)
+
+
 def test_argument_errors():
     w = synth.scaled(W["llama3_8b_2k"], batch=1, prefix=(40, 40), n_nodes=8, depth=3, branch=3, vocab=100,
                      temperatures=(0.0,))
