@@ -1,4 +1,4 @@
-"""Thin ctypes binding of libfspad.so: argument marshalling only.
+"""Thin binding of libfspad.so: argument marshalling only.
 
 Every function takes torch tensors (device memory, streams), checks dtype,
 shape and contiguity, and forwards raw pointers to the C ABI declared in
@@ -15,7 +15,9 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libfspad.so")
+CALLS_PATH = os.path.join(_PKG, "_pycall.so")
 _lib = None
+_native = None
 
 EXPORTS = ["fspad_create", "fspad_destroy", "fspad_status", "fspad_strerror", "fspad_launch_count",
            "fspad_tree_attn", "fspad_tree_accept", "fspad_accept_stats", "fspad_kv_compact",
@@ -74,13 +76,24 @@ def load():
     return lib
 
 
+def _calls():
+    """The calls a decoding loop makes, with their arguments taken from the tensors by native code."""
+    global _native
+    if _native is None:
+        load()
+        if not os.path.exists(CALLS_PATH):
+            raise RuntimeError("_pycall.so is missing: build it with `python -m paper_2408_15562_b200.build`")
+        from . import _pycall
+        _native = _pycall
+    return _native
+
+
 def strerror(code: int) -> str:
     return load().fspad_strerror(code).decode()
 
 
-# A step hands over some twenty tensors: identity of the dtype, the `is_cuda` flag and a plain integer address instead of a
-# comparison, a device object and a ctypes object each, and the stream without building a Stream object
-# (60-node sampling step: 35 -> 26 us of host time, six calls of a draft phase 97 -> 49).
+# The calls outside a decoding loop go through ctypes; those inside it through `_pycall` (csrc/pycall.cpp), which makes the same
+# checks.
 def _ptr(t: Optional[torch.Tensor], dtype, device_type: str = "cuda"):
     if t is None:
         return None
@@ -145,9 +158,8 @@ class Context:
         if out is None:
             out = torch.empty_like(q)
         bf = torch.bfloat16
-        rc = load().fspad_tree_attn(self._h, _ptr(q, bf), _ptr(k_cache, bf), _ptr(v_cache, bf),
-                                    _ptr(tree_k, bf), _ptr(tree_v, bf), _ptr(parent, torch.int32),
-                                    _ptr(prefix_len, torch.int32), N, B, _ptr(out, bf), _stream(stream))
+        rc = _calls().tree_attn(self._h.value, q, k_cache, v_cache, tree_k, tree_v, parent, prefix_len, N, B, out,
+                                _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_tree_attn")
         return out
@@ -163,10 +175,8 @@ class Context:
         if bonus_token is None:
             bonus_token = torch.empty((B,), dtype=torch.int32, device=dev)
         f32, i32 = torch.float32, torch.int32
-        rc = load().fspad_tree_accept(self._h, _ptr(target_logits, f32), _ptr(draft_probs, f32),
-                                      _ptr(draft_tokens, i32), _ptr(parent, i32), _ptr(temperature, f32),
-                                      _ptr(uniforms, f32), N, B, _ptr(accepted_path, i32),
-                                      _ptr(n_accepted, i32), _ptr(bonus_token, i32), _stream(stream))
+        rc = _calls().tree_accept(self._h.value, target_logits, draft_probs, draft_tokens, parent, temperature,
+                                  uniforms, N, B, accepted_path, n_accepted, bonus_token, _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_tree_accept")
         return accepted_path, n_accepted, bonus_token
@@ -195,9 +205,8 @@ class Context:
         if out is None:
             out = torch.empty_like(q)
         bf, i32 = torch.bfloat16, torch.int32
-        rc = load().fspad_tree_attn_paged(self._h, _ptr(q, bf), _ptr(k_pool, bf), _ptr(v_pool, bf), _ptr(block_table, i32),
-                                          block_table.shape[1], k_pool.shape[0], _ptr(tree_k, bf), _ptr(tree_v, bf),
-                                          _ptr(parent, i32), _ptr(prefix_len, i32), N, B, _ptr(out, bf), _stream(stream))
+        rc = _calls().tree_attn_paged(self._h.value, q, k_pool, v_pool, block_table, block_table.shape[1],
+                                      k_pool.shape[0], tree_k, tree_v, parent, prefix_len, N, B, out, _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_tree_attn_paged")
         return out
@@ -208,9 +217,8 @@ class Context:
         i32 = torch.int32
         if new_len is None:
             new_len = torch.empty((B,), dtype=i32, device=pool.device)
-        rc = load().fspad_kv_compact_paged(self._h, _ptr(pool, torch.bfloat16), _ptr(block_table, i32), block_table.shape[1],
-                                           pool.shape[2], _ptr(accepted_path, i32), _ptr(n_accepted, i32), _ptr(prefix_len, i32),
-                                           B, _ptr(new_len, i32), _stream(stream))
+        rc = _calls().kv_compact_paged(self._h.value, pool, block_table, block_table.shape[1], pool.shape[2],
+                                       accepted_path, n_accepted, prefix_len, B, new_len, _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_kv_compact_paged")
         return new_len
@@ -244,10 +252,9 @@ class Context:
             n_accepted = torch.empty((B,), dtype=i32, device=dev)
         if bonus_token is None:
             bonus_token = torch.empty((B,), dtype=i32, device=dev)
-        rc = load().fspad_lm_head_accept(self._h, _ptr(hidden, bf), _ptr(lm_head, bf), H, _ptr(draft_probs, f32),
-                                         _ptr(draft_tokens, i32), _ptr(parent, i32), _ptr(temperature, f32),
-                                         _ptr(uniforms, f32), N, B, _ptr(logits, f32), _ptr(accepted_path, i32),
-                                         _ptr(n_accepted, i32), _ptr(bonus_token, i32), _stream(stream))
+        rc = _calls().lm_head_accept(self._h.value, hidden, lm_head, H, draft_probs, draft_tokens, parent,
+                                     temperature, uniforms, N, B, logits, accepted_path, n_accepted, bonus_token,
+                                     _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_lm_head_accept")
         return accepted_path, n_accepted, bonus_token
@@ -264,9 +271,8 @@ class Context:
         need = load().fspad_feature_sampler_workspace_bytes(rows, H, I)
         if workspace is None:
             workspace = torch.empty((need,), dtype=torch.uint8, device=f.device)
-        rc = load().fspad_feature_sampler(self._h, _ptr(f, bf), _ptr(e, bf), _ptr(w_up, bf), _ptr(w_gate, bf), _ptr(w_down, bf),
-                                          rows, H, I, _ptr(inter, bf), _ptr(eta, bf), _ptr(workspace, torch.uint8),
-                                          workspace.numel(), _stream(stream))
+        rc = _calls().feature_sampler(self._h.value, f, e, w_up, w_gate, w_down, rows, H, I, inter, eta, workspace,
+                                      workspace.numel(), _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_feature_sampler")
         return eta, inter
@@ -277,9 +283,8 @@ class Context:
         i32 = torch.int32
         if new_len is None:
             new_len = torch.empty((B,), dtype=i32, device=cache.device)
-        rc = load().fspad_kv_append(self._h, _ptr(cache, torch.bfloat16), _ptr(tree_kv, torch.bfloat16), _ptr(accepted_path, i32),
-                                    _ptr(n_accepted, i32), _ptr(prefix_len, i32), tree_kv.shape[4], B, _ptr(new_len, i32),
-                                    _stream(stream))
+        rc = _calls().kv_append(self._h.value, cache, tree_kv, accepted_path, n_accepted, prefix_len,
+                                tree_kv.shape[4], B, new_len, _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_kv_append")
         return new_len
@@ -289,9 +294,8 @@ class Context:
         if new_len is None:
             new_len = torch.empty((B,), dtype=torch.int32, device=cache.device)
         i32 = torch.int32
-        rc = load().fspad_kv_compact(self._h, _ptr(cache, torch.bfloat16), _ptr(accepted_path, i32),
-                                     _ptr(n_accepted, i32), _ptr(prefix_len, i32), B, _ptr(new_len, i32),
-                                     _stream(stream))
+        rc = _calls().kv_compact(self._h.value, cache, accepted_path, n_accepted, prefix_len, B, new_len,
+                                 _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_kv_compact")
         return new_len
@@ -306,11 +310,8 @@ class Context:
             out = tuple(torch.empty((B, n_nodes), dtype=i32, device=dev) for _ in range(3)) + \
                 (torch.empty((B,), dtype=i32, device=dev),)
         parent, token, cand, n_out = out
-        rc = load().fspad_tree_build(self._h, _ptr(cand_parent, i32), _ptr(cand_token, i32),
-                                     _ptr(cand_logp, torch.float32), _ptr(root_token, i32), C, n_nodes, B,
-                                     _ptr(parent, i32), _ptr(token, i32), _ptr(cand, i32),
-                                     _ptr(anc, torch.int64) if anc is not None else None, _ptr(n_out, i32),
-                                     _stream(stream))
+        rc = _calls().tree_build(self._h.value, cand_parent, cand_token, cand_logp, root_token, C, n_nodes, B, parent,
+                                 token, cand, anc, n_out, _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_tree_build")
         return parent, token, cand, n_out
@@ -326,10 +327,9 @@ class Context:
             next_cand = torch.empty((B, width), dtype=i32, device=logprobs.device)
         if next_logp is None:
             next_logp = torch.empty((B, width), dtype=f32, device=logprobs.device)
-        rc = load().fspad_draft_expand(self._h, _ptr(logprobs, f32), _ptr(frontier_logp, f32), _ptr(frontier_cand, i32),
-                                       F, top_k, width, base, cand_parent.shape[1], B, _ptr(cand_parent, i32),
-                                       _ptr(cand_token, i32), _ptr(cand_logp, f32), _ptr(next_cand, i32),
-                                       _ptr(next_logp, f32), _stream(stream))
+        rc = _calls().draft_expand(self._h.value, logprobs, frontier_logp, frontier_cand, F, top_k, width, base,
+                                   cand_parent.shape[1], B, cand_parent, cand_token, cand_logp, next_cand, next_logp,
+                                   _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_draft_expand")
         return next_cand, next_logp
@@ -341,11 +341,9 @@ class Context:
         acceptance, then compaction; outputs are written in place."""
         B, N = q.shape[0], q.shape[1]
         bf, f32, i32 = torch.bfloat16, torch.float32, torch.int32
-        rc = load().fspad_verify_step(
-            self._h, _ptr(cache, bf), attn_layer, _ptr(q, bf), _ptr(tree_k, bf), _ptr(tree_v, bf), _ptr(parent, i32),
-            _ptr(prefix_len, i32), _ptr(target_logits, f32), _ptr(draft_probs, f32), _ptr(draft_tokens, i32),
-            _ptr(temperature, f32), _ptr(uniforms, f32), N, B, _ptr(attn_out, bf), _ptr(accepted_path, i32),
-            _ptr(n_accepted, i32), _ptr(bonus_token, i32), _ptr(new_len, i32), _stream(stream))
+        rc = _calls().verify_step(self._h.value, cache, attn_layer, q, tree_k, tree_v, parent, prefix_len,
+                                  target_logits, draft_probs, draft_tokens, temperature, uniforms, N, B, attn_out,
+                                  accepted_path, n_accepted, bonus_token, new_len, _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_verify_step")
         return attn_out, accepted_path, n_accepted, bonus_token, new_len
@@ -355,14 +353,9 @@ class Context:
                          bonus_token, new_len, stream=None):
         """All tensors except `cache` are HOST tensors (pinned recommended); outputs are written in place."""
         B, N = q.shape[0], q.shape[1]
-        bf, f32, i32 = torch.bfloat16, torch.float32, torch.int32
-        h = "cpu"
-        rc = load().fspad_verify_step_host(
-            self._h, _ptr(cache, bf), _ptr(q, bf, h), _ptr(tree_k, bf, h), _ptr(tree_v, bf, h),
-            _ptr(parent, i32, h), _ptr(prefix_len, i32, h), _ptr(target_logits, f32, h),
-            _ptr(draft_probs, f32, h), _ptr(draft_tokens, i32, h), _ptr(temperature, f32, h),
-            _ptr(uniforms, f32, h), N, B, _ptr(attn_out, bf, h), _ptr(accepted_path, i32, h),
-            _ptr(n_accepted, i32, h), _ptr(bonus_token, i32, h), _ptr(new_len, i32, h), _stream(stream))
+        rc = _calls().verify_step_host(self._h.value, cache, q, tree_k, tree_v, parent, prefix_len, target_logits,
+                                       draft_probs, draft_tokens, temperature, uniforms, N, B, attn_out,
+                                       accepted_path, n_accepted, bonus_token, new_len, _stream(stream))
         if rc != 0:
             raise FspadError(rc, "fspad_verify_step_host")
         return attn_out, accepted_path, n_accepted, bonus_token, new_len

@@ -4,11 +4,15 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libfspad.so")
+HEADER = os.path.join(ROOT, "include", "fspad.h")
+CALLS = os.path.join(PKG, "_pycall.so")
+CALLS_SRC = os.path.join(CSRC, "pycall.cpp")
 SOURCES = ["api.cu", "accept_stats.cu", "accept_walk.cu", "kv_compact.cu", "tree_attn.cu", "tree_attn_umma.cu", "tree_build.cu", "draft_expand.cu", "lm_head.cu", "feature_sampler.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
@@ -22,13 +26,34 @@ def _nvcc() -> str:
 
 
 def _newest_source() -> float:
-    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "fspad.h")]
+    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != os.path.basename(CALLS_SRC)] + [HEADER]
     return max(os.path.getmtime(f) for f in files)
 
 
+def _build_calls(force: bool) -> None:
+    """The Python calls of the C ABI (g++ against torch's headers), linked with the library beside it."""
+    if not force and os.path.exists(CALLS) and os.path.getmtime(CALLS) >= max(os.path.getmtime(CALLS_SRC), os.path.getmtime(HEADER)):
+        return
+    import torch
+    t = os.path.join(os.path.dirname(torch.__file__))
+    tmp = CALLS + ".tmp.%d" % os.getpid()
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I" + os.path.dirname(HEADER),
+                           "-I" + os.path.join(t, "include"), "-I" + os.path.join(t, "include", "torch", "csrc", "api", "include"),
+                           "-I" + sysconfig.get_paths()["include"], "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+                           CALLS_SRC, "-o", tmp, "-L" + PKG, "-l:" + os.path.basename(LIB), "-L" + os.path.join(t, "lib"),
+                           "-ltorch_python", "-ltorch_cpu", "-lc10", "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + os.path.join(t, "lib")])
+    os.replace(tmp, CALLS)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    _build_library(force, verbose)
+    _build_calls(force)
+    return LIB
+
+
+def _build_library(force: bool, verbose: bool) -> None:
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source():
-        return LIB
+        return
     objdir = os.path.join(PKG, "_build")
     os.makedirs(objdir, exist_ok=True)
     procs = []
@@ -50,7 +75,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + ".tmp.%d" % os.getpid()
     subprocess.check_call([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp] + objs)
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":
