@@ -15,8 +15,9 @@
 //
 // What bounds it: HBM with many rows, otherwise a chain of latencies.  As three kernels (one CTA per 4096 tokens, then a
 // 1024-entry sorting network per row, then one per sequence) a level of ten rows took 15 us at V = 32000 and 40 us with
-// 16 sequences at V = 128256 (82 MB); now 8.5 and 23.  Pieces are as long as one wave of four CTAs per SM allows (a short piece
-// pays the ranking for few tokens), and at most 16 per row, so that the lists merged for a row stay short.
+// 16 sequences at V = 128256 (82 MB); now 8.1 and 23.  Pieces are at most 16 per row, so that the lists merged for a row stay short.
+// (Prefetching rounds further ahead into L2 or asking for the second round before the bound is known made it slower: it is not HBM's
+// latency that the rounds wait for.)
 #include "common.cuh"
 #include "sort_key.cuh"
 
@@ -31,7 +32,7 @@ constexpr int kMaxPieces = 16;
 struct DraftArgs {
     const float *logprobs, *frontier_logp;
     const int *frontier_cand;
-    int V, F, k, width, base, cap, pieces, len;        // len: tokens of a piece (a multiple of kRound / 4)
+    int V, F, k, width, base, cap, pieces, len;        // len: tokens of a piece (a multiple of 32)
     uint2 *part;                                       // [rows][pieces][k] (value, token)
     int *seq_done;                                     // pieces of a sequence's rows that have finished
     int *cand_parent, *cand_token;
@@ -85,7 +86,10 @@ __device__ __forceinline__ int rank_of(const unsigned long long *list, int n, un
     return rank;
 }
 
-__global__ void __launch_bounds__(kThreads, 4)
+// PER_SM: CTAs an SM holds.  Four leave a thread 32 registers, which is a few too few; with three a level's chain is shorter (ten rows:
+// 8.9 -> 8.1 us at 32000 tokens, 12.7 -> 11.1 at 151936).
+template <int PER_SM>
+__global__ void __launch_bounds__(kThreads, PER_SM)
 draft_expand_kernel(const DraftArgs a)
 {
     __shared__ DraftShared s;
@@ -195,9 +199,9 @@ draft_expand_kernel(const DraftArgs a)
     }
     // ---- the last piece of the sequence ----
     const int b = row / a.F;
-    __threadfence();
     __syncthreads();
     if (tid == 0) {
+        __threadfence();                             // (behind the barrier it stands for the whole CTA's lists)
         s.last = atomicAdd(a.seq_done + b, 1) == a.F * a.pieces - 1;
         if (s.last) a.seq_done[b] = 0;
         __threadfence();
@@ -302,12 +306,26 @@ cudaError_t fspad_launch_draft_expand(fspad_ctx *ctx, const float *logprobs, con
     DraftArgs a;
     a.V = ctx->cfg.vocab;
     const int rows = B * F;
-    int pieces = (int)((long long)ctx->sm_count * 4 / rows);         // one wave of four CTAs per SM
-    const int most = fspad_draft_expand_pieces(a.V);                 // about a round of 4096 tokens at least (and what `part` is sized for)
-    if (pieces > most) pieces = most;
-    if (pieces > kMaxPieces) pieces = kMaxPieces;
-    if (pieces < 1) pieces = 1;
-    const int quantum = kRound / 4;
+    // One wave of CTAs at most.  Pieces of two rounds, or of one where the rows are too few to give every SM a CTA (a piece's ranking
+    // and hand-over cost what two rounds do: four sequences of ten rows at 50257 tokens 16.3 -> 10 us a level); where a CTA per SM
+    // leaves a row eight pieces or more, no more than that, because the SMs with two would set the pace.
+    const int sms = ctx->sm_count;
+    const int most = fspad_draft_expand_pieces(a.V);                 // a round of 4096 tokens (and what `part` is sized for)
+    const int fill = sms / rows < most ? sms / rows : most, two = (most + 1) / 2;
+    auto pieces_of = [&](int per_sm) {
+        int n = (int)((long long)sms * per_sm / rows);
+        const int want = two > fill ? two : fill;
+        if (n > want) n = want;
+        if (n > kMaxPieces) n = kMaxPieces;
+        if ((long long)rows * n > sms && sms / rows >= 8) n = sms / rows;
+        return n < 1 ? 1 : n;
+    };
+    // Three CTAs per SM, or four where whole pieces would leave three's wave a fifth empty and four's does not: 160 rows of 128256
+    // tokens are 320 CTAs (72 %) against 480, 26 against 23 us a level; 80 rows 400 (90 %) against 560, 15.4 against 16.0.
+    const int three = pieces_of(3), four = pieces_of(4);
+    const bool use_four = four > three && (long long)rows * three * 5 < 4ll * 3 * sms;
+    const int pieces = use_four ? four : three;
+    const int quantum = 32;                                          // a line; pieces of equal length, or the last one sets a bound of its own from few tokens
     a.len = (((a.V + 3 + pieces - 1) / pieces) + quantum - 1) / quantum * quantum;    // (up to three empty positions in front)
     a.pieces = (a.V + 3 + a.len - 1) / a.len;
     a.logprobs = logprobs; a.frontier_logp = frontier_logp; a.frontier_cand = frontier_cand;
@@ -317,5 +335,5 @@ cudaError_t fspad_launch_draft_expand(fspad_ctx *ctx, const float *logprobs, con
     a.cand_parent = cand_parent; a.cand_token = cand_token; a.cand_logp = cand_logp;
     a.next_cand = next_cand; a.next_logp = next_logp;
     ctx->launches++;
-    return fspad_launch_opt(!aside, draft_expand_kernel, dim3(a.pieces, rows), dim3(kThreads), 0, st, 0, a);
+    return fspad_launch_opt(!aside, use_four ? draft_expand_kernel<4> : draft_expand_kernel<3>, dim3(a.pieces, rows), dim3(kThreads), 0, st, 0, a);
 }

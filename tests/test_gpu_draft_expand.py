@@ -144,3 +144,20 @@ def test_next_frontier_over_the_current_one(batch, F, k, width, shift):
         for g, r in zip(got, ref):
             assert np.array_equal(g.cpu().numpy(), r)
         assert np.array_equal(nxt[0].cpu().numpy(), nc_ref) and np.array_equal(nxt[1].cpu().numpy(), nl_ref)
+
+
+@pytest.mark.parametrize("vocab,batch,F", [
+    (151937, 1, 10),       # 14 pieces: one CTA per SM
+    (36865, 1, 14),        # ten pieces, the last one shorter
+    (50257, 4, 10),        # seven pieces of two rounds
+    (20003, 16, 10),       # three pieces, four CTAs per SM
+    (20003, 16, 16),       # two pieces, four CTAs per SM
+    (32003, 16, 16),       # the same with longer ones
+])
+def test_pieces_by_rows_and_vocabulary(vocab, batch, F):
+    ctx = binding.Context(8, 2, vocab, 256, max_nodes=64, max_batch=batch)
+    rng = np.random.default_rng(vocab + batch)
+    lp = np.round(rng.standard_normal((batch, F, vocab), dtype=np.float32) * 3, 2)      # with ties
+    flp = rng.standard_normal((batch, F)).astype(np.float32)
+    fc = rng.integers(0, 5, (batch, F)).astype(np.int32)
+    _check(ctx, lp, flp, fc, 10, 10, 7, 7 + F * 10)
