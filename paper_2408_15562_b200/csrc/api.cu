@@ -89,18 +89,20 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample)
         p.chain = walk <= sms / 2 && (ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges);
         p.scan_first = !p.chain && sms - attn_ctas < sms / 4;
         if (p.chain || p.scan_first) p.attn_sms = beside;
-    } else if (attn_ctas > sms / 2) {
+    } else {
         // An all-greedy acceptance is a scan and a one-CTA walk: beside an attention that holds most SMs the
         // scan's CTAs only get going when the attention's leave.  Where the context is short enough for the
         // attention to stay short on half the SMs (at most 8 chunks per CTA by the context's max_len), it
         // gets half and the two really run side by side (17.2 against 20.5 us on the 26-node greedy workload); and where the scan
         // is short, too (8 MB: 1.3 us of HBM, 3.6 us in all), it goes first on all SMs and the attention follows in the same
-        // stream: four launches without an event between them, 17.2 -> 15.0 us on that workload.
+        // stream: four launches without an event between them, 17.2 -> 15.0 us on that workload.  With one key range (no merge) that
+        // holds for an attention of few CTAs, too: 8 KV heads called one by one 18.7 -> 12.3 us, from a graph 11.8 -> 12.3; with
+        // more ranges the graph loses more (8 chunks: 18.3 -> 14.5 and 12.5 -> 14.2) and the two streams stay.
         const int s_half = fspad_attn_umma_splits(ctx, n_nodes, batch, sms / 2);
         const int max_chunks = (c.max_len + 127) / 128;
         const bool short_attn = (max_chunks + s_half - 1) / s_half <= 8;
-        p.chain = short_attn && (long long)batch * n_nodes * c.vocab <= 2 << 20;
-        if (short_attn && !p.chain) p.attn_sms = sms / 2;
+        p.chain = short_attn && (attn_ctas > sms / 2 || fspad_attn_umma_splits(ctx, n_nodes, batch) == 1) && (long long)batch * n_nodes * c.vocab <= 2 << 20;
+        if (short_attn && !p.chain && attn_ctas > sms / 2) p.attn_sms = sms / 2;
     }
     return p;
 }

@@ -745,13 +745,17 @@ cudaError_t fspad_launch_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t s
                             (uint32_t)polls);
 }
 
-// Key ranges per row: one CTA per SM, never a partial second wave.
+// Key ranges per row: one CTA per SM, never a partial second wave; and one where the context is so short that walking all of its
+// chunks takes no longer than the merge of the ranges (2.5 us and a launch, a chunk 1.05).  A greedy step of 26 nodes and 32 heads, us with
+// ranges and without: 3 chunks 14.4 and 12.8, 4 chunks 14.3 and 12.6, 5 chunks 14.6 and 14.1, 6 chunks 15.5 and 15.2, 8 chunks 15.6 and 17.0.
+constexpr int kOneRange = 5;
 static int ranges_per_row(const fspad_ctx *ctx, int B, int mtiles, int sms)
 {
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
     const long long base = (long long)B * ctx->cfg.n_kv_heads * mtiles;
     long long s = sms / base;
     const int max_chunks = (ctx->cfg.max_len + umma::BK - 1) / umma::BK;
+    if (max_chunks <= kOneRange) return 1;
     if (s > max_chunks) s = max_chunks;
     if (s > 64) s = 64;
     if (s < 1) s = 1;
