@@ -550,9 +550,10 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
             // only has to bound the scores loosely: it follows the row maximum when some row of the warp
             // would otherwise see a P above 2^kLazyLog2, and stays put - no pass over O - when not.
             // (The decision is taken per warp because the tensor-memory accesses are warp-collective;
-            // a comparison with -inf - -inf = NaN is false and so counts as a move.)
+            // a comparison with -inf - -inf = NaN is false and so counts as a move.  Lanes whose row does not exist have no say: by
+            // TMA they hold the next sequence's queries, and what that one asks must not decide how this one's P is rounded.)
             const float m_cand = fmaxf(m_run, mx * scale);
-            const bool move = !__all_sync(0xffffffffu, m_cand - m_run <= kLazyLog2);
+            const bool move = !__all_sync(0xffffffffu, !row_ok || m_cand - m_run <= kLazyLog2);
             const float m_new = move ? m_cand : m_run;
             const float m_safe = (m_new == -INFINITY) ? 0.f : m_new;
             const float alpha = move ? ex2f(m_run - m_safe) : 1.f;

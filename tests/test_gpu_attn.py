@@ -198,3 +198,32 @@ def test_rows_behind_the_tree_may_hold_anything(hq, hkv, prefix, n):
         for plane in (inp.k_cache, inp.v_cache):
             plane[:, :, prefix + (n if alias else 0):] = 0x7FC0
         _check(inp, alias_cache=alias)
+
+
+@pytest.mark.parametrize("hq,hkv,n,batch,prefix", [
+    (32, 8, 60, 2, 300),       # lone CTAs: 240 rows, half of a warp's rows do not exist
+    (32, 8, 60, 2, 768),       # a chunk of tree rows alone
+    (16, 2, 33, 3, 700),       # 264 rows
+    (8, 8, 19, 2, 200),        # one head a group: 19 rows
+    (24, 8, 33, 2, 300),       # Q gathered
+    (32, 8, 60, 12, 300),      # pairs of CTAs
+])
+def test_a_sequence_does_not_depend_on_its_neighbours_queries(hq, hkv, n, batch, prefix):
+    """Rows of a tile past a sequence's last node hold the next sequence's queries: whatever these are, the sequence's own
+    output stays the same bit for bit."""
+    w = synth.scaled(W["batch16_ragged"], batch=batch, n_q_heads=hq, n_kv_heads=hkv, prefix=(prefix, prefix), n_nodes=n, depth=6,
+                     branch=10, vocab=16, temperatures=(0.0,) * batch, n_layers=1)
+    inp = synth.generate(w, 5, with_accept=False)
+    ctx = helpers.make_ctx(inp)
+    d = helpers.upload_attn(inp)
+
+    def call(q):
+        out = ctx.tree_attn(q, d["k_cache"], d["v_cache"], d["tree_k"], d["tree_v"], d["parent"], d["prefix_len"])
+        ctx.check()
+        return out
+
+    ref = call(d["q"])
+    for fill in (float("nan"), float("inf"), None):
+        q = d["q"].clone()
+        q[1::2] = q[1::2] * 64 if fill is None else fill
+        assert torch.equal(call(q)[0::2], ref[0::2]), fill
