@@ -227,3 +227,32 @@ def test_a_sequence_does_not_depend_on_its_neighbours_queries(hq, hkv, n, batch,
         q = d["q"].clone()
         q[1::2] = q[1::2] * 64 if fill is None else fill
         assert torch.equal(call(q)[0::2], ref[0::2]), fill
+
+
+@pytest.mark.parametrize("batch,n", [(1, 60), (12, 60), (1, 200)])
+def test_the_largest_weight_is_exact_behind_chunks_of_tree_rows(batch, n):
+    """The first 128 keys are the prefix, one of them 5 to 7.7 in log2 above the tree's keys (whose V is 0), the others 25 and more
+    below.  Taken against the largest score its weight is exactly 1, and the result is its V row over a sum kept in 32 bits: what is
+    left is the output's own rounding, half a unit in the last place of bf16, and a few of 32 bits."""
+    hq, hkv, L, j = 32, 8, 128, 10
+    w = synth.scaled(W["batch16_ragged"], batch=batch, n_q_heads=hq, n_kv_heads=hkv, prefix=(L, L), n_nodes=n, depth=8, branch=10,
+                     vocab=16, temperatures=(0.0,) * batch, n_layers=1)
+    inp = synth.generate(w, 7, with_accept=False)
+    n = inp.parent.shape[1]
+    rng = np.random.default_rng(3)
+    bf = lambda x: (np.ascontiguousarray(x, np.float32).view(np.uint32) >> 16).astype(np.uint16)      # (exact values only)
+    inp.q[...] = 0
+    inp.q[..., 0] = bf(40 + 0.25 * rng.integers(0, 80, inp.q.shape[:-1]))
+    inp.k_cache[...] = 0
+    inp.k_cache[:, :, :L, 0] = bf([-4.0])
+    inp.k_cache[:, :, j, 0] = bf([1.0])
+    inp.tree_k[...] = 0
+    inp.tree_v[...] = 0
+    ctx = helpers.make_ctx(inp)
+    d = helpers.upload_attn(inp)
+    out = ctx.tree_attn(d["q"], d["k_cache"], d["v_cache"], d["tree_k"], d["tree_v"], d["parent"], d["prefix_len"])
+    ctx.check()
+    ref = oracle.tree_attn(inp.q, inp.k_cache, inp.v_cache, inp.tree_k, inp.tree_v, inp.parent, inp.prefix_len)
+    err = np.abs(out.float().cpu().numpy().astype(np.float64) - ref)
+    half_ulp = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(ref), 2.0 ** -20))) - 8)
+    assert (err <= half_ulp + 4e-6).all(), (err / half_ulp).max()
