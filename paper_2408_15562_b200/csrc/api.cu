@@ -257,7 +257,7 @@ int fspad_tree_attn(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 *k_cac
     if (n_nodes > ctx->cfg.max_len) return FSPAD_ERR_RANGE;
     if (batch == 0) return FSPAD_OK;
     cudaError_t e = fspad_launch_tree_attn(ctx, q, k_cache, v_cache, tree_k, tree_v, parent, prefix_len,
-                                           n_nodes, batch, out, fspad_stream(stream));
+                                           n_nodes, batch, out, fspad_stream(stream), 0, FspadPaged{nullptr, 0, 0, false, true});
     return e == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;
 }
 
@@ -387,7 +387,7 @@ int fspad_tree_attn_paged(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 
     // a CTA keeps the blocks of its chunks in shared memory: at most 128 of them
     const int splits = fspad_attn_umma_splits(ctx, n_nodes, batch);
     if ((blocks_per_seq + splits - 1) / splits > 128) return FSPAD_ERR_TOO_LARGE;
-    const FspadPaged pg{block_table, blocks_per_seq, n_blocks};
+    const FspadPaged pg{block_table, blocks_per_seq, n_blocks, false, true};
     return fspad_launch_tree_attn(ctx, q, k_pool, v_pool, tree_k, tree_v, parent, prefix_len, n_nodes, batch, out,
                                   fspad_stream(stream), 0, pg) == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;
 }

@@ -311,10 +311,11 @@ cudaError_t fspad_launch_kv_compact(fspad_ctx *ctx, fspad_bf16 *cache, const int
 // of sequence b (table == NULL: contiguous cache).
 // early: the attention is launched beside the kernel before it in the stream, which has only been started when all that
 // precedes the two of them, and so every input of the attention, is complete; the attention's end waits for that kernel's.
+// alone: nothing else of the call runs beside the attention, which then leaves its row tiles to lone CTAs (see fspad_attn_pairs).
 struct FspadPaged {
     const int *table;
     int stride, n_blocks;
-    bool early = false;
+    bool early = false, alone = false;
 };
 // sms: how many SMs the call may fill with CTAs (0 = all of them).  merge_pdl: the merge kernel is a programmatic
 // dependent of the attention kernel (its CTAs become resident, waiting, as the attention's last CTAs finish).

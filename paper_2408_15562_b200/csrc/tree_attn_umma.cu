@@ -766,9 +766,14 @@ static int ranges_per_row(const fspad_ctx *ctx, int B, int mtiles, int sms)
     return (int)s;
 }
 
-// Row tiles of a kv head.  Where they alone fill the SMs (a batch: one key range per row, long loops) two or more go in pairs,
-// the last pair possibly with an empty half: 86 -> 77 us on 16 sequences of 240 rows a head, 93 -> 74 us on 4 of 520
-// (five tiles, six in pairs).  Where the keys are split as well, the loops are short and the pair's hand-shakes cost more than
+// Row tiles of a kv head.  In a step's attention, which shares the SMs with the scan and the walk, tiles that fill the SMs by
+// themselves (a batch: one key range per row, long loops) go in pairs where there are two or more, the last pair possibly with an empty half.
+// us a step, pairs against lone CTAs, called one by one / from a graph: 16 ragged sequences 193 / 189 against 186 / 198, five of 4 K
+// keys 139 / 105 against 144 / 110, twelve of 100 to 400 130 / 128 against 130 / 133; nine at 32000 tokens 86 / 86 against 80 / 80.
+// A call that has the SMs for itself (FspadPaged::alone) takes lone CTAs: faster at every one of 120 shapes (33 to 250 nodes, 1 to 8 heads a
+// group, 5 to 16 sequences, 150 to 4096 keys): 58.5 -> 42.9 us on eight sequences of 4 K (whose chunks take pairs in step with one another
+// 1.4 us, lone CTAs 1.0), 69 -> 62 on 16 ragged ones, 41.4 -> 30.9 on four of 130 nodes.
+// Where the keys are split as well, the loops are short and the pair's hand-shakes cost more than
 // it saves: 23.6 against 19.5 us with two chunks a CTA, 40 against 38 us with 17.
 bool fspad_attn_pairs(const fspad_ctx *ctx, int N, int B, int sms)
 {
@@ -857,7 +862,8 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     a.N = N; a.Hq = c.n_q_heads; a.Hkv = c.n_kv_heads; a.G = c.n_q_heads / c.n_kv_heads;
     a.M = N * a.G; a.max_len = paged.table ? paged.stride * umma::BK : c.max_len; a.n_splits = n_splits;
     a.block_table = paged.table; a.table_stride = paged.stride; a.n_blocks = paged.n_blocks;
-    a.mtiles = fspad_attn_mtiles(ctx, N, B, sms);
+    const bool in_pairs = !paged.alone && fspad_attn_pairs(ctx, N, B, sms);
+    a.mtiles = in_pairs ? fspad_attn_mtiles(ctx, N, B, sms) : (a.M + umma::BM - 1) / umma::BM;
     // (every CTA ranks all sequences itself, B loads each for B / 320 of its threads: kept to batches where that is small change)
     a.longest_first = (B > 1 && B <= 128 && (long long)B * c.n_kv_heads * a.mtiles * n_splits > ctx->sm_count) ? 1 : 0;
     a.scale_log2 = scale_log2;
@@ -882,7 +888,7 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
         ctx->attn_tmap_kptr = kc; ctx->attn_tmap_vptr = vc; ctx->attn_tmap_rows = rows;
     }
     a.use_tma = ctx->attn_tmap_ok ? 1 : 0;
-    const bool pair = a.use_tma && fspad_attn_pairs(ctx, N, B, sms);      // (without maps the tiles go to lone CTAs, one of them perhaps empty)
+    const bool pair = a.use_tma && in_pairs;      // (without maps the tiles go to lone CTAs, one of them perhaps empty)
     a.early = paged.early ? 1 : 0;
     CUtensorMap mq = {};
     a.q_tma = make_q_map(&mq, q, (size_t)B * N, c.n_q_heads, a.G) ? 1 : 0;

@@ -137,6 +137,32 @@ def test_step_in_one_stream(mode, heads, prefix, n_layers, aliased):
     _check(inp, outs, cache, *ref)
 
 
+@pytest.mark.parametrize("n_nodes,group", [(33, 4), (64, 4), (60, 5), (60, 8), (130, 3), (200, 2)])
+@pytest.mark.parametrize("alias", [False, True])
+def test_row_tiles_in_pairs_of_ctas(n_nodes, group, alias):
+    """A batch whose row tiles fill the SMs goes on pairs of CTAs inside a step and on lone ones in a call of the attention alone
+    (which is checked against the oracle at these shapes): the same bits, with 1 .. 12 chunks a sequence, an empty half of the last
+    pair, the boundary between the tiles inside a node's heads, tree rows apart and in the cache."""
+    B = 12
+    L = np.array([0, 100, 128, 129, 383, 500, 640, 700, 900, 1151, 1280, 1400], np.int32)
+    w = synth.scaled(W["batch16_ragged"], batch=B, n_q_heads=8 * group, n_kv_heads=8, n_nodes=n_nodes, depth=6, branch=12,
+                     prefix=(int(L.max()), int(L.max())), temperatures=(0.0,) * B, vocab=64, n_layers=1)
+    inp = synth.generate(w, n_nodes)
+    N = inp.parent.shape[1]
+    inp.prefix_len[:] = L
+    ctx = helpers.make_ctx(inp, n_layers=1)
+    cache_host = synth.make_cache(inp, 1)
+    cache_host[0, 0], cache_host[0, 1] = inp.k_cache, inp.v_cache
+    for b in range(B):
+        cache_host[0, 0, b, :, L[b]:L[b] + N], cache_host[0, 1, b, :, L[b]:L[b] + N] = inp.tree_k[b], inp.tree_v[b]
+    d, a, outs, cache = _device_inputs(inp, cache_host)
+    tree = (None, None) if alias else (a["tree_k"], a["tree_v"])
+    want = ctx.tree_attn(a["q"], cache[0, 0].clone(), cache[0, 1].clone(), *tree, a["parent"], a["prefix_len"])
+    _call(ctx, cache, a, d, outs, alias, 0)
+    ctx.check()
+    assert torch.equal(outs["attn_out"], want)
+
+
 def test_argument_errors():
     w = synth.scaled(W["llama3_8b_2k"], batch=1, prefix=(40, 40), n_nodes=8, depth=3, branch=3, vocab=100,
                      temperatures=(0.0,))
