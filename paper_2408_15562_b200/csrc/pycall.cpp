@@ -3,6 +3,7 @@
 // phase of six calls on new buffers 106 -> 67 us on one box).  What each argument has to be follows from the prototypes in fspad.h: a
 // pointer to fspad_bf16, float, int32_t, uint64_t is a contiguous tensor of that type on the GPU (of the host entry point: in
 // host memory, the cache apart) or None, a void pointer a uint8 tensor, an address or None, everything else a number.
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <tuple>
@@ -80,10 +81,12 @@ bool convert(PyObject *o, bool on_gpu, A *out)
     }
 }
 
-// host_from: the first argument whose tensors lie in host memory
+// host_from: the first argument whose tensors lie in host memory.  A tensor may throw when it is asked for its strides or its address
+// (one inside vmap or grad, for instance): as in torch's own methods that becomes the Python exception.
 template <typename... A, size_t... I>
 PyObject *invoke(int (*fn)(A...), PyObject *const *args, Py_ssize_t n, size_t host_from, std::index_sequence<I...>)
 {
+    HANDLE_TH_ERRORS
     if (n != (Py_ssize_t)sizeof...(A)) {
         PyErr_Format(PyExc_TypeError, "%zd arguments, not %zd", (Py_ssize_t)sizeof...(A), n);
         return nullptr;
@@ -95,6 +98,7 @@ PyObject *invoke(int (*fn)(A...), PyObject *const *args, Py_ssize_t n, size_t ho
     rc = fn(std::get<I>(a)...);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
 }
 template <typename... A>
 PyObject *invoke(int (*fn)(A...), PyObject *const *args, Py_ssize_t n, size_t host_from = 99)
