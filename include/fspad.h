@@ -399,8 +399,8 @@ int fspad_kv_append(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *tree_kv
  *               (rows 0 .. L_b + n_nodes - 1) must be distinct within a sequence and not shared between sequences
  * Everything else - the other arguments, the results, the error reporting - is as in fspad_tree_attn and
  * fspad_kv_compact with max_len = 128 * blocks_per_seq; a table entry out of range is reported as
- * FSPAD_ERR_RANGE (device-checked, accesses stay inside the pool).  FSPAD_ERR_TOO_LARGE: more than 128
- * blocks would fall to one CTA (blocks_per_seq above 128 times the number of key ranges the call uses).
+ * FSPAD_ERR_RANGE (device-checked, accesses stay inside the pool).  FSPAD_ERR_TOO_LARGE
+ * (fspad_tree_attn_paged): 2^31 rows or more a sequence.
  * Trees of up to 256 nodes, as in the contiguous calls.
  */
 int fspad_tree_attn_paged(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 *k_pool, const fspad_bf16 *v_pool,

@@ -1,6 +1,7 @@
 // C ABI of libfspad.so: context management, argument validation and the
 // host-buffer entry point.  All arithmetic of the verify step lives in the
 // kernel translation units; nothing here computes on the host.
+#include <climits>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -155,12 +156,12 @@ int fspad_create(const fspad_config *cfg, fspad_ctx **out)
 
     const int G = cfg->n_q_heads / cfg->n_kv_heads;
     const size_t B = (size_t)cfg->max_batch, Nmax = (size_t)cfg->max_nodes;
-    // split-KV partials: worst case over every (n_nodes, batch) a call may pass
+    // split-KV partials: worst case over every (n_nodes, batch) a call may pass, and any length of a paged call's table
     size_t part_rows = 0;
     int max_splits = 1;
     for (int n = 1; n <= cfg->max_nodes; ++n)
         for (int b = 1; b <= cfg->max_batch; ++b) {
-            const int s = fspad_attn_umma_splits(ctx, n, b);
+            const int s = fspad_attn_ranges(ctx, n, b, 0, INT_MAX);
             const size_t rows = (size_t)b * cfg->n_kv_heads * s * n * G;
             if (rows > part_rows) part_rows = rows;
             if (s > max_splits) max_splits = s;
@@ -384,9 +385,7 @@ int fspad_tree_attn_paged(fspad_ctx *ctx, const fspad_bf16 *q, const fspad_bf16 
         return FSPAD_ERR_ALIGN;
     if (blocks_per_seq < 1 || n_blocks < 1 || (long long)blocks_per_seq * 128 < n_nodes) return FSPAD_ERR_SHAPE;
     if (batch == 0) return FSPAD_OK;
-    // a CTA keeps the blocks of its chunks in shared memory: at most 128 of them
-    const int splits = fspad_attn_umma_splits(ctx, n_nodes, batch);
-    if ((blocks_per_seq + splits - 1) / splits > 128) return FSPAD_ERR_TOO_LARGE;
+    if (blocks_per_seq > INT_MAX / 128) return FSPAD_ERR_TOO_LARGE;      // rows are counted in 32 bits
     const FspadPaged pg{block_table, blocks_per_seq, n_blocks, false, true};
     return fspad_launch_tree_attn(ctx, q, k_pool, v_pool, tree_k, tree_v, parent, prefix_len, n_nodes, batch, out,
                                   fspad_stream(stream), 0, pg) == cudaSuccess ? FSPAD_OK : FSPAD_ERR_CUDA;

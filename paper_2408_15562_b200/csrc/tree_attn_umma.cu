@@ -749,18 +749,21 @@ cudaError_t fspad_launch_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t s
                             (uint32_t)polls);
 }
 
-// Key ranges per row: one CTA per SM, never a partial second wave; and one where the context is so short that walking all of its
+// Key ranges per row: one CTA per SM, never a partial second wave; and one where the call's sequences are so short that walking all of their
 // chunks takes no longer than the merge of the ranges (2.5 us and a launch, a chunk 1.05).  A greedy step of 26 nodes and 32 heads, us with
 // ranges and without: 3 chunks 14.4 and 12.8, 4 chunks 14.3 and 12.6, 5 chunks 14.6 and 14.1, 6 chunks 15.5 and 15.2, 8 chunks 15.6 and 17.0.
+// chunks: how many a sequence may have, by the context's max_len or by the block table of a paged call.  The scratch is sized for
+// as many ranges as the context's own sequences have chunks.
 constexpr int kOneRange = 5;
-static int ranges_per_row(const fspad_ctx *ctx, int B, int mtiles, int sms)
+int fspad_attn_ranges(const fspad_ctx *ctx, int N, int B, int sms, int chunks)
 {
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
-    const long long base = (long long)B * ctx->cfg.n_kv_heads * mtiles;
+    const long long base = (long long)B * ctx->cfg.n_kv_heads * fspad_attn_mtiles(ctx, N, B, sms);
     long long s = sms / base;
-    const int max_chunks = (ctx->cfg.max_len + umma::BK - 1) / umma::BK;
-    if (max_chunks <= kOneRange) return 1;
-    if (s > max_chunks) s = max_chunks;
+    const int held = (ctx->cfg.max_len + umma::BK - 1) / umma::BK;
+    if (chunks <= kOneRange) return 1;
+    if (s > chunks) s = chunks;
+    if (s > held) s = held;
     if (s > 64) s = 64;
     if (s < 1) s = 1;
     return (int)s;
@@ -789,7 +792,7 @@ int fspad_attn_mtiles(const fspad_ctx *ctx, int N, int B, int sms)
 
 int fspad_attn_umma_splits(const fspad_ctx *ctx, int N, int B, int sms)
 {
-    return ranges_per_row(ctx, B, fspad_attn_mtiles(ctx, N, B, sms), sms);
+    return fspad_attn_ranges(ctx, N, B, sms, (ctx->cfg.max_len + umma::BK - 1) / umma::BK);
 }
 
 // ---- TMA descriptors of the K and V cache planes ----------------------------------------

@@ -91,6 +91,25 @@ def test_attention_wide_trees_in_pairs_of_row_tiles(n_nodes, group, aliased):
     _check_attn(inp, n_nodes, aliased)
 
 
+@pytest.mark.parametrize("max_len,blocks", [(640, 129), (640, 300), (128, 140), (4096, 3)])
+def test_table_of_another_length_than_the_context(max_len, blocks):
+    """The table alone says how long a sequence may be: longer than the context's own by any number of blocks, or shorter."""
+    L = blocks * 128 - 70
+    w = synth.scaled(W["llama3_8b_2k"], batch=1, n_q_heads=8, n_kv_heads=8, prefix=(L, L), n_nodes=19, depth=4, branch=3, vocab=16)
+    inp = synth.generate(w, 2, with_accept=False)
+    k_pool, v_pool, table = _paged_from(inp, np.random.default_rng(blocks))
+    assert table.shape[1] == blocks
+    ctx = binding.Context(8, 8, 16, max_len, max_nodes=19)
+    b16 = binding.bf16_tensor
+    out = ctx.tree_attn_paged(b16(inp.q), b16(k_pool), b16(v_pool), helpers.dev(table), b16(inp.tree_k), b16(inp.tree_v),
+                              helpers.dev(inp.parent), helpers.dev(inp.prefix_len))
+    ctx.check()
+    ref = oracle.tree_attn(inp.q, oracle.paged_to_contiguous(k_pool, table), oracle.paged_to_contiguous(v_pool, table), inp.tree_k,
+                           inp.tree_v, inp.parent, inp.prefix_len)
+    mx, mean = helpers.attn_errors(out, ref)
+    assert mx <= 1e-2 and mean <= 1e-3, (mx, mean)
+
+
 def test_compaction_paged():
     rng = np.random.default_rng(9)
     B, N, Hkv, nl, nb = 4, 60, 3, 3, 5
