@@ -752,6 +752,8 @@ cudaError_t fspad_launch_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t s
 // Key ranges per row: one CTA per SM, never a partial second wave; and one where the call's sequences are so short that walking all of their
 // chunks takes no longer than the merge of the ranges (2.5 us and a launch, a chunk 1.05).  A greedy step of 26 nodes and 32 heads, us with
 // ranges and without: 3 chunks 14.4 and 12.8, 4 chunks 14.3 and 12.6, 5 chunks 14.6 and 14.1, 6 chunks 15.5 and 15.2, 8 chunks 15.6 and 17.0.
+// A wide tree on few CTAs is cut all the same: its up to three gathered chunks are a third of the loop and would all be one CTA's (8 heads on 2,
+// 250 nodes and 380 keys, the attention alone: 14.6 us in ranges, 18.7 in one; 32 heads on 8, 64 CTAs: 20.7 and 18.7).
 // chunks: how many a sequence may have, by the context's max_len or by the block table of a paged call.  The scratch is sized for
 // as many ranges as the context's own sequences have chunks.
 constexpr int kOneRange = 5;
@@ -761,7 +763,7 @@ int fspad_attn_ranges(const fspad_ctx *ctx, int N, int B, int sms, int chunks)
     const long long base = (long long)B * ctx->cfg.n_kv_heads * fspad_attn_mtiles(ctx, N, B, sms);
     long long s = sms / base;
     const int held = (ctx->cfg.max_len + umma::BK - 1) / umma::BK;
-    if (chunks <= kOneRange) return 1;
+    if (chunks <= kOneRange && (N <= FSPAD_MAX_NODES || base * 4 >= sms)) return 1;
     if (s > chunks) s = chunks;
     if (s > held) s = held;
     if (s > 64) s = 64;
