@@ -75,9 +75,10 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample)
     // CTA of the walk has its SM.  (On a second stream behind an event the attention was there 3 to 5 us later, or now and then
     // ahead of a cluster, which then had no 16 SMs side by side before the attention had left: 80 us in place of 38 on 52 heads.
     // One B200, us a step, two streams against one: 50.7 and 38.1 on 52 heads and 4 K keys, 44.2 and 42.4 on 8 x 8 and 8 K,
-    // both 17 chunks a CTA.)  The merge of the key ranges then comes when the walk is complete, too, which costs its 2.5 us
-    // where the attention would have been through before: 36.5 against 38.9 on 2 chunks a CTA.  An attention of 12 chunks (19 us)
-    // is as long as the shorter walks; with one range there is no merge.
+    // both 17 chunks a CTA.)  What is known here is how long the sequences may be, not how long they are; so the merge of the key ranges
+    // waits for the attention alone, not for the walk (when it did, a 2 K sequence in a context of 12 K rows or more took 37.1 us, two
+    // streams 34.2, and 31.1 now; 52 heads and 4 K keys 38.6 -> 39.0).  Below 12 chunks a range by max_len the two streams stay: no case there
+    // was slower on them, and what one stream would give has not been measured over the range.
     // Otherwise, and with more clusters, the attention is forked behind the scan onto the second stream.
     const fspad_config &c = ctx->cfg;
     const int sms = ctx->sm_count;
@@ -173,6 +174,7 @@ int fspad_create(const fspad_config *cfg, fspad_ctx **out)
     bool ok = dev_alloc(&ctx->d_status, 1);
     ok = ok && dev_alloc(&ctx->part_o, part_rows * FSPAD_HEAD_DIM);
     ok = ok && dev_alloc(&ctx->part_ml, part_rows * 2);
+    ok = ok && dev_alloc(&ctx->attn_done, 1);
     ok = ok && dev_alloc(&ctx->st_part, rows * ctx->stats_slots);
     ok = ok && dev_alloc(&ctx->row_max, rows);
     ok = ok && dev_alloc(&ctx->row_sum, rows);
@@ -190,6 +192,7 @@ int fspad_create(const fspad_config *cfg, fspad_ctx **out)
     ok = ok && cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) == cudaSuccess;
     if (ok) {
         ok = cudaMemset(ctx->d_status, 0, sizeof(int)) == cudaSuccess &&
+             cudaMemset(ctx->attn_done, 0, sizeof(int)) == cudaSuccess &&
              cudaMemset(ctx->dx_done, 0, B * sizeof(int)) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
     }
     if (!ok) {
@@ -204,7 +207,7 @@ void fspad_destroy(fspad_ctx *ctx)
 {
     if (!ctx) return;
     cudaDeviceSynchronize();
-    void *ptrs[] = {ctx->lm_parts, ctx->dx_part, ctx->dx_done, ctx->dx_front, ctx->d_status, ctx->part_o, ctx->part_ml, ctx->st_part, ctx->row_max, ctx->row_sum, ctx->row_arg, ctx->h_q, ctx->h_tk,
+    void *ptrs[] = {ctx->lm_parts, ctx->dx_part, ctx->dx_done, ctx->dx_front, ctx->d_status, ctx->part_o, ctx->part_ml, ctx->attn_done, ctx->st_part, ctx->row_max, ctx->row_sum, ctx->row_arg, ctx->h_q, ctx->h_tk,
                     ctx->h_tv, ctx->h_out, ctx->h_parent, ctx->h_prefix, ctx->h_tokens, ctx->h_path,
                     ctx->h_nacc, ctx->h_bonus, ctx->h_newlen, ctx->h_logits, ctx->h_draft, ctx->h_temp,
                     ctx->h_unif};

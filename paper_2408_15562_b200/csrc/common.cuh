@@ -38,6 +38,7 @@ struct fspad_ctx {
     int attn_tmap_ok;
     float *part_o;            // [batch][Hkv][splits][M][d]
     float *part_ml;           // [batch][Hkv][splits][M][2]  (running max in log2 units, sum)
+    int *attn_done;           // CTAs of the attention whose partials are written; zero between calls
 
     // per-node vocabulary scan
     int stats_slots;          // partial slots per row in st_part
@@ -227,7 +228,8 @@ __device__ __forceinline__ void fspad_stats_merge_warp(const FspadStatsPart *__r
 // because the two kernels that can precede it, the vocabulary scan and the LM head's merge, let it start only after their own
 // wait, when everything queued before them is complete, and themselves write nothing but scan partials, which the walk reads
 // after its wait.  The attention of a step called as one is the other: launched behind the walk, it starts when every CTA of the
-// walk has, reads what was complete before the scan started, and waits for the walk at its end.  Kernels whose predecessor is not one kernel of the same stream (behind a fork, a join or a copy) may be
+// walk has, reads what was complete before the scan started, and waits for the walk at its end.  The merge of its key ranges reads
+// the partials as soon as a count of the attention's CTAs says that they are there, and waits for the attention at its end.  Kernels whose predecessor is not one kernel of the same stream (behind a fork, a join or a copy) may be
 // launched without the attribute.
 #ifdef __CUDACC__
 __device__ __forceinline__ void fspad_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

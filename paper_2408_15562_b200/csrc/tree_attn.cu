@@ -20,6 +20,7 @@ struct AttnArgs {
     float *part_o, *part_ml;
     fspad_bf16 *out;
     int *status;
+    int *done, ctas;                    // see the merge kernel (done == NULL: no count)
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
@@ -31,16 +32,27 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 // Merge the split partials of one output row by log-sum-exp; one warp per row.  kBatch = how many
 // ranges' rows a lane requests at once (few ranges: a small batch keeps the kernel light; many:
 // a large one saves dependent round trips through L2).
+// done: the attention's CTAs count themselves there when their partials are written, because the attention itself ends no sooner than
+// the walk beside it.  This kernel starts when all of them have; a warp that finds the count complete goes ahead, any other (the
+// count may have been put back already) waits for the attention's end.  The last CTA waits in any case, so that what follows finds
+// everything complete, and puts the count back to zero.
 template <int kBatch>
 __global__ void __launch_bounds__(128)
 tree_attn_combine_kernel(const AttnArgs a, int B)
 {
     fspad_pdl_trigger();
-    fspad_pdl_wait();
+    const bool last = a.done != nullptr && blockIdx.x == gridDim.x - 1;
+    bool there = false;
+    if (a.done != nullptr) {
+        int n;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(n) : "l"(a.done) : "memory");
+        there = __all_sync(0xffffffffu, n == a.ctas) != 0;
+    }
+    if (!there) fspad_pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);   // over [B][Hkv][M]
     const long long total = (long long)B * a.Hkv * a.M;
-    if (row >= total) return;
+    if (row >= total) return;                     // (never the last CTA's first warp)
     const int gr = (int)(row % a.M);
     const int g = (int)((row / a.M) % a.Hkv);
     const int b = (int)(row / ((long long)a.M * a.Hkv));
@@ -92,6 +104,10 @@ tree_attn_combine_kernel(const AttnArgs a, int B)
     pk.x = pack_bf16(acc.x * inv, acc.y * inv);
     pk.y = pack_bf16(acc.z * inv, acc.w * inv);
     *reinterpret_cast<uint2 *>(dst) = pk;
+    if (last && threadIdx.x == 0) {
+        fspad_pdl_wait();
+        *a.done = 0;
+    }
 }
 
 }  // namespace
@@ -111,6 +127,8 @@ cudaError_t fspad_launch_tree_attn(fspad_ctx *ctx, const fspad_bf16 *q, const fs
     a.mtiles = (a.M + 127) / 128;
     a.scale_log2 = ctx->scale * kLog2e;
     a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.out = out; a.status = ctx->d_status;
+    a.done = paged.early ? ctx->attn_done : nullptr;
+    a.ctas = a.n_splits * c.n_kv_heads * a.mtiles * B;           // (keys in several ranges: never pairs, so these are the launch's CTAs)
     cudaError_t e = fspad_launch_attn_umma_split(ctx, q, kc, vc, tk, tv, parent, prefix_len, N, B, sms, a.n_splits,
                                                  a.scale_log2, out, st, paged);
     // One key range per row (a batch that fills the SMs): the attention kernel has written the result, nothing to merge

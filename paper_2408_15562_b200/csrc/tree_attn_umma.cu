@@ -64,6 +64,7 @@ struct Args {
     float scale_log2;
     float *part_o, *part_ml;
     fspad_bf16 *out;                    // one key range per row: the result itself, and no partials (NULL otherwise)
+    int *done;                          // counts the CTAs whose partials are written, for a merge that does not wait for this kernel's end (or NULL)
     int *status;
 };
 
@@ -196,6 +197,10 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
 
     if (n_ch <= 0) {                              // nothing to do for this split: empty partial (never in a pair: one range per row)
         if (row_ok && grp == 0) { float *ml = a.part_ml + (prow * M + gr) * 2; ml[0] = -INFINITY; ml[1] = 0.f; }
+        if (a.done != nullptr) {
+            __syncthreads();
+            if (tid == 0) { __threadfence(); atomicAdd(a.done, 1); fspad_pdl_trigger(); }
+        }
         if (last_cta) fspad_pdl_wait();
         return;
     }
@@ -687,7 +692,14 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
                 if (to >= 0) reinterpret_cast<uint4 *>(a.part_o + (prow * M + to) * D)[lane] = ld_shared16(stage + (uint32_t)(r * FROW + lane * 16));
             }
         }
-        fspad_pdl_trigger();                      // partial written: the merge kernel may start launching
+        // partial written: the merge kernel may start launching, and where it does not wait for this kernel's end, not before the
+        // count says that the partial is there (behind the barrier the fence stands for all eight warps' stores)
+        if (a.done != nullptr) {
+            asm volatile("bar.sync 1, 256;\n" ::: "memory");
+            if (tid == 0) { __threadfence(); atomicAdd(a.done, 1); fspad_pdl_trigger(); }
+        } else {
+            fspad_pdl_trigger();
+        }
         tc_fence_before();
         __syncthreads();
         if (PAIR) cluster_sync_all();             // neither CTA leaves while the other may still reach it
@@ -895,6 +907,7 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     a.use_tma = ctx->attn_tmap_ok ? 1 : 0;
     const bool pair = a.use_tma && in_pairs;      // (without maps the tiles go to lone CTAs, one of them perhaps empty)
     a.early = paged.early ? 1 : 0;
+    a.done = paged.early && n_splits > 1 ? ctx->attn_done : nullptr;
     CUtensorMap mq = {};
     a.q_tma = make_q_map(&mq, q, (size_t)B * N, c.n_q_heads, a.G) ? 1 : 0;
     const dim3 grid = pair ? dim3(c.n_kv_heads * a.mtiles, n_splits, B) : dim3(n_splits, c.n_kv_heads * a.mtiles, B);

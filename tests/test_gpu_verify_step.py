@@ -137,6 +137,43 @@ def test_step_in_one_stream(mode, heads, prefix, n_layers, aliased):
     _check(inp, outs, cache, *ref)
 
 
+@pytest.mark.parametrize("prefix,heads", [(60, 8), (300, 8), (2048, 8), (9000, 8), (1000, 40)])
+def test_sequence_of_any_length_in_a_long_context(prefix, heads):
+    """A context of 16384 rows cuts the keys into eight (three) ranges, some of them empty for a short sequence, and the step goes through
+    one stream: the merge of the ranges reads them while the walk may still be under way.  Two different steps in turn, three times
+    over, each checked against the oracle."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=1, n_q_heads=32 if heads == 8 else heads, n_kv_heads=heads,
+                     prefix=(prefix, prefix), n_nodes=40, depth=5, branch=5, vocab=33000, temperatures=(1.0,))
+    cap = 16384
+    ctx, steps = None, []
+    for seed in (1, 2):
+        inp = synth.generate(w, seed)
+        N, L = inp.parent.shape[1], int(inp.prefix_len[0])
+        ctx = ctx or binding.Context(w.n_q_heads, heads, w.vocab, cap, max_nodes=N)
+        ref_o, r, _, _ = _oracle_step(inp, synth.make_cache(inp, 1), 0)
+        d, a, outs, _ = _device_inputs(inp, np.zeros((1, 2, 1, 1, 1, 1), np.uint16))
+        cache = torch.zeros((1, 2, 1, heads, cap, 128), dtype=torch.bfloat16, device="cuda")
+        cache[0, 0, :, :, :L], cache[0, 1, :, :, :L] = a["k_cache"][:, :, :L], a["v_cache"][:, :, :L]
+        cache[0, 0, :, :, L:L + N], cache[0, 1, :, :, L:L + N] = a["tree_k"], a["tree_v"]
+        steps.append((inp, d, a, outs, cache, cache.clone(), ref_o, r))
+    for _ in range(3):
+        for inp, d, a, outs, cache, fresh, _, _ in steps:
+            outs["attn_out"].fill_(float("nan"))
+            cache.copy_(fresh)
+            _call(ctx, cache, a, d, outs, False, 0)
+        ctx.check()
+        for inp, d, a, outs, cache, fresh, ref_o, r in steps:
+            mx, mean = helpers.attn_errors(outs["attn_out"], ref_o)
+            assert mx <= 1e-2 and mean <= 1e-3, (mx, mean)
+            hard, near, msgs = helpers.compare_accept(inp, outs["path"].cpu().numpy(), outs["n_acc"].cpu().numpy(),
+                                                      outs["bonus"].cpu().numpy())
+            assert hard == 0 and near == 0, msgs
+            L, n = int(inp.prefix_len[0]), int(outs["n_acc"][0])
+            rows = L + outs["path"][0, :n].long()
+            assert torch.equal(cache[:, :, :, :, L:L + n], fresh[:, :, :, :, rows])
+            assert int(outs["new_len"][0]) == L + n
+
+
 @pytest.mark.parametrize("n_nodes,group", [(33, 4), (64, 4), (60, 5), (60, 8), (130, 3), (200, 2)])
 @pytest.mark.parametrize("alias", [False, True])
 def test_row_tiles_in_pairs_of_ctas(n_nodes, group, alias):
