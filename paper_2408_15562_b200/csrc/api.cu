@@ -66,7 +66,18 @@ struct StepPlan {
     bool scan_first;            // two streams: the scan goes first on all SMs, the attention behind it beside the walk
     int attn_sms;               // SMs the attention may fill (0: all)
 };
-StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample)
+// A call that is being captured into a graph: its events cost nothing there.
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return s == cudaStreamCaptureStatusActive;
+}
+// captured: decides on the order alone, never on attn_sms.
+StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool captured)
 {
     // Which of the two goes first.  The acceptance is a streaming scan over every SM followed by a walk
     // that one cluster per sampling sequence carries out; the attention is one CTA per SM.  Where the walk's clusters
@@ -79,32 +90,42 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample)
     // waits for the attention alone, not for the walk (when it did, a 2 K sequence in a context of 12 K rows or more took 37.1 us, two
     // streams 34.2, and 31.1 now; 52 heads and 4 K keys 38.6 -> 39.0).  Below 12 chunks a range by max_len the two streams stay: no case there
     // was slower on them, and what one stream would give has not been measured over the range.
+    // In a graph, where events cost nothing, the fork is the better way if the attention's CTAs find room beside the walk's: 29.7 against
+    // 30.4 us (one stream) on the 2 K sequence, 37.8 and 38.4 on 52 heads, 17.3 and 18.1 at 580 keys, 45.3 and 46.5 on two such
+    // sequences; where they do not, four short sequences of 32 heads take 33.8 in one stream and 44.8 forked.  A walk of single CTAs (less than 4096
+    // tokens) has next to no scan before it and goes beside the attention from the start: 12.8 against 14.2 (one stream) and 16.2 (scan first).
     // Otherwise, and with more clusters, the attention is forked behind the scan onto the second stream.
     const fspad_config &c = ctx->cfg;
     const int sms = ctx->sm_count;
-    const long long attn_ctas = (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch) *
-                                fspad_attn_umma_splits(ctx, n_nodes, batch);
+    auto ctas_on = [&](int n) {
+        return (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch, n) * fspad_attn_umma_splits(ctx, n_nodes, batch, n);
+    };
+    const long long attn_ctas = ctas_on(sms);
     StepPlan p = {false, false, 0};
     if (may_sample) {
         const int walk = fspad_walk_ctas(ctx, batch, c.vocab);
         const int beside = sms - (walk < sms / 2 ? walk : sms / 2), ranges = fspad_attn_umma_splits(ctx, n_nodes, batch, beside);
-        p.chain = walk <= sms / 2 && (ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges);
-        p.scan_first = !p.chain && sms - attn_ctas < sms / 4;
-        if (p.chain || p.scan_first) p.attn_sms = beside;
+        const bool one_stream = walk <= sms / 2 && (ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges);
+        const bool fork = !one_stream || (captured && ctas_on(beside) <= beside);
+        p.chain = !fork;
+        p.scan_first = fork && (one_stream ? walk > batch : sms - attn_ctas < sms / 4);
+        if (one_stream || p.scan_first) p.attn_sms = beside;
     } else {
         // An all-greedy acceptance is a scan and a one-CTA walk: beside an attention that holds most SMs the
         // scan's CTAs only get going when the attention's leave.  Where the context is short enough for the
         // attention to stay short on half the SMs (at most 8 chunks per CTA by the context's max_len), it
         // gets half and the two really run side by side (17.2 against 20.5 us on the 26-node greedy workload); and where the scan
-        // is short, too (8 MB: 1.3 us of HBM, 3.6 us in all), it goes first on all SMs and the attention follows in the same
-        // stream: four launches without an event between them, 17.2 -> 15.0 us on that workload.  With one key range (no merge) that
-        // holds for an attention of few CTAs, too: 8 KV heads called one by one 18.7 -> 12.3 us, from a graph 11.8 -> 12.3; with
-        // more ranges the graph loses more (8 chunks: 18.3 -> 14.5 and 12.5 -> 14.2) and the two streams stay.
+        // is short, too (8 MB: 1.3 us of HBM, 3.6 us in all), and the step is called and not captured, the scan goes first and the attention
+        // follows in the same stream: four launches without an event between them, 16.5 -> 12.7 us on that workload (in one range; in two,
+        // with 1024 rows, 16.5 -> 13.9).  With one key range (no merge) that holds for an attention of few CTAs, too: 8 KV heads called one
+        // by one 16.5 -> 12.4 us.  From a graph the two streams take 11.4 us on that workload against 12.8 in one (1024 rows: 12.2 and 13.7;
+        // 8 KV heads: 11.4 and 12.4).
         const int s_half = fspad_attn_umma_splits(ctx, n_nodes, batch, sms / 2);
         const int max_chunks = (c.max_len + 127) / 128;
         const bool short_attn = (max_chunks + s_half - 1) / s_half <= 8;
-        p.chain = short_attn && (attn_ctas > sms / 2 || fspad_attn_umma_splits(ctx, n_nodes, batch) == 1) && (long long)batch * n_nodes * c.vocab <= 2 << 20;
-        if (short_attn && !p.chain && attn_ctas > sms / 2) p.attn_sms = sms / 2;
+        if (short_attn && attn_ctas > sms / 2) p.attn_sms = sms / 2;
+        p.chain = !captured && short_attn && (attn_ctas > sms / 2 || fspad_attn_umma_splits(ctx, n_nodes, batch) == 1) &&
+                  (long long)batch * n_nodes * c.vocab <= 2 << 20;
     }
     return p;
 }
@@ -504,7 +525,7 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
 
     const int sms = ctx->sm_count;
     const bool may_sample = draft_probs != nullptr;
-    const StepPlan plan = step_plan(ctx, n_nodes, batch, may_sample);
+    const StepPlan plan = step_plan(ctx, n_nodes, batch, may_sample, capturing(st));
     const bool scan_first = plan.scan_first;
     const int attn_sms = plan.attn_sms;
     cudaError_t ce = cudaSuccess;
@@ -678,7 +699,7 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     if (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess)
         return give_up(FSPAD_ERR_CUDA);
     const size_t plane = (size_t)batch * c.n_kv_heads * (size_t)c.max_len * FSPAD_HEAD_DIM;
-    const StepPlan plan = step_plan(ctx, n_nodes, batch, draft_probs != nullptr);
+    const StepPlan plan = step_plan(ctx, n_nodes, batch, draft_probs != nullptr, false);
     const bool attn_ok = fspad_launch_tree_attn(ctx, ctx->h_q, cache, cache + plane, nullptr, nullptr, ctx->h_parent, ctx->h_prefix,
                                                 n_nodes, batch, ctx->h_out, ctx->side, plan.attn_sms) == cudaSuccess;
     h2d(ctx->h_tokens, draft_tokens, B * N * sizeof(int));

@@ -19,6 +19,7 @@ std::map<std::string, int> g_fail;                       // name -> calls until 
 struct Range { const char *lo; size_t bytes; };
 std::vector<Range> g_pinned;
 const int kSms = 148;
+bool g_capturing = false;
 
 cudaError_t call(const char *name, const char *fmt = "", ...)
 {
@@ -46,6 +47,7 @@ extern "C" {
 
 const char *fake_log() { return g_log.c_str(); }
 void fake_reset() { g_log.clear(); g_fail.clear(); g_pinned.clear(); }
+void fake_capture(int on) { g_capturing = on != 0; }
 void fake_fail(const char *name, int nth) { g_fail[name] = nth; }
 void fake_pin(const void *p, size_t bytes) { g_pinned.push_back({(const char *)p, bytes}); }
 
@@ -62,6 +64,11 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { static size_t n
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t s) { return call("event_record", "stream=%x", id(s)); }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t, unsigned) { return call("stream_wait", "stream=%x", id(s)); }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s)
+{
+    *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t s) { return call("sync", "stream=%x", id(s)); }
 cudaError_t cudaMemcpyAsync(void *dst, const void *src, size_t n, cudaMemcpyKind k, cudaStream_t s)
 {
@@ -97,13 +104,13 @@ cudaError_t cudaGetDriverEntryPoint(const char *, void **fn, unsigned long long,
 
 }  // extern "C"
 
-int fspad_attn_umma_splits(const fspad_ctx *c, int, int B, int sms)
+int fspad_attn_mtiles(const fspad_ctx *c, int N, int, int) { return (N * (c->cfg.n_q_heads / c->cfg.n_kv_heads) + 127) / 128; }
+int fspad_attn_umma_splits(const fspad_ctx *c, int N, int B, int sms)
 {
-    const int s = (sms > 0 ? sms : kSms) / (B * c->cfg.n_kv_heads), chunks = (c->cfg.max_len + 127) / 128;
-    return s < 1 ? 1 : s < chunks ? s : chunks;
+    const int s = (sms > 0 ? sms : kSms) / (B * c->cfg.n_kv_heads * fspad_attn_mtiles(c, N, B, sms)), chunks = (c->cfg.max_len + 127) / 128;
+    return chunks <= 5 || s < 1 ? 1 : s < chunks ? s : chunks;
 }
 int fspad_attn_ranges(const fspad_ctx *c, int N, int B, int sms, int) { return fspad_attn_umma_splits(c, N, B, sms); }
-int fspad_attn_mtiles(const fspad_ctx *c, int N, int, int) { return (N * (c->cfg.n_q_heads / c->cfg.n_kv_heads) + 127) / 128; }
 int fspad_draft_expand_pieces(int V) { return (V + 4095) / 4096; }
 int fspad_lm_head_tiles(int V) { return (V + 127) / 128; }
 int fspad_walk_ctas(fspad_ctx *, int B, int) { return 16 * B; }
@@ -112,9 +119,9 @@ FspadStatsGeom fspad_lm_head_geom(int, int, bool, int) { return FspadStatsGeom()
 
 cudaError_t fspad_launch_tree_attn(fspad_ctx *, const fspad_bf16 *, const fspad_bf16 *, const fspad_bf16 *, const fspad_bf16 *,
                                    const fspad_bf16 *, const int *, const int *, int, int, fspad_bf16 *, cudaStream_t st, int sms,
-                                   FspadPaged, bool)
+                                   FspadPaged paged, bool)
 {
-    return call("attention", "sms=%d stream=%x", sms, id(st));
+    return call("attention", "sms=%d early=%d stream=%x", sms, (int)paged.early, id(st));
 }
 cudaError_t fspad_launch_accept_walk(fspad_ctx *, const float *, const float *draft, const int *, const int *, const float *,
                                      const float *, const FspadStatsGeom &, int, int, int, int *, int *, int *, cudaStream_t st,

@@ -89,6 +89,38 @@ def test_host_entry_cuts_the_attention_as_the_device_entry_does(lib, hq, hkv, no
     assert _field(log_h, "attention", "sms") == want
 
 
+@pytest.mark.parametrize("sampling,hq,hkv,nodes,batch,max_len,called,captured", [
+    (True, 32, 8, 60, 1, 2176, "fork", "fork"),          # several ranges of three chunks
+    (True, 52, 52, 60, 1, 4224, "one", "fork"),          # two ranges of 17 chunks
+    (True, 32, 8, 60, 1, 16384, "one", "fork"),          # eight ranges of 16
+    (True, 32, 32, 60, 4, 320, "one", "one"),            # 128 CTAs, more than the walk leaves room for
+    (True, 32, 32, 60, 16, 4224, "fork", "fork"),        # walks on more than half of the SMs
+    (False, 32, 32, 26, 1, 320, "one", "fork"),          # short greedy step
+    (False, 32, 32, 26, 1, 1024, "one", "fork"),         # the same with two ranges
+    (False, 32, 32, 26, 1, 8320, "fork", "fork"),        # long greedy step
+])
+def test_capture_decides_on_the_order_and_not_on_the_cut(lib, sampling, hq, hkv, nodes, batch, max_len, called, captured):
+    """One stream: scan, walk, attention beside the walk, no event.  Fork: the attention on the second stream between two events.
+    The SMs the attention is cut for, and with them the results' bits, are the same either way."""
+    sms = set()
+    for on, want in ((0, called), (1, captured)):
+        step = Step(lib, hq, hkv, nodes, batch, 32768 if sampling else 4096, max_len, sampling)
+        lib.fake_capture(on)
+        try:
+            rc, log = step.device()
+        finally:
+            lib.fake_capture(0)
+        assert rc == 0
+        sms.add(_field(log, "attention", "sms"))
+        events = [x for x in log if x.startswith("event_record ") or x.startswith("stream_wait ")]
+        if want == "one":
+            assert not events and _field(log, "attention", "early") == "1" and _field(log, "attention", "stream") == "%x" % STREAM
+            assert [x.split()[0] for x in log][:3] == ["scan", "walk", "attention"]
+        else:
+            assert len(events) == 4 and _field(log, "attention", "early") == "0" and _field(log, "attention", "stream") != "%x" % STREAM
+    assert len(sms) == 1
+
+
 @pytest.mark.parametrize("pins,in_place", [(((0, 1.0),), True), ((), False), (((0, 0.5),), False), (((0, 0.999),), False),
                                            (((0.5, 0.5),), False), (((0, 0.25), (0.75, 0.25)), False), (((0, 0.5), (0.5, 0.5)), False)])
 def test_draft_rows_are_read_in_place_only_where_all_of_them_are_pinned(lib, pins, in_place):
