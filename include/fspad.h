@@ -426,8 +426,8 @@ int fspad_kv_compact_paged(fspad_ctx *ctx, fspad_bf16 *pool, const int32_t *bloc
  * reads the cache rows compaction rewrites); when they are NULL (tree rows
  * taken from cache rows L_b ..) compaction waits for the attention as well.
  * In the first case, when a sequence has at most 64 (layer, K/V, kv head)
- * slices (256 where a sampling step stays in one stream), the kernel that walks the tree makes the compaction's moves itself,
- * greedy or sampling (same result; an invalid prefix length is then reported by
+ * slices (where a sampling step stays in one stream, 32 for each CTA of the walk's cluster, up to 256), the kernel
+ * that walks the tree makes the compaction's moves itself, greedy or sampling (same result; an invalid prefix length is then reported by
  * that kernel).
  * Work queued on `stream` after the call sees every output.  The call only
  * enqueues work and records / waits on events, so it may be captured into a

@@ -532,11 +532,18 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
     FspadStatsGeom geom;
     const int rows = batch * n_nodes;
     // With the tree rows given apart from the cache the compaction depends on the walk alone, and when the
-    // sequence's slices are few (one warp each among the 16 x 16 warps of a sampling walk's cluster, four each for the 16
-    // warps of a greedy one) the walk makes the moves itself at its end: one dependent launch less on the step's
+    // sequence's slices are few (a warp takes one after another: four each for the 16 warps of a greedy walk's CTA) the walk makes the moves itself at its end: one dependent launch less on the step's
     // longest chain (all-greedy step of 26 nodes and 64 slices: 29.3 -> 23.7 us called one by one, 13.1 against 13.3 from a graph).
+    // In one stream, where the compaction kernel would come behind the attention, that pays up to two slices a warp of the cluster's CTAs, 16
+    // warps each: 256 slices at 32000 tokens (eight CTAs) 22.3 us against 23.5 with the kernel, at 128256 (16) 28.5 and 30.7; a single CTA
+    // (4000 tokens) 29.4 and 24.9.  A sequence of temperature 0 among them has one CTA whatever the cluster: 256 slices 23 us and 22.4.
     const bool aliased = tree_k == nullptr;      // attention reads the cache rows that compaction rewrites
-    const bool walk_compacts = !aliased && c.n_layers * 2 * c.n_kv_heads <= (plan.chain && may_sample ? 256 : 64);
+    int most_slices = 64;
+    if (plan.chain && may_sample) {
+        const int by_cluster = 32 * (fspad_walk_ctas(ctx, batch, c.vocab) / batch);
+        most_slices = by_cluster < 64 ? 64 : by_cluster > 256 ? 256 : by_cluster;
+    }
+    const bool walk_compacts = !aliased && c.n_layers * 2 * c.n_kv_heads <= most_slices;
     FspadWalkCompact kv;
     if (walk_compacts) { kv.cache = cache; kv.prefix_len = prefix_len; kv.new_len = new_len; }
     if (plan.chain) {

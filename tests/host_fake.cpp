@@ -113,7 +113,12 @@ int fspad_attn_umma_splits(const fspad_ctx *c, int N, int B, int sms)
 int fspad_attn_ranges(const fspad_ctx *c, int N, int B, int sms, int) { return fspad_attn_umma_splits(c, N, B, sms); }
 int fspad_draft_expand_pieces(int V) { return (V + 4095) / 4096; }
 int fspad_lm_head_tiles(int V) { return (V + 127) / 128; }
-int fspad_walk_ctas(fspad_ctx *, int B, int) { return 16 * B; }
+int fspad_walk_ctas(fspad_ctx *, int B, int V)
+{
+    int c = 16;
+    while (c > 1 && (V + c - 1) / c < 2048) c >>= 1;
+    return B * c;
+}
 size_t fspad_feature_sampler_scratch_floats(int, int, int) { return 0; }
 FspadStatsGeom fspad_lm_head_geom(int, int, bool, int) { return FspadStatsGeom(); }
 
@@ -125,9 +130,9 @@ cudaError_t fspad_launch_tree_attn(fspad_ctx *, const fspad_bf16 *, const fspad_
 }
 cudaError_t fspad_launch_accept_walk(fspad_ctx *, const float *, const float *draft, const int *, const int *, const float *,
                                      const float *, const FspadStatsGeom &, int, int, int, int *, int *, int *, cudaStream_t st,
-                                     FspadWalkCompact, bool far)
+                                     FspadWalkCompact kv, bool far)
 {
-    return call("walk", "draft=%llx far=%d stream=%x", (unsigned long long)(uintptr_t)draft, (int)far, id(st));
+    return call("walk", "draft=%llx far=%d compacts=%d stream=%x", (unsigned long long)(uintptr_t)draft, (int)far, (int)(kv.cache != nullptr), id(st));
 }
 cudaError_t fspad_launch_stats_partials(fspad_ctx *, const float *, const float *, int, int, int, FspadStatsGeom *, cudaStream_t st,
                                         bool, int)

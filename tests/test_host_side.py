@@ -39,9 +39,9 @@ def lib(tmp_path_factory):
 class Step:
     """One context and one set of (never read) buffers for both entry points."""
 
-    def __init__(self, lib, hq=32, hkv=8, nodes=60, batch=1, vocab=4096, max_len=2176, sampling=True):
+    def __init__(self, lib, hq=32, hkv=8, nodes=60, batch=1, vocab=4096, max_len=2176, sampling=True, layers=1):
         self.lib, self.n, self.batch, self.vocab, self.sampling = lib, nodes, batch, vocab, sampling
-        cfg = binding.FspadConfig(hq, hkv, 128, nodes, vocab, 1, max_len, batch, 0.0)
+        cfg = binding.FspadConfig(hq, hkv, 128, nodes, vocab, layers, max_len, batch, 0.0)
         self.ctx = ctypes.c_void_p()
         assert lib.fspad_create(ctypes.byref(cfg), ctypes.byref(self.ctx)) == 0
         raw = np.zeros(batch * nodes * vocab + 8, np.float32)
@@ -61,10 +61,10 @@ class Step:
                                              big, p, p, p, p, STREAM)
         return rc, self.lib.fake_log().decode().splitlines()
 
-    def device(self):
+    def device(self, tree=None):
         big = 0x1000
         draft, unif = (big, big) if self.sampling else (None, None)
-        rc = self.lib.fspad_verify_step(self.ctx, big, 0, big, None, None, big, big, big, draft, big, big, unif, self.n, self.batch, big,
+        rc = self.lib.fspad_verify_step(self.ctx, big, 0, big, tree, tree, big, big, big, draft, big, big, unif, self.n, self.batch, big,
                                         big, big, big, big, STREAM)
         return rc, self.lib.fake_log().decode().splitlines()
 
@@ -87,6 +87,21 @@ def test_host_entry_cuts_the_attention_as_the_device_entry_does(lib, hq, hkv, no
     rc_h, log_h = step.host()
     assert rc == 0 and rc_h == 0
     assert _field(log_h, "attention", "sms") == want
+
+
+@pytest.mark.parametrize("sampling,vocab,hkv,layers,max_len,by_walk", [
+    (True, 32000, 32, 1, 320, True), (True, 32000, 32, 4, 320, True), (True, 32000, 43, 3, 320, False),       # one stream: 64, 256, 258 slices
+    (True, 4000, 32, 1, 320, True), (True, 4000, 33, 1, 320, False),         # a single CTA walks: 64, 66
+    (True, 8192, 32, 2, 320, True), (True, 8192, 33, 2, 320, False),         # a cluster of four: 128, 132
+    (True, 128256, 8, 4, 2176, True), (True, 128256, 8, 5, 2176, False),     # two streams: 64, 80
+    (False, 4000, 32, 1, 320, True), (False, 4000, 33, 1, 320, False),       # greedy, one stream
+])
+def test_who_compacts(lib, sampling, vocab, hkv, layers, max_len, by_walk):
+    """The walk moves the cache rows where a warp of its CTAs gets two slices at most (64 slices in any case), else the kernel does."""
+    step = Step(lib, 4 * hkv if hkv == 8 else hkv, hkv, 60 if hkv == 8 else 8, 1, vocab, max_len, sampling, layers)
+    rc, log = step.device(0x1000)
+    assert rc == 0 and _field(log, "walk", "compacts") == str(int(by_walk))
+    assert any(x.startswith("compact ") for x in log) != by_walk
 
 
 @pytest.mark.parametrize("sampling,hq,hkv,nodes,batch,max_len,called,captured", [
