@@ -15,9 +15,9 @@
 // is V in its [key][d] layout (MN-major).  O stays in tensor memory across chunks.
 // The work is split over three kinds of warps that meet only on mbarriers (see the
 // kernel's comment); K/V chunks go through a ring of 128-byte-swizzled tiles (three
-// whole chunks in a lone CTA, half of each of five in a pair's) from the last chunk
+// whole chunks in a lone CTA, half of each of five in a pair's): one chunk of the prefix, then from the last one
 // down, filled by TMA, as Q is; only the chunks with rows of an explicit tree array or
-// zero padding, which come first, are gathered with 16-byte asynchronous copies, and
+// zero padding, which come early, are gathered with 16-byte asynchronous copies, and
 // Q where a group of query heads does not divide the tile.  Where a row's keys are
 // split over several CTAs the partials are merged by the combine kernel; with one
 // range per row the kernel writes the result itself.
@@ -236,14 +236,23 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
     };
     const fspad_bf16 *tkb = a.tk ? a.tk + ((size_t)b * a.Hkv + g) * (size_t)N * D : nullptr;
     const fspad_bf16 *tvb = a.tv ? a.tv + ((size_t)b * a.Hkv + g) * (size_t)N * D : nullptr;
-    // The chunks are taken from the last one down, so that those TMA cannot describe come first: the ones with rows of an
+    // The chunks are taken from the last one down, so that those TMA cannot describe come early: the ones with rows of an
     // explicit tree array, and the one that ends in zero padding (at most three of them: 256 nodes).  The softmax warps, idle until
     // the first scores are there, gather them side by side with the copies of the others.  (Gathered where they stood, at
     // the end of the range and by the copy warp alone, they held everything up: 2.5 us for each operand.)
+    // Before them goes one chunk of the prefix alone, where the range has one and the ring room: a row's reference maximum then comes
+    // from whole groups of keys and not from the row's few ancestors.  (With the tree's chunks first either the reference lags behind
+    // the prefix's scores, and the largest weight, an exact one otherwise, is rounded: three sequences of 110 keys 2.17e-3 off 64 bits against
+    // 2.09e-3; or it follows, with a pass over O behind the product: us, pass / this: 16 sequences of 1 K keys, the attention alone 40.2 / 38.8, 32 heads
+    // and 570 keys 14.0 / 13.8, 32 heads and 1.5 K 18.2 / 17.8; the other way round 52 heads and 4 K in a step 38.6 / 39.0.)
+    const int n_mask = max(0, c1 - max(c0, L / BK));                  // chunks of the range that reach past the prefix
+    const bool lead = n_mask > 0 && n_mask < n_ch && n_mask < ring_slots(false);       // (the same on pairs, and with it the bits)
+    auto chunk_at = [&](int c) { return c1 - 1 - (!lead || c > n_mask ? c : c == 0 ? n_mask : c - 1); };      // c-th chunk to be taken
     const int key_tma = tkb ? L : Ltot;           // rows in front of this key lie in the cache
     auto is_tma = [&](int ch) { return tma_ok && (ch + 1) * BK <= key_tma; };
-    int n_gather = 0;                             // chunks of the first ring filling that are gathered
-    while (n_gather < NS && n_gather < n_ch && !is_tma(c1 - 1 - n_gather)) ++n_gather;
+    const int g0 = lead && tma_ok ? 1 : 0;        // chunks g0 .. g0 + n_gather - 1 of the first ring filling are gathered
+    int n_gather = 0;
+    while (g0 + n_gather < NS && g0 + n_gather < n_ch && !is_tma(chunk_at(g0 + n_gather))) ++n_gather;
 
     // Gather chunk `ch` into ring slot `buf` with 16-byte asynchronous copies by threads t0, t0 + nt, ... (nt a multiple of 16):
     // 16-byte piece c of every row that falls to a thread is the same, so all its addresses follow from one.
@@ -307,12 +316,12 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
         }
     };
     const bool in_tree = c1 * BK > L;             // this range's keys reach into the tree
-    int blk_row = 0;                              // copy warp: first plane row of chunk 32 i + lane (counted from the range's end)
+    int blk_row = 0;                              // copy warp: first plane row of the (32 i + lane)-th chunk to be taken
     auto first_fills = [&](int u0, int u1) {      // copy warp: ring slots u0 .. u1 - 1, for the first time
         for (int u = u0; u < u1 && u < n_ch; ++u) {
             const int y = __shfl_sync(0xffffffffu, blk_row, u);
             if (lane == 0) {
-                if (u >= n_gather) { tma_fill(y, u, false); tma_fill(y, u, true); }
+                if (u < g0 || u >= g0 + n_gather) { tma_fill(y, u, false); tma_fill(y, u, true); }
                 else if (rank == 0) { mbar_arrive(kfull(u)); mbar_arrive(vfull(u)); }       // (gkfull and gvfull tell when they are there)
             }
             __syncwarp();
@@ -322,7 +331,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
     // for all of it.  So the rest of the ring is asked for when the first scores are there.
     constexpr int kFirst = PAIR ? 3 : 2;
     if (warp == 8) {
-        if (lane < n_ch) blk_row = chunk_row(c1 - 1 - lane);
+        if (lane < n_ch) blk_row = chunk_row(chunk_at(lane));
         peer_ready();
         if (lane == 0 && q_tma) {
             const int nd = b * N + mt * (BM / G);
@@ -338,7 +347,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
         }
         first_fills(0, kFirst);
     } else if (warp < 8) {
-        // What TMA cannot describe: Q where a group of query heads does not divide the tile, and the first n_gather chunks.
+        // What TMA cannot describe: Q where a group of query heads does not divide the tile, and n_gather of the first chunks.
         if (!q_tma) {
             const int c = tid & 15;
             int r = tid >> 4;                     // 16 rows a step
@@ -352,9 +361,9 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
                 if (hh >= G) { hh -= G; ++nd; }
             }
         }
-        for (int u = 0; u < n_gather; ++u) gather(c1 - 1 - u, u, false, tid, 256);
+        for (int u = g0; u < g0 + n_gather; ++u) gather(chunk_at(u), u, false, tid, 256);
         cp_async_commit();
-        for (int u = 0; u < n_gather; ++u) gather(c1 - 1 - u, u, true, tid, 256);
+        for (int u = g0; u < g0 + n_gather; ++u) gather(chunk_at(u), u, true, tid, 256);
         cp_async_commit();
         peer_ready();
     } else {
@@ -381,10 +390,10 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
         if (n_ch > kFirst && !mbar_wait(kfree(0), 0u)) failed = true;
         if (!failed) first_fills(kFirst, NS);
         auto fill = [&](int c, int y, int buf, bool is_v) {
-            if (is_tma(c1 - 1 - c)) {
+            if (is_tma(chunk_at(c))) {
                 if (lane == 0) tma_fill(y, buf, is_v);
             } else {
-                gather(c1 - 1 - c, buf, is_v, lane, 32);
+                gather(chunk_at(c), buf, is_v, lane, 32);
                 cp_async_commit();
                 cp_async_wait<0>();
                 fence_async_smem();
@@ -397,7 +406,7 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
         uint32_t ph = 0;                         // flips each time the ring wraps
         for (int i = 0; i + NS < n_ch; ++i) {
             const int c = i + NS;
-            if ((c & 31) == 0 && c + lane < n_ch) blk_row = chunk_row(c1 - 1 - c - lane);
+            if ((c & 31) == 0 && c + lane < n_ch) blk_row = chunk_row(chunk_at(c + lane));
             const int y = __shfl_sync(0xffffffffu, blk_row, c & 31);
             // the K buffer of chunk i is free once S(i) has completed, its V buffer once O += P(i) V(i) has
             if (!failed && !mbar_wait(kfree(buf), ph)) failed = true;
@@ -444,14 +453,15 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
                 if (++kbuf == NS) { kbuf = 0; kph ^= 1u; }
             };
             if ((PAIR || q_tma) && !mbar_wait(qfull, 0u)) failed = true;
-            if ((n_gather > 0 || !q_tma) && !failed && !mbar_wait(gkfull, 0u)) failed = true;
+            if (((n_gather > 0 && g0 == 0) || !q_tma) && !failed && !mbar_wait(gkfull, 0u)) failed = true;
             issue_s(0);
+            if (n_gather > 0 && !failed && !mbar_wait(gkfull, 0u)) failed = true;
             if (n_ch > 1) issue_s(1);
-            if (n_gather > 0 && !failed && !mbar_wait(gvfull, 0u)) failed = true;
             for (int c = 0; c < n_ch; ++c) {
                 const int p = c & 1;
                 const uint32_t ph = (uint32_t)(c >> 1) & 1u;
                 const uint32_t vb = v_lo + (uint32_t)vbuf * (SLOT >> 4);
+                if (n_gather > 0 && c == g0 && !failed && !mbar_wait(gvfull, 0u)) failed = true;
 #pragma unroll
                 for (int g2 = 0; g2 < 2; ++g2) {
                     // O[g2] += P_g2(c) V(c)[64 g2 .. 64 g2 + 63]: P from the four warps of group g2 (in tensor
@@ -501,12 +511,12 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
         int cur = in_tree && row_ok ? gr / G : -1;         // this row's node, then its ancestors: how far the chunks so far have taken them
 
         for (int c = 0; c < n_ch; ++c) {
-            const int ch = c1 - 1 - c, p = c & 1;      // (from the last chunk down)
+            const int ch = chunk_at(c), p = c & 1;
             const uint32_t tS = tmem + lanes + (uint32_t)p * 128u + (uint32_t)grp * 64u;   // scores, then P
             const bool masked = (ch + 1) * BK > L;   // only chunks that reach past the cached prefix
             // Validity of this group's 64 keys for this row: prefix keys are valid, tree key L + t is valid iff t is the row's node
             // or one of its ancestors (which also rules out the zero padding).  Parents come before their children and the
-            // chunks from the last one down, so every chunk takes the walk to the root on from where the one before it left off;
+            // tree's chunks from the last one down, so every chunk takes the walk to the root on from where the one before it left off;
             // no mask is kept, whatever the tree's size.
             unsigned long long valid = ~0ull;
             if (masked) {
@@ -557,10 +567,9 @@ tree_attn_umma_kernel(const Args a, const __grid_constant__ CUtensorMap tmQ, con
             // (The decision is taken per warp because the tensor-memory accesses are warp-collective;
             // a comparison with -inf - -inf = NaN is false and so counts as a move.  Lanes whose row does not exist have no say: by
             // TMA they hold the next sequence's queries, and what that one asks must not decide how this one's P is rounded.)
-            // The chunks with tree rows come first and offer a row only its few ancestors: up to the first chunk of the prefix alone
-            // the reference follows every larger score, so that the largest weight is an exact one there.  (With the lag from the
-            // start, three sequences of 110 keys were 2.17e-3 off 64 bits, against 2.09e-3.)
-            const float m_cand = fmaxf(m_run, mx * scale), lag = (ch + 2) * BK > L ? 0.f : kLazyLog2;
+            // Where the tree's chunks do come first (no chunk of the prefix alone, or three of the tree's), the reference follows every larger
+            // score up to the first chunk behind them.
+            const float m_cand = fmaxf(m_run, mx * scale), lag = !lead && (ch + 2) * BK > L ? 0.f : kLazyLog2;
             const bool move = !__all_sync(0xffffffffu, !row_ok || m_cand - m_run <= lag);
             const float m_new = move ? m_cand : m_run;
             const float m_safe = (m_new == -INFINITY) ? 0.f : m_new;
