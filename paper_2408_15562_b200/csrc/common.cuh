@@ -329,8 +329,8 @@ cudaError_t fspad_launch_tree_attn(fspad_ctx *ctx, const fspad_bf16 *q, const fs
 cudaError_t fspad_launch_tree_scatter(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *tk,
                                       const fspad_bf16 *tv, const int *prefix_len, int N, int B,
                                       cudaStream_t st);
-int fspad_attn_ranges(const fspad_ctx *ctx, int N, int B, int sms, int chunks);   // key ranges per row of sequences of up to that many chunks
-int fspad_attn_umma_splits(const fspad_ctx *ctx, int N, int B, int sms = 0);      // ... of the context's max_len
+int fspad_attn_ranges(const fspad_ctx *ctx, int N, int B, int sms, int chunks, bool alone);   // key ranges per row of sequences of up to that many chunks
+int fspad_attn_umma_splits(const fspad_ctx *ctx, int N, int B, int sms = 0);      // ... of a step's attention, by the context's max_len
 bool fspad_attn_pairs(const fspad_ctx *ctx, int N, int B, int sms = 0);      // row tiles go in pairs of CTAs
 int fspad_attn_mtiles(const fspad_ctx *ctx, int N, int B, int sms = 0);     // row tiles (CTAs) per kv head and key range
 int fspad_lm_head_tiles(int V);

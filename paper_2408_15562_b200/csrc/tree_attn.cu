@@ -123,7 +123,7 @@ cudaError_t fspad_launch_tree_attn(fspad_ctx *ctx, const fspad_bf16 *q, const fs
     a.q = q; a.kc = kc; a.vc = vc; a.tk = tk; a.tv = tv; a.parent = parent; a.prefix_len = prefix_len;
     a.N = N; a.Hq = c.n_q_heads; a.Hkv = c.n_kv_heads; a.G = c.n_q_heads / c.n_kv_heads;
     a.M = N * a.G; a.max_len = paged.table ? paged.stride * 128 : c.max_len;
-    a.n_splits = paged.table ? fspad_attn_ranges(ctx, N, B, sms, paged.stride) : fspad_attn_umma_splits(ctx, N, B, sms);
+    a.n_splits = fspad_attn_ranges(ctx, N, B, sms, paged.table ? paged.stride : (c.max_len + 127) / 128, paged.alone);
     a.mtiles = (a.M + 127) / 128;
     a.scale_log2 = ctx->scale * kLog2e;
     a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.out = out; a.status = ctx->d_status;

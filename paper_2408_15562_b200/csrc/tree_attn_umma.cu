@@ -775,16 +775,20 @@ cudaError_t fspad_launch_wait_selftest(fspad_ctx *ctx, int polls, cudaStream_t s
 // ranges and without: 3 chunks 14.4 and 12.8, 4 chunks 14.3 and 12.6, 5 chunks 14.6 and 14.1, 6 chunks 15.5 and 15.2, 8 chunks 15.6 and 17.0.
 // A wide tree on few CTAs is cut all the same: its up to three gathered chunks are a third of the loop and would all be one CTA's (8 heads on 2,
 // 250 nodes and 380 keys, the attention alone: 14.6 us in ranges, 18.7 in one; 32 heads on 8, 64 CTAs: 20.7 and 18.7).
+// So is a call of the attention alone on few CTAs at five chunks: without a step around it, whose order goes by the ranges, the merge costs less
+// than the fifth chunk (us from a graph, ranges and one: 8 heads on one 11.9 and 12.9, 4 heads of 26 nodes 12.1 and 13.5, 32 on 8 13.1 and 13.4; with 32
+// CTAs, 64 heads on 8, 13.4 and 13.1).
 // chunks: how many a sequence may have, by the context's max_len or by the block table of a paged call.  The scratch is sized for
 // as many ranges as the context's own sequences have chunks.
 constexpr int kOneRange = 5;
-int fspad_attn_ranges(const fspad_ctx *ctx, int N, int B, int sms, int chunks)
+int fspad_attn_ranges(const fspad_ctx *ctx, int N, int B, int sms, int chunks, bool alone)
 {
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
     const long long base = (long long)B * ctx->cfg.n_kv_heads * fspad_attn_mtiles(ctx, N, B, sms);
     long long s = sms / base;
     const int held = (ctx->cfg.max_len + umma::BK - 1) / umma::BK;
-    if (chunks <= kOneRange && (N <= FSPAD_MAX_NODES || base * 4 >= sms)) return 1;
+    const bool few = (N > FSPAD_MAX_NODES && base * 4 < sms) || (alone && chunks == kOneRange && base * 8 < sms);
+    if (chunks <= kOneRange && !few) return 1;
     if (s > chunks) s = chunks;
     if (s > held) s = held;
     if (s > 64) s = 64;
@@ -815,7 +819,7 @@ int fspad_attn_mtiles(const fspad_ctx *ctx, int N, int B, int sms)
 
 int fspad_attn_umma_splits(const fspad_ctx *ctx, int N, int B, int sms)
 {
-    return fspad_attn_ranges(ctx, N, B, sms, (ctx->cfg.max_len + umma::BK - 1) / umma::BK);
+    return fspad_attn_ranges(ctx, N, B, sms, (ctx->cfg.max_len + umma::BK - 1) / umma::BK, false);
 }
 
 // ---- TMA descriptors of the K and V cache planes ----------------------------------------

@@ -110,7 +110,7 @@ int fspad_attn_umma_splits(const fspad_ctx *c, int N, int B, int sms)
     const int s = (sms > 0 ? sms : kSms) / (B * c->cfg.n_kv_heads * fspad_attn_mtiles(c, N, B, sms)), chunks = (c->cfg.max_len + 127) / 128;
     return chunks <= 5 || s < 1 ? 1 : s < chunks ? s : chunks;
 }
-int fspad_attn_ranges(const fspad_ctx *c, int N, int B, int sms, int) { return fspad_attn_umma_splits(c, N, B, sms); }
+int fspad_attn_ranges(const fspad_ctx *c, int N, int B, int sms, int, bool) { return fspad_attn_umma_splits(c, N, B, sms); }
 int fspad_draft_expand_pieces(int V) { return (V + 4095) / 4096; }
 int fspad_lm_head_tiles(int V) { return (V + 127) / 128; }
 int fspad_walk_ctas(fspad_ctx *, int B, int V)
