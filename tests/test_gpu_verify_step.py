@@ -200,6 +200,74 @@ def test_row_tiles_in_pairs_of_ctas(n_nodes, group, alias):
     assert torch.equal(outs["attn_out"], want)
 
 
+@pytest.mark.parametrize("mode", ["sample", "mixed", "zero"])
+@pytest.mark.parametrize("vocab,heads,n_layers", [
+    (33000, 10, 4),        # clusters of 16 CTAs, 80 slices: half a slice a warp
+    (33000, 32, 4),        # 256 slices
+    (16500, 32, 2),        # clusters of eight, 128 slices
+])
+def test_step_in_one_stream_beside_clusters(mode, vocab, heads, n_layers):
+    """Three sequences whose walks take a cluster each, the attention beside them, the cache compacted by the walk's CTAs (a sequence
+    of temperature 0: by one of them).  Three launches and no more say that it went this way."""
+    temps = {"sample": (1.0, 0.8, 1.0), "mixed": (0.0, 1.0, 0.0), "zero": (0.0, 0.0, 0.0)}[mode]
+    w = synth.scaled(W["llama3_8b_2k"], batch=3, n_q_heads=heads, n_kv_heads=heads, prefix=(40, 500), n_nodes=24, depth=4, branch=4,
+                     vocab=vocab, temperatures=temps if mode != "zero" else (1.0, 1.0, 1.0))
+    inp = synth.generate(w, 21)
+    inp.temperature[:] = temps
+    B, N = inp.parent.shape
+    cache_host = synth.make_cache(inp, n_layers)
+    for b, L in enumerate(inp.prefix_len.tolist()):
+        cache_host[0, 0, b, :, L:L + N], cache_host[0, 1, b, :, L:L + N] = inp.tree_k[b], inp.tree_v[b]
+    ref = _oracle_step(inp, cache_host, 0)
+    ctx = helpers.make_ctx(inp, n_layers=n_layers)
+    d, a, outs, cache = _device_inputs(inp, cache_host)
+    before = ctx.launch_count()
+    _call(ctx, cache, a, d, outs, False, 0)
+    assert ctx.launch_count() - before == 3              # scan, walk, attention
+    ctx.check()
+    _check(inp, outs, cache, *ref)
+
+
+@pytest.mark.parametrize("mode,heads,prefix,max_len", [("sample", 32, 300, 400), ("sample", 8, 1000, 16384), ("greedy", 32, 300, 400),
+                                                       ("sample", 8, 1000, 1100)])
+def test_inputs_rewritten_between_steps(mode, heads, prefix, max_len):
+    """Trees, lengths, queries and logits rewritten in place by kernels right before each step, with nothing waited for: every step
+    sees its own, whichever stream its attention takes and however early that starts."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=1, n_q_heads=heads, n_kv_heads=heads, prefix=(prefix, prefix), n_nodes=24, depth=4, branch=4,
+                     vocab=33000, temperatures=(1.0 if mode == "sample" else 0.0,))
+    sets = []
+    for k in range(3):
+        inp = synth.generate(w, 30 + k)
+        assert inp.parent.shape[1] == 24
+        inp.prefix_len[:] = prefix - 37 * k
+        d, a, outs, _ = _device_inputs(inp, np.zeros((1, 2, 1, 1, 1, 1), np.uint16))
+        cache = torch.randn((1, 2, 1, heads, max_len, 128), device="cuda").to(torch.bfloat16)
+        sets.append((d, a, cache))
+    ctx = binding.Context(heads, heads, w.vocab, max_len, max_nodes=24)
+    live = ({k: None if t is None else t.clone() for k, t in sets[0][0].items()}, {k: t.clone() for k, t in sets[0][1].items()}, sets[0][2].clone())
+
+    def step(k, wait):
+        for src, dst in ((sets[k][0], live[0]), (sets[k][1], live[1]), ({"c": sets[k][2]}, {"c": live[2]})):
+            for name, t in src.items():
+                if t is not None:
+                    torch.add(t, 0, out=dst[name])       # (a kernel, not a copy)
+        if wait:
+            torch.cuda.synchronize()
+        res = {key: torch.empty_like(t) for key, t in outs.items()}
+        _call(ctx, live[2], live[1], live[0], res, False, 0)
+        if wait:
+            ctx.check()
+        return [res[key] for key in ("attn_out", "path", "n_acc", "bonus", "new_len")] + [live[2].clone()]
+
+    want = [step(k, True) for k in range(3)]
+    assert not torch.equal(want[0][0], want[1][0]) and len({tuple(x[1][0].tolist()) for x in want}) > 1
+    got = [step(k % 3, False) for k in range(12)]
+    ctx.check()
+    for k, res in enumerate(got):
+        for g, r in zip(res, want[k % 3]):
+            assert torch.equal(g, r), k
+
+
 def test_argument_errors():
     w = synth.scaled(W["llama3_8b_2k"], batch=1, prefix=(40, 40), n_nodes=8, depth=3, branch=3, vocab=100,
                      temperatures=(0.0,))

@@ -33,6 +33,31 @@ def test_attention(tree, n, hq, hkv, prefix):
     _attn_check(synth.generate(w, 1, with_accept=False), alias=(n == 128))
 
 
+@pytest.mark.parametrize("hq,hkv,prefix,n", [(8, 2, 700, 200), (4, 4, 1000, 130), (8, 1, 900, 256), (4, 4, 641, 65), (8, 2, 1151, 129)])
+@pytest.mark.parametrize("alias", [False, True])
+def test_tree_across_key_ranges(hq, hkv, prefix, n, alias):
+    """One or two chunks a range: the tree's rows fall into two or three of them, and a row's way to the root begins above the last key of
+    the lower ones; what lies behind the last row (or, with the rows apart, behind the prefix) is NaN."""
+    w = synth.scaled(W["llama3_8b_2k"], n_q_heads=hq, n_kv_heads=hkv, prefix=(prefix, prefix), n_nodes=n, depth=8, branch=10, vocab=16)
+    inp = synth.generate(w, n, with_accept=False)
+    N = inp.parent.shape[1]
+    for plane in (inp.k_cache, inp.v_cache):
+        plane[:, :, prefix + (N if alias else 0):] = 0x7FC0
+    _attn_check(inp, alias)
+
+
+@pytest.mark.parametrize("bad", [(60, 70), (199, -2), (5, 5)])
+def test_bad_tree_across_key_ranges_is_reported(bad):
+    """Parents behind their child, missing, or the node itself, in a range with the root and in ranges without it."""
+    w = synth.scaled(W["llama3_8b_2k"], n_q_heads=8, n_kv_heads=2, prefix=(720, 720), n_nodes=200, depth=8, branch=10, vocab=16)
+    inp = synth.generate(w, 0, with_accept=False)
+    inp.parent[0, bad[0]] = bad[1]
+    ctx = helpers.make_ctx(inp)
+    d = helpers.upload_attn(inp)
+    ctx.tree_attn(d["q"], d["k_cache"], d["v_cache"], d["tree_k"], d["tree_v"], d["parent"], d["prefix_len"])
+    assert ctx.status() == -8
+
+
 def test_attention_bad_tree_is_reported():
     w = synth.scaled(W["llama3_8b_2k"], n_q_heads=8, n_kv_heads=2, prefix=(100, 100), n_nodes=150, depth=8, branch=10, vocab=16)
     inp = synth.generate(w, 0, with_accept=False)
