@@ -8,14 +8,16 @@ no fallback: if the library has not been built the first call raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
 import torch
 
+from .build import calls_path
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libfspad.so")
-CALLS_PATH = os.path.join(_PKG, "_pycall.so")
 _lib = None
 _native = None
 
@@ -81,10 +83,13 @@ def _calls():
     global _native
     if _native is None:
         load()
-        if not os.path.exists(CALLS_PATH):
-            raise RuntimeError("_pycall.so is missing: build it with `python -m paper_2408_15562_b200.build`")
-        from . import _pycall
-        _native = _pycall
+        path = calls_path()
+        if not os.path.exists(path):
+            raise RuntimeError("%s is missing: build it with `python -m paper_2408_15562_b200.build`" % os.path.basename(path))
+        spec = importlib.util.spec_from_file_location(__package__ + "._pycall", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native = module
     return _native
 
 

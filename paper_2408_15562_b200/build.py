@@ -11,7 +11,6 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libfspad.so")
 HEADER = os.path.join(ROOT, "include", "fspad.h")
-CALLS = os.path.join(PKG, "_pycall.so")
 CALLS_SRC = os.path.join(CSRC, "pycall.cpp")
 SOURCES = ["api.cu", "accept_stats.cu", "accept_walk.cu", "kv_compact.cu", "tree_attn.cu", "tree_attn_umma.cu", "tree_build.cu", "draft_expand.cu", "lm_head.cu", "feature_sampler.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -30,19 +29,31 @@ def _newest_source() -> float:
     return max(os.path.getmtime(f) for f in files)
 
 
+def calls_path() -> str:
+    """The Python calls are built for one torch and one interpreter, which the file's name says: another torch lays out its tensors
+    in another way, and must not come upon this file."""
+    import torch
+    return os.path.join(PKG, "_pycall.torch-%s%s" % (torch.__version__, sysconfig.get_config_var("EXT_SUFFIX")))
+
+
 def _build_calls(force: bool) -> None:
-    """The Python calls of the C ABI (g++ against torch's headers), linked with the library beside it."""
-    if not force and os.path.exists(CALLS) and os.path.getmtime(CALLS) >= max(os.path.getmtime(CALLS_SRC), os.path.getmtime(HEADER)):
+    """The Python calls of the C ABI (g++ against torch's headers), linked with the library beside it.  torch's own libraries are in
+    the process by the time it is imported and are found by their names."""
+    calls = calls_path()
+    if not force and os.path.exists(calls) and os.path.getmtime(calls) >= max(os.path.getmtime(CALLS_SRC), os.path.getmtime(HEADER)):
         return
     import torch
-    t = os.path.join(os.path.dirname(torch.__file__))
-    tmp = CALLS + ".tmp.%d" % os.getpid()
+    t = os.path.dirname(torch.__file__)
+    tmp = calls + ".tmp.%d" % os.getpid()
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I" + os.path.dirname(HEADER),
                            "-I" + os.path.join(t, "include"), "-I" + os.path.join(t, "include", "torch", "csrc", "api", "include"),
                            "-I" + sysconfig.get_paths()["include"], "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
                            CALLS_SRC, "-o", tmp, "-L" + PKG, "-l:" + os.path.basename(LIB), "-L" + os.path.join(t, "lib"),
-                           "-ltorch_python", "-ltorch_cpu", "-lc10", "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + os.path.join(t, "lib")])
-    os.replace(tmp, CALLS)
+                           "-ltorch_python", "-ltorch_cpu", "-lc10", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, calls)
+    for f in os.listdir(PKG):
+        if f.startswith("_pycall") and f.endswith(".so") and f != os.path.basename(calls):
+            os.remove(os.path.join(PKG, f))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -53,3 +53,15 @@ def test_an_argument_without_ordinary_storage_raises(what, want):
     r = subprocess.run([sys.executable, "-c", SCRIPT, what], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0, (r.returncode, r.stderr[-500:])
     assert "Error" in r.stdout and r.stdout.startswith(want), r.stdout
+
+
+def test_calls_built_for_another_torch_are_not_loaded(monkeypatch):
+    import torch
+
+    from paper_2408_15562_b200 import binding, build
+    build.build()
+    assert binding._calls() is not None and torch.__version__ in build.calls_path()
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    with pytest.raises(RuntimeError, match="missing"):
+        binding._calls()
