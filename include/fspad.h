@@ -95,10 +95,11 @@ long long fspad_launch_count(const fspad_ctx *ctx);
 
 /*
  * Self-test of the library's bounded device-side waits (error handling of the
- * library; no passage of the paper).  Every wait of a kernel on a barrier has
- * a poll limit; when it runs out the kernel records FSPAD_ERR_TIMEOUT in the
- * status word and returns.  This call queues one warp that waits, with a limit
- * of `polls` polls (1 .. 4096), on a barrier nothing ever arrives on, and then a
+ * library; no passage of the paper).  Every wait of a kernel on a barrier is
+ * limited to a number of tries, of a microsecond at most where the thread sleeps
+ * in hardware (some 0.2 s a wait); when they run out the kernel records
+ * FSPAD_ERR_TIMEOUT in the status word and returns.  This call queues one warp that waits,
+ * with a limit of `polls` tries (1 .. 4096), on a barrier nothing ever arrives on, and then a
  * pair of CTAs of which one waits in the same way for the other's message: after
  * it fspad_status() returns FSPAD_ERR_TIMEOUT, and the context stays usable.
  */
@@ -419,15 +420,18 @@ int fspad_kv_compact_paged(fspad_ctx *ctx, fspad_bf16 *pool, const int32_t *bloc
  * `attn_layer` of `cache`), fspad_tree_accept and fspad_kv_compact queued one
  * after the other on `stream`, with the same arguments, outputs and errors, but
  * the attention runs beside the acceptance (they share no data): as a
- * programmatic dependent in `stream` where it is the longer of the two, else on a
- * second stream owned by the context, forked from and joined back into `stream`
- * with events.  Compaction follows the
+ * programmatic dependent in `stream`, or on a second stream owned by the context, forked
+ * from and joined back into `stream` with events.  Which of the two, and into how many ranges
+ * the keys are cut, follows from the context (max_len among it: up to 640 rows there is
+ * one range), n_nodes and batch; the order, not the cut and so not the results, also from whether `stream` is being
+ * captured.  Compaction follows the
  * acceptance directly when tree_k / tree_v are given (attention then never
  * reads the cache rows compaction rewrites); when they are NULL (tree rows
  * taken from cache rows L_b ..) compaction waits for the attention as well.
  * In the first case, when a sequence has at most 64 (layer, K/V, kv head)
- * slices (where a sampling step stays in one stream, 32 for each CTA of the walk's cluster, up to 256), the kernel
- * that walks the tree makes the compaction's moves itself, greedy or sampling (same result; an invalid prefix length is then reported by
+ * slices (where a sampling step stays in one stream, 32 for each CTA of the walk's cluster,
+ * up to 256), the kernel that walks the tree makes the compaction's moves itself,
+ * greedy or sampling (same result; an invalid prefix length is then reported by
  * that kernel).
  * Work queued on `stream` after the call sees every output.  The call only
  * enqueues work and records / waits on events, so it may be captured into a

@@ -99,15 +99,15 @@ def strerror(code: int) -> str:
 
 # The calls outside a decoding loop go through ctypes; those inside it through `_pycall` (csrc/pycall.cpp), which makes the same
 # checks.
-def _ptr(t: Optional[torch.Tensor], dtype, device_type: str = "cuda"):
+def _ptr(t: Optional[torch.Tensor], dtype):
     if t is None:
         return None
     if t.dtype is not dtype:
         raise TypeError("expected %s, got %s" % (dtype, t.dtype))
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    if not t.is_cuda if device_type == "cuda" else t.device.type != device_type:
-        raise ValueError("tensor must live on %s, not %s" % (device_type, t.device))
+    if not t.is_cuda:
+        raise ValueError("tensor must live on cuda, not %s" % t.device)
     return t.data_ptr()
 
 
@@ -162,7 +162,6 @@ class Context:
         B, N = q.shape[0], q.shape[1]
         if out is None:
             out = torch.empty_like(q)
-        bf = torch.bfloat16
         rc = _calls().tree_attn(self._h.value, q, k_cache, v_cache, tree_k, tree_v, parent, prefix_len, N, B, out,
                                 _stream(stream))
         if rc != 0:
@@ -179,7 +178,6 @@ class Context:
             n_accepted = torch.empty((B,), dtype=torch.int32, device=dev)
         if bonus_token is None:
             bonus_token = torch.empty((B,), dtype=torch.int32, device=dev)
-        f32, i32 = torch.float32, torch.int32
         rc = _calls().tree_accept(self._h.value, target_logits, draft_probs, draft_tokens, parent, temperature,
                                   uniforms, N, B, accepted_path, n_accepted, bonus_token, _stream(stream))
         if rc != 0:
@@ -209,7 +207,6 @@ class Context:
         B, N = q.shape[0], q.shape[1]
         if out is None:
             out = torch.empty_like(q)
-        bf, i32 = torch.bfloat16, torch.int32
         rc = _calls().tree_attn_paged(self._h.value, q, k_pool, v_pool, block_table, block_table.shape[1],
                                       k_pool.shape[0], tree_k, tree_v, parent, prefix_len, N, B, out, _stream(stream))
         if rc != 0:
@@ -250,7 +247,7 @@ class Context:
         """hidden [B][N][H] -> acceptance result, the logits' scan fused behind the LM-head product."""
         B, N, H = hidden.shape
         dev = hidden.device
-        i32, f32, bf = torch.int32, torch.float32, torch.bfloat16
+        i32 = torch.int32
         if accepted_path is None:
             accepted_path = torch.empty((B, self.cfg.max_nodes), dtype=i32, device=dev)
         if n_accepted is None:
@@ -298,7 +295,6 @@ class Context:
         B = prefix_len.shape[0]
         if new_len is None:
             new_len = torch.empty((B,), dtype=torch.int32, device=cache.device)
-        i32 = torch.int32
         rc = _calls().kv_compact(self._h.value, cache, accepted_path, n_accepted, prefix_len, B, new_len,
                                  _stream(stream))
         if rc != 0:
@@ -345,7 +341,6 @@ class Context:
         """The whole verify step on device tensors: attention beside
         acceptance, then compaction; outputs are written in place."""
         B, N = q.shape[0], q.shape[1]
-        bf, f32, i32 = torch.bfloat16, torch.float32, torch.int32
         rc = _calls().verify_step(self._h.value, cache, attn_layer, q, tree_k, tree_v, parent, prefix_len,
                                   target_logits, draft_probs, draft_tokens, temperature, uniforms, N, B, attn_out,
                                   accepted_path, n_accepted, bonus_token, new_len, _stream(stream))

@@ -90,7 +90,7 @@ skinny_gemm_kernel(const Args a, const __grid_constant__ CUtensorMap tmA0, const
 
     if (warp == 0) {
         // ================= copy warp =================
-        // one thread's loop (its waits are plain polls; nothing is shuffled to the other lanes)
+        // one thread's loop (which waits on its own; nothing is shuffled to the other lanes)
         int it = 0;
         if (lane == 0) {
             for (int j = 0; j < my_items; ++j) {

@@ -150,7 +150,7 @@ lm_head_stats_kernel(const Args a, const __grid_constant__ CUtensorMap tmW, cons
     bool failed = false;
 
     if (warp == 0) {
-        // ================= copy warp: one thread runs the whole loop (its waits are plain polls) =================
+        // ================= copy warp: one thread runs the whole loop (and waits on its own) =================
         if (lane == 0) {
             int s = 0;
             uint32_t ph = 0;                     // flips each time the ring wraps

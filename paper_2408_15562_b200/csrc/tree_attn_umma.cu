@@ -894,7 +894,7 @@ cudaError_t fspad_launch_attn_umma_split(fspad_ctx *ctx, const fspad_bf16 *q, co
     a.block_table = paged.table; a.table_stride = paged.stride; a.n_blocks = paged.n_blocks;
     const bool in_pairs = !paged.alone && fspad_attn_pairs(ctx, N, B, sms);
     a.mtiles = in_pairs ? fspad_attn_mtiles(ctx, N, B, sms) : (a.M + umma::BM - 1) / umma::BM;
-    // (every CTA ranks all sequences itself, B loads each for B / 320 of its threads: kept to batches where that is small change)
+    // (every warp ranks all sequences itself, up to four loads a lane and a shuffle a sequence: kept to batches where that is small change)
     a.longest_first = (B > 1 && B <= 128 && (long long)B * c.n_kv_heads * a.mtiles * n_splits > ctx->sm_count) ? 1 : 0;
     a.scale_log2 = scale_log2;
     a.part_o = ctx->part_o; a.part_ml = ctx->part_ml; a.out = n_splits == 1 ? out : nullptr; a.status = ctx->d_status;
