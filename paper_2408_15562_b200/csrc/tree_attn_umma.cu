@@ -25,10 +25,10 @@
 // What bounds it.  A chunk takes a CTA 2000 cycles: the softmax threads' own chain (wait,
 // scores from tensor memory, maximum, 64 exponentials, P back, arrival: 1500 to 1600 busy, of which
 // 1024 are the special-function units' when both groups are at it), beside 1050 of the tensor cores.  Around the
-// loop stand, in cycles, 5000 to the first scores and 5000 from the last product to the end (9600 and
-// 10000 before the tail's gather, the wide prologue's barriers and the row-by-row stores went).  One B200, us a call:
-// 52 heads and 4 K keys 34.8 -> 29.5, 8 heads of 8 and 8 K 33.3 -> 28.4, 16 ragged sequences 84.8 -> 66.6, four paged
-// sequences of 130 nodes 56.9 -> 40.2.
+// loop stood 9600 cycles to the first scores (18500 in a pair), 5500 and 4700 of the tail's gather by the copy warp and 4000 (7000)
+// behind the last product, before Q came by TMA, the gather went ahead of the loop and the rows left as whole lines.  One B200, us a
+// call, that kernel and this one: 52 heads and 4 K keys 34.2 -> 29.9, 8 heads of 8 and 8 K 32.6 -> 28.6, 16 sequences of 2.2 K
+// 70.3 -> 56.8, four paged sequences of 130 nodes and 1.3 K keys 74.2 -> 39.1.
 //
 // Every wait on an mbarrier is bounded; on expiry the CTA records
 // FSPAD_ERR_TIMEOUT, skips the remaining tensor-core work, frees its tensor
@@ -800,9 +800,10 @@ int fspad_attn_ranges(const fspad_ctx *ctx, int N, int B, int sms, int chunks, b
 // themselves (a batch: one key range per row, long loops) go in pairs where there are two or more, the last pair possibly with an empty half.
 // us a step, pairs against lone CTAs, called one by one / from a graph: 16 ragged sequences 193 / 189 against 186 / 198, five of 4 K
 // keys 139 / 105 against 144 / 110, twelve of 100 to 400 130 / 128 against 130 / 133; nine at 32000 tokens 86 / 86 against 80 / 80.
-// A call that has the SMs for itself (FspadPaged::alone) takes lone CTAs: faster at every one of 120 shapes (33 to 250 nodes, 1 to 8 heads a
-// group, 5 to 16 sequences, 150 to 4096 keys): 58.5 -> 42.9 us on eight sequences of 4 K (whose chunks take pairs in step with one another
-// 1.4 us, lone CTAs 1.0), 69 -> 62 on 16 ragged ones, 41.4 -> 30.9 on four of 130 nodes.
+// A call that has the SMs for itself (FspadPaged::alone) takes lone CTAs: of 160 shapes (33 to 250 nodes, 1 to 8 heads a group, 5 to 16
+// sequences, 150 to 4096 keys) they were slower at a few of nine sequences or more and 4 K keys, by up to 3 %, and faster at all others:
+// 58.5 -> 42.9 us on eight sequences of 4 K (whose chunks take pairs in step with one another 1.4 us, lone CTAs 1.0), 69 -> 62 on 16
+// ragged ones, 41.4 -> 30.9 on four of 130 nodes.
 // Where the keys are split as well, the loops are short and the pair's hand-shakes cost more than
 // it saves: 23.6 against 19.5 us with two chunks a CTA, 40 against 38 us with 17.
 bool fspad_attn_pairs(const fspad_ctx *ctx, int N, int B, int sms)
