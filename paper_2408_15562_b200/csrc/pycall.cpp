@@ -6,6 +6,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <exception>
 #include <tuple>
 #include <utility>
 
@@ -82,23 +83,26 @@ bool convert(PyObject *o, bool on_gpu, A *out)
 }
 
 // host_from: the first argument whose tensors lie in host memory.  A tensor may throw when it is asked for its strides or its address
-// (one inside vmap or grad, for instance): as in torch's own methods that becomes the Python exception.
+// (one inside vmap or grad, for instance): by torch's own translation that becomes the Python exception.
 template <typename... A, size_t... I>
 PyObject *invoke(int (*fn)(A...), PyObject *const *args, Py_ssize_t n, size_t host_from, std::index_sequence<I...>)
 {
-    HANDLE_TH_ERRORS
     if (n != (Py_ssize_t)sizeof...(A)) {
         PyErr_Format(PyExc_TypeError, "%zd arguments, not %zd", (Py_ssize_t)sizeof...(A), n);
         return nullptr;
     }
     std::tuple<A...> a{};
-    if (!(convert(args[I], I < host_from, &std::get<I>(a)) && ...)) return nullptr;
+    try {
+        if (!(convert(args[I], I < host_from, &std::get<I>(a)) && ...)) return nullptr;
+    } catch (...) {
+        torch::translate_exception_to_python(std::current_exception());
+        return nullptr;
+    }
     int rc;
     Py_BEGIN_ALLOW_THREADS
     rc = fn(std::get<I>(a)...);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
-    END_HANDLE_TH_ERRORS
 }
 template <typename... A>
 PyObject *invoke(int (*fn)(A...), PyObject *const *args, Py_ssize_t n, size_t host_from = 99)
