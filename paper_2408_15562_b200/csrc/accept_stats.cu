@@ -3,7 +3,9 @@
 // maximum, its lowest index and the sum of exponentials at the row's
 // temperature.  The strict comparison of the paper's verification stage
 // (Section "Preliminaries") needs the target's result for every tree node;
-// this kernel produces all of them in one HBM-bound sweep.
+// this kernel produces all of them in one HBM-bound sweep.  The walk that follows an acceptance's scan reads only
+// rows it comes to, and of a node without children only one, its last: on large arrays the scan of an acceptance
+// goes by the trees and leaves those nodes' rows out (accept_stats_inner_kernel).
 //
 // Layout: logits [rows][V] fp32, viewed as one flat array that is cut into
 // equal contiguous ranges, one per CTA (1024 threads per SM in a single wave:
@@ -215,6 +217,222 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
     }
 }
 
+// The same scan over the rows of the nodes that have children (a quarter of a 60-node tree's): the walk stops at a node without
+// children at most once, at its end, and looks at that row itself.  A parent that is no lower node counts as the root, as in the
+// walk.  Two ways of finding the rows:
+//   SHARED = false  few rows: a CTA for every piece of every row, gridDim.x pieces by gridDim.y rows, and those of a row that is
+//                   nobody's parent leave at once
+//   SHARED = true   every CTA marks the nodes that are somebody's parent, a bit a row, and numbers them; where their pieces are no
+//                   more than the CTAs it takes one, else an equal share of their rows laid end to end, the first loads of a run
+//                   being in flight while the one before it is reduced
+// Bound by HBM where the rows are many (240 of 128256: 26 us, 4.7 TB/s; the scan of all 960 80 us), by the chain of launch, parents,
+// loads and reduction where they are few (15 of 60 rows: 4.5 us; all 60 9.4).  A share may cross rows.  The run of a row that a CTA takes is reduced as a whole, and its result goes to slot 0 if the run begins
+// the row, else to the one behind the stretch of `wide` units it starts in: every share is at least that long, so no two meet.  The
+// slots in between are empty.
+template <bool SHARED>
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads)
+accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restrict__ temperature, int N, int rows, int V,
+                          const FspadStatsGeom g, int wide, FspadStatsPart *__restrict__ parts)
+{
+    typedef Unit<4> U4;
+    constexpr int kStep = kThreads * kDeep, kWords = SHARED ? FSPAD_INNER_MAX_ROWS / 32 : 1, kList = SHARED ? FSPAD_INNER_LIST : 1;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, upr = g.upr;
+    __shared__ unsigned word[kWords];
+    __shared__ int list[kList], warp_n[kThreads / 32];
+    __shared__ Acc wacc[kThreads / 32];
+    __shared__ float s_bmax;
+    __shared__ int s_barg;
+    unsigned hi = 0;                             // SHARED: end of the share, in units of the rows laid end to end (below 2^31)
+    int first = 0, last = 0;                     // the rows it touches, by number
+    bool one_piece = true;
+    if constexpr (SHARED)
+        if (tid < kWords) word[tid] = 0u;
+    static_assert(kWords <= kThreads, "a word to a thread");
+    struct Run {
+        const float4 *x;                         // its units off .. off + n - 1 of the row, from token j0 on (up to three in front of the row)
+        int row, off, j0, n, n_load;             // n_load: how many of them can be loaded whole (the rest has no token or ends the array)
+        float k;
+    };
+    auto open = [&](int row, int off, int n) {
+        Run q;
+        q.row = row;
+        q.off = off;
+        q.n = n;
+        q.j0 = 4 * off - (int)(((size_t)row * V) & 3);
+        q.x = reinterpret_cast<const float4 *>(logits + (size_t)row * V + q.j0);
+        q.n_load = min(n, (V - q.j0 + (row + 1 < rows ? 3 : 0)) >> 2);
+        const float T = temperature ? temperature[(unsigned)row / (unsigned)N] : 1.0f;
+        q.k = kLog2e / (T > 0.0f ? T : 1.0f);
+        return q;
+    };
+    // A unit that reaches out of its row is loaded whole, but for one that ends the array, and clipped when it is used: the threads
+    // that have one do not hold up their warp's loads.
+    auto batch = [&](float4 (&v)[kDeep], const Run &q, int base) {
+#pragma unroll
+        for (int u = 0; u < kDeep; ++u) {
+            const int i = base + u * kThreads + tid;
+            v[u] = i < q.n_load ? __ldg(q.x + i) : U4::pad();
+        }
+    };
+    fspad_pdl_wait();                            // (the order of the two: see the scan of all rows)
+    fspad_pdl_trigger();
+    Run q;
+    if constexpr (SHARED) {
+        __syncthreads();
+        int c = (int)((unsigned)tid % (unsigned)N);
+        const int step = (int)((unsigned)kThreads % (unsigned)N);
+#pragma unroll 4
+        for (int i = tid; i < rows; i += kThreads) {
+            const int p = __ldg(g.parent + i), r = i - c + ((unsigned)p < (unsigned)c ? p : 0);
+            atomicOr(&word[r >> 5], 1u << (r & 31));
+            c += step;
+            c -= c >= N ? N : 0;
+        }
+        __syncthreads();
+        unsigned mine = tid < kWords ? word[tid] : 0u;
+        const int cnt = __popc(mine);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) warp_n[wid] = incl;
+        __syncthreads();
+        int n_inner = 0, rank = incl - cnt;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) {
+            if (w < wid) rank += warp_n[w];
+            n_inner += warp_n[w];
+        }
+        one_piece = n_inner * g.per_row <= (int)gridDim.x;
+        int off;
+        if (one_piece) {
+            first = last = (int)((unsigned)blockIdx.x / (unsigned)g.per_row);
+            off = ((int)blockIdx.x - first * g.per_row) * (int)g.chunk;
+            if (first >= n_inner) return;
+            hi = (unsigned)(first * upr + min(upr, off + (int)g.chunk));
+        } else {
+            const unsigned total = (unsigned)(n_inner * upr), each = max((total + gridDim.x - 1) / gridDim.x, (unsigned)wide);
+            const unsigned lo = min(total, blockIdx.x * each);
+            hi = min(total, lo + each);
+            if (lo >= hi) return;
+            first = (int)(lo / (unsigned)upr);
+            last = (int)((hi - 1) / (unsigned)upr);
+            off = (int)(lo - (unsigned)(first * upr));
+        }
+        for (; mine != 0u && rank <= last; mine &= mine - 1u, ++rank)
+            if (rank >= first) list[rank - first] = tid * 32 + __ffs((int)mine) - 1;
+        __syncthreads();
+        q = open(list[0], off, min(upr - off, (int)(hi - (unsigned)(first * upr + off))));
+    } else {
+        const int row = (int)blockIdx.y, root = row - (int)((unsigned)row % (unsigned)N);
+        bool inner = row == root;
+        for (int c = tid + 1; c < N; c += kThreads) {
+            const int p = __ldg(g.parent + root + c);
+            inner |= p == row - root && p < c;
+        }
+        const int off = (int)blockIdx.x * (int)g.chunk, n = min((int)g.chunk, upr - off);
+        if (!__syncthreads_or(inner)) return;
+        q = open(row, off, n);                   // (n below 1: the piece is empty)
+    }
+    float4 cur[kDeep], nxt[kDeep];
+    batch(cur, q, 0);
+    for (int r = first;;) {
+        Run following = q;
+        Acc p{-INFINITY, 0.f, 0x7fffffff};
+        for (int base = 0; base < q.n; base += kStep) {
+            if (base + kStep < q.n) {
+                batch(nxt, q, base + kStep);
+            } else if (SHARED && r < last) {
+                following = open(list[r + 1 - first], 0, min(upr, (int)(hi - (unsigned)((r + 1) * upr))));
+                batch(nxt, following, 0);
+            }
+            if (g.shift) {
+#pragma unroll
+                for (int u = 0; u < kDeep; ++u) {
+                    const int i = base + u * kThreads + tid, j = q.j0 + 4 * i;
+                    if (i < q.n && j < V && (j < 0 || j + 4 > V)) {
+                        if (i >= q.n_load) {
+                            cur[u] = fspad_edge4(logits + (size_t)q.row * V, j, V, -INFINITY);
+                        } else {
+                            if (j < 0) cur[u].x = -INFINITY;
+                            if (j < -1 || j + 1 >= V) cur[u].y = -INFINITY;
+                            if (j < -2 || j + 2 >= V) cur[u].z = -INFINITY;
+                            if (j + 3 >= V) cur[u].w = -INFINITY;
+                        }
+                    }
+                }
+            }
+            float bm = U4::vmax(cur[0]);
+#pragma unroll
+            for (int u = 1; u < kDeep; ++u) bm = fmaxf(bm, U4::vmax(cur[u]));
+            if (bm > p.m) {
+                p.s = (p.m == -INFINITY) ? 0.f : p.s * ex2((p.m - bm) * q.k);
+                p.m = bm;
+                p.a = base;
+            }
+            if (p.m != -INFINITY) {
+                float s0 = 0.f;
+#pragma unroll
+                for (int u = 0; u < kDeep; ++u) s0 += U4::vsum(cur[u], p.m, q.k);
+                p.s += s0;
+            }
+#pragma unroll
+            for (int u = 0; u < kDeep; ++u) cur[u] = nxt[u];
+        }
+        const float my_m = p.m;
+        const int my_base = p.a;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float om = __shfl_xor_sync(0xffffffffu, p.m, o);
+            const float os = __shfl_xor_sync(0xffffffffu, p.s, o);
+            acc_merge(p, om, os, q.k);
+        }
+        if (lane == 0) wacc[wid] = p;
+        if (tid == 0) s_barg = 0x7fffffff;
+        __syncthreads();
+        if (wid == 0) {
+            Acc t = (lane < kThreads / 32) ? wacc[lane] : Acc{-INFINITY, 0.f, 0};
+#pragma unroll
+            for (int o = kThreads / 64; o > 0; o >>= 1) {
+                const float om = __shfl_xor_sync(0xffffffffu, t.m, o);
+                const float os = __shfl_xor_sync(0xffffffffu, t.s, o);
+                acc_merge(t, om, os, q.k);
+            }
+            if (lane == 0) { wacc[0] = t; s_bmax = t.m; }
+        }
+        __syncthreads();
+        const float bmax = s_bmax;
+        if (my_m == bmax && bmax != -INFINITY) {
+            int b = 0x7fffffff;
+#pragma unroll 1
+            for (int u = kDeep - 1; u >= 0; --u) {
+                const int i = my_base + u * kThreads + tid, j = q.j0 + 4 * i;
+                if (i < q.n) b = U4::first_eq(fspad_load4(logits + (size_t)q.row * V, j, V, -INFINITY), bmax, j, b);
+            }
+            atomicMin(&s_barg, b);
+        }
+        __syncthreads();
+        int own = SHARED ? q.off / (int)g.chunk : (int)blockIdx.x, stop = own + 1;
+        if (!one_piece) {
+            const int end = q.off + q.n;
+            own = q.off == 0 ? 0 : 1 + q.off / wide;
+            stop = end >= upr ? g.per_row : 1 + end / wide;
+        }
+        if (tid >= own && tid < stop) {
+            FspadStatsPart out;
+            out.m = -INFINITY; out.s = 0.f; out.a = 0x7fffffff; out.pad = 0;
+            if (tid == own) { out.m = wacc[0].m; out.s = wacc[0].s; out.a = s_barg; }
+            parts[(size_t)q.row * g.slots + tid] = out;
+        }
+        if (!SHARED || r == last) break;
+        __syncthreads();
+        ++r;
+        q = following;
+    }
+}
+
 // rows -> (max, sum, argmax) from the partials; one warp per row
 __global__ void __launch_bounds__(128)
 accept_stats_merge_kernel(const FspadStatsPart *__restrict__ parts, const FspadStatsGeom g,
@@ -263,6 +481,17 @@ cudaError_t fspad_launch_stats_partials(fspad_ctx *ctx, const float *logits, con
 {
     const bool aligned = (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
+    if (geom->parent != nullptr && aligned && rows % rows_per_seq == 0 && fspad_scan_inner(sms, rows, V)) {
+        *geom = fspad_stats_geom_inner(sms, rows, V, ctx->stats_slots, geom->parent);
+        const FspadStatsGeom &g = *geom;
+        const int wide = (g.upr + g.per_row - 2) / (g.per_row - 1);
+        ctx->launches++;
+        if (g.n_cta == rows * g.per_row)
+            return fspad_launch_opt(pdl, accept_stats_inner_kernel<false>, dim3(g.per_row, rows), dim3(kThreads), 0, st, 0, logits,
+                                    temperature, rows_per_seq, rows, V, g, wide, ctx->st_part);
+        return fspad_launch_opt(pdl, accept_stats_inner_kernel<true>, dim3(g.n_cta), dim3(kThreads), 0, st, 0, logits, temperature,
+                                rows_per_seq, rows, V, g, wide, ctx->st_part);
+    }
     *geom = fspad_stats_geom(sms, rows, V, aligned, ctx->stats_slots, true);
     ctx->launches++;
     return launch_partials(logits, temperature, rows_per_seq, V, *geom, ctx->st_part, st, pdl);

@@ -51,6 +51,7 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kMaxCluster = 16;
+constexpr int kGreedyCluster = 8;          // all sequences greedy, rows of nodes without children not scanned
 constexpr int kWalkThreads = 512;          // 128 registers each: a thread keeps 16 tokens of the node's rows in them
 constexpr int kWarps = kWalkThreads / 32;
 constexpr int kTile = 16;                  // tokens of a thread's chunk that later residual sweeps take from registers
@@ -107,7 +108,8 @@ struct Child {
 };
 
 // MAXN: capacity in tree nodes of this instance of the kernel (64 or FSPAD_MAX_NODES_WIDE)
-template <int MAXN> struct TreeShared {
+// INNER: the scan has gone by the trees and left out the rows of nodes without children
+template <int MAXN, bool INNER> struct TreeShared {
     int parent[MAXN];
     int tok[MAXN];
     int path[MAXN];
@@ -116,8 +118,14 @@ template <int MAXN> struct TreeShared {
     int len;
     int kv_L;                       // prefix length (where the walk compacts the cache)
 };
-template <int MAXN> struct SharedT {
-    TreeShared<MAXN> t;
+template <int MAXN> struct TreeShared<MAXN, true> : TreeShared<MAXN, false> {
+    unsigned char known[MAXN];      // the scan has been over the node's row
+    int last;                       // greedy: the node the walk ended at, if its row is still to be looked at, else -1
+    unsigned long long best;        // ... the row's maximum and where it is (see argmax_key)
+};
+// (The functions that are not inlined are instantiated by it, too, so that what one kind of walk calls has no say in the other's registers.)
+template <int MAXN, bool INNER> struct SharedT {
+    TreeShared<MAXN, INNER> t;
     alignas(128) double exp_tbl[kExpTable];      // 2^(i/16)
     // what thread 0 asks for and about which node (written by thread 0, read by all after a barrier)
     double S, C;                    // sum of exponentials in use, coefficient of the draft row
@@ -558,6 +566,80 @@ __device__ __noinline__ double block_scan(Shared &sh, double v, double *excl_out
     return woff + incl;
 }
 
+// The bonus draw from a row that the scan has left out: inverse CDF of its softmax.  Every CTA takes its own slice's maximum for the
+// row's; the slices' masses are brought to the largest of them when all have come, in one exchange.  `last`: the thread has the last
+// tokens of its CTA.  false: a wait ran out.
+template <class Shared>
+__device__ __forceinline__ bool draw_from_row(Shared &sh, const float *__restrict__ x, Chunk ck, bool last, int rank, int C, int par,
+                                           uint32_t phase, double invT, int V, int *bonus)
+{
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    float m = -INFINITY;
+#pragma unroll 1
+    for (int j = ck.lo; j < ck.hi; j += 16) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = fspad_load4(x, j + 4 * u, ck.hi, -INFINITY);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) m = fmaxf(m, fmaxf(fmaxf(v[u].x, v[u].y), fmaxf(v[u].z, v[u].w)));
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if (lane == 0) sh.warp_v[1][wid] = (double)m;
+    __syncthreads();
+    m = (float)sh.warp_v[1][lane % kWarps];
+#pragma unroll
+    for (int off = kWarps / 2; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    const ExpArg arg = exp_arg(m, invT);
+    double mine = 0.0;
+#pragma unroll 1
+    for (int j = ck.lo; j < ck.hi; j += 4) {
+        const float4 v = fspad_load4(x, j, ck.hi, -INFINITY);
+        mine += exp_neg(v.x, arg, sh.exp_tbl);
+        mine += exp_neg(v.y, arg, sh.exp_tbl);
+        mine += exp_neg(v.z, arg, sh.exp_tbl);
+        mine += exp_neg(v.w, arg, sh.exp_tbl);
+    }
+    double E, total;
+    const double P = block_scan(sh, mine, &E, &total);
+    const uint32_t bar = smem_addr(&sh.bar[par]);
+    if (tid == 0) expect_bytes(bar, C * 16);
+    if (tid < C) {
+        send_double(smem_addr(&sh.slot[par][0][rank]), bar, tid, total);
+        send_double(smem_addr(&sh.slot[par][1][rank]), bar, tid, (double)m);
+    }
+    if (!wait_cluster_all(sh, bar, phase)) return false;
+    const float own = lane < C ? (float)sh.slot[par][1][lane & (kMaxCluster - 1)] : -INFINITY;
+    float top = own;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
+    const double scale = exp_neg(own, exp_arg(top, invT), sh.exp_tbl);       // (lane r: CTA r's)
+    double cum = lane < C ? sh.slot[par][0][lane & (kMaxCluster - 1)] * scale : 0.0;
+#pragma unroll
+    for (int off = 1; off < kMaxCluster; off <<= 1) {
+        const double t = __shfl_up_sync(0xffffffffu, cum, off);
+        if (lane >= off) cum += t;
+    }
+    const double target = (double)sh.ubonus * __shfl_sync(0xffffffffu, cum, C - 1);
+    const double before = __shfl_sync(0xffffffffu, cum, rank > 0 ? rank - 1 : 0);
+    const int owner = __ffs((int)__ballot_sync(0xffffffffu, lane < C && cum > target)) - 1;
+    if (owner == rank) {
+        const double local = (target - (rank > 0 ? before : 0.0)) / __shfl_sync(0xffffffffu, scale, rank);
+        if (tid == 0) sh.sel = 0x7fffffff;
+        __syncthreads();
+        if (P > local) atomicMin(&sh.sel, tid);
+        __syncthreads();
+        // (the rounding of the two levels can leave no thread above the target: the last tokens of the CTA then take the draw)
+        if (tid == sh.sel || (sh.sel == 0x7fffffff && last && ck.lo < ck.hi)) {
+            int found = -1;
+            sweep_row(MODE_CDF, sh, x, x, nullptr, nullptr, 0, ck, false, arg, 0.0, -1, E, local, &found);
+            *bonus = found < 0 ? min(max(ck.lo, 0), V - 1) : found;
+        }
+    }
+    if (owner < 0 && rank == 0 && tid == 0) *bonus = 0;       // no positive weight anywhere
+    return true;
+}
+
 // Compaction of the accepted path by the CTAs that walked it (every CTA of the cluster holds the same path in
 // its shared memory): row L + path[j] -> row L + j of every (layer, K/V, head) slice of the sequence, one warp
 // per slice, eight rows in flight, every load of a batch before any of its stores (path[j] >= j and the path
@@ -618,10 +700,57 @@ __device__ __forceinline__ void check_node(int c, int V, int &p, int &t, int *st
     }
 }
 
+// The row of a node without children, which the scan by the trees has left out.  Maximum and lowest index in one word: the larger
+// word is the larger value or, of equal ones (the two zeros are), the lower index.
+__device__ __forceinline__ unsigned long long argmax_key(float m, int a)
+{
+    const unsigned u = __float_as_uint(m + 0.0f);
+    return ((unsigned long long)(u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u)) << 32) | (0xffffffffu - (unsigned)a);
+}
+// The largest key of row positions [lo, hi) of a row that starts `ph` positions behind a 16-byte boundary, into t.best (set to 0
+// before; the caller's barrier comes after).  Eight loads in flight a thread: on one CTA a 128256-token row is bound by what one SM
+// can have under way.
+template <typename Tree>
+__device__ __noinline__ void argmax_row(Tree &t, const float *__restrict__ x, int lo, int hi, int tid, int nthr)
+{
+    constexpr int kLoads = 8;
+    float m = -INFINITY;
+    int a = 0x7fffffff;
+#pragma unroll 1
+    for (int j0 = lo + 4 * tid; j0 < hi; j0 += 4 * kLoads * nthr) {
+        float4 v[kLoads];
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+            const int j = j0 + 4 * u * nthr;
+            v[u] = fspad_load4(x, j, hi, -INFINITY);
+        }
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+            const int j = j0 + 4 * u * nthr;
+            if (v[u].x > m) { m = v[u].x; a = j; }
+            if (v[u].y > m) { m = v[u].y; a = j + 1; }
+            if (v[u].z > m) { m = v[u].z; a = j + 2; }
+            if (v[u].w > m) { m = v[u].w; a = j + 3; }
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const float om = __shfl_xor_sync(0xffffffffu, m, off);
+        const int oa = __shfl_xor_sync(0xffffffffu, a, off);
+        if (om > m || (om == m && oa < a)) { m = om; a = oa; }
+    }
+    if ((tid & 31) == 0) atomicMax(&t.best, argmax_key(m, a));
+}
+__device__ __forceinline__ int argmax_of(unsigned long long key)
+{
+    const unsigned a = 0xffffffffu - (unsigned)key;
+    return a == 0x7fffffffu ? 0 : (int)a;        // (nothing above -inf anywhere)
+}
+
 // Greedy walk of one sequence by one CTA: strict comparison of the draft tokens with the target's argmax.  Every node looks
 // at its parent's argmax side by side; what is left for one thread is to follow the chain of matches.
-template <int MAXN>
-__device__ __forceinline__ void greedy_walk(TreeShared<MAXN> &t, const WalkArgs &args, int b, int N, int tid, int nthr, bool writer)
+template <bool INNER, int MAXN>
+__device__ __forceinline__ void greedy_walk(TreeShared<MAXN, INNER> &t, const WalkArgs &args, int b, int N, int tid, int nthr, bool writer)
 {
     if (tid < MAXN) t.next[tid] = MAXN;
     __syncthreads();
@@ -636,7 +765,16 @@ __device__ __forceinline__ void greedy_walk(TreeShared<MAXN> &t, const WalkArgs 
             cur = nx;
         }
         t.len = len;
-        if (writer) { args.n_acc[b] = len; args.bonus[b] = t.rowA[cur]; }
+        bool known = true;
+        if constexpr (INNER) {
+            known = t.known[cur] != 0;
+            t.last = known ? -1 : cur;
+            t.best = 0ull;
+        }
+        if (writer) {
+            args.n_acc[b] = len;
+            if (known) args.bonus[b] = t.rowA[cur];
+        }
     }
     __syncthreads();
     if (writer) {
@@ -646,14 +784,22 @@ __device__ __forceinline__ void greedy_walk(TreeShared<MAXN> &t, const WalkArgs 
     }
 }
 
-// All sequences greedy: one CTA per sequence, nothing of the sampling walk's apparatus.
-template <int MAXN>
+// All sequences greedy: one CTA per sequence, nothing of the sampling walk's apparatus.  INNER: the scan has gone by the trees, and
+// a cluster of CTAs shares the row of a node without children that the walk ends in.
+template <int MAXN, bool INNER>
 __global__ void __launch_bounds__(kWalkThreads)
 accept_greedy_kernel(const __grid_constant__ WalkArgs args)
 {
-    __shared__ TreeShared<MAXN> t;
-    const int b = blockIdx.x, tid = threadIdx.x, nthr = blockDim.x, N = args.N;
+    __shared__ TreeShared<MAXN, INNER> t;
+    __shared__ unsigned long long peer_best[kGreedyCluster];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int C = INNER ? (int)cluster.num_blocks() : 1, rank = INNER ? (int)cluster.block_rank() : 0;
+    const int b = blockIdx.x / C, tid = threadIdx.x, nthr = blockDim.x, N = args.N;
     fspad_pdl_trigger();
+    if constexpr (INNER) {
+        if (tid < MAXN) t.known[tid] = tid == 0;
+        __syncthreads();
+    }
     // (read before the scan has finished: see the sampling kernel)
     const float Tf = args.temperature[b];
     int p = -1, tk = 0;
@@ -663,6 +809,12 @@ accept_greedy_kernel(const __grid_constant__ WalkArgs args)
         check_node(tid, args.V, p, tk, args.status);
         t.parent[tid] = p;
         t.tok[tid] = tk;
+        if constexpr (INNER)
+            if (tid > 0) t.known[p] = 1;
+    }
+    if constexpr (INNER) {
+        __syncthreads();
+        cluster.barrier_arrive();
     }
     if (tid == 0 && args.kv_cache != nullptr) t.kv_L = args.kv_prefix[b];
     if (tid == 0 && !(Tf >= 0.0f)) fspad_report(args.status, FSPAD_ERR_RANGE);
@@ -673,19 +825,39 @@ accept_greedy_kernel(const __grid_constant__ WalkArgs args)
     for (int r0 = 0; r0 < N; r0 += nthr >> 3) {      // whole warps iterate together
         const int row = r0 + (tid >> 3);
         float M; double S; int A;
-        merge_row(args.parts, args.geom, b * N + row, row < N, 0.f, l8, M, S, A, nullptr, nullptr);
+        bool scanned = row < N;
+        if constexpr (INNER) scanned = scanned && t.known[row];
+        merge_row(args.parts, args.geom, b * N + row, scanned, 0.f, l8, M, S, A, nullptr, nullptr);
         if (l8 == 0 && row < N) t.rowA[row] = A;
     }
     __syncthreads();
-    greedy_walk(t, args, b, N, tid, nthr, true);
-    if (args.kv_cache != nullptr) compact_accepted(args, t, b, 0, 1, tid, nthr);
+    if constexpr (INNER) cluster.barrier_wait();     // (every CTA of the cluster is there before anything is written to it)
+    greedy_walk<INNER>(t, args, b, N, tid, nthr, rank == 0);       // every CTA of the cluster: same data, same path
+    if constexpr (INNER) {
+        if (t.last >= 0) {
+            const size_t start = ((size_t)b * N + t.last) * args.V;
+            const int ph = (int)(start & 3), each = (((args.V + 3 + C - 1) / C) + 3) & ~3;
+            argmax_row(t, args.logits + start, rank * each - ph, min(args.V, (rank + 1) * each - ph), tid, nthr);
+            __syncthreads();
+            if (tid == 0) *cluster.map_shared_rank(&peer_best[rank], 0) = t.best;  // (a word each: maxima of 64 bits sent to one word of a peer got lost)
+            cluster.sync();
+            if (rank == 0 && tid == 0) {
+                unsigned long long best = peer_best[0];
+                for (int r = 1; r < C; ++r) best = max(best, peer_best[r]);
+                args.bonus[b] = argmax_of(best);
+            }
+        }
+    }
+    if (args.kv_cache != nullptr) compact_accepted(args, t, b, rank, C, tid, nthr);
 }
 
-template <int MAXN>
+// INNER: the scan has gone by the trees.  (An instance of its own: the few instructions more cost a walk behind a scan of all rows half
+// a microsecond, and this one has no use for the pieces' masses.)
+template <int MAXN, bool INNER>
 __global__ void __launch_bounds__(kWalkThreads, 1)
 accept_walk_kernel(const __grid_constant__ WalkArgs args)
 {
-    typedef SharedT<MAXN> Shared;
+    typedef SharedT<MAXN, INNER> Shared;
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
@@ -734,7 +906,10 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     if (tid == 32 && args.kv_cache != nullptr) sh.t.kv_L = args.kv_prefix[b];
     // (the loads above are under way)
     if (tid < kExpTable) sh.exp_tbl[tid] = kExp2Tbl[tid];
-    if (tid < MAXN) sh.first_child[tid] = MAXN;
+    if (tid < MAXN) {
+        sh.first_child[tid] = MAXN;
+        if constexpr (INNER) sh.t.known[tid] = tid == 0;
+    }
     if (tid == 0) {
         sh.fail = 0;
         for (int i = 0; i < 2; ++i)
@@ -762,6 +937,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         sh.t.tok[tid] = t;
         if (tid >= 1) {
             atomicMin(&sh.first_child[p], tid);
+            if constexpr (INNER) sh.t.known[p] = 1;
             if (sampling) {
                 const size_t at = (size_t)p * V + t;
                 xv = lg[at];
@@ -812,7 +988,8 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     for (int r0 = 0; r0 < N; r0 += kWalkThreads / 8) {           // whole warps iterate together
         const int row = r0 + (tid >> 3), rs = row < N ? row : 0;
         float M; double S; int A;
-        merge_row(args.parts, args.geom, b * N + row, row < N, kT, l8, M, S, A, piece_w[rs], &sh.piece_cnt[rs]);
+        if constexpr (INNER) merge_row(args.parts, args.geom, b * N + row, row < N && sh.t.known[rs], kT, l8, M, S, A, nullptr, nullptr);
+        else merge_row(args.parts, args.geom, b * N + row, row < N, kT, l8, M, S, A, piece_w[rs], &sh.piece_cnt[rs]);
         if (l8 == 0 && row < N) { sh.rowM[row] = M; sh.rowS[row] = S; sh.t.rowA[row] = A; }
     }
     const double invT = 1.0 / (double)(sampling ? Tf : 1.0f);
@@ -833,7 +1010,15 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     __syncthreads();
 
     if (!sampling) {
-        greedy_walk(sh.t, args, b, N, tid, kWalkThreads, true);
+        greedy_walk<INNER>(sh.t, args, b, N, tid, kWalkThreads, true);
+        if constexpr (INNER) {
+            if (sh.t.last >= 0) {
+                const size_t start = (row0 + sh.t.last) * V;
+                argmax_row(sh.t, args.logits + start, -(int)(start & 3), V, tid, kWalkThreads);
+                __syncthreads();
+                if (tid == 0) args.bonus[b] = argmax_of(sh.t.best);
+            }
+        }
         if (args.kv_cache != nullptr) compact_accepted(args, sh.t, b, 0, 1, tid, kWalkThreads);
         return;   // (rank 0 of the cluster; no peer memory is touched)
     }
@@ -841,7 +1026,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     // ---- sampling ----
     const bool cache_ok = args.cache_ok != 0, in_regs = cache_ok && per_thr <= kTile;
     // parked values: [k][thread] (k-th position of each thread's chunk), conflict-free
-    unsigned char *node_cache = dyn_smem + N * kPieceBytes;
+    unsigned char *node_cache = dyn_smem + (INNER ? 0 : N * kPieceBytes);
     double *se = reinterpret_cast<double *>(node_cache) + tid;
     float *sq = reinterpret_cast<float *>(node_cache + (size_t)per_thr * kWalkThreads * sizeof(double)) + tid;
     int n_exch = 0;                              // exchanges so far
@@ -1145,8 +1330,20 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     // uncertainty of all the approximations together.  Otherwise, and for every other kind of
     // draw, the cluster sweeps the whole row exactly.
     bool settled = false;
-    const int n_piece = sh.piece_cnt[cur];
-    if (!sh.bonus_ok && c == 0.0 && sh.nrem == 0 && n_piece > 0) {
+    if constexpr (INNER) {
+        if (!sh.t.known[cur]) {                               // (a node without children: nothing was rejected there)
+            const Chunk ck = chunk_of((row0 + cur) * V, V, per_cta, per_thr, rank, tid);
+            const bool last = tid == kWalkThreads - 1 || ck.hi == V || ck.hi - ck.lo < per_thr || (tid + 1) * per_thr >= per_cta;
+            if (!draw_from_row(sh, x, ck, last, rank, C, n_exch & 1, (uint32_t)(n_exch >> 1) & 1u, invT, V, args.bonus + b)) {
+                if (tid == 0) fspad_report(args.status, FSPAD_ERR_TIMEOUT);
+                cluster.sync();                               // nobody leaves while a peer may still write to its shared memory
+                return;
+            }
+            settled = true;
+        }
+    }
+    const int n_piece = INNER ? 0 : sh.piece_cnt[cur];
+    if (!INNER && !sh.bonus_ok && c == 0.0 && sh.nrem == 0 && n_piece > 0) {
         // every warp scans the pieces' masses: prefix of the piece the target falls into
         double cum = lane < n_piece ? piece_w[cur][lane & (kPieceSlots - 1)] : 0.0;
         const double own = cum;
@@ -1318,39 +1515,42 @@ cudaError_t fspad_launch_walk_wait_selftest(fspad_ctx *ctx, int polls, cudaStrea
     return fspad_launch_opt(false, walk_wait_selftest_kernel, dim3(2), dim3(64), 0, st, 2u, ctx->d_status, (uint32_t)polls);
 }
 
+typedef void (*WalkKernel)(const WalkArgs);
+static WalkKernel walk_kernel(bool narrow, bool inner)
+{
+    if (narrow) return inner ? accept_walk_kernel<64, true> : accept_walk_kernel<64, false>;
+    return inner ? accept_walk_kernel<FSPAD_MAX_NODES_WIDE, true> : accept_walk_kernel<FSPAD_MAX_NODES_WIDE, false>;
+}
+
 // Cluster size of the sampling walk.  Once per context: raise the dynamic shared-memory limit and find
-// the largest cluster the device can co-schedule for this kernel: 16 (opt-in), else 8.  Small
+// the largest cluster the device can co-schedule for these kernels: 16 (opt-in), else 8.  Small
 // vocabularies do not need the whole cluster.  (Halving the clusters of a batch whose CTAs outnumber the
 // SMs was measured and not kept: on 16 sequences, half of them greedy and gone at once, the acceptance
 // took 186 us with clusters of 8 against 143 us with clusters of 16 in two waves.)
 static int walk_cluster_size(fspad_ctx *ctx, int B, int V)
 {
     if (ctx->walk_cluster == 0) {
-        ctx->walk_cluster = 8;
         constexpr int most = kSmemBudget + 64 * kPieceBytes, most_wide = kSmemBudgetWide + FSPAD_MAX_NODES_WIDE * kPieceBytes;
-        static_assert(most + sizeof(SharedT<64>) <= 227 * 1024 && most_wide + sizeof(SharedT<FSPAD_MAX_NODES_WIDE>) <= 227 * 1024,
+        static_assert(most + sizeof(SharedT<64, true>) <= 227 * 1024 && most_wide + sizeof(SharedT<FSPAD_MAX_NODES_WIDE, true>) <= 227 * 1024,
                       "shared memory of a CTA");
-        cudaFuncSetAttribute(accept_walk_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        cudaFuncSetAttribute(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most_wide);
-        if (cudaFuncSetAttribute(accept_walk_kernel<64>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaFuncSetAttribute(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                cudaSuccess) {
+        bool all = true;
+        for (int i = 0; i < 4; ++i) {
+            const WalkKernel k = walk_kernel(i & 1, i & 2);
+            const int bytes = i & 1 ? most : most_wide;
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            if (!all || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { all = false; continue; }
             cudaLaunchConfig_t probe = {};
             probe.gridDim = dim3(kMaxCluster);
             probe.blockDim = dim3(kWalkThreads);
-            probe.dynamicSmemBytes = most;
+            probe.dynamicSmemBytes = bytes;
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
             at[0].val.clusterDim.x = kMaxCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
             probe.attrs = at; probe.numAttrs = 1;
             int n = 0;
-            int n2 = 0;
-            cudaLaunchConfig_t probe2 = probe;
-            probe2.dynamicSmemBytes = most_wide;
-            if (cudaOccupancyMaxActiveClusters(&n, accept_walk_kernel<64>, &probe) == cudaSuccess && n >= 1 &&
-                cudaOccupancyMaxActiveClusters(&n2, accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, &probe2) == cudaSuccess && n2 >= 1)
-                ctx->walk_cluster = kMaxCluster;
+            all = cudaOccupancyMaxActiveClusters(&n, k, &probe) == cudaSuccess && n >= 1;
         }
+        ctx->walk_cluster = all ? kMaxCluster : 8;
         (void)cudaGetLastError();
     }
     int cluster = ctx->walk_cluster;
@@ -1375,11 +1575,15 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     a.N = N; a.V = V; a.path_stride = ctx->cfg.max_nodes; a.cache_ok = 0; a.draft_far = draft_far ? 1 : 0; a.B = B; a.sampled_first = 0;
     a.path = path; a.n_acc = n_acc; a.bonus = bonus; a.status = ctx->d_status;
 
+    const bool inner = geom.parent != nullptr;
     ctx->launches++;
     if (draft == nullptr || uniforms == nullptr) {               // every sequence greedy
-        if (N <= FSPAD_MAX_NODES)
-            return fspad_launch(accept_greedy_kernel<FSPAD_MAX_NODES>, dim3((unsigned)B), dim3(kWalkThreads), 0, st, 0, a);
-        return fspad_launch(accept_greedy_kernel<FSPAD_MAX_NODES_WIDE>, dim3((unsigned)B), dim3(kWalkThreads), 0, st, 0, a);
+        // a row that the scan has left out is looked at by a cluster of eight, 64 KB a CTA at 128256 tokens
+        unsigned c = inner ? (unsigned)kGreedyCluster : 1u;
+        while (c > 1 && (V + (int)c - 1) / (int)c < 4096) c >>= 1;
+        return fspad_launch(N <= 64 ? inner ? accept_greedy_kernel<64, true> : accept_greedy_kernel<64, false>
+                                    : inner ? accept_greedy_kernel<FSPAD_MAX_NODES_WIDE, true> : accept_greedy_kernel<FSPAD_MAX_NODES_WIDE, false>,
+                            dim3((unsigned)B * c), dim3(kWalkThreads), 0, st, inner ? c : 0u, a);
     }
     const int cluster = walk_cluster_size(ctx, B, V);
     // (16 sequences, half of them sampling: the walk 75 -> 68 us beside the attention, the step 202 -> 199; with one wave of clusters
@@ -1388,11 +1592,8 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     const size_t per_cta = (size_t)((((V + 3 + cluster - 1) / cluster) + 3) & ~3);       // as the kernel shares a row out
     const size_t per_thr = ((per_cta + kWalkThreads - 1) / kWalkThreads + 3) & ~(size_t)3;
     const size_t need = per_thr * kWalkThreads * (sizeof(double) + sizeof(float));
-    size_t smem = (size_t)N * kPieceBytes;
+    size_t smem = inner ? 0 : (size_t)N * kPieceBytes;
     if (need <= (size_t)(N <= 64 ? kSmemBudget : kSmemBudgetWide)) { smem += need; a.cache_ok = 1; }
     // trees of up to 64 nodes and of up to FSPAD_MAX_NODES_WIDE nodes are two instances of the kernel
-    if (N <= 64)
-        return fspad_launch(accept_walk_kernel<64>, dim3((unsigned)(B * cluster)), dim3(kWalkThreads), smem, st, (unsigned)cluster, a);
-    return fspad_launch(accept_walk_kernel<FSPAD_MAX_NODES_WIDE>, dim3((unsigned)(B * cluster)), dim3(kWalkThreads), smem, st,
-                        (unsigned)cluster, a);
+    return fspad_launch(walk_kernel(N <= 64, inner), dim3((unsigned)(B * cluster)), dim3(kWalkThreads), smem, st, (unsigned)cluster, a);
 }

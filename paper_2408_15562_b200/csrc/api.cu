@@ -321,6 +321,7 @@ int fspad_tree_accept(fspad_ctx *ctx, const float *target_logits, const float *d
     if (batch == 0) return FSPAD_OK;
     cudaStream_t st = fspad_stream(stream);
     FspadStatsGeom geom;
+    geom.parent = parent;
     cudaError_t e = fspad_launch_stats_partials(ctx, target_logits, temperature, batch * n_nodes, n_nodes,
                                                 ctx->cfg.vocab, &geom, st);
     if (e != cudaSuccess) return FSPAD_ERR_CUDA;
@@ -530,6 +531,7 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
     const int attn_sms = plan.attn_sms;
     cudaError_t ce = cudaSuccess;
     FspadStatsGeom geom;
+    geom.parent = parent;
     const int rows = batch * n_nodes;
     // With the tree rows given apart from the cache the compaction depends on the walk alone, and when the
     // sequence's slices are few (a warp takes one after another: four each for the 16 warps of a greedy walk's CTA) the walk makes the moves itself at its end: one dependent launch less on the step's
@@ -721,6 +723,7 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
          cudaMemcpyAsync(attn_out, ctx->h_out, q_bytes, cudaMemcpyDeviceToHost, ctx->side) == cudaSuccess;
     const bool joined = cudaEventRecord(ctx->ev_join, ctx->side) == cudaSuccess;
     FspadStatsGeom geom;
+    geom.parent = ctx->h_parent;
     ok = ok && fspad_launch_stats_partials(ctx, ctx->h_logits, ctx->h_temp, batch * n_nodes, n_nodes, c.vocab, &geom, st) == cudaSuccess;
     ok = ok && fspad_launch_accept_walk(ctx, ctx->h_logits, draft, ctx->h_tokens, ctx->h_parent, ctx->h_temp,
                                         draft_probs ? ctx->h_unif : nullptr, geom, n_nodes, batch, c.vocab, ctx->h_path, ctx->h_nacc,

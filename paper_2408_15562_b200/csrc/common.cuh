@@ -87,6 +87,10 @@ struct FspadStatsGeom {
     long long total;   // rows * upr
     int per_row;       // > 0: ranges are cut at the rows, this many per row (the last may be shorter); 0: they may cross rows
     int threads;       // threads per CTA of the scan: FSPAD_STATS_THREADS, or half of it for a small array
+    // The trees [rows / rows_per_seq][rows_per_seq] the rows belong to: rows of nodes without children (other than a root) have
+    // then no partials, and whoever walks into such a node looks at its row itself.  NULL: every row has them.  Set by the
+    // caller of fspad_launch_stats_partials, which puts it back to NULL where the scan reads every row after all.
+    const int *parent = nullptr;
 };
 
 // small_ctas: the scan may use CTAs of half the size when the array is small (the pieces, one of which the
@@ -150,6 +154,42 @@ static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, boo
     g.n_cta = (int)((g.total + g.chunk - 1) / g.chunk);
     g.per_row = g.upr % g.chunk == 0 ? (int)(g.upr / g.chunk) : 0;
     return g;
+}
+
+// Rows of the nodes that have children, of a batch of trees.
+#define FSPAD_INNER_MAX_ROWS 8192      /* one bit each, a word to a thread of the scan's CTAs */
+#define FSPAD_INNER_LIST 128           /* rows one CTA may be given pieces of */
+// How the rows of the nodes with children are cut: into at most 16 pieces each, as many as the walk merges at once, with two units for
+// each thread of a CTA at least.  How many rows there are is known to the kernel alone.  Where a CTA for every piece of every row is
+// one wave, most of which leaves at once, the CTAs are the pieces; else the kernel numbers the rows first (16 and 30 rows of 128256: the
+// step 0.7 us shorter without; 60 rows, in two waves, 2 us longer).
+static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int V, int slots, const int *parent)
+{
+    FspadStatsGeom g;
+    g.unit = 4;
+    g.shift = V % 4 != 0;
+    g.upr = g.shift ? (V + 6) / 4 : V / 4;
+    g.slots = slots;
+    g.total = (long long)rows * g.upr;
+    int k = g.upr / (2 * FSPAD_STATS_THREADS);
+    k = k < 2 ? 2 : k > 16 ? 16 : k;
+    g.chunk = (g.upr + k - 1) / k;
+    g.per_row = k;
+    const long long n = (long long)sm_count * (1024 / FSPAD_STATS_THREADS);
+    g.threads = FSPAD_STATS_THREADS;
+    g.n_cta = (int)((long long)rows * k <= n ? rows * k : n);
+    g.parent = parent;
+    return g;
+}
+// Whether the scan of these rows goes by the trees.  Looking for the rows takes about a microsecond, and a walk that ends in a node
+// without children two more; against that stand three quarters of the scan.  Us a step, all rows and by the trees: 60 x 32000
+// 21.2 and 22.6, 40 x 64000 28.9 and 29.2, 60 x 50257 32.8 and 33.0 (greedy 21.2 and 20.8), 120 x 32000 32.6 and 32.9, 240 x 32000 36.7
+// and 35.9, 60 x 128256 35.0 and 32.3, 960 x 128256 191 and 126.  Few rows of 128256 tokens are read by the trees whatever their
+// number, because all SMs share a row otherwise and the walk has more pieces to merge than it takes at once: 8 rows 31.1 and 25.0, 30 32.4 and 29.7.
+static inline bool fspad_scan_inner(int sm_count, int rows, int V)
+{
+    return rows <= FSPAD_INNER_MAX_ROWS && ((long long)rows * V >= 7 << 19 || V > 98304) && (long long)rows * (V + 6) < 1ll << 31 &&
+           rows / (sm_count * (1024 / FSPAD_STATS_THREADS)) + 2 <= FSPAD_INNER_LIST;
 }
 
 #ifdef __CUDACC__

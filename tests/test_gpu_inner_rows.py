@@ -1,0 +1,86 @@
+"""Acceptance on arrays that are scanned by the trees: the rows of nodes without children have no scan results, and the walk looks
+at the one it ends in itself.  Against the oracle, bit-exact (the 1e-6 band excepted and counted)."""
+import numpy as np
+import pytest
+
+from paper_2408_15562_b200 import synth
+from tests import helpers
+from tests.test_gpu_accept import _run
+
+pytestmark = pytest.mark.gpu
+
+W = synth.WORKLOADS
+
+
+def _parity(inp, allow_near=1):
+    path, n_acc, bonus = _run(inp)
+    hard, near, msgs = helpers.compare_accept(inp, path, n_acc, bonus)
+    assert hard == 0, msgs
+    assert near <= allow_near, msgs
+    return path, n_acc, bonus
+
+
+def _leaf_ends(inp, path, n_acc):
+    return sum(int(path[b, n_acc[b] - 1]) not in set(inp.parent[b].tolist()) for b in range(len(n_acc)))
+
+
+# one CTA per sequence up to clusters of 16; rows that start on and off 16-byte boundaries; trees on either side of 64 nodes;
+# fewer and more items than CTAs
+@pytest.mark.parametrize("vocab,nodes,batch", [(4099, 64, 15), (8192, 200, 3), (16381, 130, 2), (32000, 60, 2), (50257, 60, 3), (128256, 33, 1),
+                                                (128256, 1, 17), (5003, 60, 16)])
+@pytest.mark.parametrize("mode", ["greedy", "sample", "mixed"])
+def test_rows_without_children(vocab, nodes, batch, mode):
+    temps = {"greedy": (0.0,) * 16, "sample": (1.0, 0.7) * 8, "mixed": (0.0, 1.0, 0.6) * 6}[mode]
+    temps = (temps * 2)[:batch]
+    at_leaf = 0
+    for variant in range(3):
+        w = synth.scaled(W["llama3_8b_2k"], batch=batch, vocab=vocab, n_nodes=nodes, depth=3, branch=8 if nodes <= 64 else 16,
+                         temperatures=temps, prefix=(8, 8))
+        if nodes == 1:
+            w = synth.scaled(w, depth=1)
+        inp = synth.generate(w, variant, with_attention=False)
+        assert inp.parent.size * vocab >= 7 << 19 or vocab > 98304         # (else every row is scanned)
+        path, n_acc, _ = _parity(inp)
+        at_leaf += _leaf_ends(inp, path, n_acc)
+    assert at_leaf > 0 or batch == 1 or nodes == 1
+
+
+@pytest.mark.parametrize("temps", [(0.0, 0.0), (1.0, 0.0), (0.3, 2.0)])
+@pytest.mark.parametrize("where", [0, 1, 31998, 49999, 50256])
+def test_ends_of_the_row(temps, where):
+    """A star whose only child is certain to be accepted; the leaf's mass lies at one token, also twice (the lower index counts), or
+    nowhere."""
+    w = synth.scaled(W["tiny_greedy"], batch=2, vocab=50257, n_nodes=48, tree="star", temperatures=temps, prefix=(8, 8))
+    inp = synth.generate(w, 0, with_attention=False)
+    inp.target_logits[:, 0] = -np.inf
+    inp.target_logits[0, 0, inp.draft_tokens[0, 1]] = 1.0
+    inp.target_logits[1, 0, inp.draft_tokens[1, 1]] = 1.0
+    for b in range(2):
+        inp.target_logits[b, 1] = -np.inf
+        if b == 0:
+            inp.target_logits[b, 1, where] = -3.0
+        else:
+            inp.target_logits[b, 1, where] = 4.0
+            inp.target_logits[b, 1, 50256] = 4.0
+    path, n_acc, bonus = _parity(inp, allow_near=0)
+    assert n_acc.tolist() == [2, 2] and bonus[0] == where
+    if temps[1] == 0.0:
+        assert bonus[1] == where
+    inp.target_logits[:, 1] = -np.inf
+    _, _, bonus = _run(inp)
+    assert bonus.tolist() == [0, 0]
+
+
+def test_zeros_of_either_sign_and_chains():
+    w = synth.scaled(W["tiny_greedy"], batch=1, vocab=65536, n_nodes=60, tree="star", temperatures=(0.0,), prefix=(8, 8))
+    inp = synth.generate(w, 0, with_attention=False)
+    inp.target_logits[:] = -1.0
+    inp.target_logits[0, 0, inp.draft_tokens[0, 5]] = 1.0
+    inp.target_logits[0, :, 40000] = 0.0
+    inp.target_logits[0, :, 123] = -0.0
+    path, n_acc, bonus = _parity(inp, allow_near=0)
+    assert path[0, 1] in (1, 2, 3, 4, 5) and bonus[0] == 123
+    for temps in ((0.0, 0.0), (1.0, 1.0)):
+        w = synth.scaled(W["tiny_greedy"], batch=2, vocab=32000, n_nodes=60, tree="chain", temperatures=temps, prefix=(8, 8))
+        for variant in range(3):
+            _parity(synth.generate(w, variant, with_attention=False))
