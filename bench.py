@@ -465,9 +465,11 @@ def main():
         e2e_step(i)
     barrier()
     e2e_us = (time.perf_counter() - t0) * 1e6 / e2e_steps
-    h2d = sum(t.numel() * t.element_size() for t in (hq, htk, htv, hpar, hpre, htok, htemp, hlg) if t is not None)
+    h2d = sum(t.numel() * t.element_size() for t in (hq, htk, htv, hpar, hpre, htok, htemp) if t is not None)
+    # page-locked logits and draft rows are read where they are: of the logits the rows of nodes with children (and of a walk that ends
+    # in another node that one, and a logit and a draft probability of every node, which are not counted, nor are the few draft rows)
+    h2d += sum(len(set(p[1:].tolist()) | {0}) for p in inp.parent) * w.vocab * 4
     h2d += hun.numel() * hun.element_size() if hun is not None else 0
-    # (page-locked draft rows are not copied: the walk reads the few it needs where they are)
     d2h = sum(t.numel() * t.element_size() for t in (hout, hpath, hn, hb, hl))
 
     # max over ranks
@@ -536,8 +538,9 @@ def main():
                 "note": "draft side: eta = Wdown(silu(Wgate e) * Wup f) + f on the frontier rows; three matrices streamed once; "
                         "not part of value"}),
             "e2e": {"value": e2e_us, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
-                    "steps": e2e_steps, "note": "fspad_verify_step_host: pinned host inputs, device-resident KV cache; draft rows are read in place, "
-                            "not copied, and not counted in h2d_bytes_per_step"},
+                    "steps": e2e_steps, "note": "fspad_verify_step_host: pinned host inputs, device-resident KV cache; logits and draft rows are "
+                            "read over the link by the kernels where they need them, not copied: the logits rows of nodes with "
+                            "children are counted in h2d_bytes_per_step, draft rows are not"},
             "gpu_launches": int(launches),
             "clocks": clocks,
         }

@@ -458,9 +458,9 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
  * are those of fspad_verify_step on the same inputs, bit for bit.  The KV cache
  * is device-resident state that persists between steps (the caller's device
  * pointer `cache`, layout as in fspad_kv_compact); everything else is host
- * memory (pinned memory makes the copies asynchronous; draft_probs that lie in
- * one pinned allocation or registration as a whole and start on a 16-byte
- * boundary are not copied at all: the kernel reads the rows it needs where they
+ * memory (pinned memory makes the copies asynchronous; draft_probs or target_logits
+ * that lie in one pinned allocation or registration as a whole and start on a 16-byte
+ * boundary are not copied at all: the kernels read the rows they need where they
  * are, before the call returns).  An error, too, is returned only when nothing
  * queued by the call uses host memory any more.  Host outputs:
  * attn_out [batch][n_nodes][Hq][d] bf16, accepted_path [batch][max_nodes],

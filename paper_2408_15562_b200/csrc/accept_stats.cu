@@ -217,6 +217,17 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
     }
 }
 
+// Positions j .. j + 3 of a row, from memory this thread has written itself.
+static __device__ __noinline__ float4 own4(const float *x, int j, int V)
+{
+    float4 r = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    if (j >= 0 && j < V) r.x = x[j];
+    if (j + 1 >= 0 && j + 1 < V) r.y = x[j + 1];
+    if (j + 2 >= 0 && j + 2 < V) r.z = x[j + 2];
+    if (j + 3 >= 0 && j + 3 < V) r.w = x[j + 3];
+    return r;
+}
+
 // The same scan over the rows of the nodes that have children (a quarter of a 60-node tree's): the walk stops at a node without
 // children at most once, at its end, and looks at that row itself.  A parent that is no lower node counts as the root, as in the
 // walk.  Two ways of finding the rows:
@@ -229,7 +240,8 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
 // loads and reduction where they are few (15 of 60 rows: 4.5 us; all 60 9.4).  A share may cross rows.  The run of a row that a CTA takes is reduced as a whole, and its result goes to slot 0 if the run begins
 // the row, else to the one behind the stretch of `wide` units it starts in: every share is at least that long, so no two meet.  The
 // slots in between are empty.
-template <bool SHARED>
+// STAGE: the logits are in host memory, and the rows read are left at g.stage for the walk.
+template <bool SHARED, bool STAGE>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restrict__ temperature, int N, int rows, int V,
                           const FspadStatsGeom g, int wide, FspadStatsPart *__restrict__ parts)
@@ -364,6 +376,21 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
                     }
                 }
             }
+            if constexpr (STAGE) {
+                float *to = g.stage + (size_t)q.row * V;
+#pragma unroll
+                for (int u = 0; u < kDeep; ++u) {
+                    const int i = base + u * kThreads + tid, j = q.j0 + 4 * i;
+                    if (i < q.n && j >= 0 && j + 4 <= V) {
+                        *reinterpret_cast<float4 *>(to + j) = cur[u];
+                    } else if (i < q.n) {
+                        if (j >= 0 && j < V) to[j] = cur[u].x;
+                        if (j + 1 >= 0 && j + 1 < V) to[j + 1] = cur[u].y;
+                        if (j + 2 >= 0 && j + 2 < V) to[j + 2] = cur[u].z;
+                        if (j + 3 >= 0 && j + 3 < V) to[j + 3] = cur[u].w;
+                    }
+                }
+            }
             float bm = U4::vmax(cur[0]);
 #pragma unroll
             for (int u = 1; u < kDeep; ++u) bm = fmaxf(bm, U4::vmax(cur[u]));
@@ -409,7 +436,8 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
 #pragma unroll 1
             for (int u = kDeep - 1; u >= 0; --u) {
                 const int i = my_base + u * kThreads + tid, j = q.j0 + 4 * i;
-                if (i < q.n) b = U4::first_eq(fspad_load4(logits + (size_t)q.row * V, j, V, -INFINITY), bmax, j, b);
+                const float *from = STAGE ? g.stage : logits;         // (what this thread has stored there itself: no read-only load)
+                if (i < q.n) b = U4::first_eq(STAGE ? own4(from + (size_t)q.row * V, j, V) : fspad_load4(from + (size_t)q.row * V, j, V, -INFINITY), bmax, j, b);
             }
             atomicMin(&s_barg, b);
         }
@@ -481,17 +509,19 @@ cudaError_t fspad_launch_stats_partials(fspad_ctx *ctx, const float *logits, con
 {
     const bool aligned = (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
-    if (geom->parent != nullptr && aligned && rows % rows_per_seq == 0 && fspad_scan_inner(sms, rows, V)) {
-        *geom = fspad_stats_geom_inner(sms, rows, V, ctx->stats_slots, geom->parent);
+    if (geom->parent != nullptr && aligned && rows % rows_per_seq == 0 &&
+        (geom->stage != nullptr ? fspad_scan_inner_fits(sms, rows, V) : fspad_scan_inner(sms, rows, V))) {
+        *geom = fspad_stats_geom_inner(sms, rows, V, ctx->stats_slots, geom->parent, geom->stage);
         const FspadStatsGeom &g = *geom;
         const int wide = (g.upr + g.per_row - 2) / (g.per_row - 1);
         ctx->launches++;
-        if (g.n_cta == rows * g.per_row)
-            return fspad_launch_opt(pdl, accept_stats_inner_kernel<false>, dim3(g.per_row, rows), dim3(kThreads), 0, st, 0, logits,
-                                    temperature, rows_per_seq, rows, V, g, wide, ctx->st_part);
-        return fspad_launch_opt(pdl, accept_stats_inner_kernel<true>, dim3(g.n_cta), dim3(kThreads), 0, st, 0, logits, temperature,
-                                rows_per_seq, rows, V, g, wide, ctx->st_part);
+        const bool pieces = g.n_cta == rows * g.per_row, stage = g.stage != nullptr;
+        return fspad_launch_opt(pdl, pieces ? stage ? accept_stats_inner_kernel<false, true> : accept_stats_inner_kernel<false, false>
+                                            : stage ? accept_stats_inner_kernel<true, true> : accept_stats_inner_kernel<true, false>,
+                                pieces ? dim3(g.per_row, rows) : dim3(g.n_cta), dim3(kThreads), 0, st, 0, logits, temperature, rows_per_seq,
+                                rows, V, g, wide, ctx->st_part);
     }
+    if (geom->stage != nullptr) return cudaErrorInvalidValue;        // (the caller looks first)
     *geom = fspad_stats_geom(sms, rows, V, aligned, ctx->stats_slots, true);
     ctx->launches++;
     return launch_partials(logits, temperature, rows_per_seq, V, *geom, ctx->st_part, st, pdl);

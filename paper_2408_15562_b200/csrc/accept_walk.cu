@@ -77,6 +77,8 @@ __constant__ double kExp2Tbl[16] = {
 
 struct WalkArgs {
     const float *logits, *draft, *temperature, *uniforms;
+    const float *given;                 // the caller's logits: other than `logits` where they lie in host memory and the scan has brought
+                                        // the rows that it reads to the device
     const int *tokens, *parent;
     const FspadStatsPart *parts;
     FspadStatsGeom geom;
@@ -567,11 +569,11 @@ __device__ __noinline__ double block_scan(Shared &sh, double v, double *excl_out
 }
 
 // The bonus draw from a row that the scan has left out: inverse CDF of its softmax.  Every CTA takes its own slice's maximum for the
-// row's; the slices' masses are brought to the largest of them when all have come, in one exchange.  `last`: the thread has the last
-// tokens of its CTA.  false: a wait ran out.
+// row's; the slices' masses are brought to the largest of them when all have come, in one exchange.  The row is read once and kept in
+// shared memory (`park`, NULL where it does not fit).  `last`: the thread has the last tokens of its CTA.  false: a wait ran out.
 template <class Shared>
-__device__ __forceinline__ bool draw_from_row(Shared &sh, const float *__restrict__ x, Chunk ck, bool last, int rank, int C, int par,
-                                           uint32_t phase, double invT, int V, int *bonus)
+__device__ __forceinline__ bool draw_from_row(Shared &sh, const float *__restrict__ x, float *__restrict__ park, Chunk ck, int per_thr,
+                                              bool last, int rank, int C, int par, uint32_t phase, double invT, int V, int *bonus)
 {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     float m = -INFINITY;
@@ -581,8 +583,19 @@ __device__ __forceinline__ bool draw_from_row(Shared &sh, const float *__restric
 #pragma unroll
         for (int u = 0; u < 4; ++u) v[u] = fspad_load4(x, j + 4 * u, ck.hi, -INFINITY);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) m = fmaxf(m, fmaxf(fmaxf(v[u].x, v[u].y), fmaxf(v[u].z, v[u].w)));
+        for (int u = 0; u < 4; ++u) {
+            m = fmaxf(m, fmaxf(fmaxf(v[u].x, v[u].y), fmaxf(v[u].z, v[u].w)));
+            const int k = j - ck.lo + 4 * u;
+            if (park != nullptr && k < per_thr) {
+                park[k * kWalkThreads] = v[u].x;
+                park[(k + 1) * kWalkThreads] = v[u].y;
+                park[(k + 2) * kWalkThreads] = v[u].z;
+                park[(k + 3) * kWalkThreads] = v[u].w;
+            }
+        }
     }
+    const int n = max(ck.hi - ck.lo, 0);
+    auto token = [&](int k) { return park != nullptr ? park[k * kWalkThreads] : ck.lo + k < 0 ? -INFINITY : x[ck.lo + k]; };
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     if (lane == 0) sh.warp_v[1][wid] = (double)m;
@@ -592,14 +605,8 @@ __device__ __forceinline__ bool draw_from_row(Shared &sh, const float *__restric
     for (int off = kWarps / 2; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     const ExpArg arg = exp_arg(m, invT);
     double mine = 0.0;
-#pragma unroll 1
-    for (int j = ck.lo; j < ck.hi; j += 4) {
-        const float4 v = fspad_load4(x, j, ck.hi, -INFINITY);
-        mine += exp_neg(v.x, arg, sh.exp_tbl);
-        mine += exp_neg(v.y, arg, sh.exp_tbl);
-        mine += exp_neg(v.z, arg, sh.exp_tbl);
-        mine += exp_neg(v.w, arg, sh.exp_tbl);
-    }
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) mine += exp_neg(token(k), arg, sh.exp_tbl);
     double E, total;
     const double P = block_scan(sh, mine, &E, &total);
     const uint32_t bar = smem_addr(&sh.bar[par]);
@@ -631,9 +638,16 @@ __device__ __forceinline__ bool draw_from_row(Shared &sh, const float *__restric
         __syncthreads();
         // (the rounding of the two levels can leave no thread above the target: the last tokens of the CTA then take the draw)
         if (tid == sh.sel || (sh.sel == 0x7fffffff && last && ck.lo < ck.hi)) {
-            int found = -1;
-            sweep_row(MODE_CDF, sh, x, x, nullptr, nullptr, 0, ck, false, arg, 0.0, -1, E, local, &found);
-            *bonus = found < 0 ? min(max(ck.lo, 0), V - 1) : found;
+            double run = E;
+            int found = max(ck.lo, 0);                        // the first token above the target, else the last of positive weight
+#pragma unroll 1
+            for (int k = 0; k < n; ++k) {
+                const double w = exp_neg(token(k), arg, sh.exp_tbl);
+                run += w;
+                if (w > 0.0) found = ck.lo + k;
+                if (w > 0.0 && run > local) break;
+            }
+            *bonus = found;
         }
     }
     if (owner < 0 && rank == 0 && tid == 0) *bonus = 0;       // no positive weight anywhere
@@ -837,7 +851,7 @@ accept_greedy_kernel(const __grid_constant__ WalkArgs args)
         if (t.last >= 0) {
             const size_t start = ((size_t)b * N + t.last) * args.V;
             const int ph = (int)(start & 3), each = (((args.V + 3 + C - 1) / C) + 3) & ~3;
-            argmax_row(t, args.logits + start, rank * each - ph, min(args.V, (rank + 1) * each - ph), tid, nthr);
+            argmax_row(t, args.given + start, rank * each - ph, min(args.V, (rank + 1) * each - ph), tid, nthr);
             __syncthreads();
             if (tid == 0) *cluster.map_shared_rank(&peer_best[rank], 0) = t.best;  // (a word each: maxima of 64 bits sent to one word of a peer got lost)
             cluster.sync();
@@ -940,7 +954,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             if constexpr (INNER) sh.t.known[p] = 1;
             if (sampling) {
                 const size_t at = (size_t)p * V + t;
-                xv = lg[at];
+                xv = INNER ? args.given[row0 * V + at] : lg[at];       // (the scan may still be bringing the row)
                 qv = dp[at];
             }
         }
@@ -1014,7 +1028,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         if constexpr (INNER) {
             if (sh.t.last >= 0) {
                 const size_t start = (row0 + sh.t.last) * V;
-                argmax_row(sh.t, args.logits + start, -(int)(start & 3), V, tid, kWalkThreads);
+                argmax_row(sh.t, args.given + start, -(int)(start & 3), V, tid, kWalkThreads);
                 __syncthreads();
                 if (tid == 0) args.bonus[b] = argmax_of(sh.t.best);
             }
@@ -1334,7 +1348,8 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         if (!sh.t.known[cur]) {                               // (a node without children: nothing was rejected there)
             const Chunk ck = chunk_of((row0 + cur) * V, V, per_cta, per_thr, rank, tid);
             const bool last = tid == kWalkThreads - 1 || ck.hi == V || ck.hi - ck.lo < per_thr || (tid + 1) * per_thr >= per_cta;
-            if (!draw_from_row(sh, x, ck, last, rank, C, n_exch & 1, (uint32_t)(n_exch >> 1) & 1u, invT, V, args.bonus + b)) {
+            if (!draw_from_row(sh, args.given + (row0 + cur) * V, cache_ok ? sq : nullptr, ck, per_thr, last, rank, C, n_exch & 1,
+                               (uint32_t)(n_exch >> 1) & 1u, invT, V, args.bonus + b)) {
                 if (tid == 0) fspad_report(args.status, FSPAD_ERR_TIMEOUT);
                 cluster.sync();                               // nobody leaves while a peer may still write to its shared memory
                 return;
@@ -1569,7 +1584,7 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     WalkArgs a;
     a.kv_cache = reinterpret_cast<uint4 *>(kv.cache); a.kv_prefix = kv.prefix_len; a.kv_new_len = kv.new_len;
     a.kv_layers = ctx->cfg.n_layers; a.kv_B = B; a.kv_H = ctx->cfg.n_kv_heads; a.kv_max_len = ctx->cfg.max_len;
-    a.logits = logits; a.draft = draft; a.temperature = temperature; a.uniforms = uniforms;
+    a.logits = geom.stage != nullptr ? geom.stage : logits; a.given = logits; a.draft = draft; a.temperature = temperature; a.uniforms = uniforms;
     a.tokens = tokens; a.parent = parent;
     a.parts = ctx->st_part; a.geom = geom;
     a.N = N; a.V = V; a.path_stride = ctx->cfg.max_nodes; a.cache_ok = 0; a.draft_far = draft_far ? 1 : 0; a.B = B; a.sampled_first = 0;

@@ -91,6 +91,9 @@ struct FspadStatsGeom {
     // then no partials, and whoever walks into such a node looks at its row itself.  NULL: every row has them.  Set by the
     // caller of fspad_launch_stats_partials, which puts it back to NULL where the scan reads every row after all.
     const int *parent = nullptr;
+    // With the trees: the logits lie in host memory, and the rows that the scan reads are left here, [rows][V] on the device.  NULL: they
+    // are on the device.  Set by the caller, too.
+    float *stage = nullptr;
 };
 
 // small_ctas: the scan may use CTAs of half the size when the array is small (the pieces, one of which the
@@ -163,7 +166,7 @@ static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, boo
 // each thread of a CTA at least.  How many rows there are is known to the kernel alone.  Where a CTA for every piece of every row is
 // one wave, most of which leaves at once, the CTAs are the pieces; else the kernel numbers the rows first (16 and 30 rows of 128256: the
 // step 0.7 us shorter without; 60 rows, in two waves, 2 us longer).
-static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int V, int slots, const int *parent)
+static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int V, int slots, const int *parent, float *stage)
 {
     FspadStatsGeom g;
     g.unit = 4;
@@ -179,17 +182,22 @@ static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int 
     g.threads = FSPAD_STATS_THREADS;
     g.n_cta = (int)((long long)rows * k <= n ? rows * k : n);
     g.parent = parent;
+    g.stage = stage;
     return g;
 }
-// Whether the scan of these rows goes by the trees.  Looking for the rows takes about a microsecond, and a walk that ends in a node
+// Whether the scan of these rows can go by the trees, and whether it does.  Looking for the rows takes about a microsecond, and a walk that ends in a node
 // without children two more; against that stand three quarters of the scan.  Us a step, all rows and by the trees: 60 x 32000
 // 21.2 and 22.6, 40 x 64000 28.9 and 29.2, 60 x 50257 32.8 and 33.0 (greedy 21.2 and 20.8), 120 x 32000 32.6 and 32.9, 240 x 32000 36.7
 // and 35.9, 60 x 128256 35.0 and 32.3, 960 x 128256 191 and 126.  Few rows of 128256 tokens are read by the trees whatever their
 // number, because all SMs share a row otherwise and the walk has more pieces to merge than it takes at once: 8 rows 31.1 and 25.0, 30 32.4 and 29.7.
+static inline bool fspad_scan_inner_fits(int sm_count, int rows, int V)
+{
+    return rows <= FSPAD_INNER_MAX_ROWS && (long long)rows * (V + 6ll) < 1ll << 31 &&
+           rows / (sm_count * (1024 / FSPAD_STATS_THREADS)) + 2 <= FSPAD_INNER_LIST;
+}
 static inline bool fspad_scan_inner(int sm_count, int rows, int V)
 {
-    return rows <= FSPAD_INNER_MAX_ROWS && ((long long)rows * V >= 7 << 19 || V > 98304) && (long long)rows * (V + 6) < 1ll << 31 &&
-           rows / (sm_count * (1024 / FSPAD_STATS_THREADS)) + 2 <= FSPAD_INNER_LIST;
+    return fspad_scan_inner_fits(sm_count, rows, V) && ((long long)rows * V >= 7 << 19 || V > 98304);
 }
 
 #ifdef __CUDACC__

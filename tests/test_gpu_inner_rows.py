@@ -2,8 +2,9 @@
 at the one it ends in itself.  Against the oracle, bit-exact (the 1e-6 band excepted and counted)."""
 import numpy as np
 import pytest
+import torch
 
-from paper_2408_15562_b200 import synth
+from paper_2408_15562_b200 import binding, synth
 from tests import helpers
 from tests.test_gpu_accept import _run
 
@@ -84,3 +85,31 @@ def test_zeros_of_either_sign_and_chains():
         w = synth.scaled(W["tiny_greedy"], batch=2, vocab=32000, n_nodes=60, tree="chain", temperatures=temps, prefix=(8, 8))
         for variant in range(3):
             _parity(synth.generate(w, variant, with_attention=False))
+
+
+@pytest.mark.parametrize("vocab,nodes,batch", [(1000, 9, 1), (3001, 70, 3), (4099, 256, 2), (50257, 40, 2)])
+@pytest.mark.parametrize("mode", ["greedy", "mixed"])
+def test_logits_read_where_they_are(vocab, nodes, batch, mode):
+    """The host entry point on logits that the kernels read over the link (pinned, on a 16-byte boundary) and on ones that are copied
+    (pinned off the boundary; pageable): the oracle's acceptance each time, also in a second call with other logits in the same memory."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=batch, prefix=(40, 300), n_nodes=nodes, depth=4, branch=16, vocab=vocab,
+                     temperatures=((0.0,) * 3 if mode == "greedy" else (1.0, 0.0, 0.7))[:batch])
+    inps = [synth.generate(w, v) for v in (3, 4)]
+    ctx = helpers.make_ctx(inps[0], n_layers=1)
+    pin = lambda a: torch.from_numpy(np.ascontiguousarray(a)).pin_memory()   # noqa: E731
+    flat = torch.from_numpy(inps[0].target_logits)
+    for where in (flat.clone().pin_memory(), torch.empty(flat.numel() + 4).pin_memory()[1:1 + flat.numel()].view(flat.shape), flat.clone()):
+        for inp in inps:
+            where.copy_(torch.from_numpy(inp.target_logits))
+            sampling = inp.draft_probs is not None
+            cache = binding.bf16_tensor(synth.make_cache(inp, 1))
+            out = torch.empty(inp.q.shape, dtype=torch.bfloat16).pin_memory()
+            path = torch.empty(inp.parent.shape, dtype=torch.int32)
+            n, bonus, new_len = (torch.empty((batch,), dtype=torch.int32) for _ in range(3))
+            ctx.verify_step_host(cache, *(binding.bf16_tensor(a, "cpu").pin_memory() for a in (inp.q, inp.tree_k, inp.tree_v)),
+                                 pin(inp.parent), pin(inp.prefix_len), where, pin(inp.draft_probs) if sampling else None,
+                                 pin(inp.draft_tokens), pin(inp.temperature), pin(inp.uniforms) if sampling else None, out, path, n, bonus,
+                                 new_len)
+            hard, near, msgs = helpers.compare_accept(inp, path.numpy(), n.numpy(), bonus.numpy())
+            assert hard == 0 and near == 0, msgs
+            assert np.array_equal(new_len.numpy(), inp.prefix_len + n.numpy())

@@ -152,6 +152,18 @@ def test_draft_rows_are_read_in_place_only_where_all_of_them_are_pinned(lib, pin
         assert int(_field(log, "walk", "draft"), 16) == step.draft.ctypes.data
 
 
+@pytest.mark.parametrize("share,nodes,batch,vocab,in_place", [(1.0, 60, 1, 4096, True), (1.0, 200, 2, 33, True), (0.99, 60, 1, 4096, False), (0, 60, 1, 4096, False),
+                                                              (1.0, 256, 33, 8, False)])        # 8448 rows: more than the scan by the trees takes
+def test_logits_stay_where_all_of_them_are_pinned(lib, share, nodes, batch, vocab, in_place):
+    step = Step(lib, nodes=nodes, batch=batch, vocab=vocab, sampling=False)
+    bytes_ = batch * nodes * vocab * 4
+    if share:
+        lib.fake_pin(0x1000, int(share * bytes_))
+    rc, log = step.host()
+    copied = any(x.startswith("h2d host=1000 bytes=%d " % bytes_) for x in log)
+    assert rc == 0 and copied != in_place and any(x.startswith("scan ") for x in log)
+
+
 FAILING = [("h2d", k) for k in range(1, 10)] + [("d2h", k) for k in range(1, 7)] + \
     [(name, 1) for name in ("scatter", "attention", "scan", "walk", "compact", "sync")] + \
     [("event_record", k) for k in (1, 2)] + [("stream_wait", k) for k in (1, 2)]
