@@ -5,7 +5,8 @@
 // One kernel per call, grid (pieces of a row, rows):
 //   1. every CTA streams its piece: the half-warp maxima of the first 4096 tokens give a lower
 //      bound of the piece's k-th largest value, the tokens that reach it are listed in
-//      shared memory, and the list's members are ranked by counting; the one HBM pass over the rows;
+//      shared memory, a warp cuts the list by a bound of the same kind and ranks what is left by counting; the one HBM pass over
+//      the rows;
 //   2. the CTA that finishes a sequence's last piece (told by a counter per sequence that it then puts back to zero; nobody
 //      waits for anybody) takes one warp to a row and ranks the pieces' lists the same way; the first k
 //      become candidates base + f k + r with the frontier node as parent and the joint
@@ -15,7 +16,10 @@
 //
 // What bounds it: HBM with many rows, otherwise a chain of latencies.  As three kernels (one CTA per 4096 tokens, then a
 // 1024-entry sorting network per row, then one per sequence) a level of ten rows took 15 us at V = 32000 and 40 us with
-// 16 sequences at V = 128256 (82 MB); now 8.1 and 23.  Pieces are at most 16 per row, so that the lists merged for a row stay short.
+// 16 sequences at V = 128256 (82 MB); with lists ranked by all threads, every member against every other, 8.1 and 23; now 7.2 and 20
+// (11 sequences, 16 of 151936 tokens a row, where lists of 265 keys now and then outgrew what was ranked and were cut bit by bit: 45 -> 31).  What
+// is left behind the stream is mostly a chain of code that each CTA runs once: code inlined twice, or fetched early by a call
+// that does nothing, made a level 0.5 us longer, and so did lists handed on unranked.  Pieces are at most 16 per row, so that the lists merged for a row stay short.
 // (Prefetching rounds further ahead into L2 or asking for the second round before the bound is known made it slower: it is not HBM's
 // latency that the rounds wait for.)
 #include "common.cuh"
@@ -26,14 +30,15 @@ namespace {
 constexpr int kThreads = 512;                          // one warp for each of a sequence's up to 16 rows
 constexpr int kPerThread = 8;                         // tokens per thread and round
 constexpr int kRound = kThreads * kPerThread;          // 4096 tokens
-constexpr int kKeep = 512;                             // longest list that is ranked by counting
+constexpr int kKeep = 512;                             // longest list left by a round where lists are cut between rounds
+constexpr int kShort = 128;                            // longest list that is ranked by counting
 constexpr int kMaxPieces = 16;
 
 struct DraftArgs {
     const float *logprobs, *frontier_logp;
     const int *frontier_cand;
     int V, F, k, width, base, cap, pieces, len;        // len: tokens of a piece (a multiple of 32)
-    uint2 *part;                                       // [rows][pieces][k] (value, token)
+    unsigned long long *part;                          // [rows][pieces][k] keys, 0 where a piece has fewer tokens
     int *seq_done;                                     // pieces of a sequence's rows that have finished
     int *cand_parent, *cand_token;
     float *cand_logp;
@@ -45,6 +50,7 @@ struct DraftShared {
     unsigned long long list[kKeep + kRound];           // keys of the tokens that reach the bound
     unsigned long long top[FSPAD_MAX_FRONTIER];
     float hmax[kThreads / 16];
+    alignas(16) uint32_t scratch[kThreads / 32][32];
     float joint[FSPAD_MAX_FRONTIER * FSPAD_MAX_FRONTIER];
     float bound;
     int cnt, n, hits, last;
@@ -84,6 +90,37 @@ __device__ __forceinline__ int rank_of(const unsigned long long *list, int n, un
 #pragma unroll 4
     for (int o = 0; o < n; ++o) rank += list[o] > me ? 1 : 0;
     return rank;
+}
+
+// One warp, the n keys of `list` (0: no key): those that can be among its k <= 32 largest are moved to its front, and their number
+// is returned.  The k-th largest of the lanes' maxima is a bound that k keys reach; few others do (150 keys, k = 10: about 13 are left), and
+// ranking those takes a tenth of what ranking all of them against one another took (3 us of a level of 16 sequences).
+__device__ __noinline__ int shorten(unsigned long long *list, int n, int k, uint32_t *scratch, int lane)
+{
+    uint32_t top = 0u;                                 // (the high words, the values, are enough for a bound)
+    for (int i = lane; i < n; i += 32) top = max(top, (uint32_t)(list[i] >> 32));
+    scratch[lane] = top;
+    __syncwarp();
+    int rank = 0;
+#pragma unroll 2
+    for (int o = 0; o < 32; o += 4) {
+        const uint4 t = *reinterpret_cast<const uint4 *>(scratch + o);
+        rank += (t.x > top || (t.x == top && o < lane)) + (t.y > top || (t.y == top && o + 1 < lane)) +
+                (t.z > top || (t.z == top && o + 2 < lane)) + (t.w > top || (t.w == top && o + 3 < lane));
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, rank == k - 1);
+    const uint32_t bound = max(__shfl_sync(0xffffffffu, top, __ffs((int)who) - 1), 1u);      // (a key's value is never 0)
+    int m = 0;
+#pragma unroll 1
+    for (int i = 0; i < n; i += 32) {
+        const unsigned long long key = i + lane < n ? list[i + lane] : 0ull;
+        const bool stays = (uint32_t)(key >> 32) >= bound;
+        const unsigned all = __ballot_sync(0xffffffffu, stays);
+        if (stays) list[m + __popc(all & ((1u << lane) - 1u))] = key;      // (behind every key already read, or that one itself)
+        m += __popc(all);
+    }
+    __syncwarp();
+    return m;
 }
 
 // PER_SM: CTAs an SM holds.  Four leave a thread 32 registers, which is a few too few; with three a level's chain is shorter (ten rows:
@@ -183,62 +220,65 @@ draft_expand_kernel(const DraftArgs a)
             __syncthreads();
             if (s.cnt > kKeep) cut_list(s, k, tid);
         }
-    } else if (s.cnt > kKeep) {
-        cut_list(s, k, tid);
+    } else if (s.cnt > kShort) {                                 // cut it here only if a warp would be long about it: many equal values
+        const int n = s.cnt;
+        __syncthreads();
+        if (tid < 32) {
+            const int m = shorten(s.list, n, k, s.scratch[0], lane);
+            if (lane == 0) s.cnt = m;
+        }
+        __syncthreads();
+        if (s.cnt > kShort) cut_list(s, k, tid);
     }
     __syncthreads();
-    {
-        const int n = s.cnt;
-        uint2 *out = a.part + ((size_t)row * a.pieces + piece) * k;
-        for (int i = tid; i < n; i += kThreads) {
+    // ---- the piece's list, and whether it is the sequence's last: one warp ----
+    const int b = row / a.F;
+    if (tid < 32) {
+        const int n = s.cnt > 32 ? shorten(s.list, s.cnt, k, s.scratch[0], lane) : s.cnt;
+        unsigned long long *out = a.part + ((size_t)row * a.pieces + piece) * k;
+        for (int i = lane; i < n; i += 32) {
             const unsigned long long me = s.list[i];
             const int rank = rank_of(s.list, n, me);
-            if (rank < k) __stcg(out + rank, make_uint2(__float_as_uint(fspad_key_value(me)), fspad_key_index(me)));
+            if (rank < k) __stcg(out + rank, me);
         }
-        for (int r = n + tid; r < k; r += kThreads) __stcg(out + r, make_uint2(__float_as_uint(-INFINITY), 0x7fffffffu));   // empty slots
-    }
-    // ---- the last piece of the sequence ----
-    const int b = row / a.F;
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();                             // (behind the barrier it stands for the whole CTA's lists)
-        s.last = atomicAdd(a.seq_done + b, 1) == a.F * a.pieces - 1;
-        if (s.last) a.seq_done[b] = 0;
-        __threadfence();
+        for (int r = n + lane; r < k; r += 32) __stcg(out + r, 0ull);          // empty slots
+        __syncwarp();
+        if (lane == 0) {
+            int done;                                // (release: behind the warp's barrier it stands for the whole list)
+            asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(done) : "l"(a.seq_done + b) : "memory");
+            s.last = done == a.F * a.pieces - 1;
+            if (s.last) a.seq_done[b] = 0;
+        }
     }
     __syncthreads();
     if (s.last == 0) return;
-    // the pieces' lists of a row -> candidates, one warp to a row
+    // ---- the last piece of the sequence: the pieces' lists of a row -> candidates, one warp to a row ----
     const int n2 = a.pieces * k;                                     // at most 256: eight entries per lane
     unsigned long long *list = s.list + (tid >> 5) * (kMaxPieces * FSPAD_MAX_FRONTIER);
     for (int f = tid >> 5; f < a.F; f += kThreads / 32) {
-        const uint2 *in = a.part + (size_t)(b * a.F + f) * n2;
+        const unsigned long long *in = a.part + (size_t)(b * a.F + f) * n2;
         const float above = a.frontier_logp[b * a.F + f];
         const int parent = a.frontier_cand[b * a.F + f];
-        uint2 e[kMaxPieces * FSPAD_MAX_FRONTIER / 32];
+        unsigned long long e[kMaxPieces * FSPAD_MAX_FRONTIER / 32];
 #pragma unroll
-        for (int u = 0; u < kMaxPieces * FSPAD_MAX_FRONTIER / 32; ++u) {
-            e[u] = make_uint2(0u, 0x7fffffffu);
-            if (lane + 32 * u < n2) e[u] = __ldcg(in + lane + 32 * u);
-        }
+        for (int u = 0; u < kMaxPieces * FSPAD_MAX_FRONTIER / 32; ++u) e[u] = lane + 32 * u < n2 ? __ldcg(in + lane + 32 * u) : 0ull;
         // The lists are in descending order: at least k entries are as large as the smallest of the pieces' j-th, j = k / pieces
         // rounded up.  What is below that needs no ranking.
-        uint2 jth = make_uint2(0u, 0x7fffffffu);
+        unsigned long long jth = ~0ull;
         if (lane < a.pieces) jth = __ldcg(in + lane * k + (k + a.pieces - 1) / a.pieces - 1);
-        const uint32_t low = jth.y == 0x7fffffffu ? 0u : fspad_orderable(__uint_as_float(jth.x) + 0.0f);
-        const uint32_t bound = __reduce_min_sync(0xffffffffu, lane < a.pieces ? low : 0xffffffffu);
+        const uint32_t bound = max(__reduce_min_sync(0xffffffffu, (uint32_t)(jth >> 32)), 1u);
         int n = 0;
 #pragma unroll
         for (int u = 0; u < kMaxPieces * FSPAD_MAX_FRONTIER / 32; ++u) {
-            const unsigned long long key = e[u].y == 0x7fffffffu ? 0ull : fspad_sort_key(__uint_as_float(e[u].x), e[u].y);
-            const bool in_list = key != 0ull && (uint32_t)(key >> 32) >= bound;
+            if (32 * u >= n2) break;
+            const bool in_list = (uint32_t)(e[u] >> 32) >= bound;
             const unsigned m = __ballot_sync(0xffffffffu, in_list);
-            if (in_list) list[n + __popc(m & ((1u << lane) - 1u))] = key;
+            if (in_list) list[n + __popc(m & ((1u << lane) - 1u))] = e[u];
             n += __popc(m);
         }
-        __syncwarp();
         if (lane < k) s.joint[f * k + lane] = -INFINITY;
         __syncwarp();
+        if (n > 32) n = shorten(list, n, k, s.scratch[tid >> 5], lane);      // (many short lists: the bound is a low one)
         for (int i = lane; i < n; i += 32) {
             const unsigned long long me = list[i];
             const int rank = rank_of(list, n, me);
@@ -254,19 +294,20 @@ draft_expand_kernel(const DraftArgs a)
         __syncwarp();
     }
     __syncthreads();
-    // the new joint values -> next frontier
-    const int n_new = a.F * k;                                       // at most 256: one entry per thread
-    unsigned long long me = 0ull;
-    if (tid < n_new) {
-        me = fspad_sort_key(s.joint[tid], (uint32_t)tid);
-        s.list[tid] = me;
-    }
+    // the new joint values -> next frontier: a warp where it has few places, else every value's rank
+    const int n_new = a.F * k;                                       // at most 256
+    if (tid < n_new) s.list[tid] = fspad_sort_key(s.joint[tid], (uint32_t)tid);
     __syncthreads();
-    if (tid < n_new) {
-        const int rank = rank_of(s.list, n_new, me);
+    const bool few = a.width <= 32;
+    if (few && tid >= 32) return;
+    const int n = few ? shorten(s.list, n_new, a.width, s.scratch[0], lane) : n_new;
+    for (int i = tid; i < n; i += few ? 32 : kThreads) {
+        const unsigned long long me = s.list[i];
+        const int rank = rank_of(s.list, n, me);
         if (rank < a.width) {
-            a.next_cand[(size_t)b * a.width + rank] = a.base + tid;
-            a.next_logp[(size_t)b * a.width + rank] = s.joint[tid];
+            const int at = (int)fspad_key_index(me);
+            a.next_cand[(size_t)b * a.width + rank] = a.base + at;
+            a.next_logp[(size_t)b * a.width + rank] = s.joint[at];
         }
     }
 }
@@ -330,7 +371,7 @@ cudaError_t fspad_launch_draft_expand(fspad_ctx *ctx, const float *logprobs, con
     a.pieces = (a.V + 3 + a.len - 1) / a.len;
     a.logprobs = logprobs; a.frontier_logp = frontier_logp; a.frontier_cand = frontier_cand;
     a.F = F; a.k = k; a.width = width; a.base = base; a.cap = cap;
-    a.part = reinterpret_cast<uint2 *>(ctx->dx_part);
+    a.part = static_cast<unsigned long long *>(ctx->dx_part);
     a.seq_done = ctx->dx_done;
     a.cand_parent = cand_parent; a.cand_token = cand_token; a.cand_logp = cand_logp;
     a.next_cand = next_cand; a.next_logp = next_logp;

@@ -161,3 +161,23 @@ def test_pieces_by_rows_and_vocabulary(vocab, batch, F):
     flp = rng.standard_normal((batch, F)).astype(np.float32)
     fc = rng.integers(0, 5, (batch, F)).astype(np.int32)
     _check(ctx, lp, flp, fc, 10, 10, 7, 7 + F * 10)
+
+
+@pytest.mark.parametrize("more", [0, 22, 23, 118, 119, 502, 503, 4598, 4599])
+@pytest.mark.parametrize("values", ["apart", "equal"])
+@pytest.mark.parametrize("k,width", [(10, 32), (10, 33), (16, 16)])
+def test_lengths_of_a_piece_s_list(more, values, k, width):
+    """A row's list takes the tokens that reach the k-th largest half-warp maximum of its first 4096: k of those and `more` behind them,
+    on either side of what a warp ranks as it is (32), cuts first (128), what is kept between rounds (512) and what there is room for."""
+    V, F, B = 16384, 16, 8
+    ctx = binding.Context(8, 2, V, 256, max_nodes=64, max_batch=B)
+    rng = np.random.default_rng(more)
+    lp = np.full((B, F, V), -50.0, np.float32)
+    lp[:, :, :4096:4096 // 32][:, :, :k] = -10.0                 # tokens 0, 128, ...: one for each of k half-warps
+    for b in range(B):
+        for f in range(F):
+            at = 4096 + rng.choice(V - 4096, more, replace=False)
+            lp[b, f, at] = -10.0 if values == "equal" else -10.0 + 9.0 * rng.random(more, dtype=np.float32)
+    flp = (-rng.random((B, F)) * 4).astype(np.float32)
+    fc = rng.integers(-1, 50, size=(B, F)).astype(np.int32)
+    _check(ctx, lp, flp, fc, k, width, 0, F * k)
