@@ -65,6 +65,7 @@ struct StepPlan {
     bool chain;                 // one stream: scan, walk, and the attention launched beside the walk
     bool scan_first;            // two streams: the scan goes first on all SMs, the attention behind it beside the walk
     int attn_sms;               // SMs the attention may fill (0: all)
+    bool compact_far;           // a compaction kernel would come behind a long attention
 };
 // A call that is being captured into a graph: its events cost nothing there.
 bool capturing(cudaStream_t st)
@@ -88,8 +89,10 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool
     // One B200, us a step, two streams against one: 50.7 and 38.1 on 52 heads and 4 K keys, 44.2 and 42.4 on 8 x 8 and 8 K,
     // both 17 chunks a CTA.)  What is known here is how long the sequences may be, not how long they are; so the merge of the key ranges
     // waits for the attention alone, not for the walk (when it did, a 2 K sequence in a context of 12 K rows or more took 37.1 us, two
-    // streams 34.2, and 31.1 now; 52 heads and 4 K keys 38.6 -> 39.0).  Below 12 chunks a range by max_len the two streams stay: no case there
-    // was slower on them, and what one stream would give has not been measured over the range.
+    // streams 34.2, and 31.1 now; 52 heads and 4 K keys 38.6 -> 39.0).  Behind a scan by the trees, which is short, one stream is the better
+    // way for an attention of any length: called one by one, 8 KV heads and 60 x 128256 at 1 K, 2 K and 4 K keys 31.2 -> 27.6, 32.2 -> 28.9 and
+    // 32.3 -> 28.8, 64 heads at 2 K 32.1 -> 28.5, two sequences 35.1 -> 33.8.  (60 x 32000 would gain as much, 28.3 -> 25.2, 60 x 50257 and 4 KV heads
+    // at 3 K 32.3 -> 29.1; below 12 chunks a range by max_len the order of calls behind a full scan is the one tests/test_host_side.py states.)
     // In a graph, where events cost nothing, the fork is the better way if the attention's CTAs find room beside the walk's: 29.7 against
     // 30.4 us (one stream) on the 2 K sequence, 37.8 and 38.4 on 52 heads, 17.3 and 18.1 at 580 keys, 45.3 and 46.5 on two such
     // sequences; where they do not, four short sequences of 32 heads take 33.8 in one stream and 44.8 forked.  A walk of single CTAs (less than 4096
@@ -101,15 +104,18 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool
         return (long long)batch * c.n_kv_heads * fspad_attn_mtiles(ctx, n_nodes, batch, n) * fspad_attn_umma_splits(ctx, n_nodes, batch, n);
     };
     const long long attn_ctas = ctas_on(sms);
-    StepPlan p = {false, false, 0};
+    StepPlan p = {false, false, 0, false};
     if (may_sample) {
         const int walk = fspad_walk_ctas(ctx, batch, c.vocab);
         const int beside = sms - (walk < sms / 2 ? walk : sms / 2), ranges = fspad_attn_umma_splits(ctx, n_nodes, batch, beside);
-        const bool one_stream = walk <= sms / 2 && (ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges);
+        const bool long_attn = ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges;
+        const bool one_stream = walk <= sms / 2 && (long_attn || fspad_scan_inner(sms, batch * n_nodes, c.vocab));
         const bool fork = !one_stream || (captured && ctas_on(beside) <= beside);
+        const bool scan_first = walk <= sms / 2 && long_attn ? walk > batch : sms - attn_ctas < sms / 4;
         p.chain = !fork;
-        p.scan_first = fork && (one_stream ? walk > batch : sms - attn_ctas < sms / 4);
-        if (one_stream || p.scan_first) p.attn_sms = beside;
+        p.scan_first = fork && scan_first;
+        p.compact_far = p.chain && long_attn;
+        if (scan_first || (walk <= sms / 2 && long_attn)) p.attn_sms = beside;
     } else {
         // An all-greedy acceptance is a scan and a one-CTA walk: beside an attention that holds most SMs the
         // scan's CTAs only get going when the attention's leave.  Where the context is short enough for the
@@ -541,7 +547,7 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
     // (4000 tokens) 29.4 and 24.9.  A sequence of temperature 0 among them has one CTA whatever the cluster: 256 slices 23 us and 22.4.
     const bool aliased = tree_k == nullptr;      // attention reads the cache rows that compaction rewrites
     int most_slices = 64;
-    if (plan.chain && may_sample) {
+    if (plan.compact_far) {
         const int by_cluster = 32 * (fspad_walk_ctas(ctx, batch, c.vocab) / batch);
         most_slices = by_cluster < 64 ? 64 : by_cluster > 256 ? 256 : by_cluster;
     }
