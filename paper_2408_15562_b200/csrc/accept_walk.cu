@@ -42,6 +42,8 @@
 // 0.5), the walk of a 60-node sampling step with eight rejections 53 -> 29 us.  (Masses
 // in double throughout, exact conversions of q and differences taken before scaling,
 // which came after these stamps, cost a step 0.3 to 0.7 us.)
+#include <climits>
+
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -51,6 +53,7 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kMaxCluster = 16;
+constexpr int kSmallerCluster = 10;        // where a batch needs more clusters than fit at once
 constexpr int kGreedyCluster = 8;          // all sequences greedy, rows of nodes without children not scanned
 constexpr int kWalkThreads = 512;          // 128 registers each: a thread keeps 16 tokens of the node's rows in them
 constexpr int kWarps = kWalkThreads / 32;
@@ -1530,6 +1533,14 @@ cudaError_t fspad_launch_walk_wait_selftest(fspad_ctx *ctx, int polls, cudaStrea
     return fspad_launch_opt(false, walk_wait_selftest_kernel, dim3(2), dim3(64), 0, st, 2u, ctx->d_status, (uint32_t)polls);
 }
 
+// Shared memory that parks a CTA's slice of a row (as the kernel shares it out): e_j in double, q_j in float.
+static size_t walk_parked_bytes(int cluster, int V)
+{
+    const size_t per_cta = (size_t)((((V + 3 + cluster - 1) / cluster) + 3) & ~3);
+    const size_t per_thr = ((per_cta + kWalkThreads - 1) / kWalkThreads + 3) & ~(size_t)3;
+    return per_thr * kWalkThreads * (sizeof(double) + sizeof(float));
+}
+
 typedef void (*WalkKernel)(const WalkArgs);
 static WalkKernel walk_kernel(bool narrow, bool inner)
 {
@@ -1539,9 +1550,10 @@ static WalkKernel walk_kernel(bool narrow, bool inner)
 
 // Cluster size of the sampling walk.  Once per context: raise the dynamic shared-memory limit and find
 // the largest cluster the device can co-schedule for these kernels: 16 (opt-in), else 8.  Small
-// vocabularies do not need the whole cluster.  (Halving the clusters of a batch whose CTAs outnumber the
-// SMs was measured and not kept: on 16 sequences, half of them greedy and gone at once, the acceptance
-// took 186 us with clusters of 8 against 143 us with clusters of 16 in two waves.)
+// vocabularies do not need the whole cluster.  A cluster's CTAs lie side by side, so fewer fit than the SMs
+// would hold: 7 of 16, 11 of 10, 15 of 8.  Where a batch may need more than the 7, clusters of 10 are taken, as long as a thread's
+// share of a row can be parked in shared memory.  us a step at 128256 tokens, clusters of 16, 10 and 8: 8 sequences 71, 63, 70; 11 73, 65, 78;
+// 16, half of them greedy, 124, 115, 145; 16 sampled 146, 129, 125; 10 at 50257 61, 53, 51.
 static int walk_cluster_size(fspad_ctx *ctx, int B, int V)
 {
     if (ctx->walk_cluster == 0) {
@@ -1549,6 +1561,7 @@ static int walk_cluster_size(fspad_ctx *ctx, int B, int V)
         static_assert(most + sizeof(SharedT<64, true>) <= 227 * 1024 && most_wide + sizeof(SharedT<FSPAD_MAX_NODES_WIDE, true>) <= 227 * 1024,
                       "shared memory of a CTA");
         bool all = true;
+        int fit = INT_MAX;
         for (int i = 0; i < 4; ++i) {
             const WalkKernel k = walk_kernel(i & 1, i & 2);
             const int bytes = i & 1 ? most : most_wide;
@@ -1564,12 +1577,17 @@ static int walk_cluster_size(fspad_ctx *ctx, int B, int V)
             probe.attrs = at; probe.numAttrs = 1;
             int n = 0;
             all = cudaOccupancyMaxActiveClusters(&n, k, &probe) == cudaSuccess && n >= 1;
+            fit = n < fit ? n : fit;
         }
         ctx->walk_cluster = all ? kMaxCluster : 8;
+        ctx->walk_fit = all ? fit : ctx->sm_count / 8;
         (void)cudaGetLastError();
     }
     int cluster = ctx->walk_cluster;
     while (cluster > 1 && (V + cluster - 1) / cluster < 2048) cluster >>= 1;
+    if (cluster == kMaxCluster && B > ctx->walk_fit &&
+        walk_parked_bytes(kSmallerCluster, V) <= (size_t)(ctx->cfg.max_nodes <= 64 ? kSmemBudget : kSmemBudgetWide))
+        cluster = kSmallerCluster;
     return cluster;
 }
 
@@ -1603,10 +1621,8 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *ctx, const float *logits, const 
     const int cluster = walk_cluster_size(ctx, B, V);
     // (16 sequences, half of them sampling: the walk 75 -> 68 us beside the attention, the step 202 -> 199; with one wave of clusters
     // the order does not matter and the look at the temperatures is saved)
-    a.sampled_first = B > 1 && B <= kWalkThreads && B * cluster > ctx->sm_count;     // (one thread looks at each sequence)
-    const size_t per_cta = (size_t)((((V + 3 + cluster - 1) / cluster) + 3) & ~3);       // as the kernel shares a row out
-    const size_t per_thr = ((per_cta + kWalkThreads - 1) / kWalkThreads + 3) & ~(size_t)3;
-    const size_t need = per_thr * kWalkThreads * (sizeof(double) + sizeof(float));
+    a.sampled_first = B > 1 && B <= kWalkThreads && (B * cluster > ctx->sm_count || cluster == kSmallerCluster);     // (one thread looks at each sequence)
+    const size_t need = walk_parked_bytes(cluster, V);
     size_t smem = inner ? 0 : (size_t)N * kPieceBytes;
     if (need <= (size_t)(N <= 64 ? kSmemBudget : kSmemBudgetWide)) { smem += need; a.cache_ok = 1; }
     // trees of up to 64 nodes and of up to FSPAD_MAX_NODES_WIDE nodes are two instances of the kernel

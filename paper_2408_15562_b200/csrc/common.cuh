@@ -46,7 +46,8 @@ struct fspad_ctx {
     float *row_max;           // [rows]
     double *row_sum;
     int *row_arg;
-    int walk_cluster;         // cluster size used by the sampling walk (0 = not probed yet)
+    int walk_cluster;         // largest cluster of the sampling walk (0 = not probed yet)
+    int walk_fit;             // how many of that size the device holds at once
 
     // whole-step entry point: attention runs on `side`, forked from and joined into the caller's stream
     cudaStream_t side;

@@ -113,3 +113,15 @@ def test_logits_read_where_they_are(vocab, nodes, batch, mode):
             hard, near, msgs = helpers.compare_accept(inp, path.numpy(), n.numpy(), bonus.numpy())
             assert hard == 0 and near == 0, msgs
             assert np.array_equal(new_len.numpy(), inp.prefix_len + n.numpy())
+
+
+@pytest.mark.parametrize("vocab,nodes,batch", [(32753, 20, 7), (32753, 20, 8), (50257, 12, 9), (128256, 10, 12), (151936, 66, 8)])
+@pytest.mark.parametrize("mode", ["sample", "mixed"])
+def test_batches_of_more_clusters_than_fit_at_once(vocab, nodes, batch, mode):
+    """Clusters of 16 up to seven sequences, of ten beyond (but where a slice of the row would not fit into shared memory), sampling
+    sequences first: every number of rejections, draws at leaves and inside."""
+    temps = ((1.0, 0.7) * 8 if mode == "sample" else (0.0, 1.0, 0.6, 1.0) * 4)[:batch]
+    for variant in range(2):
+        w = synth.scaled(W["llama3_8b_2k"], batch=batch, vocab=vocab, n_nodes=nodes, depth=3, branch=9 if nodes <= 64 else 12,
+                         temperatures=temps, prefix=(8, 8))
+        _parity(synth.generate(w, variant, with_attention=False))
