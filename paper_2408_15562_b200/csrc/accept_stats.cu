@@ -510,7 +510,7 @@ cudaError_t fspad_launch_stats_partials(fspad_ctx *ctx, const float *logits, con
     const bool aligned = (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
     if (geom->parent != nullptr && aligned && rows % rows_per_seq == 0 &&
-        (geom->stage != nullptr ? fspad_scan_inner_fits(sms, rows, V) : fspad_scan_inner(sms, rows, V))) {
+        (geom->stage != nullptr ? fspad_scan_inner_fits(sms, rows, V) : fspad_scan_inner(sms, rows, rows_per_seq, V))) {
         *geom = fspad_stats_geom_inner(sms, rows, V, ctx->stats_slots, geom->parent, geom->stage);
         const FspadStatsGeom &g = *geom;
         const int wide = (g.upr + g.per_row - 2) / (g.per_row - 1);

@@ -91,8 +91,9 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool
     // waits for the attention alone, not for the walk (when it did, a 2 K sequence in a context of 12 K rows or more took 37.1 us, two
     // streams 34.2, and 31.1 now; 52 heads and 4 K keys 38.6 -> 39.0).  Behind a scan by the trees, which is short, one stream is the better
     // way for an attention of any length: called one by one, 8 KV heads and 60 x 128256 at 1 K, 2 K and 4 K keys 31.2 -> 27.6, 32.2 -> 28.9 and
-    // 32.3 -> 28.8, 64 heads at 2 K 32.1 -> 28.5, two sequences 35.1 -> 33.8.  (60 x 32000 would gain as much, 28.3 -> 25.2, 60 x 50257 and 4 KV heads
-    // at 3 K 32.3 -> 29.1; below 12 chunks a range by max_len the order of calls behind a full scan is the one tests/test_host_side.py states.)
+    // 32.3 -> 28.8, 64 heads at 2 K 32.1 -> 28.5, two sequences 35.1 -> 33.8.  (60 x 32000 would gain as much, 28.3 -> 25.2;
+    // below 12 chunks a range by max_len the order of calls behind a full scan is the one tests/test_host_side.py states.)  Captured, such a
+    // step forks only where the scan goes first: beside an attention on most SMs it is the longer way (52 heads and 1 K keys 38.7).
     // In a graph, where events cost nothing, the fork is the better way if the attention's CTAs find room beside the walk's: 29.7 against
     // 30.4 us (one stream) on the 2 K sequence, 37.8 and 38.4 on 52 heads, 17.3 and 18.1 at 580 keys, 45.3 and 46.5 on two such
     // sequences; where they do not, four short sequences of 32 heads take 33.8 in one stream and 44.8 forked.  A walk of single CTAs (less than 4096
@@ -109,9 +110,9 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool
         const int walk = fspad_walk_ctas(ctx, batch, c.vocab);
         const int beside = sms - (walk < sms / 2 ? walk : sms / 2), ranges = fspad_attn_umma_splits(ctx, n_nodes, batch, beside);
         const bool long_attn = ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges;
-        const bool one_stream = walk <= sms / 2 && (long_attn || fspad_scan_inner(sms, batch * n_nodes, c.vocab));
-        const bool fork = !one_stream || (captured && ctas_on(beside) <= beside);
+        const bool one_stream = walk <= sms / 2 && (long_attn || fspad_scan_inner(sms, batch * n_nodes, n_nodes, c.vocab));
         const bool scan_first = walk <= sms / 2 && long_attn ? walk > batch : sms - attn_ctas < sms / 4;
+        const bool fork = !one_stream || (captured && ctas_on(beside) <= beside && (long_attn || scan_first));
         p.chain = !fork;
         p.scan_first = fork && scan_first;
         p.compact_far = p.chain && long_attn;

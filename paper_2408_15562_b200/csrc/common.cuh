@@ -187,18 +187,19 @@ static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int 
     return g;
 }
 // Whether the scan of these rows can go by the trees, and whether it does.  Looking for the rows takes about a microsecond, and a walk that ends in a node
-// without children two more; against that stand three quarters of the scan.  Us a step, all rows and by the trees: 60 x 32000
-// 21.2 and 22.6, 40 x 64000 28.9 and 29.2, 60 x 50257 32.8 and 33.0 (greedy 21.2 and 20.8), 120 x 32000 32.6 and 32.9, 240 x 32000 36.7
-// and 35.9, 60 x 128256 35.0 and 32.3, 960 x 128256 191 and 126.  Few rows of 128256 tokens are read by the trees whatever their
-// number, because all SMs share a row otherwise and the walk has more pieces to merge than it takes at once: 8 rows 31.1 and 25.0, 30 32.4 and 29.7.
+// without children one or two more; against that stand three quarters of the scan (less of small trees: half of 11 nodes have children),
+// and a step behind the short scan stays in one stream.  Us a step, all rows and by the trees: 60 x 32000 21.2 and 22.6, 40 x 64000 28.7
+// and 26.9, 60 x 50257 32.6 and 29.7 (greedy 21.6 and 19.5), 2 x 40 x 32000 31.9 and 28.3, 4 x 20 x 32000 27.6 and 24.9, but 7 x 11 x 32001 32.5 and 34.0, 5 x 9 x 128256 26.9 and 28.8;
+// 240 x 32000 36.7 and 35.9, 60 x 128256 35.0 and 32.3, 960 x 128256 191 and 126.  Few rows of 128256 tokens are read by the trees whatever the
+// trees, because all SMs share a row otherwise and the walk has more pieces to merge than it takes at once: 8 rows 31.1 and 25.0, 2 x 10 31.8 and 28.4.
 static inline bool fspad_scan_inner_fits(int sm_count, int rows, int V)
 {
     return rows <= FSPAD_INNER_MAX_ROWS && (long long)rows * (V + 6ll) < 1ll << 31 &&
            rows / (sm_count * (1024 / FSPAD_STATS_THREADS)) + 2 <= FSPAD_INNER_LIST;
 }
-static inline bool fspad_scan_inner(int sm_count, int rows, int V)
+static inline bool fspad_scan_inner(int sm_count, int rows, int nodes, int V)
 {
-    return fspad_scan_inner_fits(sm_count, rows, V) && ((long long)rows * V >= 7 << 19 || V > 98304);
+    return fspad_scan_inner_fits(sm_count, rows, V) && ((long long)rows * V >= (nodes >= 16 ? 1 << 21 : 1 << 23) || (V > 98304 && rows <= 32));
 }
 
 #ifdef __CUDACC__
