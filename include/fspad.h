@@ -166,7 +166,8 @@ int fspad_tree_accept(fspad_ctx *ctx, const float *target_logits, const float *d
                       int32_t *n_accepted, int32_t *bonus_token, void *stream);
 
 /*
- * The first stage of fspad_tree_accept on its own: one pass over every row of
+ * The first stage of fspad_tree_accept on its own, over every row (which fspad_tree_accept
+ * itself takes on small arrays; on large ones it leaves out the rows of nodes without children): one pass over
  * logits [rows][V] giving row_max (fp32 maximum), row_arg (its lowest index)
  * and row_sum = sum_j exp((x_j - max)/T_row) accumulated from fp32 exponentials
  * (relative accuracy about 1e-6; the acceptance walk re-derives exact sums
@@ -429,7 +430,7 @@ int fspad_kv_compact_paged(fspad_ctx *ctx, fspad_bf16 *pool, const int32_t *bloc
  * reads the cache rows compaction rewrites); when they are NULL (tree rows
  * taken from cache rows L_b ..) compaction waits for the attention as well.
  * In the first case, when a sequence has at most 64 (layer, K/V, kv head)
- * slices (where a sampling step stays in one stream, 32 for each CTA of the walk's cluster,
+ * slices (where a sampling step with a long attention stays in one stream, 32 for each CTA of the walk's cluster,
  * up to 256), the kernel that walks the tree makes the compaction's moves itself,
  * greedy or sampling (same result; an invalid prefix length is then reported by
  * that kernel).

@@ -28,6 +28,10 @@
 // c into c + U / D, which is exactly p <- norm(max(p - q, 0)), q <- norm(q
 // without x) written without materialising either vector.
 //
+// Where the scan has gone by the trees it has left out the rows of nodes without
+// children.  A walk comes to one of them at its end at most: it then draws from the row, or
+// takes its argmax, itself.
+//
 // The per-row maximum and argmax come exact from the vocabulary scan; its sum
 // of exponentials is fp32-accurate and is trusted only when a decision clears
 // a 1e-4 relative margin, otherwise (and before any residual) the exact sum is
