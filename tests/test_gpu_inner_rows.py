@@ -4,6 +4,8 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
+
 from paper_2408_15562_b200 import binding, synth
 from tests import helpers
 from tests.test_gpu_accept import _run
@@ -125,3 +127,62 @@ def test_batches_of_more_clusters_than_fit_at_once(vocab, nodes, batch, mode):
         w = synth.scaled(W["llama3_8b_2k"], batch=batch, vocab=vocab, n_nodes=nodes, depth=3, branch=9 if nodes <= 64 else 12,
                          temperatures=temps, prefix=(8, 8))
         _parity(synth.generate(w, variant, with_attention=False))
+
+
+@pytest.mark.parametrize("hq,hkv,prefix,nodes,batch,vocab,temps", [
+    (32, 8, 1500, 60, 1, 50257, (1.0,)),                 # several key ranges behind the walk in one stream, from a graph forked behind the scan
+    (52, 52, 700, 48, 1, 50257, (1.0,)),                 # an attention on most SMs: one stream either way
+    (32, 8, 700, 40, 2, 50257, (0.8, 0.0)),
+    (32, 8, 300, 24, 9, 32753, (1.0, 0.0, 0.7) * 3),     # more clusters than fit at once: forked
+])
+def test_step_called_and_captured(hq, hkv, prefix, nodes, batch, vocab, temps):
+    """The step behind a scan by the trees: called, and replayed from a graph twice, it gives the same bits, and the acceptance and the
+    compacted cache are those of the separate calls."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=batch, prefix=(prefix, prefix + 40), n_q_heads=hq, n_kv_heads=hkv, n_nodes=nodes, depth=4,
+                     branch=12, vocab=vocab, temperatures=temps, n_layers=1)
+    inp = synth.generate(w, 6)
+    assert inp.parent.size * vocab >= 1 << 21
+    B, N = inp.parent.shape
+    ctx = helpers.make_ctx(inp, n_layers=1)
+    cache0 = binding.bf16_tensor(synth.make_cache(inp, 1))
+    d, a = helpers.upload_accept(inp), helpers.upload_attn(inp)
+    L = inp.prefix_len
+    for b in range(B):
+        cache0[0, 0, b, :, L[b]:L[b] + N] = a["tree_k"][b]
+        cache0[0, 1, b, :, L[b]:L[b] + N] = a["tree_v"][b]
+    i32 = dict(dtype=torch.int32, device="cuda")
+
+    def outputs():
+        return [torch.zeros_like(a["q"]), torch.zeros((B, N), **i32)] + [torch.zeros((B,), **i32) for _ in range(3)]
+
+    def step(cache, out):
+        ctx.verify_step(cache, a["q"], a["tree_k"], a["tree_v"], d["parent"], a["prefix_len"], d["target_logits"], d["draft_probs"],
+                        d["draft_tokens"], d["temperature"], d["uniforms"], *out)
+
+    called, cache = outputs(), cache0.clone()
+    step(cache, called)
+    ctx.check()
+    path, n, bonus = ctx.tree_accept(d["target_logits"], d["draft_probs"], d["draft_tokens"], d["parent"], d["temperature"], d["uniforms"])
+    want = cache0.clone()
+    new_len = ctx.kv_compact(want, path, n, a["prefix_len"])
+    for got, ref in zip(called[1:] + [cache], [path, n, bonus, new_len, want]):
+        assert torch.equal(got.view(torch.int16), ref.view(torch.int16))
+    hard, near, msgs = helpers.compare_accept(inp, path.cpu().numpy(), n.cpu().numpy(), bonus.cpu().numpy())
+    assert hard == 0, msgs
+    replayed, cache_g = outputs(), cache0.clone()
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        step(cache_g, replayed)
+    for _ in range(2):
+        cache_g.copy_(cache0)
+        for t in replayed:
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        ctx.check()
+        for got, ref in zip(replayed + [cache_g], called + [cache]):
+            assert torch.equal(got.view(torch.int16), ref.view(torch.int16))
+    ref_o = oracle.tree_attn(inp.q, inp.k_cache, inp.v_cache, inp.tree_k, inp.tree_v, inp.parent, L)
+    mx, mean = helpers.attn_errors(called[0], ref_o)
+    assert mx <= 1e-2 and mean <= 1e-3
