@@ -217,14 +217,15 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
     }
 }
 
-// Positions j .. j + 3 of a row, from memory this thread has written itself.
+// Positions j .. j + 3 of a row, from memory this thread has written itself.  (Past the first-level cache: the other half of a line's
+// 32 bytes may be another CTA's and not there yet.)
 static __device__ __noinline__ float4 own4(const float *x, int j, int V)
 {
     float4 r = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-    if (j >= 0 && j < V) r.x = x[j];
-    if (j + 1 >= 0 && j + 1 < V) r.y = x[j + 1];
-    if (j + 2 >= 0 && j + 2 < V) r.z = x[j + 2];
-    if (j + 3 >= 0 && j + 3 < V) r.w = x[j + 3];
+    if (j >= 0 && j < V) r.x = __ldcg(x + j);
+    if (j + 1 >= 0 && j + 1 < V) r.y = __ldcg(x + j + 1);
+    if (j + 2 >= 0 && j + 2 < V) r.z = __ldcg(x + j + 2);
+    if (j + 3 >= 0 && j + 3 < V) r.w = __ldcg(x + j + 3);
     return r;
 }
 

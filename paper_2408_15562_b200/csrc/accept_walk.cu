@@ -132,8 +132,12 @@ template <int MAXN> struct TreeShared<MAXN, true> : TreeShared<MAXN, false> {
     int last;                       // greedy: the node the walk ended at, if its row is still to be looked at, else -1
     unsigned long long best;        // ... the row's maximum and where it is (see argmax_key)
 };
+// The logits' rows as the walk sweeps them: those that the scan has gone over by the trees it may have brought to the device itself.
+template <bool INNER> struct LogitsRow { typedef const float *__restrict__ T; };
+template <> struct LogitsRow<true> { typedef FspadLateRow T; };
 // (The functions that are not inlined are instantiated by it, too, so that what one kind of walk calls has no say in the other's registers.)
 template <int MAXN, bool INNER> struct SharedT {
+    typedef typename LogitsRow<INNER>::T Row;
     TreeShared<MAXN, INNER> t;
     alignas(128) double exp_tbl[kExpTable];      // 2^(i/16)
     // what thread 0 asks for and about which node (written by thread 0, read by all after a barrier)
@@ -324,7 +328,7 @@ enum { MODE_EXP = 0, MODE_RESID = 1, MODE_CDF = 2 };
 // With `found` the running sum starts at run and *found receives the first token where it exceeds target (else the
 // last positive-weight token).
 template <class Shared>
-__device__ __noinline__ double sweep_row(int mode, const Shared &sh, const float *__restrict__ x, const float *__restrict__ q,
+__device__ __noinline__ double sweep_row(int mode, const Shared &sh, typename Shared::Row x, const float *__restrict__ q,
                                          const double *__restrict__ se, const float *__restrict__ sq, int stride, Chunk ck,
                                          bool parked, const ExpArg &arg, double C, int xnew, double run, double target, int *found)
 {
@@ -429,7 +433,7 @@ __device__ __forceinline__ double residual_of_tile(const double (&er)[kTile], co
 // four in flight): it runs two or three times per launch, and eight unrolled tokens spent longer on their first pass
 // through the instruction cache (3 us) than on the work.
 template <class Shared>
-__device__ __forceinline__ void fused_reject_sweep(const Shared &sh, const float *__restrict__ x, const float *__restrict__ q,
+__device__ __forceinline__ void fused_reject_sweep(const Shared &sh, typename Shared::Row x, const float *__restrict__ q,
                                                    double *__restrict__ se, float *__restrict__ sq, int stride, Chunk ck,
                                                    int per_thr, bool park, const ExpArg &arg, double S, int xnew, int node,
                                                    int n_nodes, double (&v)[5])
@@ -911,7 +915,8 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         b = sh.cur;
     }
     // The vocabulary scan that precedes this kernel in the stream lets it start only after the scan's
-    // own predecessor has completed, and the scan writes nothing but its partial results.  So the
+    // own predecessor has completed, and the scan writes nothing of the caller's: only its partial
+    // results and, of logits in host memory, the rows that it brings to the device.  So the
     // caller's arrays may be read before the scan has finished: the prologue's two round trips of
     // dependent loads run under the scan's tail.
     // Round trip 1: everything that depends on nothing - temperature, tree arrays, uniforms.
@@ -946,7 +951,9 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
     }
     const bool sampling = Tf > 0.0f;
     const size_t row0 = (size_t)b * N;           // the sequence's first row
-    const float *lg = args.logits + row0 * V, *dp = args.draft + row0 * V;
+    typedef typename Shared::Row Row;
+    const Row lg{args.logits + row0 * V};
+    const float *dp = args.draft + row0 * V;
     const float kT = kLog2eF / (sampling ? Tf : 1.0f);
 
     // Round trip 2: thread c owns node c (tree arrays, and the scalars its accept test needs: target logit and draft
@@ -961,7 +968,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
             if constexpr (INNER) sh.t.known[p] = 1;
             if (sampling) {
                 const size_t at = (size_t)p * V + t;
-                xv = INNER ? args.given[row0 * V + at] : lg[at];       // (the scan may still be bringing the row)
+                xv = args.given[row0 * V + at];                        // (the scan may still be bringing the row)
                 qv = dp[at];
             }
         }
@@ -1250,7 +1257,8 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         const int req = sh.req;
         if (req == REQ_DONE) break;                           // uniform
         const int cur = sh.cur, xn = sh.xnew;
-        const float *x = lg + (size_t)cur * V, *q = dp + (size_t)cur * V;
+        const Row x = lg + (size_t)cur * V;
+        const float *q = dp + (size_t)cur * V;
         const Chunk ck = chunk_of((row0 + cur) * V, V, per_cta, per_thr, rank, tid);
         const ExpArg arg = exp_arg(sh.rowM[cur], invT);
         got = GOT_RESIDUAL;
@@ -1340,7 +1348,8 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
 
     // ---- bonus token: inverse CDF of the current residual at the last node ----
     const int cur = sh.cur;
-    const float *x = lg + (size_t)cur * V, *q = dp + (size_t)cur * V;
+    const Row x = lg + (size_t)cur * V;
+    const float *q = dp + (size_t)cur * V;
     const double c = sh.C;
     // A draw at a node where nothing was rejected (a leaf, typically) is taken from the softmax
     // of the row itself.  The scan left the mass of every piece of the row, accurate to kScanRel:
@@ -1365,7 +1374,7 @@ accept_walk_kernel(const __grid_constant__ WalkArgs args)
         }
     }
     const int n_piece = INNER ? 0 : sh.piece_cnt[cur];
-    if (!INNER && !sh.bonus_ok && c == 0.0 && sh.nrem == 0 && n_piece > 0) {
+    if constexpr (!INNER) if (!sh.bonus_ok && c == 0.0 && sh.nrem == 0 && n_piece > 0) {
         // every warp scans the pieces' masses: prefix of the piece the target falls into
         double cum = lane < n_piece ? piece_w[cur][lane & (kPieceSlots - 1)] : 0.0;
         const double own = cum;

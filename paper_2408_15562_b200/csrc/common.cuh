@@ -222,6 +222,30 @@ __device__ __forceinline__ float4 fspad_load4(const float *__restrict__ x, int j
     return fspad_edge4(x, j, hi, pad);
 }
 
+// A row that an earlier kernel may still be writing when this one starts: read behind fspad_pdl_wait, and by plain loads.  The loads
+// above go by the read-only path, which is for data that nobody writes during the reading kernel's life.  (A type of its own, so that
+// such a row cannot come to them.)
+struct FspadLateRow {
+    const float *p;
+    __device__ __forceinline__ FspadLateRow operator+(size_t n) const { return FspadLateRow{p + n}; }
+    __device__ __forceinline__ float operator[](int j) const { return p[j]; }
+};
+static __device__ __noinline__ float4 fspad_late_edge4(FspadLateRow x, int j, int hi, float pad)
+{
+    float4 r = make_float4(pad, pad, pad, pad);
+    if (j >= 0 && j < hi) r.x = x[j];
+    if (j + 1 >= 0 && j + 1 < hi) r.y = x[j + 1];
+    if (j + 2 >= 0 && j + 2 < hi) r.z = x[j + 2];
+    if (j + 3 >= 0 && j + 3 < hi) r.w = x[j + 3];
+    return r;
+}
+__device__ __forceinline__ float4 fspad_load4(FspadLateRow x, int j, int hi, float pad)
+{
+    if (j >= 0 && j + 4 <= hi) return *reinterpret_cast<const float4 *>(x.p + j);
+    if (j + 4 <= 0 || j >= hi) return make_float4(pad, pad, pad, pad);
+    return fspad_late_edge4(x, j, hi, pad);
+}
+
 // Merge the per-CTA partials of one row (warp-collective: all 32 lanes call it and all get
 // the result): maximum, its lowest index, and the sum of exponentials rescaled to that
 // maximum (k = log2(e)/T).  Every lane fetches up to two partial slots, so the loads of a
@@ -276,8 +300,8 @@ __device__ __forceinline__ void fspad_stats_merge_warp(const FspadStatsPart *__r
 // while results stay exactly those of plain stream order.
 // The acceptance walk is the exception: it reads the caller's arrays (trees, logits, draft rows) before its wait.  It may,
 // because the two kernels that can precede it, the vocabulary scan and the LM head's merge, let it start only after their own
-// wait, when everything queued before them is complete, and themselves write nothing but scan partials, which the walk reads
-// after its wait.  The attention of a step called as one is the other: launched behind the walk, it starts when every CTA of the
+// wait, when everything queued before them is complete, and themselves write nothing but what the walk reads after its wait and not by
+// the read-only path: scan partials and, of logits in host memory, the rows that the scan brings to the device (FspadLateRow).  The attention of a step called as one is the other: launched behind the walk, it starts when every CTA of the
 // walk has, reads what was complete before the scan started, and waits for the walk at its end.  The merge of its key ranges reads
 // the partials as soon as a count of the attention's CTAs says that they are there, and waits for the attention at its end.  Kernels whose predecessor is not one kernel of the same stream (behind a fork, a join or a copy) may be
 // launched without the attribute.

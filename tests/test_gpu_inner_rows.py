@@ -186,3 +186,40 @@ def test_step_called_and_captured(hq, hkv, prefix, nodes, batch, vocab, temps):
     ref_o = oracle.tree_attn(inp.q, inp.k_cache, inp.v_cache, inp.tree_k, inp.tree_v, inp.parent, L)
     mx, mean = helpers.attn_errors(called[0], ref_o)
     assert mx <= 1e-2 and mean <= 1e-3
+
+
+def _host_step(ctx, inp, logits):
+    """The host entry point on `inp` with its logits in `logits`: the outputs and the cache."""
+    B, N = inp.parent.shape
+    sampling = inp.draft_probs is not None
+    pin = lambda a: torch.from_numpy(np.ascontiguousarray(a)).pin_memory()   # noqa: E731
+    cache = binding.bf16_tensor(synth.make_cache(inp, 1))
+    out = torch.empty(inp.q.shape, dtype=torch.bfloat16).pin_memory()
+    path = torch.empty((B, N), dtype=torch.int32)
+    n, bonus, new_len = (torch.empty((B,), dtype=torch.int32) for _ in range(3))
+    ctx.verify_step_host(cache, *(binding.bf16_tensor(a, "cpu").pin_memory() for a in (inp.q, inp.tree_k, inp.tree_v)), pin(inp.parent),
+                         pin(inp.prefix_len), logits, pin(inp.draft_probs) if sampling else None, pin(inp.draft_tokens),
+                         pin(inp.temperature), pin(inp.uniforms) if sampling else None, out, path, n, bonus, new_len)
+    return out, path, n, bonus, new_len, cache
+
+
+# every row, or every other one, has children: more pieces of rows than CTAs
+@pytest.mark.parametrize("tree,branch,nodes,batch,vocab", [("chain", 1, 60, 1, 50257), ("chain", 1, 40, 2, 32000), ("bfs", 2, 120, 1, 32753)])
+@pytest.mark.parametrize("mode", ["greedy", "sample"])
+def test_most_rows_read_where_they_are(tree, branch, nodes, batch, vocab, mode):
+    """Rows that the scan brings to the device while the walk that sweeps them is already resident: other logits in the same memory at
+    every call, and the oracle's acceptance each time (children are rejected at the root at least once)."""
+    w = synth.scaled(W["llama3_8b_2k"], batch=batch, prefix=(40, 300), n_nodes=nodes, tree=tree, branch=branch, vocab=vocab,
+                     temperatures=((0.0, 0.0) if mode == "greedy" else (1.0, 0.7))[:batch])
+    inps = [synth.generate(w, v) for v in (1, 2, 3, 4)]
+    ctx = helpers.make_ctx(inps[0], n_layers=1)
+    logits = torch.empty(inps[0].target_logits.shape).pin_memory()
+    rejected = 0
+    for inp in inps:
+        logits.copy_(torch.from_numpy(inp.target_logits))
+        _, path, n, bonus, new_len, _ = _host_step(ctx, inp, logits)
+        hard, near, msgs = helpers.compare_accept(inp, path.numpy(), n.numpy(), bonus.numpy())
+        assert hard == 0 and near == 0, msgs
+        assert np.array_equal(new_len.numpy(), inp.prefix_len + n.numpy())
+        rejected += int((n.numpy() < 2).sum())
+    assert rejected > 0
