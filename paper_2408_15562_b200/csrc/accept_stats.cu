@@ -273,7 +273,7 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
         q.n = n;
         q.j0 = 4 * off - (int)(((size_t)row * V) & 3);
         q.x = reinterpret_cast<const float4 *>(logits + (size_t)row * V + q.j0);
-        q.n_load = min(n, (V - q.j0 + (row + 1 < rows ? 3 : 0)) >> 2);
+        q.n_load = fspad_whole_units(rows, row, V, q.j0, n);
         const float T = temperature ? temperature[(unsigned)row / (unsigned)N] : 1.0f;
         q.k = kLog2e / (T > 0.0f ? T : 1.0f);
         return q;

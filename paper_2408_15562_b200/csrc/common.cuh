@@ -202,6 +202,17 @@ static inline bool fspad_scan_inner(int sm_count, int rows, int nodes, int V)
     return fspad_scan_inner_fits(sm_count, rows, V) && ((long long)rows * V >= (nodes >= 16 ? 1 << 21 : 1 << 23) || (V > 98304 && rows <= 32));
 }
 
+// How many of the first n units of four positions of row `row`, from position j0 of it on, can be loaded whole: the last one may reach
+// into the next rows (its caller leaves out what is not the row's), but not past the end of the array [rows][V].
+#ifdef __CUDACC__
+__device__
+#endif
+static inline int fspad_whole_units(int rows, int row, int V, int j0, int n)
+{
+    const int behind = (rows - 1 - row) * V, whole = (V - j0 + (behind < 3 ? behind : 3)) >> 2;
+    return n < whole ? n : whole;
+}
+
 #ifdef __CUDACC__
 // ---- rows read 16 bytes at a time whatever their length ----
 // Positions j .. j + 3 of a row whose valid positions are [0, hi); x + j is 16-byte aligned.  A group that reaches past either

@@ -45,5 +45,6 @@ int load4(const float *x, int j, int hi, int late, float *out)
 }
 // whether a late row can come to a load of the read-only path
 int late_row_is_a_pointer() { return std::is_convertible<FspadLateRow, const float *>::value; }
+int whole_units(int rows, int row, int V, int j0, int n) { return fspad_whole_units(rows, row, V, j0, n); }
 
 }  // extern "C"

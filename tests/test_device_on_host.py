@@ -42,3 +42,17 @@ def test_the_walk_takes_rows_that_the_scan_brings_as_late_ones(lib):
     walk = open(os.path.join(CSRC, "accept_walk.cu")).read()
     assert re.search(r"struct LogitsRow<true> \{ typedef FspadLateRow T; \}", walk)
     assert re.findall(r"args\.logits\b[^;]*", walk) == ["args.logits + row0 * V}"] and "const Row lg{args.logits" in walk
+
+
+@pytest.mark.parametrize("vocab", [1, 2, 3, 4, 5, 6, 7, 9])
+def test_units_loaded_whole_lie_in_the_array(lib, vocab):
+    """The scan by the trees loads a row's units of four whole where they end in a row behind it, however short those rows are: all
+    that it loads whole lies in the array, and every unit of the row that does is loaded whole."""
+    for rows in range(1, 8):
+        for row in range(rows):
+            start = row * vocab
+            j0 = -(start & 3)
+            units = (vocab - j0 + 3) // 4
+            whole = [i for i in range(units) if start + j0 + 4 * i + 4 <= rows * vocab]
+            for n in range(units + 1):
+                assert max(0, lib.whole_units(rows, row, vocab, j0, n)) == len([i for i in whole if i < n]), (rows, row, n)

@@ -223,3 +223,18 @@ def test_most_rows_read_where_they_are(tree, branch, nodes, batch, vocab, mode):
         assert np.array_equal(new_len.numpy(), inp.prefix_len + n.numpy())
         rejected += int((n.numpy() < 2).sum())
     assert rejected > 0
+
+
+@pytest.mark.parametrize("vocab", [1, 2, 3, 5])
+@pytest.mark.parametrize("mode", ["greedy", "sample"])
+def test_rows_of_less_than_a_unit(vocab, mode):
+    """The host entry point on rows shorter than the unit they are read by, from logits that end where their allocation ends."""
+    nodes, batch = 6, 3
+    w = synth.scaled(W["llama3_8b_2k"], batch=batch, prefix=(8, 40), n_nodes=nodes, tree="chain", vocab=vocab,
+                     temperatures=(0.0,) * batch if mode == "greedy" else (1.0, 0.0, 0.7))
+    for variant in range(3):
+        inp = synth.generate(w, variant)
+        ctx = helpers.make_ctx(inp, n_layers=1)
+        _, path, n, bonus, _, _ = _host_step(ctx, inp, torch.from_numpy(inp.target_logits).pin_memory())
+        hard, near, msgs = helpers.compare_accept(inp, path.numpy(), n.numpy(), bonus.numpy())
+        assert hard == 0 and near == 0, msgs
