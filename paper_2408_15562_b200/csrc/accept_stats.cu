@@ -217,6 +217,14 @@ accept_stats_kernel(const float *__restrict__ logits, const float *__restrict__ 
     }
 }
 
+// The largest of a warp's values.
+static __device__ __forceinline__ float warp_max(float v)
+{
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+    return m;
+}
+
 // Positions j .. j + 3 of a row, from memory this thread has written itself.  (Past the first-level cache: the other half of a line's
 // 32 bytes may be another CTA's and not there yet.)
 static __device__ __noinline__ float4 own4(const float *x, int j, int V)
@@ -234,13 +242,18 @@ static __device__ __noinline__ float4 own4(const float *x, int j, int V)
 // walk.  Two ways of finding the rows:
 //   SHARED = false  few rows: a CTA for every piece of every row, gridDim.x pieces by gridDim.y rows, and those of a row that is
 //                   nobody's parent leave at once
-//   SHARED = true   every CTA marks the nodes that are somebody's parent, a bit a row, and numbers them; where their pieces are no
-//                   more than the CTAs it takes one, else an equal share of their rows laid end to end, the first loads of a run
-//                   being in flight while the one before it is reduced
-// Bound by HBM where the rows are many (240 of 128256: 26 us, 4.7 TB/s; the scan of all 960 80 us), by the chain of launch, parents,
-// loads and reduction where they are few (15 of 60 rows: 4.5 us; all 60 9.4).  A share may cross rows.  The run of a row that a CTA takes is reduced as a whole, and its result goes to slot 0 if the run begins
-// the row, else to the one behind the stretch of `wide` units it starts in: every share is at least that long, so no two meet.  The
-// slots in between are empty.
+//   SHARED = true   every CTA marks the nodes that are somebody's parent, a bit a row, and every warp numbers them for itself.  A row is
+//                   cut into as many pieces as give every CTA one, up to g.per_row; where that leaves two fifths of the CTAs idle, or
+//                   there are more rows than CTAs, each takes an equal share of the rows laid end to end instead, the first loads of
+//                   a run being in flight while the one before it is reduced
+// Bound by HBM where the rows are many, else by the chain of launch, parents, loads and reduction: parents marked 0.7 us after the start,
+// piece known 1.3 to 1.6, loads back 2.2 to 2.7, partials written 3.3 to 3.8 (60 nodes of 50257 and 128256 tokens).  One piece to a CTA wherever
+// that fills three fifths of them, because a second run costs a reduction (1.1 us) more than the idle CTAs do.  Acceptance alone, greedy, us
+// from a graph, all rows / shares with pairs of (maximum, sum) merged step by step / this: 60 x 32000 eight times 18.0 / 15.3 / 11.7, 25 x 32001
+// six times 8.2 / 13.0 / 9.8, 60 x 128256 16 times 83.5 / 33.8 / 32.3, a chain of 60 x 128256 12.3 / 15.6 / 12.3.
+//   The run of a row that a CTA takes is reduced as a whole.  Of a share its result goes to slot 0 if the run begins the row, else to the
+// one behind the stretch of `wide` units it starts in: every share is at least that long, so no two meet.  Slots without a run of their
+// own are empty.
 // STAGE: the logits are in host memory, and the rows read are left at g.stage for the walk.
 template <bool SHARED, bool STAGE>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
@@ -249,18 +262,17 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
 {
     typedef Unit<4> U4;
     constexpr int kStep = kThreads * kDeep, kWords = SHARED ? FSPAD_INNER_MAX_ROWS / 32 : 1, kList = SHARED ? FSPAD_INNER_LIST : 1;
+    constexpr int kWarps = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, upr = g.upr;
-    __shared__ unsigned word[kWords];
-    __shared__ int list[kList], warp_n[kThreads / 32];
-    __shared__ Acc wacc[kThreads / 32];
-    __shared__ float s_bmax;
-    __shared__ int s_barg;
-    unsigned hi = 0;                             // SHARED: end of the share, in units of the rows laid end to end (below 2^31)
-    int first = 0, last = 0;                     // the rows it touches, by number
-    bool one_piece = true;
+    __shared__ unsigned word[kWords];            // SHARED: a bit a row, set where it is somebody's parent
+    __shared__ int list[kList];                  // the rows of the CTA's share
+    __shared__ float2 wacc[2][kWarps];           // (by the parity of the run, as s_at: what one run leaves is read while the next begins)
+    __shared__ int s_at[2];
+    static_assert(kWords <= kThreads, "a word to a thread");
     if constexpr (SHARED)
         if (tid < kWords) word[tid] = 0u;
-    static_assert(kWords <= kThreads, "a word to a thread");
+    if (tid < 2) s_at[tid] = 0x7fffffff;
+    __syncthreads();
     struct Run {
         const float4 *x;                         // its units off .. off + n - 1 of the row, from token j0 on (up to three in front of the row)
         int row, off, j0, n, n_load;             // n_load: how many of them can be loaded whole (the rest has no token or ends the array)
@@ -289,9 +301,11 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
     };
     fspad_pdl_wait();                            // (the order of the two: see the scan of all rows)
     fspad_pdl_trigger();
+    unsigned hi = 0;                             // end of the share, in units of the rows laid end to end (below 2^31)
+    int first = 0, last = 0;                     // the rows it touches, by number
+    int piece = (int)blockIdx.x, pieces = g.per_row;   // pieces: 0 where the rows are shared out laid end to end
     Run q;
     if constexpr (SHARED) {
-        __syncthreads();
         int c = (int)((unsigned)tid % (unsigned)N);
         const int step = (int)((unsigned)kThreads % (unsigned)N);
 #pragma unroll 4
@@ -302,42 +316,57 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
             c -= c >= N ? N : 0;
         }
         __syncthreads();
-        unsigned mine = tid < kWords ? word[tid] : 0u;
-        const int cnt = __popc(mine);
+        // the marked rows, numbered by every warp for itself: a lane has `wpl` words of marks, `incl` rows up to its last
+        const int wpl = (rows + 1023) >> 10;
+        int cnt = 0;
+#pragma unroll 1
+        for (int u = 0; u < wpl; ++u) cnt += __popc(word[lane * wpl + u]);
         int incl = cnt;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += t;
         }
-        if (lane == 31) warp_n[wid] = incl;
-        __syncthreads();
-        int n_inner = 0, rank = incl - cnt;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) {
-            if (w < wid) rank += warp_n[w];
-            n_inner += warp_n[w];
-        }
-        one_piece = n_inner * g.per_row <= (int)gridDim.x;
-        int off;
-        if (one_piece) {
-            first = last = (int)((unsigned)blockIdx.x / (unsigned)g.per_row);
-            off = ((int)blockIdx.x - first * g.per_row) * (int)g.chunk;
+        const int n_inner = __shfl_sync(0xffffffffu, incl, 31);
+        auto row_of = [&](int number) {          // (whole warps)
+            const int owner = __ffs((int)__ballot_sync(0xffffffffu, incl > number)) - 1;
+            int nth = number - __shfl_sync(0xffffffffu, incl - cnt, owner), w = owner * wpl;
+            unsigned bits = word[w];
+#pragma unroll 1
+            for (int c = __popc(bits); nth >= c; c = __popc(bits)) {
+                nth -= c;
+                bits = word[++w];
+            }
+            const bool is = ((bits >> lane) & 1u) != 0u && __popc(bits & ((1u << lane) - 1u)) == nth;
+            return 32 * w + __ffs((int)__ballot_sync(0xffffffffu, is)) - 1;
+        };
+        const unsigned ctas = gridDim.x;
+        pieces = min(g.per_row, (int)(ctas / (unsigned)n_inner));
+        if (pieces < g.per_row && 10u * (unsigned)(pieces * n_inner) < 6u * ctas) pieces = 0;
+        int off, n;
+        if (pieces > 0) {
+            const int chunk = (int)((unsigned)(upr + pieces - 1) / (unsigned)pieces);
+            first = last = (int)((unsigned)blockIdx.x / (unsigned)pieces);
             if (first >= n_inner) return;
-            hi = (unsigned)(first * upr + min(upr, off + (int)g.chunk));
+            piece = (int)blockIdx.x - first * pieces;
+            off = piece * chunk;
+            n = min(chunk, upr - off);
         } else {
-            const unsigned total = (unsigned)(n_inner * upr), each = max((total + gridDim.x - 1) / gridDim.x, (unsigned)wide);
+            const unsigned total = (unsigned)(n_inner * upr), each = max((total + ctas - 1) / ctas, (unsigned)wide);
             const unsigned lo = min(total, blockIdx.x * each);
             hi = min(total, lo + each);
             if (lo >= hi) return;
             first = (int)(lo / (unsigned)upr);
             last = (int)((hi - 1) / (unsigned)upr);
             off = (int)(lo - (unsigned)(first * upr));
+            n = min(upr - off, (int)(hi - lo));
+            for (int r = first + wid; r <= last; r += kWarps) {
+                const int row = row_of(r);
+                if (lane == 0) list[r - first] = row;
+            }
+            __syncthreads();
         }
-        for (; mine != 0u && rank <= last; mine &= mine - 1u, ++rank)
-            if (rank >= first) list[rank - first] = tid * 32 + __ffs((int)mine) - 1;
-        __syncthreads();
-        q = open(list[0], off, min(upr - off, (int)(hi - (unsigned)(first * upr + off))));
+        q = open(row_of(first), off, n);
     } else {
         const int row = (int)blockIdx.y, root = row - (int)((unsigned)row % (unsigned)N);
         bool inner = row == root;
@@ -345,13 +374,13 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
             const int p = __ldg(g.parent + root + c);
             inner |= p == row - root && p < c;
         }
-        const int off = (int)blockIdx.x * (int)g.chunk, n = min((int)g.chunk, upr - off);
+        const int off = piece * (int)g.chunk;
         if (!__syncthreads_or(inner)) return;
-        q = open(row, off, n);                   // (n below 1: the piece is empty)
+        q = open(row, off, min((int)g.chunk, upr - off));          // (n below 1: the piece is empty)
     }
     float4 cur[kDeep], nxt[kDeep];
     batch(cur, q, 0);
-    for (int r = first;;) {
+    for (int r = first, par = 0;; par ^= 1) {
         Run following = q;
         Acc p{-INFINITY, 0.f, 0x7fffffff};
         for (int base = 0; base < q.n; base += kStep) {
@@ -361,7 +390,7 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
                 following = open(list[r + 1 - first], 0, min(upr, (int)(hi - (unsigned)((r + 1) * upr))));
                 batch(nxt, following, 0);
             }
-            if (g.shift) {
+            if (g.shift && ((base == 0 && q.j0 < 0) || q.j0 + 4 * (base + kStep) > V)) {         // (the row's first or last batch)
 #pragma unroll
                 for (int u = 0; u < kDeep; ++u) {
                     const int i = base + u * kThreads + tid, j = q.j0 + 4 * i;
@@ -409,42 +438,36 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
 #pragma unroll
             for (int u = 0; u < kDeep; ++u) cur[u] = nxt[u];
         }
-        const float my_m = p.m;
-        const int my_base = p.a;
+        // The run's maximum first, by warps and then by all warps' results, then the sums, brought to it once each: half the time of
+        // merging pairs of (maximum, sum) step by step.
+        const float wm = warp_max(p.m);
+        float ws = p.m == -INFINITY ? 0.f : p.s * ex2((p.m - wm) * q.k);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float om = __shfl_xor_sync(0xffffffffu, p.m, o);
-            const float os = __shfl_xor_sync(0xffffffffu, p.s, o);
-            acc_merge(p, om, os, q.k);
-        }
-        if (lane == 0) wacc[wid] = p;
-        if (tid == 0) s_barg = 0x7fffffff;
+        for (int o = 16; o > 0; o >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, o);
+        if (lane == 0) wacc[par][wid] = make_float2(wm, ws);
         __syncthreads();
-        if (wid == 0) {
-            Acc t = (lane < kThreads / 32) ? wacc[lane] : Acc{-INFINITY, 0.f, 0};
+        float bmax = wacc[par][0].x;
 #pragma unroll
-            for (int o = kThreads / 64; o > 0; o >>= 1) {
-                const float om = __shfl_xor_sync(0xffffffffu, t.m, o);
-                const float os = __shfl_xor_sync(0xffffffffu, t.s, o);
-                acc_merge(t, om, os, q.k);
+        for (int w = 1; w < kWarps; ++w) bmax = fmaxf(bmax, wacc[par][w].x);
+        if (p.m == bmax && bmax != -INFINITY) {
+            // the batch at p.a holds the maximum: fetch it again (cache hit) and look for it
+            const float *from = (STAGE ? g.stage : logits) + (size_t)q.row * V;      // (what this thread has stored there itself)
+            float4 v[kDeep];
+#pragma unroll
+            for (int u = 0; u < kDeep; ++u) {
+                const int i = p.a + u * kThreads + tid, j = q.j0 + 4 * i;
+                v[u] = U4::pad();
+                if (i < q.n) v[u] = STAGE ? own4(from, j, V) : fspad_load4(from, j, V, -INFINITY);
             }
-            if (lane == 0) { wacc[0] = t; s_bmax = t.m; }
+            int at = 0x7fffffff;
+#pragma unroll
+            for (int u = kDeep - 1; u >= 0; --u) at = U4::first_eq(v[u], bmax, q.j0 + 4 * (p.a + u * kThreads + tid), at);
+            atomicMin(&s_at[par], at);
         }
         __syncthreads();
-        const float bmax = s_bmax;
-        if (my_m == bmax && bmax != -INFINITY) {
-            int b = 0x7fffffff;
-#pragma unroll 1
-            for (int u = kDeep - 1; u >= 0; --u) {
-                const int i = my_base + u * kThreads + tid, j = q.j0 + 4 * i;
-                const float *from = STAGE ? g.stage : logits;         // (what this thread has stored there itself: no read-only load)
-                if (i < q.n) b = U4::first_eq(STAGE ? own4(from + (size_t)q.row * V, j, V) : fspad_load4(from + (size_t)q.row * V, j, V, -INFINITY), bmax, j, b);
-            }
-            atomicMin(&s_barg, b);
-        }
-        __syncthreads();
-        int own = SHARED ? q.off / (int)g.chunk : (int)blockIdx.x, stop = own + 1;
-        if (!one_piece) {
+        int own = piece, stop = piece + 1;
+        if (SHARED && pieces > 0 && stop == pieces) stop = g.per_row;
+        if (SHARED && pieces == 0) {
             const int end = q.off + q.n;
             own = q.off == 0 ? 0 : 1 + q.off / wide;
             stop = end >= upr ? g.per_row : 1 + end / wide;
@@ -452,11 +475,19 @@ accept_stats_inner_kernel(const float *__restrict__ logits, const float *__restr
         if (tid >= own && tid < stop) {
             FspadStatsPart out;
             out.m = -INFINITY; out.s = 0.f; out.a = 0x7fffffff; out.pad = 0;
-            if (tid == own) { out.m = wacc[0].m; out.s = wacc[0].s; out.a = s_barg; }
+            if (tid == own) {
+                out.m = bmax;
+                out.a = s_at[par];
+                s_at[par] = 0x7fffffff;                          // (for the run after next)
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) {
+                    const float2 t = wacc[par][w];
+                    out.s += t.x == -INFINITY ? 0.f : t.y * ex2((t.x - bmax) * q.k);
+                }
+            }
             parts[(size_t)q.row * g.slots + tid] = out;
         }
         if (!SHARED || r == last) break;
-        __syncthreads();
         ++r;
         q = following;
     }
@@ -510,8 +541,7 @@ cudaError_t fspad_launch_stats_partials(fspad_ctx *ctx, const float *logits, con
 {
     const bool aligned = (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
     if (sms <= 0 || sms > ctx->sm_count) sms = ctx->sm_count;
-    if (geom->parent != nullptr && aligned && rows % rows_per_seq == 0 &&
-        (geom->stage != nullptr ? fspad_scan_inner_fits(sms, rows, V) : fspad_scan_inner(sms, rows, rows_per_seq, V))) {
+    if (geom->parent != nullptr && aligned && rows % rows_per_seq == 0 && fspad_scan_inner_fits(sms, rows, V)) {
         *geom = fspad_stats_geom_inner(sms, rows, V, ctx->stats_slots, geom->parent, geom->stage);
         const FspadStatsGeom &g = *geom;
         const int wide = (g.upr + g.per_row - 2) / (g.per_row - 1);

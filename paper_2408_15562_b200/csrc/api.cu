@@ -110,7 +110,9 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool
         const int walk = fspad_walk_ctas(ctx, batch, c.vocab);
         const int beside = sms - (walk < sms / 2 ? walk : sms / 2), ranges = fspad_attn_umma_splits(ctx, n_nodes, batch, beside);
         const bool long_attn = ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges;
-        const bool one_stream = walk <= sms / 2 && (long_attn || fspad_scan_inner(sms, batch * n_nodes, n_nodes, c.vocab));
+        const int rows = batch * n_nodes;
+        const bool short_scan = (long long)rows * c.vocab >= (n_nodes >= 16 ? 1 << 21 : 1 << 23) || (c.vocab > 98304 && rows <= 32);
+        const bool one_stream = walk <= sms / 2 && (long_attn || short_scan);
         const bool scan_first = walk <= sms / 2 && long_attn ? walk > batch : sms - attn_ctas < sms / 4;
         const bool fork = !one_stream || (captured && ctas_on(beside) <= beside && (long_attn || scan_first));
         p.chain = !fork;
@@ -328,7 +330,7 @@ int fspad_tree_accept(fspad_ctx *ctx, const float *target_logits, const float *d
     if (batch == 0) return FSPAD_OK;
     cudaStream_t st = fspad_stream(stream);
     FspadStatsGeom geom;
-    geom.parent = parent;
+    if (fspad_scan_inner(ctx->sm_count, batch * n_nodes, n_nodes, ctx->cfg.vocab, draft_probs != nullptr, true)) geom.parent = parent;
     cudaError_t e = fspad_launch_stats_partials(ctx, target_logits, temperature, batch * n_nodes, n_nodes,
                                                 ctx->cfg.vocab, &geom, st);
     if (e != cudaSuccess) return FSPAD_ERR_CUDA;
@@ -538,8 +540,8 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
     const int attn_sms = plan.attn_sms;
     cudaError_t ce = cudaSuccess;
     FspadStatsGeom geom;
-    geom.parent = parent;
     const int rows = batch * n_nodes;
+    if (fspad_scan_inner(sms, rows, n_nodes, c.vocab, may_sample, false)) geom.parent = parent;
     // With the tree rows given apart from the cache the compaction depends on the walk alone, and when the
     // sequence's slices are few (a warp takes one after another: four each for the 16 warps of a greedy walk's CTA) the walk makes the moves itself at its end: one dependent launch less on the step's
     // longest chain (all-greedy step of 26 nodes and 64 slices: 29.3 -> 23.7 us called one by one, 13.1 against 13.3 from a graph).
@@ -735,7 +737,7 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
          cudaMemcpyAsync(attn_out, ctx->h_out, q_bytes, cudaMemcpyDeviceToHost, ctx->side) == cudaSuccess;
     const bool joined = cudaEventRecord(ctx->ev_join, ctx->side) == cudaSuccess;
     FspadStatsGeom geom;
-    geom.parent = ctx->h_parent;
+    if (far_logits || fspad_scan_inner(ctx->sm_count, batch * n_nodes, n_nodes, c.vocab, draft_probs != nullptr, false)) geom.parent = ctx->h_parent;
     if (far_logits) geom.stage = ctx->h_logits;
     const float *logits = far_logits ? far_logits : ctx->h_logits;
     ok = ok && fspad_launch_stats_partials(ctx, logits, ctx->h_temp, batch * n_nodes, n_nodes, c.vocab, &geom, st) == cudaSuccess;

@@ -165,8 +165,8 @@ static inline FspadStatsGeom fspad_stats_geom(int sm_count, int rows, int V, boo
 #define FSPAD_INNER_LIST 128           /* rows one CTA may be given pieces of */
 // How the rows of the nodes with children are cut: into at most 16 pieces each, as many as the walk merges at once, with two units for
 // each thread of a CTA at least.  How many rows there are is known to the kernel alone.  Where a CTA for every piece of every row is
-// one wave, most of which leaves at once, the CTAs are the pieces; else the kernel numbers the rows first (16 and 30 rows of 128256: the
-// step 0.7 us shorter without; 60 rows, in two waves, 2 us longer).
+// one wave, most of which leaves at once, the CTAs are the pieces; else the kernel numbers the rows first and may cut them into fewer
+// (16 and 30 rows of 128256: the step 0.7 us shorter without; 60 rows, in two waves, 2 us longer).
 static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int V, int slots, const int *parent, float *stage)
 {
     FspadStatsGeom g;
@@ -186,20 +186,38 @@ static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int 
     g.stage = stage;
     return g;
 }
-// Whether the scan of these rows can go by the trees, and whether it does.  Looking for the rows takes about a microsecond, and a walk that ends in a node
-// without children one or two more; against that stand three quarters of the scan (less of small trees: half of 11 nodes have children),
-// and a step behind the short scan stays in one stream.  Us a step, all rows and by the trees: 60 x 32000 21.2 and 22.6, 40 x 64000 28.7
-// and 26.9, 60 x 50257 32.6 and 29.7 (greedy 21.6 and 19.5), 2 x 40 x 32000 31.9 and 28.3, 4 x 20 x 32000 27.6 and 24.9, but 7 x 11 x 32001 32.5 and 34.0, 5 x 9 x 128256 26.9 and 28.8;
-// 240 x 32000 36.7 and 35.9, 60 x 128256 35.0 and 32.3, 960 x 128256 191 and 126.  Few rows of 128256 tokens are read by the trees whatever the
-// trees, because all SMs share a row otherwise and the walk has more pieces to merge than it takes at once: 8 rows 31.1 and 25.0, 2 x 10 31.8 and 28.4.
+// Whether the scan of these rows can go by the trees, and whether it does.  Up to nine rows (fewer than a sixteenth of the SMs) the scan
+// of all rows cuts a row into more pieces than the walk merges at once, and the draw from more than 16 pieces reads the whole row
+// again: 8 rows alone, all rows and by the trees, 22.5 and 16.0 us at 128256 tokens, 17.1 and 13.7 at 32000 (up to 8192 tokens there are no more than 16).
+//   Otherwise the rows left out stand against what finding the others costs (1.3 to 1.6 us) and, of a greedy walk, its look at the row of its last
+// node (2.4 us, which in a step passes beside the attention; `alone` says that nothing of the call does).  The gain grows with the array, and with
+// the trees: of up to 11 nodes half and more have children, of 60 a fifth.  The lines, in thousands of logits, lie where trees of branching two
+// to ten were no slower (acceptance, or step of 8 KV heads and 1 K to 2 K keys; us from a graph, all rows and by the trees):
+//   sampled, a step   40 x 32000 twice 31.1 and 28.6, 24 x 50257 four times 33.4 and 31.4, 24 x 32000 twice 23.4 and 25.0; 8 x 128256 eight times 39.3 and 35.8
+//   sampled, alone    40 x 50257 twice 23.9 and 22.9, 24 x 32000 eight times 26.7 and 26.7, 16 x 32000 eight times 21.3 and 21.9; 8 x 32000 16 times 26.6 and 29.3
+//   greedy, a step    40 x 32000 twice 21.6 and 19.2, 24 x 32000 eight times 31.2 and 31.2; 16 x 50257 eight times 29.5 and 31.0, 8 x 50257 16 times 34.5 and 38.0
+//   greedy, alone     40 x 32000 four times 11.0 and 10.3, 24 x 50257 eight times 13.0 and 11.6, 60 x 50257 twice 8.9 and 10.2; 16 x 32000 16 times 11.0 and 11.6
+// Rows whose length is no multiple of four are always cut at the rows by the scan of all of them, which makes it the faster one of small
+// arrays.  Where the CTAs are the pieces nothing is numbered: 24 x 128256, 32 x 128256 (16 nodes twice) in a sampled step 24.4 and 23.7, 28.2 and 24.8.
+// What the kernel finds is not known here: a tree most of whose nodes have children (a chain) gains nothing from it.  Chains of 40 to 60
+// nodes: acceptance alone 22.0 and 24.2 (60 x 128256 sampled), 12.3 and 12.3 (greedy), 17.5 and 20.5 at worst (40 x 50257 eight times, greedy);
+// steps level to 7 % longer.
 static inline bool fspad_scan_inner_fits(int sm_count, int rows, int V)
 {
     return rows <= FSPAD_INNER_MAX_ROWS && (long long)rows * (V + 6ll) < 1ll << 31 &&
            rows / (sm_count * (1024 / FSPAD_STATS_THREADS)) + 2 <= FSPAD_INNER_LIST;
 }
-static inline bool fspad_scan_inner(int sm_count, int rows, int nodes, int V)
+static inline bool fspad_scan_inner(int sm_count, int rows, int nodes, int V, bool may_sample, bool alone)
 {
-    return fspad_scan_inner_fits(sm_count, rows, V) && ((long long)rows * V >= (nodes >= 16 ? 1 << 21 : 1 << 23) || (V > 98304 && rows <= 32));
+    if (!fspad_scan_inner_fits(sm_count, rows, V)) return false;
+    if (rows * 16 < sm_count && V > 16 * 4 * (FSPAD_STATS_THREADS / 2)) return true;
+    const bool odd = V % 4 != 0, one_wave = rows * 16 <= sm_count * (1024 / FSPAD_STATS_THREADS);
+    int line;                                    // thousands of logits
+    if (may_sample) line = alone ? nodes >= 24 ? 4000 : nodes >= 12 ? 6000 : 8000 : nodes >= 32 ? 2500 : nodes >= 12 ? 4000 : 8000;
+    else if (alone) line = nodes >= 32 ? odd ? 9500 : 5000 : nodes >= 12 ? 9500 : 25000;
+    else line = nodes >= 32 ? odd ? 4000 : 2500 : nodes >= 12 && !odd ? 6000 : 16000;
+    if (one_wave && (may_sample || !alone)) line = !may_sample ? 4000 : alone ? 2000 : 1500;
+    return (long long)rows * V >= 1000ll * line;
 }
 
 // How many of the first n units of four positions of row `row`, from position j0 of it on, can be loaded whole: the last one may reach

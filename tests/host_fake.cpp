@@ -117,7 +117,7 @@ int fspad_walk_ctas(fspad_ctx *, int B, int V)
 {
     int c = 16;
     while (c > 1 && (V + c - 1) / c < 2048) c >>= 1;
-    return B * c;
+    return B * (c == 16 && B > 7 ? 10 : c);
 }
 size_t fspad_feature_sampler_scratch_floats(int, int, int) { return 0; }
 FspadStatsGeom fspad_lm_head_geom(int, int, bool, int) { return FspadStatsGeom(); }
@@ -134,10 +134,10 @@ cudaError_t fspad_launch_accept_walk(fspad_ctx *, const float *, const float *dr
 {
     return call("walk", "draft=%llx far=%d compacts=%d stream=%x", (unsigned long long)(uintptr_t)draft, (int)far, (int)(kv.cache != nullptr), id(st));
 }
-cudaError_t fspad_launch_stats_partials(fspad_ctx *, const float *, const float *, int, int, int, FspadStatsGeom *, cudaStream_t st,
+cudaError_t fspad_launch_stats_partials(fspad_ctx *, const float *, const float *, int, int, int, FspadStatsGeom *geom, cudaStream_t st,
                                         bool, int)
 {
-    return call("scan", "stream=%x", id(st));
+    return call("scan", "trees=%d staged=%d stream=%x", (int)(geom->parent != nullptr), (int)(geom->stage != nullptr), id(st));
 }
 cudaError_t fspad_launch_kv_compact(fspad_ctx *, fspad_bf16 *, const int *, const int *, const int *, int, int *, cudaStream_t st, bool)
 {

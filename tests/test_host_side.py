@@ -30,6 +30,7 @@ def lib(tmp_path_factory):
     lib.fspad_destroy.restype = None
     lib.fspad_verify_step.argtypes = [vp, vp, ci] + [vp] * 10 + [ci, ci] + [vp] * 6
     lib.fspad_verify_step_host.argtypes = [vp] * 12 + [ci, ci] + [vp] * 6
+    lib.fspad_tree_accept.argtypes = [vp] * 7 + [ci, ci] + [vp] * 4
     lib.fake_log.restype = ctypes.c_char_p
     lib.fake_fail.argtypes = [ctypes.c_char_p, ci]
     lib.fake_pin.argtypes = [vp, ctypes.c_size_t]
@@ -66,6 +67,13 @@ class Step:
         draft, unif = (big, big) if self.sampling else (None, None)
         rc = self.lib.fspad_verify_step(self.ctx, big, 0, big, tree, tree, big, big, big, draft, big, big, unif, self.n, self.batch, big,
                                         big, big, big, big, STREAM)
+        return rc, self.lib.fake_log().decode().splitlines()
+
+
+    def accept(self):
+        big = 0x1000
+        draft, unif = (big, big) if self.sampling else (None, None)
+        rc = self.lib.fspad_tree_accept(self.ctx, big, draft, big, big, big, unif, self.n, self.batch, big, big, big, STREAM)
         return rc, self.lib.fake_log().decode().splitlines()
 
 
@@ -162,6 +170,32 @@ def test_logits_stay_where_all_of_them_are_pinned(lib, share, nodes, batch, voca
     rc, log = step.host()
     copied = any(x.startswith("h2d host=1000 bytes=%d " % bytes_) for x in log)
     assert rc == 0 and copied != in_place and any(x.startswith("scan ") for x in log)
+
+
+# just below and on the line from which the scan goes by the trees: alone, in a step
+@pytest.mark.parametrize("sampling,nodes,batch,vocab,alone,step", [
+    (True, 9, 1, 8192, False, False), (True, 9, 1, 8193, True, True), (False, 3, 3, 32000, True, True), (False, 5, 2, 32000, False, False),
+    (True, 40, 2, 31000, False, False), (True, 40, 2, 32000, False, True), (True, 24, 6, 32000, True, True), (True, 24, 5, 32000, False, False),
+    (True, 16, 8, 46000, False, True), (True, 16, 8, 47000, True, True), (True, 8, 20, 49000, False, False), (True, 8, 20, 50000, True, True),
+    (True, 24, 1, 62000, False, False), (True, 24, 1, 64000, False, True), (True, 24, 1, 84000, True, True),            # one wave of pieces
+    (False, 40, 2, 31000, False, False), (False, 40, 2, 32000, False, True), (False, 40, 4, 32000, True, True),
+    (False, 40, 2, 32001, False, False), (False, 40, 2, 50257, False, True), (False, 40, 4, 59001, False, True), (False, 40, 4, 60001, True, True),
+    (False, 24, 7, 32000, False, False), (False, 24, 8, 32000, False, True), (False, 24, 8, 32001, False, False), (False, 24, 9, 45000, True, True),
+    (False, 8, 16, 128256, False, True), (False, 8, 25, 128256, True, True), (False, 24, 1, 128256, False, False), (False, 32, 1, 128256, False, True)])
+def test_when_the_scan_goes_by_the_trees(lib, sampling, nodes, batch, vocab, alone, step):
+    step_ = Step(lib, nodes=nodes, batch=batch, vocab=vocab, sampling=sampling, max_len=2176)
+    rc, log = step_.accept()
+    assert rc == 0 and _field(log, "scan", "trees") == str(int(alone))
+    lib.fake_reset()
+    rc, log = step_.device(0x1000)
+    assert rc == 0 and _field(log, "scan", "trees") == str(int(step)) and _field(log, "scan", "staged") == "0"
+    lib.fake_reset()
+    rc, log = step_.host()                       # pageable logits: as the step
+    assert rc == 0 and _field(log, "scan", "trees") == str(int(step)) and _field(log, "scan", "staged") == "0"
+    lib.fake_reset()
+    lib.fake_pin(0x1000, batch * nodes * vocab * 4)
+    rc, log = step_.host()                       # pinned ones: brought to the device by a scan by the trees
+    assert rc == 0 and _field(log, "scan", "trees") == "1" and _field(log, "scan", "staged") == "1"
 
 
 FAILING = [("h2d", k) for k in range(1, 10)] + [("d2h", k) for k in range(1, 7)] + \
