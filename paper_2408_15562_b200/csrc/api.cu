@@ -59,6 +59,21 @@ const void *mapped_whole(const void *p, size_t bytes)
     return first >= lo && first - lo <= size && size - (first - lo) >= bytes ? at.devicePointer : nullptr;
 }
 
+// Rows [batch][nodes] of the nodes that have children, and of the roots: what the scan by the trees reads.
+int rows_with_children(const int32_t *parent, int nodes, int batch)
+{
+    int n = 0;
+    for (int b = 0; b < batch; ++b, parent += nodes) {
+        unsigned long long mark[(FSPAD_MAX_NODES_WIDE + 63) / 64] = {1ull};
+        for (int c = 1; c < nodes; ++c) {
+            const unsigned p = (unsigned)parent[c];
+            if (p < (unsigned)c) mark[p >> 6] |= 1ull << (p & 63);
+        }
+        for (unsigned long long m : mark) n += __builtin_popcountll(m);
+    }
+    return n;
+}
+
 // How a step's attention shares the SMs with its acceptance.  Both entry points take it from here: the number of key ranges
 // follows from attn_sms, and with it which reference a probability is rounded against, so that they give the same bits.
 struct StepPlan {
@@ -703,10 +718,19 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     const float *draft = draft_probs ? static_cast<const float *>(mapped_whole(draft_probs, lg_bytes)) : nullptr;
     if (misaligned(draft)) draft = nullptr;
     const bool draft_in_place = draft != nullptr;
-    // Of the logits the scan by the trees reads a quarter, and the walk the one row that it ends in: page-locked ones, too, are left
-    // where they are (60 rows of 128256 copied whole took 557 us).
+    // Of the logits the scan by the trees reads the rows of nodes with children, a quarter of a 60-node tree's, and the walk the one row that
+    // it ends in: page-locked ones, too, are left where they are (60 rows of 128256 copied whole took 557 us).  Not where nearly all nodes
+    // have children: the kernel takes 50 GB/s from the link and the copy 55.3, every row begun costs it about 0.08 us, and what it saves is
+    // the copy's own 2 us of a greedy step and 12 us of a sampled one.  Calls in place and copied, us: chains of 60 x 128256 717 and 660
+    // (greedy), four of 30 x 8000 208 and 184, one of 8 x 128256 158 and 169; two of 16 x 32000 178 and 164 greedy, 185 and 188 sampled.  The trees
+    // are looked at here for that alone: if the stream has yet to bring them, what they hold now decides which way the logits go, and
+    // nothing else.
     const float *far_logits = nullptr;
-    if (fspad_scan_inner_fits(ctx->sm_count, batch * n_nodes, c.vocab)) far_logits = static_cast<const float *>(mapped_whole(target_logits, lg_bytes));
+    if (fspad_scan_inner_fits(ctx->sm_count, batch * n_nodes, c.vocab)) {
+        const double inner = rows_with_children(parent, n_nodes, batch), row_bytes = (double)c.vocab * sizeof(float);
+        if (inner * (1.106 * row_bytes + 4700.0) < (double)lg_bytes + (draft_probs ? 660e3 : 100e3))
+            far_logits = static_cast<const float *>(mapped_whole(target_logits, lg_bytes));
+    }
     if (misaligned(far_logits)) far_logits = nullptr;
     h2d(ctx->h_prefix, prefix_len, B * sizeof(int));
     h2d(ctx->h_parent, parent, B * N * sizeof(int));

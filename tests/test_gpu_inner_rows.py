@@ -204,14 +204,15 @@ def _host_step(ctx, inp, logits):
     return out, path, n, bonus, new_len, cache
 
 
-# every row, or every other one, has children: more pieces of rows than CTAs
-@pytest.mark.parametrize("tree,branch,nodes,batch,vocab", [("chain", 1, 60, 1, 50257), ("chain", 1, 40, 2, 32000), ("bfs", 2, 120, 1, 32753)])
+# every other row has children, or all but one of few: a CTA for every piece, fewer pieces a row than 16, shares of rows laid end to end
+@pytest.mark.parametrize("tree,branch,nodes,batch,vocab", [("chain", 1, 8, 1, 50257), ("bfs", 2, 120, 1, 32753), ("bfs", 2, 200, 3, 8001),
+                                                           ("bfs", 2, 250, 5, 2003)])
 @pytest.mark.parametrize("mode", ["greedy", "sample"])
 def test_most_rows_read_where_they_are(tree, branch, nodes, batch, vocab, mode):
     """Rows that the scan brings to the device while the walk that sweeps them is already resident: other logits in the same memory at
     every call, and the oracle's acceptance each time (children are rejected at the root at least once)."""
     w = synth.scaled(W["llama3_8b_2k"], batch=batch, prefix=(40, 300), n_nodes=nodes, tree=tree, branch=branch, vocab=vocab,
-                     temperatures=((0.0, 0.0) if mode == "greedy" else (1.0, 0.7))[:batch])
+                     temperatures=((0.0,) * 5 if mode == "greedy" else (1.0, 0.7, 1.0, 0.0, 0.7))[:batch])
     inps = [synth.generate(w, v) for v in (1, 2, 3, 4)]
     ctx = helpers.make_ctx(inps[0], n_layers=1)
     logits = torch.empty(inps[0].target_logits.shape).pin_memory()

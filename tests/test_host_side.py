@@ -49,6 +49,7 @@ class Step:
         skip = (-raw.ctypes.data // 4) % 4
         self.draft = raw[skip:skip + batch * nodes * vocab]              # 16-byte aligned
         self.small = np.zeros(batch * (max(nodes, 64) + 1) + 8, np.int32)
+        self.parent = np.zeros((batch, nodes), np.int32)                 # stars; the one array that the host entry looks at
         lib.fake_reset()
 
     def __del__(self):
@@ -58,7 +59,7 @@ class Step:
         big = 0x1000                                     # never dereferenced by the stand-ins
         p = self.small.ctypes.data
         draft, unif = (self.draft.ctypes.data, p) if self.sampling else (None, None)
-        rc = self.lib.fspad_verify_step_host(self.ctx, big, big, big, big, big, big, big, draft, big, big, unif, self.n, self.batch,
+        rc = self.lib.fspad_verify_step_host(self.ctx, big, big, big, big, self.parent.ctypes.data, big, big, draft, big, big, unif, self.n, self.batch,
                                              big, p, p, p, p, STREAM)
         return rc, self.lib.fake_log().decode().splitlines()
 
@@ -170,6 +171,25 @@ def test_logits_stay_where_all_of_them_are_pinned(lib, share, nodes, batch, voca
     rc, log = step.host()
     copied = any(x.startswith("h2d host=1000 bytes=%d " % bytes_) for x in log)
     assert rc == 0 and copied != in_place and any(x.startswith("scan ") for x in log)
+
+
+@pytest.mark.parametrize("nodes,batch,vocab,chains,in_place", [
+    (60, 1, 128256, 0, True), (60, 1, 128256, 1, False), (60, 2, 32000, 2, False), (60, 2, 32000, 1, True), (8, 1, 128256, 1, True),
+    (8, 1, 8000, 1, True), (60, 1, 2000, 1, False), (256, 32, 333, 32, False), (1, 1, 32000, 1, True)])
+def test_logits_of_chains_are_copied(lib, nodes, batch, vocab, chains, in_place):
+    """Page-locked logits: read in place unless most rows would be, where a copy is the faster way.  Parents that no tree has count as
+    the root, as they do on the device, and none is looked at outside of the array."""
+    for bad in (False, True):
+        step = Step(lib, nodes=nodes, batch=batch, vocab=vocab, sampling=False)
+        step.parent[:chains] = np.arange(-1, nodes - 1)
+        if bad:
+            step.parent[step.parent == 0] = 1 << 30
+            step.parent[:, 0] = 77
+        bytes_ = batch * nodes * vocab * 4
+        lib.fake_pin(0x1000, bytes_)
+        rc, log = step.host()
+        copied = any(x.startswith("h2d host=1000 bytes=%d " % bytes_) for x in log)
+        assert rc == 0 and copied != in_place and _field(log, "scan", "staged") == str(int(in_place))
 
 
 # just below and on the line from which the scan goes by the trees: alone, in a step
