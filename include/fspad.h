@@ -166,8 +166,8 @@ int fspad_tree_accept(fspad_ctx *ctx, const float *target_logits, const float *d
                       int32_t *n_accepted, int32_t *bonus_token, void *stream);
 
 /*
- * The first stage of fspad_tree_accept on its own, over every row (which fspad_tree_accept
- * itself takes on small arrays; on large ones it leaves out the rows of nodes without children): one pass over
+ * The first stage of fspad_tree_accept on its own, over every row (fspad_tree_accept itself leaves
+ * out the rows of nodes without children where that is the faster way, which depends on the sizes): one pass over
  * logits [rows][V] giving row_max (fp32 maximum), row_arg (its lowest index)
  * and row_sum = sum_j exp((x_j - max)/T_row) accumulated from fp32 exponentials
  * (relative accuracy about 1e-6; the acceptance walk re-derives exact sums
@@ -455,14 +455,18 @@ int fspad_verify_step(fspad_ctx *ctx, fspad_bf16 *cache, int attn_layer, const f
  * must not be made inside a stream capture), writes the tree rows into cache
  * rows L_b.. of layer 0, does what fspad_verify_step does (attention over layer
  * 0; it runs while the logits are on their way) on `stream` and the context's
- * second stream, copies the results back and synchronises the stream.  The outputs
- * are those of fspad_verify_step on the same inputs, bit for bit.  The KV cache
+ * second stream, copies the results back and synchronises the stream.  The attention's
+ * output is that of fspad_verify_step on the same inputs, bit for bit, and so is an
+ * acceptance at temperature 0.  A sampled one takes the same decisions but for such as lie
+ * within about 1e-9 (relative) of their boundary: the order in which the scan's sums are
+ * taken depends on where the logits lie and on what runs beside it (as it does between a step
+ * called and captured, and between a step and fspad_tree_accept).  The KV cache
  * is device-resident state that persists between steps (the caller's device
  * pointer `cache`, layout as in fspad_kv_compact); everything else is host
- * memory (pinned memory makes the copies asynchronous; draft_probs or target_logits
- * that lie in one pinned allocation or registration as a whole and start on a 16-byte
- * boundary are not copied at all: the kernels read the rows they need where they
- * are, before the call returns).  An error, too, is returned only when nothing
+ * memory (pinned memory makes the copies asynchronous; draft_probs, and target_logits
+ * unless nearly all of the trees' nodes have children, that lie in one pinned allocation or
+ * registration as a whole and start on a 16-byte boundary are not copied at all: the kernels
+ * read the rows they need where they are, before the call returns).  An error, too, is returned only when nothing
  * queued by the call uses host memory any more.  Host outputs:
  * attn_out [batch][n_nodes][Hq][d] bf16, accepted_path [batch][max_nodes],
  * n_accepted, bonus_token, new_len [batch].  draft_probs/uniforms may be NULL
