@@ -732,8 +732,8 @@ __device__ __forceinline__ unsigned long long argmax_key(float m, int a)
     const unsigned u = __float_as_uint(m + 0.0f);
     return ((unsigned long long)(u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u)) << 32) | (0xffffffffu - (unsigned)a);
 }
-// The largest key of row positions [lo, hi) of a row that starts `ph` positions behind a 16-byte boundary, into t.best (set to 0
-// before; the caller's barrier comes after).  Eight loads in flight a thread: on one CTA a 128256-token row is bound by what one SM
+// The largest key of row positions [lo, hi), of which lo (it may lie before the row's first) is on a 16-byte boundary, into t.best (set to
+// 0 before; the caller's barrier comes after).  Eight loads in flight a thread: on one CTA a 128256-token row is bound by what one SM
 // can have under way.
 template <typename Tree>
 __device__ __noinline__ void argmax_row(Tree &t, const float *__restrict__ x, int lo, int hi, int tid, int nthr)
@@ -864,7 +864,7 @@ accept_greedy_kernel(const __grid_constant__ WalkArgs args)
             const int ph = (int)(start & 3), each = (((args.V + 3 + C - 1) / C) + 3) & ~3;
             argmax_row(t, args.given + start, rank * each - ph, min(args.V, (rank + 1) * each - ph), tid, nthr);
             __syncthreads();
-            if (tid == 0) *cluster.map_shared_rank(&peer_best[rank], 0) = t.best;  // (a word each: maxima of 64 bits sent to one word of a peer got lost)
+            if (tid == 0) *cluster.map_shared_rank(&peer_best[rank], 0) = t.best;  // (a word each: rank 0 clears its own t.best at a time of its own, and a maximum sent there might come before)
             cluster.sync();
             if (rank == 0 && tid == 0) {
                 unsigned long long best = peer_best[0];
@@ -1566,7 +1566,8 @@ static WalkKernel walk_kernel(bool narrow, bool inner)
 // vocabularies do not need the whole cluster.  A cluster's CTAs lie side by side, so fewer fit than the SMs
 // would hold: 7 of 16, 11 of 10, 15 of 8.  Where a batch may need more than the 7, clusters of 10 are taken, as long as a thread's
 // share of a row can be parked in shared memory.  us a step at 128256 tokens, clusters of 16, 10 and 8: 8 sequences 71, 63, 70; 11 73, 65, 78;
-// 16, half of them greedy, 124, 115, 145; 16 sampled 146, 129, 125; 10 at 50257 61, 53, 51.
+// 16, half of them greedy, 124, 115, 145; 16 sampled 146, 129, 125; 10 at 50257 61, 53, 51.  (Of these only the last two are faster
+// with eight, by 3 and 4 %.)
 static int walk_cluster_size(fspad_ctx *ctx, int B, int V)
 {
     if (ctx->walk_cluster == 0) {

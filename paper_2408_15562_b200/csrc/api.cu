@@ -104,11 +104,12 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool
     // One B200, us a step, two streams against one: 50.7 and 38.1 on 52 heads and 4 K keys, 44.2 and 42.4 on 8 x 8 and 8 K,
     // both 17 chunks a CTA.)  What is known here is how long the sequences may be, not how long they are; so the merge of the key ranges
     // waits for the attention alone, not for the walk (when it did, a 2 K sequence in a context of 12 K rows or more took 37.1 us, two
-    // streams 34.2, and 31.1 now; 52 heads and 4 K keys 38.6 -> 39.0).  Behind a scan by the trees, which is short, one stream is the better
-    // way for an attention of any length: called one by one, 8 KV heads and 60 x 128256 at 1 K, 2 K and 4 K keys 31.2 -> 27.6, 32.2 -> 28.9 and
-    // 32.3 -> 28.8, 64 heads at 2 K 32.1 -> 28.5, two sequences 35.1 -> 33.8.  (60 x 32000 would gain as much, 28.3 -> 25.2;
-    // below 12 chunks a range by max_len the order of calls behind a full scan is the one tests/test_host_side.py states.)  Captured, such a
-    // step forks only where the scan goes first: beside an attention on most SMs it is the longer way (52 heads and 1 K keys 38.7).
+    // streams 34.2, and 31.1 now; 52 heads and 4 K keys 38.6 -> 39.0).  On larger arrays of logits one stream is the better way for an
+    // attention of any length (`any_attn`): called one by one, 8 KV heads and 60 x 128256 at 1 K, 2 K and 4 K keys 31.2 -> 27.6, 32.2 -> 28.9
+    // and 32.3 -> 28.8, 64 heads at 2 K 32.1 -> 28.5, two sequences 35.1 -> 33.8, all behind a scan by the trees; behind a scan of all rows
+    // 60 x 50257 32.3 -> 27.4, 24 x 128256 28.9 -> 24.1, 24 x 50257 twice 26.6 -> 24.6.  (The line lies higher than it need: 60 x 32000, below it, takes
+    // 28.3 us in two streams and 25.2 in one.)  Captured, such a step forks only where the scan goes first: beside an attention on most SMs
+    // it is the longer way (52 heads and 1 K keys 38.7).
     // In a graph, where events cost nothing, the fork is the better way if the attention's CTAs find room beside the walk's: 29.7 against
     // 30.4 us (one stream) on the 2 K sequence, 37.8 and 38.4 on 52 heads, 17.3 and 18.1 at 580 keys, 45.3 and 46.5 on two such
     // sequences; where they do not, four short sequences of 32 heads take 33.8 in one stream and 44.8 forked.  A walk of single CTAs (less than 4096
@@ -126,8 +127,8 @@ StepPlan step_plan(fspad_ctx *ctx, int n_nodes, int batch, bool may_sample, bool
         const int beside = sms - (walk < sms / 2 ? walk : sms / 2), ranges = fspad_attn_umma_splits(ctx, n_nodes, batch, beside);
         const bool long_attn = ranges == 1 || (c.max_len + 127) / 128 >= 12 * ranges;
         const int rows = batch * n_nodes;
-        const bool short_scan = (long long)rows * c.vocab >= (n_nodes >= 16 ? 1 << 21 : 1 << 23) || (c.vocab > 98304 && rows <= 32);
-        const bool one_stream = walk <= sms / 2 && (long_attn || short_scan);
+        const bool any_attn = (long long)rows * c.vocab >= (n_nodes >= 16 ? 1 << 21 : 1 << 23) || (c.vocab > 98304 && rows <= 32);
+        const bool one_stream = walk <= sms / 2 && (long_attn || any_attn);
         const bool scan_first = walk <= sms / 2 && long_attn ? walk > batch : sms - attn_ctas < sms / 4;
         const bool fork = !one_stream || (captured && ctas_on(beside) <= beside && (long_attn || scan_first));
         p.chain = !fork;

@@ -58,7 +58,7 @@ struct fspad_ctx {
     int lm_attr_done;
     int fs_attr_done;         // dynamic shared-memory limit raised for the Feature Sampler's product kernel
 
-    void *dx_part;            // draft step: per-piece top-k lists [max_batch * 16 rows][pieces][16] (value, token)
+    void *dx_part;            // draft step: per-piece top-k lists [max_batch * 16 rows][pieces][16], 64-bit sort keys (0: none)
     int *dx_done;             // draft step: finished pieces of each sequence [max_batch]; zero between calls
     float *dx_front;          // draft step: a frontier put aside, values and candidates [2][max_batch][16]
 
@@ -90,7 +90,7 @@ struct FspadStatsGeom {
     int threads;       // threads per CTA of the scan: FSPAD_STATS_THREADS, or half of it for a small array
     // The trees [rows / rows_per_seq][rows_per_seq] the rows belong to: rows of nodes without children (other than a root) have
     // then no partials, and whoever walks into such a node looks at its row itself.  NULL: every row has them.  Set by the
-    // caller of fspad_launch_stats_partials, which puts it back to NULL where the scan reads every row after all.
+    // caller of fspad_launch_stats_partials where the scan is to go by them, put back to NULL there if it cannot.
     const int *parent = nullptr;
     // With the trees: the logits lie in host memory, and the rows that the scan reads are left here, [rows][V] on the device.  NULL: they
     // are on the device.  Set by the caller, too.

@@ -102,7 +102,7 @@ def test_host_entry_cuts_the_attention_as_the_device_entry_does(lib, hq, hkv, no
     (True, 32000, 32, 1, 320, True), (True, 32000, 32, 4, 320, True), (True, 32000, 43, 3, 320, False),       # one stream: 64, 256, 258 slices
     (True, 4000, 32, 1, 320, True), (True, 4000, 33, 1, 320, False),         # a single CTA walks: 64, 66
     (True, 8192, 32, 2, 320, True), (True, 8192, 33, 2, 320, False),         # a cluster of four: 128, 132
-    (True, 128256, 8, 4, 2176, True), (True, 128256, 8, 5, 2176, False),     # two streams: 64, 80
+    (True, 128256, 8, 4, 2176, True), (True, 128256, 8, 5, 2176, False),     # one stream, the attention a short one: 64, 80
     (False, 4000, 32, 1, 320, True), (False, 4000, 33, 1, 320, False),       # greedy, one stream
 ])
 def test_who_compacts(lib, sampling, vocab, hkv, layers, max_len, by_walk):
@@ -142,6 +142,39 @@ def test_capture_decides_on_the_order_and_not_on_the_cut(lib, sampling, hq, hkv,
             assert [x.split()[0] for x in log][:3] == ["scan", "walk", "attention"]
         else:
             assert len(events) == 4 and _field(log, "attention", "early") == "0" and _field(log, "attention", "stream") != "%x" % STREAM
+    assert len(sms) == 1
+
+
+@pytest.mark.parametrize("hq,hkv,nodes,batch,max_len,vocab,called,captured", [
+    (32, 8, 60, 1, 2176, 128256, "one", "scan first"),       # 16 CTAs to a range, nine ranges: 144 of 148 SMs
+    (64, 8, 24, 1, 2176, 128256, "one", "scan first"),       # few rows of a large vocabulary
+    (32, 8, 40, 2, 2176, 50257, "one", "scan first"),
+    (52, 52, 60, 1, 1100, 50257, "one", "one"),              # 104 SMs, the scan does not go first
+    (32, 8, 60, 1, 2176, 32768, "fork", "fork"),             # below the line
+    (32, 8, 24, 9, 1024, 128256, "fork", "fork"),            # walks (clusters of ten) on more than half of the SMs
+    (32, 8, 12, 5, 2176, 50257, "fork", "fork"),             # small trees: below their line
+])
+def test_order_behind_larger_scans(lib, hq, hkv, nodes, batch, max_len, vocab, called, captured):
+    """A sampled step with a short attention: one stream from a number of logits on, captured only where the scan would not go first
+    of two streams; the scan goes by the trees or not by a line of its own.  The attention's cut is the same either way."""
+    sms = set()
+    for on, want in ((0, called), (1, captured)):
+        step = Step(lib, hq, hkv, nodes, batch, vocab, max_len, True)
+        lib.fake_capture(on)
+        try:
+            rc, log = step.device(0x1000)
+        finally:
+            lib.fake_capture(0)
+        assert rc == 0
+        sms.add(_field(log, "attention", "sms"))
+        order = [x.split()[0] for x in log]
+        events = [x for x in order if x in ("event_record", "stream_wait")]
+        if want == "one":
+            assert not events and order[:3] == ["scan", "walk", "attention"] and _field(log, "attention", "early") == "1"
+        else:
+            assert len(events) == 4 and _field(log, "attention", "early") == "0"
+            if want == "scan first":
+                assert order[:3] == ["scan", "event_record", "stream_wait"] and order[3] == "walk"
     assert len(sms) == 1
 
 
