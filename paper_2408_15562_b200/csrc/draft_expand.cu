@@ -54,16 +54,42 @@ struct DraftShared {
     float joint[FSPAD_MAX_FRONTIER * FSPAD_MAX_FRONTIER];
     float bound;
     int cnt, n, hits, last;
+    uint32_t lowest;
 };
 
-// The list cut to its k largest keys (a list of more than kKeep: ascending or constant values).  The k-th largest key is
-// found bit by bit: 64 counts, whatever the list holds.
-__device__ __noinline__ void cut_list(DraftShared &s, int k, int tid)
+// The list cut to its k largest keys (a long list: ascending or constant values).  The k-th largest key is found bit by bit, a count
+// of the list to a bit (0.6 us).  Tokens are below V: a key's low word has the bits above those of V - 1 set, whatever the token.  equal:
+// the list was cut by a bound before, so what makes it long are keys of one value as a rule, its lowest, and the values' bits need no search.
+// Constant rows, ten of 32000 tokens, 64 bits searched behind nothing / 64 behind a warp's bound / this: 42, 55 and 32 us.
+__device__ __noinline__ void cut_list(DraftShared &s, int k, int V, bool equal, int tid)
 {
-    const int n = s.cnt;
+    const int n = s.cnt, token_bits = 32 - __clz((V - 1) | 1);
     unsigned long long t = 0ull;
-    for (int bit = 63; bit >= 0; --bit) {
+    int bit = 63;
+    if (equal) {
+        if (tid == 0) { s.lowest = 0xffffffffu; s.hits = 0; }
+        __syncthreads();
+        uint32_t low = 0xffffffffu;
+        for (int i = tid; i < n; i += kThreads) low = min(low, (uint32_t)(s.list[i] >> 32));
+        atomicMin(&s.lowest, low);
+        __syncthreads();
+        low = s.lowest;
+        int above = 0;
+        for (int i = tid; i < n; i += kThreads) above += (uint32_t)(s.list[i] >> 32) > low ? 1 : 0;
+        if (above) atomicAdd(&s.hits, above);
+        __syncthreads();
+        if (s.hits < k) {
+            t = (unsigned long long)low << 32;
+            bit = 31;
+        }
+        __syncthreads();
+    }
+    for (; bit >= 0; --bit) {
         const unsigned long long with = t | (1ull << bit);
+        if (bit < 32 && bit >= token_bits) {
+            t = with;
+            continue;
+        }
         int c = 0;
         for (int i = tid; i < n; i += kThreads) c += s.list[i] >= with ? 1 : 0;
         if (tid == 0) s.hits = 0;
@@ -218,7 +244,7 @@ draft_expand_kernel(const DraftArgs a)
             __syncthreads();
             push(e0);
             __syncthreads();
-            if (s.cnt > kKeep) cut_list(s, k, tid);
+            if (s.cnt > kKeep) cut_list(s, k, V, false, tid);
         }
     } else if (s.cnt > kShort) {                                 // cut it here only if a warp would be long about it: many equal values
         const int n = s.cnt;
@@ -228,7 +254,7 @@ draft_expand_kernel(const DraftArgs a)
             if (lane == 0) s.cnt = m;
         }
         __syncthreads();
-        if (s.cnt > kShort) cut_list(s, k, tid);
+        if (s.cnt > kShort) cut_list(s, k, V, true, tid);
     }
     __syncthreads();
     // ---- the piece's list, and whether it is the sequence's last: one warp ----

@@ -181,3 +181,24 @@ def test_lengths_of_a_piece_s_list(more, values, k, width):
     flp = (-rng.random((B, F)) * 4).astype(np.float32)
     fc = rng.integers(-1, 50, size=(B, F)).astype(np.int32)
     _check(ctx, lp, flp, fc, k, width, 0, F * k)
+
+
+@pytest.mark.parametrize("vocab", [4096, 4097, 16385, 32000])
+@pytest.mark.parametrize("above", [0, 9, 15, 16, 20, 40])
+@pytest.mark.parametrize("k", [10, 16])
+def test_many_equal_values(vocab, above, k):
+    """Rows of one value, with a few tokens above it (of one value, or of two): what a warp's bound does not shorten is cut by a search
+    over tokens alone where fewer than k lie above the lowest value, by values and tokens elsewhere."""
+    F, B = 10, 3
+    ctx = binding.Context(8, 2, vocab, 256, max_nodes=64, max_batch=B)
+    rng = np.random.default_rng(vocab + above)
+    lp = np.full((B, F, vocab), -9.0, np.float32)
+    for b in range(B):
+        for f in range(F):
+            at = rng.choice(vocab, above, replace=False)
+            lp[b, f, at] = -8.0
+            if f % 2:
+                lp[b, f, at[:above // 3]] = -7.5
+    flp = (-rng.random((B, F)) * 4).astype(np.float32)
+    fc = rng.integers(-1, 50, size=(B, F)).astype(np.int32)
+    _check(ctx, lp, flp, fc, k, k, 0, F * k)
