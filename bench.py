@@ -210,10 +210,13 @@ def main():
     L_mean = float(inp.prefix_len.mean())
     n_layers = w.n_layers
     step_bytes = algorithmic_bytes(w, L_mean, 0)
+    inner_rows = sum(len(set(p[1:].tolist()) | {0}) for p in inp.parent)       # rows of nodes with children, and of the roots
+    inner_bytes = 4 * w.vocab * inner_rows
     # Bytes each timed function is sure to read per call (the walk reads only the draft rows of the realised
-    # path, so draft rows are not counted): the rotation is sized for the function that touches the least.
-    touched = {"step": step_bytes["attention"] + step_bytes["accept_logits"], "tree_attn": step_bytes["attention"],
-               "tree_accept": step_bytes["accept_logits"], "accept_stats_kernel": step_bytes["accept_logits"]}
+    # path, and a scan that goes by the trees only the rows of nodes with children, so the others are not counted): the
+    # rotation is sized for the function that touches the least.
+    touched = {"step": step_bytes["attention"] + inner_bytes, "tree_attn": step_bytes["attention"],
+               "tree_accept": inner_bytes, "accept_stats_kernel": step_bytes["accept_logits"]}
     cache_host = synth.make_cache(inp, n_layers)
     set_bytes = cache_host.nbytes + 2 * inp.q.nbytes + 2 * inp.tree_k.nbytes + inp.target_logits.nbytes * \
         (2 if inp.draft_probs is not None else 1)
@@ -468,7 +471,7 @@ def main():
     h2d = sum(t.numel() * t.element_size() for t in (hq, htk, htv, hpar, hpre, htok, htemp) if t is not None)
     # page-locked logits and draft rows are read where they are: of the logits the rows of nodes with children (and of a walk that ends
     # in another node that one, and a logit and a draft probability of every node, which are not counted, nor are the few draft rows)
-    h2d += sum(len(set(p[1:].tolist()) | {0}) for p in inp.parent) * w.vocab * 4
+    h2d += inner_bytes
     h2d += hun.numel() * hun.element_size() if hun is not None else 0
     d2h = sum(t.numel() * t.element_size() for t in (hout, hpath, hn, hb, hl))
 
@@ -483,15 +486,16 @@ def main():
         bytes_real = algorithmic_bytes(w, L_mean, float(n_acc_host.mean()))
         stats_bytes = bytes_real["accept_logits"]
         step_all = bytes_real["attention"] + bytes_real["accept_all_rows"] + bytes_real["compaction"]
+        step_needed = bytes_real["attention"] + inner_bytes + bytes_real["compaction"]
         achieved = stats_bytes / (stats_us * 1e-6) / 1e9
         traffic, traffic_note = recorded_traffic("accept_stats_kernel", w.name)
         cfg = workload_config(w, n_layers, L_mean)
         cfg.update({"launch": "K calls of fspad_verify_step captured in one CUDA graph; %d replays timed one by one, "
                               "value = median" % REPLAYS,
                     "l2": "inputs rotated over %d sets; bytes touched before a set is reused: step %.0f MB, tree_attn %.0f MB, "
-                          "tree_accept and the scan kernel alone %.0f MB (L2: %.0f MB); L2 flushed between replays"
-                          % (R, R * touched["step"] / 1e6, R * touched["tree_attn"] / 1e6,
-                             R * touched["tree_accept"] / 1e6, L2_BYTES / 1e6),
+                          "tree_accept %.0f MB, the scan kernel alone %.0f MB (L2: %.0f MB); L2 flushed between replays"
+                          % (R, R * touched["step"] / 1e6, R * touched["tree_attn"] / 1e6, R * touched["tree_accept"] / 1e6,
+                             R * touched["accept_stats_kernel"] / 1e6, L2_BYTES / 1e6),
                     "multi_gpu": "independent replicas, no collective"})
         line = {
             "metric": METRIC, "value": step_us, "value_median": step_us, "value_min": step_min, "replays": REPLAYS,
@@ -501,8 +505,9 @@ def main():
             "config": cfg,
             "steps_per_s_all_gpus": dist_util.aggregate_replicas(step_us, world),
             "step_hbm_gbs_all_rows_definition": step_all / (step_us * 1e-6) / 1e9,
-            "step_frac_of_hbm_peak": step_all / (step_us * 1e-6) / 1e9 / peak,
             "step_algorithmic_bytes": step_all,
+            "step_bytes_needed": step_needed,         # of the logits the rows of nodes with children alone, no draft rows
+            "step_frac_of_hbm_peak": step_needed / (step_us * 1e-6) / 1e9 / peak,
             "breakdown_us": {"three_calls_on_one_stream": three_us, "three_calls_on_one_stream_min": three_min,
                              "tree_attn": attn_us, "tree_attn_min": attn_min, "tree_accept": accept_us,
                              "tree_accept_min": accept_min, "kv_compact_warm_l2": compact_us, "kv_append_warm_l2": append_us,
@@ -514,7 +519,9 @@ def main():
             "roofline": {"kernel": "accept_stats_kernel", "bound": "hbm", "achieved": achieved, "peak": peak,
                          "peak_kind": "%s copy bandwidth (burst, kernel timed alone)" % peak_kind, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "traffic_note": traffic_note,
-                         "algorithmic_bytes_per_launch": stats_bytes, "launch_us_median": stats_us, "launch_us_min": stats_min},
+                         "algorithmic_bytes_per_launch": stats_bytes, "launch_us_median": stats_us, "launch_us_min": stats_min,
+                         "note": "the scan of all rows, alone; a step or an acceptance of large arrays scans the rows of nodes with "
+                                 "children only (accept_stats_inner_kernel, which has no entry of its own: profiles/)"},
             "tree_attn_call": attention_report(w, L_mean, attn_us, bytes_real["attention"], peak),
             "tree_build_call": {"us": tree_build_us, "candidates_per_sequence": int(cpa.shape[1]), "n_nodes": N,
                                 "batch": B, "bit_exact_vs_oracle": tree_build_ok,

@@ -284,7 +284,7 @@ def test_rows_that_shared_memory_does_not_hold(vocab, nodes):
     assert at_leaf > 0
 
 
-@pytest.mark.parametrize("nodes,batch,vocab", [(60, 1, 65536), (130, 3, 32001), (24, 2, 128256)])
+@pytest.mark.parametrize("nodes,batch,vocab", [(60, 1, 65536), (130, 3, 32001), (32, 2, 128256), (9, 1, 50257)])      # (the last in one stream)
 def test_greedy_step_whose_clusters_compact(nodes, batch, vocab):
     """All sequences greedy, few slices: the CTAs that share a leaf's row share the moves of the cache rows, too."""
     w = synth.scaled(W["llama3_8b_2k"], batch=batch, prefix=(300, 500), n_nodes=nodes, depth=5, branch=8 if nodes <= 64 else 16, vocab=vocab,
