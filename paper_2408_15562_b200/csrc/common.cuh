@@ -194,11 +194,12 @@ static inline FspadStatsGeom fspad_stats_geom_inner(int sm_count, int rows, int 
 // the trees: of up to 11 nodes half and more have children, of 60 a fifth.  The lines, in thousands of logits, lie where trees of branching two
 // to ten were no slower (acceptance, or step of 8 KV heads and 1 K to 2 K keys; us from a graph, all rows and by the trees):
 //   sampled, a step   40 x 32000 twice 31.1 and 28.6, 24 x 50257 four times 33.4 and 31.4, 24 x 32000 twice 23.4 and 25.0; 8 x 128256 eight times 39.3 and 35.8
-//   sampled, alone    40 x 50257 twice 23.9 and 22.9, 24 x 32000 eight times 26.7 and 26.7, 16 x 32000 eight times 21.3 and 21.9; 8 x 32000 16 times 26.6 and 29.3
+//   sampled, alone    40 x 32000 four times 31.4 and 29.7, 130 x 32000 21.9 and 24.7, 24 x 32000 eight times 26.7 and 26.7, 16 x 32000 eight times 21.3 and 21.9; 8 x 32000 16 times 26.6 and 29.3
 //   greedy, a step    40 x 32000 twice 21.6 and 19.2, 24 x 32000 eight times 31.2 and 31.2; 16 x 50257 eight times 29.5 and 31.0, 8 x 50257 16 times 34.5 and 38.0
 //   greedy, alone     40 x 32000 four times 11.0 and 10.3, 24 x 50257 eight times 13.0 and 11.6, 60 x 50257 twice 8.9 and 10.2; 16 x 32000 16 times 11.0 and 11.6
 // Rows whose length is no multiple of four are always cut at the rows by the scan of all of them, which makes it the faster one of small
-// arrays.  Where the CTAs are the pieces nothing is numbered: 24 x 128256, 32 x 128256 (16 nodes twice) in a sampled step 24.4 and 23.7, 28.2 and 24.8.
+// arrays.  Where the CTAs are the pieces nothing is numbered: 24 x 128256, 32 x 128256 (16 nodes twice) in a sampled step 24.4 and 23.7, 28.2 and 24.8
+// (alone 17.5 and 18.5, 22.6 and 22.1).
 // What the kernel finds is not known here: a tree most of whose nodes have children (a chain) gains nothing from it.  Chains of 40 to 60
 // nodes: acceptance alone 22.0 and 24.2 (60 x 128256 sampled), 12.3 and 12.3 (greedy), 17.5 and 20.5 at worst (40 x 50257 eight times, greedy);
 // steps level to 7 % longer.
@@ -213,10 +214,11 @@ static inline bool fspad_scan_inner(int sm_count, int rows, int nodes, int V, bo
     if (rows * 16 < sm_count && V > 16 * 4 * (FSPAD_STATS_THREADS / 2)) return true;
     const bool odd = V % 4 != 0, one_wave = rows * 16 <= sm_count * (1024 / FSPAD_STATS_THREADS);
     int line;                                    // thousands of logits
-    if (may_sample) line = alone ? nodes >= 24 ? 4000 : nodes >= 12 ? 6000 : 8000 : nodes >= 32 ? 2500 : nodes >= 12 ? 4000 : 8000;
+    if (may_sample) line = alone ? nodes >= 24 ? 4400 : nodes >= 12 ? 6000 : 8000 : nodes >= 32 ? 2500 : nodes >= 12 ? 4000 : 8000;
     else if (alone) line = nodes >= 32 ? odd ? 9500 : 5000 : nodes >= 12 ? 9500 : 25000;
     else line = nodes >= 32 ? odd ? 4000 : 2500 : nodes >= 12 && !odd ? 6000 : 16000;
-    if (one_wave && (may_sample || !alone)) line = !may_sample ? 4000 : alone ? 2000 : 1500;
+    const int few = may_sample && !alone ? 1500 : 4000;
+    if (one_wave && (may_sample || !alone) && few < line) line = few;
     return (long long)rows * V >= 1000ll * line;
 }
 

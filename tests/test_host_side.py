@@ -230,7 +230,7 @@ def test_logits_of_chains_are_copied(lib, nodes, batch, vocab, chains, in_place)
     (True, 9, 1, 8192, False, False), (True, 9, 1, 8193, True, True), (False, 3, 3, 32000, True, True), (False, 5, 2, 32000, False, False),
     (True, 40, 2, 31000, False, False), (True, 40, 2, 32000, False, True), (True, 24, 6, 32000, True, True), (True, 24, 5, 32000, False, False),
     (True, 16, 8, 46000, False, True), (True, 16, 8, 47000, True, True), (True, 8, 20, 49000, False, False), (True, 8, 20, 50000, True, True),
-    (True, 24, 1, 62000, False, False), (True, 24, 1, 64000, False, True), (True, 24, 1, 84000, True, True),            # one wave of pieces
+    (True, 24, 1, 62000, False, False), (True, 24, 1, 64000, False, True), (True, 24, 1, 84000, False, True), (True, 32, 1, 128256, True, True),            # one wave of pieces
     (False, 40, 2, 31000, False, False), (False, 40, 2, 32000, False, True), (False, 40, 4, 32000, True, True),
     (False, 40, 2, 32001, False, False), (False, 40, 2, 50257, False, True), (False, 40, 4, 59001, False, True), (False, 40, 4, 60001, True, True),
     (False, 24, 7, 32000, False, False), (False, 24, 8, 32000, False, True), (False, 24, 8, 32001, False, False), (False, 24, 9, 45000, True, True),
