@@ -59,6 +59,15 @@ const void *mapped_whole(const void *p, size_t bytes)
     return first >= lo && first - lo <= size && size - (first - lo) >= bytes ? at.devicePointer : nullptr;
 }
 
+// Whether the host can look at p: a caller's mistake (a device array for a host one) is the copy's to report.
+bool on_host(const void *p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type != cudaMemoryTypeDevice;
+    (void)cudaGetLastError();
+    return true;
+}
+
 // Rows [batch][nodes] of the nodes that have children, and of the roots: what the scan by the trees reads.
 int rows_with_children(const int32_t *parent, int nodes, int batch)
 {
@@ -727,12 +736,12 @@ int fspad_verify_step_host(fspad_ctx *ctx, fspad_bf16 *cache, const fspad_bf16 *
     // are looked at here for that alone: if the stream has yet to bring them, what they hold now decides which way the logits go, and
     // nothing else.
     const float *far_logits = nullptr;
-    if (fspad_scan_inner_fits(ctx->sm_count, batch * n_nodes, c.vocab)) {
-        const double inner = rows_with_children(parent, n_nodes, batch), row_bytes = (double)c.vocab * sizeof(float);
-        if (inner * (1.106 * row_bytes + 4700.0) < (double)lg_bytes + (draft_probs ? 660e3 : 100e3))
-            far_logits = static_cast<const float *>(mapped_whole(target_logits, lg_bytes));
-    }
+    if (fspad_scan_inner_fits(ctx->sm_count, batch * n_nodes, c.vocab)) far_logits = static_cast<const float *>(mapped_whole(target_logits, lg_bytes));
     if (misaligned(far_logits)) far_logits = nullptr;
+    if (far_logits && on_host(parent)) {
+        const double inner = rows_with_children(parent, n_nodes, batch), row_bytes = (double)c.vocab * sizeof(float);
+        if (inner * (1.106 * row_bytes + 4700.0) >= (double)lg_bytes + (draft_probs ? 660e3 : 100e3)) far_logits = nullptr;
+    }
     h2d(ctx->h_prefix, prefix_len, B * sizeof(int));
     h2d(ctx->h_parent, parent, B * N * sizeof(int));
     h2d(ctx->h_tk, tree_k, t_bytes);

@@ -18,6 +18,7 @@ std::string g_log;
 std::map<std::string, int> g_fail;                       // name -> calls until one fails
 struct Range { const char *lo; size_t bytes; };
 std::vector<Range> g_pinned;
+const void *g_device = nullptr;                          // a pointer that is said to be the device's
 const int kSms = 148;
 bool g_capturing = false;
 
@@ -46,7 +47,8 @@ unsigned id(const void *p) { return (unsigned)(uintptr_t)p; }
 extern "C" {
 
 const char *fake_log() { return g_log.c_str(); }
-void fake_reset() { g_log.clear(); g_fail.clear(); g_pinned.clear(); }
+void fake_reset() { g_log.clear(); g_fail.clear(); g_pinned.clear(); g_device = nullptr; }
+void fake_device(const void *p) { g_device = p; }
 void fake_capture(int on) { g_capturing = on != 0; }
 void fake_fail(const char *name, int nth) { g_fail[name] = nth; }
 void fake_pin(const void *p, size_t bytes) { g_pinned.push_back({(const char *)p, bytes}); }
@@ -80,7 +82,7 @@ cudaError_t cudaMemsetAsync(void *, int, size_t, cudaStream_t) { return cudaSucc
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p)
 {
     const bool in = pinned(p) != nullptr;
-    a->type = in ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
+    a->type = p == g_device ? cudaMemoryTypeDevice : in ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
     a->devicePointer = in ? const_cast<void *>(p) : nullptr;
     a->hostPointer = const_cast<void *>(p);
     return cudaSuccess;

@@ -34,6 +34,7 @@ def lib(tmp_path_factory):
     lib.fake_log.restype = ctypes.c_char_p
     lib.fake_fail.argtypes = [ctypes.c_char_p, ci]
     lib.fake_pin.argtypes = [vp, ctypes.c_size_t]
+    lib.fake_device.argtypes = [vp]
     return lib
 
 
@@ -55,11 +56,11 @@ class Step:
     def __del__(self):
         self.lib.fspad_destroy(self.ctx)
 
-    def host(self):
+    def host(self, parent=None):
         big = 0x1000                                     # never dereferenced by the stand-ins
-        p = self.small.ctypes.data
+        p, parent = self.small.ctypes.data, parent or self.parent.ctypes.data
         draft, unif = (self.draft.ctypes.data, p) if self.sampling else (None, None)
-        rc = self.lib.fspad_verify_step_host(self.ctx, big, big, big, big, self.parent.ctypes.data, big, big, draft, big, big, unif, self.n, self.batch,
+        rc = self.lib.fspad_verify_step_host(self.ctx, big, big, big, big, parent, big, big, draft, big, big, unif, self.n, self.batch,
                                              big, p, p, p, p, STREAM)
         return rc, self.lib.fake_log().decode().splitlines()
 
@@ -223,6 +224,16 @@ def test_logits_of_chains_are_copied(lib, nodes, batch, vocab, chains, in_place)
         rc, log = step.host()
         copied = any(x.startswith("h2d host=1000 bytes=%d " % bytes_) for x in log)
         assert rc == 0 and copied != in_place and _field(log, "scan", "staged") == str(int(in_place))
+
+
+def test_a_device_array_for_the_trees_is_left_to_the_copy(lib):
+    """The host entry looks at the trees only where the host can: a device array given for them is the copy's error, as it was."""
+    step = Step(lib, nodes=60, vocab=128256, sampling=False)
+    lib.fake_pin(0x1000, 60 * 128256 * 4)
+    lib.fake_device(0x5000)
+    lib.fake_fail(b"h2d", 2)                             # (what the runtime says to it)
+    rc, log = step.host(parent=0x5000)
+    assert rc == -6 and any(x.startswith("h2d host=5000 ") for x in log)
 
 
 # just below and on the line from which the scan goes by the trees: alone, in a step
